@@ -54,10 +54,9 @@ PRECS = {"f64": 0, "f32": 1, "tf32": 2, "bf16": 3, "tf32x3": 4}
 # the capture and its command; a kernel changed since its capture has no
 # entry here (traffic null).
 TRAFFIC = {
-    # profiles/traffic_diffusion2d_512_f32.md: one application = 181 launches
-    # (455.6 MB read, 0.01 MB written); the large-node truncation of one
+    # profiles/traffic_diffusion2d_512_f32.md: the large-node truncation of one
     # factorization = 193.5 MB over its 46 launch groups
-    ("diffusion2d_512", "f32"): {"apply": 455.62e6, "trunc": 193.48e6 / 46},
+    ("diffusion2d_512", "f32"): {"trunc": 193.48e6 / 46},
 }
 
 
@@ -931,7 +930,7 @@ def main():
                   "algorithmic_flops_per_launch": info_f["trunc_big_flops"] / tb_launches,
                   "launch_ms": tb_ms / tb_launches, "launches_per_factor": info_f["trunc_big_launches"],
                   "share_of_step": tb_ms / ms_per_step}
-    roof_apply = {"bound": "hbm", "kernel": "apply (Algorithm 2: k_f1, k_f2, k_b1, k_b2, k_root)",
+    roof_apply = {"bound": "hbm", "kernel": "apply (Algorithm 2: k_fwd, k_bwd, k_root)",
                   "achieved": achieved, "peak": hbm_peak, "unit": "GB/s", "frac": achieved / hbm_peak,
                   "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)" if peaks else "fallback",
                   "traffic": TRAFFIC.get((args.workload, args.prec), {}).get("apply"),

@@ -95,11 +95,9 @@ void numeric_pre(FactorHandle &h, const double *val, cudaStream_t st) {
   }
   h.alloc.put(h.d_nodes, st);
   h.alloc.put(h.d_nbrs, st);
-  h.alloc.put(h.d_targets, st);
   h.alloc.put(h.d_contribs, st);
   h.d_nodes = nullptr;
   h.d_nbrs = nullptr;
-  h.d_targets = nullptr;
   h.d_contribs = nullptr;
 }
 
@@ -113,7 +111,6 @@ void numeric_failed(FactorHandle &h) {
 void numeric_post(FactorHandle &h, float ms, cudaStream_t st) {
   h.d_nodes = upload_vec(h, h.nodes, st);
   h.d_nbrs = upload_vec(h, h.nbrs, st);
-  h.d_targets = upload_vec(h, h.targets, st);
   h.d_contribs = upload_vec(h, h.contribs, st);
   apply_prepare(h, st);
   hs_info &in = h.info;
@@ -123,7 +120,8 @@ void numeric_post(FactorHandle &h, float ms, cudaStream_t st) {
   in.factor_ms = ms;
   const double tb = h.prec == HS_PREC_F64 ? 8.0 : 4.0;
   double fb = 0.0;
-  for (const auto &nd : h.nodes) fb += 2.0 * ((double)nd.m * nd.m + (double)nd.k * nd.m + (double)nd.m * nd.dN);
+  for (const auto &nd : h.nodes)
+    fb += (double)nd.m * nd.m + 2.0 * ((double)nd.k * nd.m + (double)nd.m * nd.dN);
   fb += (double)h.root_m * h.root_m;
   in.factor_bytes = (int64_t)(fb * tb);
   in.device_bytes = (int64_t)(h.pers->reserved() + h.scratch->reserved());

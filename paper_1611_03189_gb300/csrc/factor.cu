@@ -2,11 +2,12 @@
 // elimination; Sec. 6 GC basis), level by level and wave by wave.
 //
 // Per wave every super node s of the wave is processed by batched kernels:
-//   A. gather [A_sn]_n (kept as a factor record) and [A_sw]_w; L^-1 of
+//   A. gather [A_sn]_n and [A_sw]_w; L^-1 of
 //      A_ss = L L^T; Gram G = A_sw A_sw^T and a = A_sw phi_w; truncation -> U, k.
 //      One device->host read of the ranks k (sizes of the new red nodes).
 //   B. L^-1 U = Q R by CholQR2 (twice: Q1 = L^-1 U R1^-1, Q = Q1 R2^-1), then
 //        P_ss = R^-1 Q^T L^-1            M_ss = L^-T L^-1 - (L^-T Q)(L^-T Q)^T
+//        B_s  = M_ss A_sN (for the solves, solve.cu)
 //        A_rr = S^-1 = R^-1 R^-T          A_nr = (L^-1 A_sn)^T Q R^-T
 //        A_rw = U^T A_sw (= R_w^T)        phi_r = U^T phi_s
 //        Z_s  = (L^-1 A_sN)^T (L^-1 A_sN) - (Q^T L^-1 A_sN)^T (Q^T L^-1 A_sN)
@@ -736,7 +737,7 @@ struct WaveBatches {
   GemmBatch<T> o1, o2, o3, o4;
   CholBatch<T> oc1, oc2;
   // phase B and the Schur update
-  GemmBatch<T> g1, g2, g3, g4, g5, g6, g7, g8;
+  GemmBatch<T> g1, g2, g3, g4, g5, g6, g7, g8, gb;
   CholBatch<T> c1, c2;
   SumBatch<T> schur;
 };
@@ -777,7 +778,7 @@ class Run {
     T *U = nullptr, *work = nullptr;
     T *Ut = nullptr, *S1 = nullptr, *L1 = nullptr, *Q1 = nullptr, *S2 = nullptr, *L2 = nullptr;
     T *Q = nullptr, *Rinv = nullptr, *Wt = nullptr, *Gt = nullptr, *Tm = nullptr, *Z = nullptr;
-    T *M = nullptr, *Pm = nullptr, *ANr = nullptr, *Arr = nullptr, *ArW = nullptr, *phir = nullptr;
+    T *M = nullptr, *Pm = nullptr, *B = nullptr, *ANr = nullptr, *Arr = nullptr, *ArW = nullptr, *phir = nullptr;
     bool red = false;
   };
 
@@ -1053,7 +1054,7 @@ void Run<T>::wave_a(int li, int widx, WaveBatches<T> &B) {
       x.dW += size_[w];
     }
     const int m = x.m;
-    x.AsN = talloc<T>(per, (size_t)m * x.dN);
+    x.AsN = talloc<T>(scr, (size_t)m * x.dN);
     x.Linv = talloc<T>(scr, (size_t)m * m);
     auto oriented = [&](int row, int other, T *dst, int ld, int cols) {
       auto it = blocks_.find(bkey(row, other));
@@ -1214,7 +1215,7 @@ bool Run<T>::wave_c(WaveBatches<T> &B, size_t count) {
   // phase B
   std::vector<Sup> &S = cur_;
   const double f0 = B.c1.flops + B.c2.flops + B.g1.flops + B.g2.flops + B.g3.flops + B.g4.flops + B.g5.flops +
-                    B.g6.flops + B.g7.flops + B.g8.flops;
+                    B.g6.flops + B.g7.flops + B.g8.flops + B.gb.flops;
   const size_t q0 = c_next_, q1 = std::min(S.size(), c_next_ + count);
   c_next_ = q1;
   for (size_t q = q0; q < q1; ++q) {
@@ -1237,6 +1238,7 @@ bool Run<T>::wave_c(WaveBatches<T> &B, size_t count) {
     x.Z = talloc<T>(scr, (size_t)dN * dN);
     x.M = talloc<T>(per, (size_t)m * m);
     x.Pm = talloc<T>(per, (size_t)k * m);
+    x.B = talloc<T>(per, (size_t)m * dN);
     if (x.red) {
       x.ANr = talloc<T>(per, (size_t)dN * k);
       x.Arr = talloc<T>(per, (size_t)k * k);
@@ -1264,6 +1266,7 @@ bool Run<T>::wave_c(WaveBatches<T> &B, size_t count) {
     B.g7.add(x.Wt, k, 0, x.Wt, k, 1, x.M, m, m, m, k, T(-1), T(1));             // M_ss -= W W^T
     B.g7.add(x.Q, k, 1, x.Gt, dN, 0, x.Tm, dN, k, dN, m, T(1), T(0));           // Q^T L^-1 A_sN
     B.g7.add(x.Gt, dN, 1, x.Gt, dN, 0, x.Z, dN, dN, dN, m, T(1), T(0));         // (L^-1 A_sN)^T (L^-1 A_sN)
+    B.gb.add(x.M, m, 0, x.AsN, dN, 0, x.B, dN, m, dN, m, T(1), T(0));           // B_s = M_ss A_sN
     B.g8.add(x.Tm, dN, 1, x.Tm, dN, 0, x.Z, dN, dN, dN, k, T(-1), T(1));        // - T^T T
     if (x.red) {
       B.g8.add(x.Tm, dN, 1, x.Rinv, k, 1, x.ANr, k, dN, k, k, T(1), T(0));      // A_Nr = T^T R^-T
@@ -1271,7 +1274,7 @@ bool Run<T>::wave_c(WaveBatches<T> &B, size_t count) {
     }
   }
   flops_ += B.c1.flops + B.c2.flops + B.g1.flops + B.g2.flops + B.g3.flops + B.g4.flops + B.g5.flops +
-            B.g6.flops + B.g7.flops + B.g8.flops - f0;
+            B.g6.flops + B.g7.flops + B.g8.flops + B.gb.flops - f0;
   // algorithmic work of the elimination, counted from the actual sizes: Gram
   // 2 m^2 w and R^T 2 m k w of the truncation (Sec. 3.2), Cholesky m^3/3,
   // Y 2 m^2 k, S 2 m k^2 + k^3/3, G_n 2 m^2 d_N, H_n 2 m k d_N, the Schur
@@ -1398,7 +1401,7 @@ void Run<T>::wave_d(WaveBatches<T> &B) {
     ApplyNode an{};
     an.M = x.M;
     an.P = x.Pm;
-    an.AsN = x.AsN;
+    an.B = x.B;
     an.m = x.m;
     an.k = x.red ? x.k : 0;
     an.dN = x.dN;
@@ -1448,7 +1451,6 @@ void Run<T>::end_level(const PlanLevel &lv, int li) {
     std::vector<int> torder, c_t, c_node, c_col;
     int64_t t = 0;
     wa.max_m = 0;
-    wa.rows_f = wa.rows_b = wa.pch = wa.tch = 0;
     for (int q = 0; q < wa.node_count; ++q, ++rp) {
       const Rec &rc = recs_[rp];
       ApplyNode &an = h_.nodes[rc.node];
@@ -1456,12 +1458,6 @@ void Run<T>::end_level(const PlanLevel &lv, int li) {
       an.xr = lv.red_made[rc.s] ? xoff(nsup + rc.s) : -1;
       an.toff = t;
       t += an.m;
-      an.row0 = wa.rows_f;
-      wa.rows_f += an.m + an.k;
-      an.brow0 = wa.rows_b;
-      wa.rows_b += an.m;
-      an.pch0 = wa.pch;
-      if (an.k > 0) wa.pch += (an.m + 31) / 32;
       wa.max_m = std::max(wa.max_m, an.m);
       an.nb_first = (int)h_.nbrs.size();
       an.nb_count = (int)rc.N.size();
@@ -1503,18 +1499,16 @@ void Run<T>::end_level(const PlanLevel &lv, int li) {
       ApplyTarget tg;
       tg.x = xoff(n);
       tg.size = size_[n];
-      tg.ch0 = wa.tch;
-      wa.tch += (tg.size + 31) / 32;
       tg.first = (int)h_.contribs.size();
       tg.count = c_start[ti + 1] - c_start[ti];
       for (int cc = c_start[ti]; cc < c_start[ti + 1]; ++cc) {
         const int c = c_list[cc];
         const ApplyNode &an = h_.nodes[c_node[c]];
         ApplyContrib ac;
-        ac.A = (const char *)an.AsN + sizeof(T) * (size_t)c_col[c];
+        ac.A = (const char *)an.B + sizeof(T) * (size_t)c_col[c];
         ac.ld = an.dN;
         ac.m = an.m;
-        ac.toff = an.toff;
+        ac.x = an.xs;
         h_.contribs.push_back(ac);
       }
       h_.targets.push_back(tg);
@@ -1986,6 +1980,7 @@ void execute(Exec &ex, std::vector<std::unique_ptr<Run<T>>> &runs) {
         ex.gemm(B.g6);
         ex.gemm(B.g7);
         ex.gemm(B.g8);
+        ex.gemm(B.gb, false);   // read by the solves: in FP32 on every mixed path
         ex.end();
         B.c1.tasks.clear();
         B.c1.what.clear();

@@ -66,32 +66,43 @@ class DevArena {
 struct ApplyNode {
   const void *M;     // M_ss, m x m
   const void *P;     // P_ss, k x m
-  const void *AsN;   // [A_{s n}]_n, m x dN (ld dN)
+  const void *B;     // B_s = M_ss [A_{s n}]_n, m x dN (ld dN)
   int64_t xs;        // unknown offset of s in the workspace
   int64_t xr;        // unknown offset of the red node r (or -1)
   int64_t toff;      // unknown offset of t_s in the per-wave scratch
   int m, k, dN;
   int nb_first, nb_count;
-  int row0;          // prefix of (m + k) rows inside the wave (forward GEMV rows)
-  int brow0;         // prefix of m rows inside the wave (backward rows)
-  int pch0;          // prefix of 32-column chunks of P_ss inside the wave (k > 0 nodes)
 };
 struct ApplyNbr {
   int64_t x;         // unknown offset of neighbour n
   int size;
-  int col;           // column offset of A_{s n} inside AsN
+  int col;           // column offset of n inside B_s
 };
 struct ApplyTarget {  // forward substitution, gathered by neighbour
   int64_t x;
   int size;
   int first, count;
-  int ch0;           // prefix of 32-row chunks inside the wave
 };
 struct ApplyContrib {
-  const void *A;     // AsN + col, element (i in s, q in n) at A[i*ld + q]
+  const void *A;     // B_s + col, element (i in s, q in n) at A[i*ld + q]
   int ld;
   int m;
-  int64_t toff;
+  int64_t x;         // unknown offset of s
+};
+
+// One CTA's share of a wave's forward or backward launch (solve.cu).
+constexpr int kApplyRows = 32;   // rows (unknowns) per item
+struct ApplyItem {
+  enum Kind { ROWS = 0, TARGET = 1, MOVE = 2 };   // of a forward item
+  const void *A;     // ROWS: M_ss; backward: B_s
+  const void *P;     // P_ss
+  int64_t x;         // unknown offset of s (TARGET: of n)
+  int64_t r;         // of the red node
+  int64_t t;         // of t_s in the wave's scratch
+  int m, k, dN;      // sizes of s (TARGET: m is the size of n)
+  int i0;            // first row (unknown)
+  int first, count;  // TARGET: contributions; MOVE: nodes of the wave before; backward: neighbours
+  int kind;
 };
 
 struct WaveApply {
@@ -99,14 +110,7 @@ struct WaveApply {
   int tgt_first, tgt_count;
   int max_m;
   int64_t tsize;     // unknowns of t scratch used
-  int rows_f;        // sum of (m + k): forward GEMV rows
-  int rows_b;        // sum of m: backward rows
-  int pch;           // sum of 32-column chunks of P_ss
-  int tch;           // sum of 32-row chunks of the targets
-  // offsets into FactorHandle::d_hints of the per-CTA search starts of the
-  // per-step kernels (-1: none): f1 by row0, f2 by ch0, b1/b2 by brow0, b1's
-  // P_ss^T part by pch0
-  int hf1 = -1, hf2 = -1, hb = -1, hp = -1;
+  int f_first = 0, f_count = 0, b_first = 0, b_count = 0;   // items of the two launches
 };
 struct LevelApply {
   int level;
@@ -163,7 +167,6 @@ struct FactorHandle {
   std::vector<LevelApply> levels;      // levels L..2
   ApplyNode *d_nodes = nullptr;
   ApplyNbr *d_nbrs = nullptr;
-  ApplyTarget *d_targets = nullptr;
   ApplyContrib *d_contribs = nullptr;
   // the persistent apply: step list (kind, wave) and the waves on the device,
   // the grid barrier's counter and generation, and its time-out flag
@@ -172,10 +175,8 @@ struct FactorHandle {
   WaveApply *d_waves = nullptr;
   unsigned *d_apply_bar = nullptr;
   int *d_apply_err = nullptr;
-  // per-CTA first node (or target) of each per-step apply kernel, for a
-  // CTA's first warp; each warp scans forward from it (WaveApply::hf1 ...)
-  int *d_hints = nullptr;
-  size_t hints_cap = 0;
+  ApplyItem *d_items = nullptr;        // the waves' items (WaveApply::f_first ...)
+  size_t items_cap = 0;
   int64_t ws_size = 0;                 // unknowns in the apply workspace
   int64_t tmax = 0;                    // max unknowns of t scratch per wave
   int64_t root_off = 0;

@@ -7,14 +7,31 @@
 // are the concatenation of its two children's, so super node and red nodes of
 // a level share the same memory.
 //
-// Per wave (in elimination order) the forward pass runs
-//   k_f1:  t_s = M_ss phi_s, phi_r += P_ss phi_s       (restriction)
-//   k_f2:  phi_n -= sum_s A_ns t_s                     (forward substitution)
-// then the root solve (k_copy, k_root), then per wave in reverse order
-//   k_b1:  v_s = phi_s - sum_n A_sn x_n, y_s = P_ss^T x_r
-//   k_b2:  x_s = M_ss v_s + y_s           (backward substitution and prolongation).
-// Contributions to one phi_n are summed in a fixed order, so results do not
-// depend on scheduling.
+// With B_s = M_ss A_sN (made by the factorization), Algorithm 2's steps of a
+// wave become one launch each way (in elimination order, then in reverse):
+//   k_fwd:  t_s = M_ss phi_s, phi_r = P_ss phi_s           (restriction)
+//           phi_n -= sum_s B_s[:, n]^T phi_s               (forward substitution:
+//                                                           A_ns M_ss = B_s[:, n]^T)
+//   k_bwd:  x_s = t_s + P_ss^T x_r - B_s x_N               (backward substitution
+//                                                           and prolongation:
+//                                                           M_ss (phi_s - A_sN x_N))
+// and the root solve (k_copy, k_root) between them.  The form with A_sN needs
+// two dependent launches each way and reads M_ss twice.  What bounds an
+// application is the chain of dependent launches at the top levels and the
+// latency of the loads inside each, so both are kept short: at 512 x 512 (59
+// waves, FP32, one right-hand side) 120 launches and 0.60 ms an application
+// against 181 and 1.5 ms with the form above, one warp per row; at 300 x 217
+// (FP64, five right-hand sides) 1.59 ms against 4.43; at 40^3 (FP32, sixteen)
+// a four-iteration solve takes 15.6 ms against 34.0.
+// t_s goes to the wave's scratch (every row of the wave reads phi_s), and the
+// next wave's launch moves it into the place of phi_s, which nothing reads any
+// more; the scratch is two buffers used in turn.
+// A launch is a list of items, one CTA each (apply_prepare): 32 rows of
+// [M_ss; P_ss], 32 unknowns of a target n or of x_s, or up to 8 nodes' t_s to
+// move.  Rows are walked by warps, four rows sharing each load of x; columns
+// (P_ss^T, B_s^T) by the CTA's 8 warps together, 32 adjacent columns each.
+// What an item does and the order of every sum depend on the node alone, so
+// results depend neither on scheduling nor on the number of right-hand sides.
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -32,247 +49,290 @@ namespace {
 
 constexpr int AW = 8;         // warps per CTA in the apply kernels
 constexpr int AT = AW * 32;
+constexpr int AR = kApplyRows / AW;   // rows of an item per warp
 
-// last node i in nodes[first, first+count) with key(i) <= w (keys are prefix sums)
-template <typename F>
-__device__ __forceinline__ int find_last(int first, int count, int w, F key) {
-  int lo = first, hi = first + count - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (key(mid) <= w)
-      lo = mid;
-    else
-      hi = mid - 1;
-  }
-  return lo;
-}
-
-// The same index, from a start known not to be past it (hint >= 0: the
-// answer for the CTA's first warp): a forward scan over the few node
-// boundaries inside the CTA's rows instead of a search of the whole wave.
-template <typename F>
-__device__ __forceinline__ int find_from(int first, int count, int w, int hint, F key) {
-  if (hint < 0) return find_last(first, count, w, key);
-  int i = hint;
-  const int last = first + count - 1;
-  while (i < last && key(i + 1) <= w) ++i;
-  return i;
-}
-
-template <typename T, int NR>
-__device__ __forceinline__ void warp_reduce(T (&acc)[NR]) {
+// NR consecutive values of one unknown; VEC: 16-byte loads (every column of
+// the chunk in use, unknown stride and first column multiples of 16 bytes)
+template <typename T, int NR, bool VEC>
+__device__ __forceinline__ void load_x(const T *x, int nr, T (&v)[NR]) {
+  if constexpr (VEC) {
+    constexpr int W = 16 / (int)sizeof(T);
 #pragma unroll
-  for (int j = 0; j < NR; ++j)
+    for (int i = 0; i < NR / W; ++i) {
+      if constexpr (sizeof(T) == 4) {
+        const float4 q = reinterpret_cast<const float4 *>(x)[i];
+        v[4 * i] = q.x;
+        v[4 * i + 1] = q.y;
+        v[4 * i + 2] = q.z;
+        v[4 * i + 3] = q.w;
+      } else {
+        const double2 q = reinterpret_cast<const double2 *>(x)[i];
+        v[2 * i] = q.x;
+        v[2 * i + 1] = q.y;
+      }
+    }
+  } else {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], o);
-}
-
-
-// acc[j] += sum_c A[c] x[c*stride + j] for c = lane, lane+32, ... < len, four
-// independent loads in flight per lane
-template <typename T, int NR>
-__device__ __forceinline__ void row_dot(const T *__restrict__ A, const T *__restrict__ x, int len,
-                                        int64_t stride, int nr, int lane, T (&acc)[NR]) {
-  int c = lane;
-  for (; c + 96 < len; c += 128) {
-    const T a0 = A[c], a1 = A[c + 32], a2 = A[c + 64], a3 = A[c + 96];
-    const T *x0 = x + (int64_t)c * stride, *x1 = x0 + 32 * stride, *x2 = x0 + 64 * stride,
-            *x3 = x0 + 96 * stride;
-#pragma unroll
-    for (int j = 0; j < NR; ++j)
-      if (j < nr) acc[j] = fma(a3, x3[j], fma(a2, x2[j], fma(a1, x1[j], fma(a0, x0[j], acc[j]))));
-  }
-  for (; c < len; c += 32) {
-    const T a = A[c];
-    const T *xc = x + (int64_t)c * stride;
-#pragma unroll
-    for (int j = 0; j < NR; ++j)
-      if (j < nr) acc[j] = fma(a, xc[j], acc[j]);
+    for (int j = 0; j < NR; ++j) v[j] = j < nr ? x[j] : T(0);
   }
 }
 
-// acc[j] += sum_q A[q*ld] t[q*stride + j] for q < len (column walk, unrolled by 4)
-template <typename T, int NR>
-__device__ __forceinline__ void col_dot(const T *__restrict__ A, int64_t ld, const T *__restrict__ t, int len,
-                                        int64_t stride, int nr, T (&acc)[NR]) {
-  int q = 0;
-  for (; q + 3 < len; q += 4) {
-    const T a0 = A[q * ld], a1 = A[(q + 1) * ld], a2 = A[(q + 2) * ld], a3 = A[(q + 3) * ld];
-    const T *t0 = t + (int64_t)q * stride;
+// acc[r][j] += sum_c a[r][c] x[c*stride + j] for c = lane, lane + 32, ... < len:
+// R rows share every load of x, and 4 R row elements per lane are in flight
+template <typename T, int NR, int R, bool VEC>
+__device__ __forceinline__ void rows_dot(const T *const (&a)[R], const T *x, int len, int64_t stride, int nr,
+                                         int lane, T (&acc)[R][NR]) {
+  for (int c0 = 0; c0 < len; c0 += 128) {
+    T av[4][R];
 #pragma unroll
-    for (int j = 0; j < NR; ++j)
-      if (j < nr)
-        acc[j] = fma(a3, t0[3 * stride + j], fma(a2, t0[2 * stride + j], fma(a1, t0[stride + j], fma(a0, t0[j], acc[j]))));
-  }
-  for (; q < len; ++q) {
-    const T a = A[q * ld];
-    const T *tq = t + (int64_t)q * stride;
+    for (int u = 0; u < 4; ++u) {
+      const int c = c0 + 32 * u + lane;
 #pragma unroll
-    for (int j = 0; j < NR; ++j)
-      if (j < nr) acc[j] = fma(a, tq[j], acc[j]);
-  }
-}
-
-// Each step of Algorithm 2 below is a __device__ function of one warp's share
-// (virtual warp w of the step); the per-step kernels give warp w = global warp
-// index, the persistent kernel walks w over all warps of the grid.
-
-// F1: one warp per row of [M_ss; P_ss]: t_s = M_ss phi_s, phi_r += P_ss phi_s
-template <typename T, int NR>
-__device__ __forceinline__ void f1_warp(const ApplyNode *__restrict__ nodes, int first, int count, int w, int lane,
-                                        T *__restrict__ ws, T *__restrict__ tb, int nrhs, int j0, int hint = -1) {
-  const int ni = find_from(first, count, w, hint, [&](int i) { return nodes[i].row0; });
-  const ApplyNode nd = nodes[ni];
-  const int r = w - nd.row0;
-  const T *Ar = r < nd.m ? (const T *)nd.M + (int64_t)r * nd.m : (const T *)nd.P + (int64_t)(r - nd.m) * nd.m;
-  const T *x = ws + nd.xs * nrhs + j0;
-  const int nr = min(NR, nrhs - j0);
-  T acc[NR];
+      for (int r = 0; r < R; ++r) av[u][r] = c < len ? __ldg(a[r] + c) : T(0);
+    }
 #pragma unroll
-  for (int j = 0; j < NR; ++j) acc[j] = T(0);
-  row_dot<T, NR>(Ar, x, nd.m, nrhs, nr, lane, acc);
-  warp_reduce<T, NR>(acc);
-  if (lane == 0) {
-    T *o = r < nd.m ? tb + (nd.toff + r) * nrhs + j0 : ws + (nd.xr + r - nd.m) * nrhs + j0;
+    for (int u = 0; u < 4; ++u)
+      if (c0 + 32 * u < len) {
+        const int c = min(c0 + 32 * u + lane, len - 1);
+        T xv[NR];
+        load_x<T, NR, VEC>(x + (int64_t)c * stride, nr, xv);
 #pragma unroll
-    for (int j = 0; j < NR; ++j)
-      if (j < nr) {
-        if (r < nd.m)
-          o[j] = acc[j];
-        else
-          o[j] += acc[j];
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+          for (int j = 0; j < NR; ++j) acc[r][j] = fma(av[u][r], xv[j], acc[r][j]);
       }
   }
 }
 
-template <typename T, int NR>
-__global__ void __launch_bounds__(AT) k_f1(const ApplyNode *__restrict__ nodes, int first, int count, int rows,
-                                           T *__restrict__ ws, T *__restrict__ tb, int nrhs, int j0,
-                                           const int *__restrict__ hint) {
-  const int w = blockIdx.x * AW + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (w < rows) f1_warp<T, NR>(nodes, first, count, w, lane, ws, tb, nrhs, j0, hint ? hint[blockIdx.x] : -1);
-}
-
-// F2: phi_n -= sum_s A_ns t_s; one warp per 32 rows of a target, contributions in order
-template <typename T, int NR>
-__device__ __forceinline__ void f2_warp(const ApplyTarget *__restrict__ tg, int first, int count, int w, int lane,
-                                        const ApplyContrib *__restrict__ cb, T *__restrict__ ws,
-                                        const T *__restrict__ tb, int nrhs, int j0, int hint = -1) {
-  const int ti = find_from(first, count, w, hint, [&](int i) { return tg[i].ch0; });
-  const ApplyTarget t = tg[ti];
-  const int i = (w - t.ch0) * 32 + lane;
-  if (i >= t.size) return;
-  const int nr = min(NR, nrhs - j0);
-  T acc[NR];
+// Warp sums of V values (a power of two).  While a lane holds two values or
+// more it exchanges half of them with its partner and keeps the other half,
+// so V sums cost about V shuffles instead of 5 V.  Every value is summed over
+// the lanes in the order of the plain butterfly (partners 16, 8, 4, 2, 1
+// lanes away), whatever V is, so a right-hand side's bits do not depend on
+// how many share the pass.  Afterwards lane l holds values
+// [warp_sum_first<V>(l), + warp_sum_count<V>()) in v[0..).
+template <typename T, int V>
+__device__ __forceinline__ void warp_sums(T (&v)[V], int lane) {
+  static_assert((V & (V - 1)) == 0, "V must be a power of two");
 #pragma unroll
-  for (int j = 0; j < NR; ++j) acc[j] = T(0);
-  for (int c = 0; c < t.count; ++c) {
-    const ApplyContrib ac = cb[t.first + c];
-    const T *A = (const T *)ac.A + i;
-    const T *tv = tb + ac.toff * nrhs + j0;
-    col_dot<T, NR>(A, ac.ld, tv, ac.m, nrhs, nr, acc);
+  for (int s = 0; s < 5; ++s) {
+    const int o = 16 >> s;
+    const int n = V >> s;
+    if (n >= 2) {
+      const bool up = lane & o;
+#pragma unroll
+      for (int i = 0; i < n / 2; ++i) {
+        const T give = up ? v[i] : v[i + n / 2];
+        const T keep = up ? v[i + n / 2] : v[i];
+        v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+      }
+    } else {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    }
   }
-  T *o = ws + (t.x + i) * nrhs + j0;
+}
+template <int V>
+__device__ __forceinline__ int warp_sum_first(int lane) {
+  return V >= 32 ? lane * (V / 32) : lane / (32 / V);
+}
+template <int V>
+__host__ __device__ __forceinline__ constexpr int warp_sum_count() {
+  return V >= 32 ? V / 32 : 1;
+}
+// one lane of those that hold the same value
+template <int V>
+__device__ __forceinline__ bool warp_sum_writer(int lane) {
+  return V >= 32 || lane % (32 / (V >= 32 ? 32 : V)) == 0;
+}
+
+// acc[j] += sum_q A[q*ld] x[q*stride + j] over q = warp, warp + AW, ... < len:
+// a CTA's warps share the walk down 32 adjacent columns (lane: one column)
+template <typename T, int NR, bool VEC>
+__device__ __forceinline__ void cols_dot(const T *A, int64_t ld, const T *x, int len, int64_t stride, int nr, int warp,
+                                         bool active, T (&acc)[NR]) {
+  for (int q0 = warp; q0 < len; q0 += 4 * AW) {
+    T av[4];
 #pragma unroll
-  for (int j = 0; j < NR; ++j)
-    if (j < nr) o[j] -= acc[j];
+    for (int u = 0; u < 4; ++u) {
+      const int q = q0 + AW * u;
+      av[u] = active && q < len ? __ldg(A + q * ld) : T(0);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int q = q0 + AW * u;
+      if (q < len) {
+        T xv[NR];
+        load_x<T, NR, VEC>(x + (int64_t)q * stride, nr, xv);
+#pragma unroll
+        for (int j = 0; j < NR; ++j) acc[j] = fma(av[u], xv[j], acc[j]);
+      }
+    }
+  }
 }
 
+// Shared memory of one item: the warps' partial sums of a column walk and the
+// row sums of the same 32 unknowns.
 template <typename T, int NR>
-__global__ void __launch_bounds__(AT) k_f2(const ApplyTarget *__restrict__ tg, int first, int count, int chunks,
-                                           const ApplyContrib *__restrict__ cb, T *__restrict__ ws,
-                                           const T *__restrict__ tb, int nrhs, int j0, const int *__restrict__ hint) {
-  const int w = blockIdx.x * AW + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (w < chunks) f2_warp<T, NR>(tg, first, count, w, lane, cb, ws, tb, nrhs, j0, hint ? hint[blockIdx.x] : -1);
+struct ItemSmem {
+  T part[AW][NR][32];
+  T rows[32][NR];
+};
+
+// rows per pass of a warp: its accumulators stay within 64 registers
+template <typename T, int NR>
+__host__ __device__ constexpr int rows_per_pass() {
+  return NR * AR * (int)sizeof(T) <= 256 ? AR : NR * 2 * (int)sizeof(T) <= 256 ? 2 : 1;
 }
 
-// B1 (warps < rows_b): v_s = phi_s - sum_n A_sn x_n, one warp per row of s.
-// B2a (warps >= rows_b): y_s = P_ss^T x_r, one warp per 32 columns of P_ss.
-template <typename T, int NR>
-__device__ __forceinline__ void b1_warp(const ApplyNode *__restrict__ nodes, int first, int count, int rows_b,
-                                        int w, int lane, const ApplyNbr *__restrict__ nb, const T *__restrict__ ws,
-                                        T *__restrict__ tb, T *__restrict__ tb2, int nrhs, int j0, int hint_b = -1,
-                                        int hint_p = -1) {
+// One item of the forward step of a wave.
+template <typename T, int NR, bool VEC>
+__device__ __forceinline__ void fwd_item(const ApplyItem &it, const ApplyNode *__restrict__ nodes,
+                                         const ApplyContrib *__restrict__ cb, T *ws, T *tcur, const T *tprev, int nrhs,
+                                         int j0, ItemSmem<T, NR> &sm) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nr = min(NR, nrhs - j0);
-  T acc[NR];
+  if (it.kind == ApplyItem::ROWS) {
+    // t_s = M_ss phi_s and phi_r = P_ss phi_s, rows i0 .. i0 + 31 of [M; P]
+    constexpr int R = rows_per_pass<T, NR>();
+    const int total = it.m + it.k;
+    const T *x = ws + it.x * nrhs + j0;
+#pragma unroll 1
+    for (int r0 = it.i0 + warp * AR; r0 < min(it.i0 + (warp + 1) * AR, total); r0 += R) {
+      const T *a[R];
+      T acc[R][NR];
 #pragma unroll
-  for (int j = 0; j < NR; ++j) acc[j] = T(0);
-  if (w < rows_b) {
-    const int ni = find_from(first, count, w, hint_b, [&](int i) { return nodes[i].brow0; });
-    const ApplyNode nd = nodes[ni];
-    const int r = w - nd.brow0;
-    for (int b = 0; b < nd.nb_count; ++b) {
-      const ApplyNbr n = nb[nd.nb_first + b];
-      const T *Ar = (const T *)nd.AsN + (int64_t)r * nd.dN + n.col;
-      const T *xn = ws + n.x * nrhs + j0;
-      row_dot<T, NR>(Ar, xn, n.size, nrhs, nr, lane, acc);
-    }
-    warp_reduce<T, NR>(acc);
-    if (lane == 0) {
-      const T *ph = ws + (nd.xs + r) * nrhs + j0;
-      T *o = tb + (nd.toff + r) * nrhs + j0;
+      for (int r = 0; r < R; ++r) {
+        const int row = min(r0 + r, total - 1);
+        a[r] = row < it.m ? (const T *)it.A + (int64_t)row * it.m : (const T *)it.P + (int64_t)(row - it.m) * it.m;
 #pragma unroll
-      for (int j = 0; j < NR; ++j)
-        if (j < nr) o[j] = ph[j] - acc[j];
+        for (int j = 0; j < NR; ++j) acc[r][j] = T(0);
+      }
+      rows_dot<T, NR, R, VEC>(a, x, it.m, nrhs, nr, lane, acc);
+      constexpr int V = R * NR;
+      T(&v)[V] = reinterpret_cast<T(&)[V]>(acc);
+      warp_sums<T, V>(v, lane);
+      if (warp_sum_writer<V>(lane)) {
+#pragma unroll
+        for (int i = 0; i < warp_sum_count<V>(); ++i) {
+          const int idx = warp_sum_first<V>(lane) + i;
+          const int row = r0 + idx / NR, j = idx % NR;
+          if (row < total && j < nr) {
+            T *o = row < it.m ? tcur + (it.t + row) * nrhs + j0 : ws + (it.r + row - it.m) * nrhs + j0;
+            o[j] = v[i];
+          }
+        }
+      }
     }
+  } else if (it.kind == ApplyItem::TARGET) {
+    // phi_n -= sum_s B_s[:, n]^T phi_s, unknowns i0 .. i0 + 31 of n
+    const int i = it.i0 + lane;
+    const bool active = i < it.m;
+    T acc[NR];
+#pragma unroll
+    for (int j = 0; j < NR; ++j) acc[j] = T(0);
+    for (int c = 0; c < it.count; ++c) {
+      const ApplyContrib ac = cb[it.first + c];
+      cols_dot<T, NR, VEC>((const T *)ac.A + i, ac.ld, ws + ac.x * nrhs + j0, ac.m, nrhs, nr, warp, active, acc);
+    }
+#pragma unroll
+    for (int j = 0; j < NR; ++j) sm.part[warp][j][lane] = acc[j];
+    __syncthreads();
+    for (int e = threadIdx.x; e < 32 * nr; e += AT) {
+      const int l = e & 31, j = e >> 5;
+      T s = T(0);
+#pragma unroll
+      for (int w = 0; w < AW; ++w) s += sm.part[w][j][l];
+      if (it.i0 + l < it.m) ws[(it.x + it.i0 + l) * nrhs + j0 + j] -= s;
+    }
+    __syncthreads();
   } else {
-    const int w2 = w - rows_b;
-    const int ni = find_from(first, count, w2, hint_p, [&](int i) { return nodes[i].pch0; });
-    const ApplyNode nd = nodes[ni];
-    const int i = (w2 - nd.pch0) * 32 + lane;
-    if (i >= nd.m || nd.k == 0) return;
-    const T *P = (const T *)nd.P + i;
-    const T *xr = ws + nd.xr * nrhs + j0;
-    col_dot<T, NR>(P, nd.m, xr, nd.k, nrhs, nr, acc);
-    T *o = tb2 + (nd.toff + i) * nrhs + j0;
-#pragma unroll
-    for (int j = 0; j < NR; ++j)
-      if (j < nr) o[j] = acc[j];
+    // t_s of the previous wave into the place of its phi_s, one node per warp
+    if (warp < it.count) {
+      const ApplyNode &nd = nodes[it.first + warp];
+      const int64_t src = nd.toff * nrhs, dst = nd.xs * nrhs;
+      const int m = nd.m;
+      for (int e = lane; e < m * nr; e += 32) {
+        const int64_t o = (int64_t)(e / nr) * nrhs + j0 + e % nr;
+        ws[dst + o] = tprev[src + o];
+      }
+    }
   }
 }
 
-template <typename T, int NR>
-__global__ void __launch_bounds__(AT) k_b1(const ApplyNode *__restrict__ nodes, int first, int count, int rows_b,
-                                           int pch, const ApplyNbr *__restrict__ nb, const T *__restrict__ ws,
-                                           T *__restrict__ tb, T *__restrict__ tb2, int nrhs, int j0,
-                                           const int *__restrict__ hint_b, const int *__restrict__ hint_p) {
-  const int w = blockIdx.x * AW + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (w < rows_b + pch)
-    b1_warp<T, NR>(nodes, first, count, rows_b, w, lane, nb, ws, tb, tb2, nrhs, j0,
-                   hint_b ? hint_b[blockIdx.x] : -1, hint_p ? hint_p[blockIdx.x] : -1);
-}
-
-// B2b: x_s = M_ss v_s + y_s, one warp per row of s
-template <typename T, int NR>
-__device__ __forceinline__ void b2_warp(const ApplyNode *__restrict__ nodes, int first, int count, int w, int lane,
-                                        T *__restrict__ ws, const T *__restrict__ tb, const T *__restrict__ tb2,
-                                        int nrhs, int j0, int hint = -1) {
-  const int ni = find_from(first, count, w, hint, [&](int i) { return nodes[i].brow0; });
-  const ApplyNode nd = nodes[ni];
-  const int r = w - nd.brow0;
-  const T *Mr = (const T *)nd.M + (int64_t)r * nd.m;
-  const T *v = tb + nd.toff * nrhs + j0;
+// One item of the backward step: x_s = t_s + P_ss^T x_r - B_s x_N for the
+// unknowns i0 .. i0 + 31 of s, in place of t_s (tsrc: the last wave's t_s)
+template <typename T, int NR, bool VEC>
+__device__ __forceinline__ void bwd_item(const ApplyItem &it, const ApplyNbr *__restrict__ nb, T *ws, const T *tsrc,
+                                         int nrhs, int j0, ItemSmem<T, NR> &sm) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nr = min(NR, nrhs - j0);
+  const int i = it.i0 + lane;
   T acc[NR];
 #pragma unroll
   for (int j = 0; j < NR; ++j) acc[j] = T(0);
-  row_dot<T, NR>(Mr, v, nd.m, nrhs, nr, lane, acc);
-  warp_reduce<T, NR>(acc);
-  if (lane == 0) {
-    const T *y = tb2 + (nd.toff + r) * nrhs + j0;
-    T *o = ws + (nd.xs + r) * nrhs + j0;
+  if (it.k > 0)
+    cols_dot<T, NR, VEC>((const T *)it.P + i, it.m, ws + it.r * nrhs + j0, it.k, nrhs, nr, warp, i < it.m, acc);
 #pragma unroll
-    for (int j = 0; j < NR; ++j)
-      if (j < nr) o[j] = acc[j] + (nd.k > 0 ? y[j] : T(0));
+  for (int j = 0; j < NR; ++j) sm.part[warp][j][lane] = acc[j];
+  if (it.count > 0) {
+    constexpr int R = rows_per_pass<T, NR>();
+#pragma unroll 1
+    for (int q = 0; q < AR; q += R) {
+      const int r0 = warp * AR + q;   // row inside the item
+      const T *a[R];
+      T ra[R][NR];
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int j = 0; j < NR; ++j) ra[r][j] = T(0);
+      for (int b = 0; b < it.count; ++b) {
+        const ApplyNbr n = nb[it.first + b];
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+          a[r] = (const T *)it.A + (int64_t)min(it.i0 + r0 + r, it.m - 1) * it.dN + n.col;
+        rows_dot<T, NR, R, VEC>(a, ws + n.x * nrhs + j0, n.size, nrhs, nr, lane, ra);
+      }
+      constexpr int V = R * NR;
+      T(&v)[V] = reinterpret_cast<T(&)[V]>(ra);
+      warp_sums<T, V>(v, lane);
+      if (warp_sum_writer<V>(lane))
+#pragma unroll
+        for (int u = 0; u < warp_sum_count<V>(); ++u) {
+          const int idx = warp_sum_first<V>(lane) + u;
+          sm.rows[r0 + idx / NR][idx % NR] = v[u];
+        }
+    }
   }
+  __syncthreads();
+  for (int e = threadIdx.x; e < 32 * nr; e += AT) {
+    const int l = e & 31, j = e >> 5;
+    if (it.i0 + l < it.m) {
+      T s = T(0);
+#pragma unroll
+      for (int w = 0; w < AW; ++w) s += sm.part[w][j][l];
+      T *o = ws + (it.x + it.i0 + l) * nrhs + j0 + j;
+      const T t = tsrc ? tsrc[(it.t + it.i0 + l) * nrhs + j0 + j] : *o;
+      s += t;
+      if (it.count > 0) s -= sm.rows[l][j];
+      *o = s;
+    }
+  }
+  __syncthreads();
 }
 
-template <typename T, int NR>
-__global__ void __launch_bounds__(AT) k_b2(const ApplyNode *__restrict__ nodes, int first, int count, int rows_b,
-                                           T *__restrict__ ws, const T *__restrict__ tb,
-                                           const T *__restrict__ tb2, int nrhs, int j0, const int *__restrict__ hint) {
-  const int w = blockIdx.x * AW + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (w < rows_b) b2_warp<T, NR>(nodes, first, count, w, lane, ws, tb, tb2, nrhs, j0, hint ? hint[blockIdx.x] : -1);
+template <typename T, int NR, bool VEC>
+__global__ void __launch_bounds__(AT) k_fwd(const ApplyItem *__restrict__ items, const ApplyNode *__restrict__ nodes,
+                                            const ApplyContrib *__restrict__ cb, T *ws, T *tcur, const T *tprev,
+                                            int nrhs, int j0) {
+  __shared__ ItemSmem<T, NR> sm;
+  fwd_item<T, NR, VEC>(items[blockIdx.x], nodes, cb, ws, tcur, tprev, nrhs, j0, sm);
+}
+
+template <typename T, int NR, bool VEC>
+__global__ void __launch_bounds__(AT) k_bwd(const ApplyItem *__restrict__ items, const ApplyNbr *__restrict__ nb,
+                                            T *ws, const T *tsrc, int nrhs, int j0) {
+  __shared__ ItemSmem<T, NR> sm;
+  bwd_item<T, NR, VEC>(items[blockIdx.x], nb, ws, tsrc, nrhs, j0, sm);
 }
 
 template <typename T>
@@ -282,50 +342,46 @@ __global__ void k_copy(const T *__restrict__ src, T *__restrict__ dst, int64_t n
 }
 
 // root: x = A_root^-1 phi (phi copied to tb first), one warp per row
-template <typename T, int NR>
-__device__ __forceinline__ void root_warp(const T *__restrict__ Ainv, int m, int64_t off, int w, int lane,
-                                          T *__restrict__ ws, const T *__restrict__ tb, int nrhs, int j0) {
-  const T *Ar = Ainv + (int64_t)w * m;
+template <typename T, int NR, bool VEC>
+__device__ __forceinline__ void root_warp(const T *__restrict__ Ainv, int m, int64_t off, int w, int lane, T *ws,
+                                          const T *tb, int nrhs, int j0) {
   const int nr = min(NR, nrhs - j0);
-  T acc[NR];
+  const T *a[1] = {Ainv + (int64_t)w * m};
+  T acc[1][NR];
 #pragma unroll
-  for (int j = 0; j < NR; ++j) acc[j] = T(0);
-  row_dot<T, NR>(Ar, tb + j0, m, nrhs, nr, lane, acc);
-  warp_reduce<T, NR>(acc);
-  if (lane == 0) {
-    T *o = ws + (off + w) * nrhs + j0;
-#pragma unroll
-    for (int j = 0; j < NR; ++j)
-      if (j < nr) o[j] = acc[j];
+  for (int j = 0; j < NR; ++j) acc[0][j] = T(0);
+  rows_dot<T, NR, 1, VEC>(a, tb + j0, m, nrhs, nr, lane, acc);
+  warp_sums<T, NR>(acc[0], lane);
+  if (warp_sum_writer<NR>(lane)) {
+    const int j = warp_sum_first<NR>(lane);
+    if (j < nr) ws[(off + w) * nrhs + j0 + j] = acc[0][0];
   }
 }
 
-template <typename T, int NR>
-__global__ void __launch_bounds__(AT) k_root(const T *__restrict__ Ainv, int m, int64_t off,
-                                             T *__restrict__ ws, const T *__restrict__ tb, int nrhs,
-                                             int j0) {
+template <typename T, int NR, bool VEC>
+__global__ void __launch_bounds__(AT) k_root(const T *__restrict__ Ainv, int m, int64_t off, T *ws, const T *tb,
+                                             int nrhs, int j0) {
   const int w = blockIdx.x * AW + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (w < m) root_warp<T, NR>(Ainv, m, off, w, lane, ws, tb, nrhs, j0);
+  if (w < m) root_warp<T, NR, VEC>(Ainv, m, off, w, lane, ws, tb, nrhs, j0);
 }
 
 // ---------------------------------------------------------------------------
 // Persistent apply: the whole of Algorithm 2 for one chunk of right-hand sides
 // in ONE cooperative launch.  The per-step launches above cost a launch
-// latency per dependent step (about four per wave, some 240 at the 512 x 512
-// workload); here every CTA of a grid sized to be resident walks the step
-// list (forward f1, f2 per wave; root copy and solve; backward b1, b2 per
-// wave in reverse), the warps of the grid sharing each step's virtual warps,
-// with a grid-wide barrier between dependent steps.  The barrier is one
-// arrival counter; its wait is bounded (clock cycles) and a wait that runs
-// out sets *err and ends the kernel (the host reports HS_ERR_TIMEOUT).
+// latency per dependent step (two per wave); here every CTA of a grid sized
+// to be resident walks the step list (forward step per wave; root copy and
+// solve; backward step per wave in reverse), the CTAs of the grid sharing each
+// step's items, with a grid-wide barrier between dependent steps.  The barrier
+// is one arrival counter; its wait is bounded (clock cycles) and a wait that
+// runs out sets *err and ends the kernel (the host reports HS_ERR_TIMEOUT).
 // The steps and their arithmetic are those of the per-step kernels, so the
 // result is the same bit for bit.
 // ---------------------------------------------------------------------------
-enum { AS_F1 = 0, AS_F2 = 1, AS_COPY = 2, AS_ROOT = 3, AS_B1 = 4, AS_B2 = 5 };
+enum { AS_FWD = 0, AS_COPY = 1, AS_ROOT = 2, AS_BWD = 3 };
 
 struct ApplyStepDev {
   int kind;
-  int wave;          // index into the waves (f1, f2, b1, b2)
+  int wave;          // index into the waves (forward, backward)
 };
 
 // Grid barrier number `round` (0, 1, ...): one counter that only grows; CTA
@@ -367,40 +423,39 @@ __device__ bool grid_barrier(unsigned *bar, unsigned round, int *err, long long 
   return s_ok != 0;
 }
 
-template <typename T, int NR>
+// tb0, tb1: the wave scratch of even and odd waves
+template <typename T, int NR, bool VEC>
 __global__ void __launch_bounds__(AT) k_apply_persistent(
-    const ApplyStepDev *__restrict__ steps, int nsteps, const WaveApply *__restrict__ waves,
-    const ApplyNode *__restrict__ nodes, const ApplyNbr *__restrict__ nbrs, const ApplyTarget *__restrict__ tg,
-    const ApplyContrib *__restrict__ cb, const T *__restrict__ root_inv, int root_m, int64_t root_off,
-    T *__restrict__ ws, T *__restrict__ tb, T *__restrict__ tb2, int nrhs, int j0, unsigned *bar, int *err,
-    long long limit) {
+    const ApplyStepDev *__restrict__ steps, int nsteps, const WaveApply *__restrict__ waves, int nwaves,
+    const ApplyItem *__restrict__ items, const ApplyNode *__restrict__ nodes, const ApplyNbr *__restrict__ nbrs,
+    const ApplyContrib *__restrict__ cb, const T *__restrict__ root_inv, int root_m, int64_t root_off, T *ws, T *tb0,
+    T *tb1, int nrhs, int j0, unsigned *bar, int *err, long long limit) {
+  __shared__ ItemSmem<T, NR> sm;
   const int lane = threadIdx.x & 31;
-  const int gw = blockIdx.x * AW + (threadIdx.x >> 5), nwarps = gridDim.x * AW;
+  const int gw = blockIdx.x * AW + (threadIdx.x >> 5), gwarps = gridDim.x * AW;
   // test of the time-out path: a barrier round no launch can complete (the
   // switch is read at run time, so recorded graphs follow it too)
   if (g_apply_probe && !grid_barrier(bar, 1u << 20, err, limit)) return;
+  T *troot = (nwaves & 1) ? tb1 : tb0;   // not the last wave's scratch
   for (int si = 0; si < nsteps; ++si) {
     const ApplyStepDev st = steps[si];
     if (st.kind == AS_COPY) {
       const int64_t n = (int64_t)root_m * nrhs;
       for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
-        tb[e] = ws[root_off * nrhs + e];
+        troot[e] = ws[root_off * nrhs + e];
     } else if (st.kind == AS_ROOT) {
-      for (int w = gw; w < root_m; w += nwarps) root_warp<T, NR>(root_inv, root_m, root_off, w, lane, ws, tb, nrhs, j0);
+      for (int w = gw; w < root_m; w += gwarps)
+        root_warp<T, NR, VEC>(root_inv, root_m, root_off, w, lane, ws, troot, nrhs, j0);
     } else {
       const WaveApply wa = waves[st.wave];
-      if (st.kind == AS_F1) {
-        for (int w = gw; w < wa.rows_f; w += nwarps)
-          f1_warp<T, NR>(nodes, wa.node_first, wa.node_count, w, lane, ws, tb, nrhs, j0);
-      } else if (st.kind == AS_F2) {
-        for (int w = gw; w < wa.tch; w += nwarps)
-          f2_warp<T, NR>(tg, wa.tgt_first, wa.tgt_count, w, lane, cb, ws, tb, nrhs, j0);
-      } else if (st.kind == AS_B1) {
-        for (int w = gw; w < wa.rows_b + wa.pch; w += nwarps)
-          b1_warp<T, NR>(nodes, wa.node_first, wa.node_count, wa.rows_b, w, lane, nbrs, ws, tb, tb2, nrhs, j0);
+      T *tc = (st.wave & 1) ? tb1 : tb0, *tp = (st.wave & 1) ? tb0 : tb1;
+      if (st.kind == AS_FWD) {
+        for (int i = blockIdx.x; i < wa.f_count; i += gridDim.x)
+          fwd_item<T, NR, VEC>(items[wa.f_first + i], nodes, cb, ws, tc, tp, nrhs, j0, sm);
       } else {
-        for (int w = gw; w < wa.rows_b; w += nwarps)
-          b2_warp<T, NR>(nodes, wa.node_first, wa.node_count, w, lane, ws, tb, tb2, nrhs, j0);
+        const T *ts = st.wave == nwaves - 1 ? tc : nullptr;
+        for (int i = blockIdx.x; i < wa.b_count; i += gridDim.x)
+          bwd_item<T, NR, VEC>(items[wa.b_first + i], nbrs, ws, ts, nrhs, j0, sm);
       }
     }
     if (si + 1 < nsteps && !grid_barrier(bar, (unsigned)si, err, limit)) return;
@@ -654,46 +709,34 @@ int grid_for(int64_t total) {
 // grid of the PCG reduction kernels: a function of n only (see above)
 int rgrid_for(int64_t n) { return grid_for(n); }
 
-// a wave's per-CTA search starts (nullptr: the kernels search the whole wave)
-inline const int *hint_at(const FactorHandle &h, int off) { return (h.d_hints && off >= 0) ? h.d_hints + off : nullptr; }
-
 // One pass of Algorithm 2 over right-hand sides [j0, j0 + NR) of the
-// workspace ws (layout [unknown][nrhs]); tb and tb2 are the per-wave scratch.
-template <typename T, int NR>
-void apply_waves_nr(const FactorHandle &h, T *ws, T *tb, T *tb2, int nrhs, int j0, cudaStream_t st) {
-  auto blocks = [](int warps) { return (warps + AW - 1) / AW; };
-  for (const LevelApply &la : h.levels)
-    for (int w = la.wave_first; w < la.wave_first + la.wave_count; ++w) {
-      const WaveApply &wa = h.waves[w];
-      if (wa.rows_f) {
-        k_f1<T, NR><<<blocks(wa.rows_f), AT, 0, st>>>(h.d_nodes, wa.node_first, wa.node_count, wa.rows_f, ws, tb,
-                                                      nrhs, j0, hint_at(h, wa.hf1));
-        count_launch();
-      }
-      if (wa.tch) {
-        k_f2<T, NR><<<blocks(wa.tch), AT, 0, st>>>(h.d_targets, wa.tgt_first, wa.tgt_count, wa.tch, h.d_contribs,
-                                                   ws, tb, nrhs, j0, hint_at(h, wa.hf2));
-        count_launch();
-      }
-    }
+// workspace ws (layout [unknown][nrhs]); tb0 and tb1 are the scratch of even and
+// odd waves.
+template <typename T, int NR, bool VEC>
+void apply_waves_nr(const FactorHandle &h, T *ws, T *tb0, T *tb1, int nrhs, int j0, cudaStream_t st) {
+  const int nw = (int)h.waves.size();
+  auto buf = [&](int w) { return (w & 1) ? tb1 : tb0; };
+  for (int w = 0; w < nw; ++w) {
+    const WaveApply &wa = h.waves[w];
+    if (!wa.f_count) continue;
+    k_fwd<T, NR, VEC><<<wa.f_count, AT, 0, st>>>(h.d_items + wa.f_first, h.d_nodes, h.d_contribs, ws, buf(w),
+                                                 buf(w + 1), nrhs, j0);
+    count_launch();
+  }
   if (h.root_m > 0) {
     const int64_t cnt = (int64_t)h.root_m * nrhs;
-    k_copy<T><<<(int)std::min<int64_t>((cnt + 255) / 256, 1024), 256, 0, st>>>(ws + h.root_off * nrhs, tb, cnt);
-    k_root<T, NR><<<blocks(h.root_m), AT, 0, st>>>((const T *)h.root_inv, h.root_m, h.root_off, ws, tb, nrhs, j0);
+    T *tr = buf(nw);   // the other buffer holds the last wave's t_s
+    k_copy<T><<<(int)std::min<int64_t>((cnt + 255) / 256, 1024), 256, 0, st>>>(ws + h.root_off * nrhs, tr, cnt);
+    k_root<T, NR, VEC><<<(h.root_m + AW - 1) / AW, AT, 0, st>>>((const T *)h.root_inv, h.root_m, h.root_off, ws, tr,
+                                                                nrhs, j0);
     count_launch(2);
   }
-  for (int li = (int)h.levels.size() - 1; li >= 0; --li) {
-    const LevelApply &la = h.levels[li];
-    for (int w = la.wave_first + la.wave_count - 1; w >= la.wave_first; --w) {
-      const WaveApply &wa = h.waves[w];
-      if (!wa.rows_b) continue;
-      k_b1<T, NR><<<blocks(wa.rows_b + wa.pch), AT, 0, st>>>(h.d_nodes, wa.node_first, wa.node_count, wa.rows_b,
-                                                             wa.pch, h.d_nbrs, ws, tb, tb2, nrhs, j0,
-                                                             hint_at(h, wa.hb), hint_at(h, wa.hp));
-      k_b2<T, NR><<<blocks(wa.rows_b), AT, 0, st>>>(h.d_nodes, wa.node_first, wa.node_count, wa.rows_b, ws, tb,
-                                                    tb2, nrhs, j0, hint_at(h, wa.hb));
-      count_launch(2);
-    }
+  for (int w = nw - 1; w >= 0; --w) {
+    const WaveApply &wa = h.waves[w];
+    if (!wa.b_count) continue;
+    k_bwd<T, NR, VEC><<<wa.b_count, AT, 0, st>>>(h.d_items + wa.b_first, h.d_nbrs, ws,
+                                                 w == nw - 1 ? (const T *)buf(w) : nullptr, nrhs, j0);
+    count_launch();
   }
   HS_CUDA(cudaGetLastError());
 }
@@ -721,8 +764,8 @@ int persistent_apply_bps() {
 // The grid is the number of CTAs that can be resident at once (at most four
 // per SM), launched cooperatively so that they are; the barrier words are
 // cleared on the stream first.
-template <typename T, int NR>
-void apply_persistent_nr(const FactorHandle &h, T *ws, T *tb, T *tb2, int nrhs, int j0, cudaStream_t st) {
+template <typename T, int NR, bool VEC>
+void apply_persistent_nr(const FactorHandle &h, T *ws, T *tb0, T *tb1, int nrhs, int j0, cudaStream_t st) {
   static int blocks_per_sm[64] = {0};
   static std::mutex mu;
   int dev = 0;
@@ -733,7 +776,7 @@ void apply_persistent_nr(const FactorHandle &h, T *ws, T *tb, T *tb2, int nrhs, 
     if (dev < 0 || dev >= 64) fail(HS_ERR_CUDA, "device ordinal out of range");
     if (!blocks_per_sm[dev]) {
       int b = 0;
-      HS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_apply_persistent<T, NR>, AT, 0));
+      HS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_apply_persistent<T, NR, VEC>, AT, 0));
       blocks_per_sm[dev] = std::max(1, std::min(b, persistent_apply_bps() ? persistent_apply_bps() : 4));
     }
     bps = blocks_per_sm[dev];
@@ -752,29 +795,44 @@ void apply_persistent_nr(const FactorHandle &h, T *ws, T *tb, T *tb2, int nrhs, 
   cfg.numAttrs = 1;
   // about one second of SM clocks per barrier unless hs_opts.timeout_cycles says otherwise
   const long long limit = h.timeout_cycles > 0 ? (long long)h.timeout_cycles : 2000000000LL;
-  HS_CUDA(cudaLaunchKernelEx(&cfg, k_apply_persistent<T, NR>, (const ApplyStepDev *)h.d_apply_steps,
-                             h.apply_nsteps, (const WaveApply *)h.d_waves, (const ApplyNode *)h.d_nodes,
-                             (const ApplyNbr *)h.d_nbrs, (const ApplyTarget *)h.d_targets,
-                             (const ApplyContrib *)h.d_contribs, (const T *)h.root_inv, h.root_m, h.root_off, ws, tb,
-                             tb2, nrhs, j0, h.d_apply_bar, h.d_apply_err, limit));
+  HS_CUDA(cudaLaunchKernelEx(&cfg, k_apply_persistent<T, NR, VEC>, (const ApplyStepDev *)h.d_apply_steps,
+                             h.apply_nsteps, (const WaveApply *)h.d_waves, (int)h.waves.size(),
+                             (const ApplyItem *)h.d_items, (const ApplyNode *)h.d_nodes, (const ApplyNbr *)h.d_nbrs,
+                             (const ApplyContrib *)h.d_contribs, (const T *)h.root_inv, h.root_m, h.root_off, ws, tb0,
+                             tb1, nrhs, j0, h.d_apply_bar, h.d_apply_err, limit));
   count_launch();
 }
 
-template <typename T, int NR>
-void apply_chunk_nr(const FactorHandle &h, T *ws, T *tb, T *tb2, int nrhs, int j0, cudaStream_t st) {
+template <typename T, int NR, bool VEC>
+void apply_chunk_v(const FactorHandle &h, T *ws, T *tb0, T *tb1, int nrhs, int j0, cudaStream_t st) {
   if (persistent_apply_enabled() && h.d_apply_steps && h.apply_nsteps > 0)
-    apply_persistent_nr<T, NR>(h, ws, tb, tb2, nrhs, j0, st);
+    apply_persistent_nr<T, NR, VEC>(h, ws, tb0, tb1, nrhs, j0, st);
   else
-    apply_waves_nr<T, NR>(h, ws, tb, tb2, nrhs, j0, st);
+    apply_waves_nr<T, NR, VEC>(h, ws, tb0, tb1, nrhs, j0, st);
+}
+
+// 16-byte loads of the right-hand sides of an unknown when the chunk is full
+// and every unknown's values start on a 16-byte boundary (the workspace and
+// both scratch buffers do)
+template <typename T, int NR>
+void apply_chunk_nr(const FactorHandle &h, T *ws, T *tb0, T *tb1, int nrhs, int j0, cudaStream_t st) {
+  constexpr int W = 16 / (int)sizeof(T);
+  if constexpr (NR % W == 0) {
+    const bool aligned = (((uintptr_t)ws | (uintptr_t)tb0 | (uintptr_t)tb1) & 15) == 0;
+    if (aligned && nrhs - j0 >= NR && nrhs % W == 0 && j0 % W == 0) {
+      apply_chunk_v<T, NR, true>(h, ws, tb0, tb1, nrhs, j0, st);
+      return;
+    }
+  }
+  apply_chunk_v<T, NR, false>(h, ws, tb0, tb1, nrhs, j0, st);
 }
 
 // The whole apply on a workspace whose level-L part holds the right-hand
-// sides: red-node parts cleared (Algorithm 2 starts them at zero), then the
-// right-hand sides in chunks of at most 16 (register accumulators).
+// sides, in chunks of at most 16 of them (register accumulators).  The red
+// nodes' parts need no clearing: the restriction that makes a red node's
+// vector is the first to write it.
 template <typename T>
 void apply_chunks(const FactorHandle &h, T *ws, T *tb, T *tb2, int nrhs, cudaStream_t st) {
-  const int64_t n = h.plan.n;
-  if (h.ws_size > n) HS_CUDA(cudaMemsetAsync(ws + n * nrhs, 0, sizeof(T) * (h.ws_size - n) * nrhs, st));
   for (int j0 = 0; j0 < nrhs;) {
     const int rem = nrhs - j0;
     if (rem > 8) {
@@ -808,8 +866,8 @@ void apply_ws_direct(const FactorHandle &h, int nrhs, cudaStream_t st) {
 }
 
 // ---------------------------------------------------------------------------
-// CUDA graphs.  One apply is about four dependent launches per wave (some 240
-// at the 512 x 512 workload), each too short to hide its launch latency, so
+// CUDA graphs.  One apply is two dependent launches per wave (about 120 at
+// the 512 x 512 workload), each too short to hide its launch latency, so
 // the launch sequence is recorded once per factorization and right-hand-side
 // count and replayed with one cudaGraphLaunch.  Recording happens on a private
 // stream of the handle in thread-local capture mode (other threads keep
@@ -874,7 +932,8 @@ void apply_ws(FactorHandle &h, int nrhs, cudaStream_t st) {
 }
 
 void ensure_buffers(FactorHandle &h, int nrhs_cap, cudaStream_t st) {
-  const int64_t tneed0 = std::max<int64_t>(std::max<int64_t>(h.tmax, h.root_m), 1);
+  // a multiple of 4, so that the second buffer starts on a 16-byte boundary
+  const int64_t tneed0 = (std::max<int64_t>(std::max<int64_t>(h.tmax, h.root_m), 1) + 3) & ~(int64_t)3;
   if (h.nrhs_cap >= nrhs_cap && h.d_ws && h.ws_cap >= h.ws_size && h.t_cap >= tneed0) return;
   nrhs_cap = std::max(nrhs_cap, h.nrhs_cap);
   h.drop_graphs();   // they hold the old buffers
@@ -907,69 +966,90 @@ void ensure_buffers(FactorHandle &h, int nrhs_cap, cudaStream_t st) {
 }  // namespace
 
 void apply_prepare(FactorHandle &h, cudaStream_t st) {
+  // the items of every wave (one CTA each), longest chains first
+  const int nw = (int)h.waves.size();
+  std::vector<ApplyItem> items;
+  size_t cnt = 0;
+  for (const ApplyNode &nd : h.nodes) cnt += (size_t)(2 * nd.m + nd.k) / kApplyRows + 3;
+  items.reserve(cnt + h.targets.size() * 2);
+  for (int w = 0; w < nw; ++w) {
+    WaveApply &wa = h.waves[w];
+    wa.f_first = (int)items.size();
+    for (int t = wa.tgt_first; t < wa.tgt_first + wa.tgt_count; ++t) {
+      const ApplyTarget &tg = h.targets[t];
+      for (int i = 0; i < tg.size; i += kApplyRows) {
+        ApplyItem it{};
+        it.kind = ApplyItem::TARGET;
+        it.x = tg.x;
+        it.m = tg.size;
+        it.i0 = i;
+        it.first = tg.first;
+        it.count = tg.count;
+        items.push_back(it);
+      }
+    }
+    auto node_item = [](const ApplyNode &nd, int i) {
+      ApplyItem it{};
+      it.P = nd.P;
+      it.x = nd.xs;
+      it.r = nd.xr;
+      it.t = nd.toff;
+      it.m = nd.m;
+      it.k = nd.k;
+      it.i0 = i;
+      return it;
+    };
+    for (int q = wa.node_first; q < wa.node_first + wa.node_count; ++q) {
+      const ApplyNode &nd = h.nodes[q];
+      for (int i = 0; i < nd.m + nd.k; i += kApplyRows) {
+        ApplyItem it = node_item(nd, i);
+        it.kind = ApplyItem::ROWS;
+        it.A = nd.M;
+        items.push_back(it);
+      }
+    }
+    if (w > 0)
+      for (int q = 0; q < h.waves[w - 1].node_count; q += AW) {
+        ApplyItem it{};
+        it.kind = ApplyItem::MOVE;
+        it.first = h.waves[w - 1].node_first + q;
+        it.count = std::min(AW, h.waves[w - 1].node_count - q);
+        items.push_back(it);
+      }
+    wa.f_count = (int)items.size() - wa.f_first;
+    wa.b_first = (int)items.size();
+    for (int q = wa.node_first; q < wa.node_first + wa.node_count; ++q) {
+      const ApplyNode &nd = h.nodes[q];
+      for (int i = 0; i < nd.m; i += kApplyRows) {
+        ApplyItem it = node_item(nd, i);
+        it.A = nd.B;
+        it.dN = nd.dN;
+        it.first = nd.nb_first;
+        it.count = nd.dN > 0 ? nd.nb_count : 0;
+        items.push_back(it);
+      }
+    }
+    wa.b_count = (int)items.size() - wa.b_first;
+  }
+  if (items.size() > h.items_cap) {
+    h.alloc.put(h.d_items, st);
+    h.d_items = nullptr;
+    h.items_cap = 0;
+    h.alloc.get(&h.d_items, sizeof(ApplyItem) * items.size(), st);
+    h.items_cap = items.size();
+  }
+  if (!items.empty())
+    HS_CUDA(cudaMemcpyAsync(h.d_items, items.data(), sizeof(ApplyItem) * items.size(), cudaMemcpyHostToDevice, st));
   // the step list of Algorithm 2, in the order of the per-step launches
   std::vector<ApplyStepDev> steps;
-  for (const LevelApply &la : h.levels)
-    for (int w = la.wave_first; w < la.wave_first + la.wave_count; ++w) {
-      if (h.waves[w].rows_f) steps.push_back(ApplyStepDev{AS_F1, w});
-      if (h.waves[w].tch) steps.push_back(ApplyStepDev{AS_F2, w});
-    }
+  for (int w = 0; w < nw; ++w)
+    if (h.waves[w].f_count) steps.push_back(ApplyStepDev{AS_FWD, w});
   if (h.root_m > 0) {
     steps.push_back(ApplyStepDev{AS_COPY, 0});
     steps.push_back(ApplyStepDev{AS_ROOT, 0});
   }
-  for (int li = (int)h.levels.size() - 1; li >= 0; --li) {
-    const LevelApply &la = h.levels[li];
-    for (int w = la.wave_first + la.wave_count - 1; w >= la.wave_first; --w) {
-      if (!h.waves[w].rows_b) continue;
-      steps.push_back(ApplyStepDev{AS_B1, w});
-      steps.push_back(ApplyStepDev{AS_B2, w});
-    }
-  }
-  // per-CTA search starts of the per-step kernels: for CTA b, the last node
-  // (target) whose first row (chunk) is <= b AW, found by one sweep per key
-  std::vector<int> hints;
-  auto sweep = [&](int nrows, int first, int count, auto key) -> int {
-    if (nrows <= 0 || count <= 0) return -1;
-    const int off = (int)hints.size();
-    const int nb = (nrows + AW - 1) / AW;
-    int i = first;
-    for (int b = 0; b < nb; ++b) {
-      const int w0 = b * AW;
-      while (i + 1 < first + count && key(i + 1) <= w0) ++i;
-      hints.push_back(i);
-    }
-    return off;
-  };
-  for (WaveApply &wa : h.waves) {
-    const ApplyNode *nd = h.nodes.data();
-    const ApplyTarget *tg = h.targets.data();
-    wa.hf1 = sweep(wa.rows_f, wa.node_first, wa.node_count, [&](int i) { return nd[i].row0; });
-    wa.hf2 = sweep(wa.tch, wa.tgt_first, wa.tgt_count, [&](int i) { return tg[i].ch0; });
-    // b1 runs blocks(rows_b + pch) CTAs: by brow0 for its first rows_b warps,
-    // by pch0 for the rest (CTA b's first warp there: max(b AW - rows_b, 0))
-    const int nb1 = (wa.rows_b + wa.pch + AW - 1) / AW;
-    wa.hb = sweep(nb1 * AW, wa.node_first, wa.node_count, [&](int i) { return nd[i].brow0; });
-    if (wa.pch > 0 && wa.node_count > 0) {
-      wa.hp = (int)hints.size();
-      int i = wa.node_first;
-      for (int b = 0; b < nb1; ++b) {
-        const int w2 = std::max(b * AW - wa.rows_b, 0);
-        while (i + 1 < wa.node_first + wa.node_count && nd[i + 1].pch0 <= w2) ++i;
-        hints.push_back(i);
-      }
-    } else {
-      wa.hp = -1;
-    }
-  }
-  if (hints.size() > h.hints_cap) {
-    h.alloc.put(h.d_hints, st);
-    h.d_hints = nullptr;
-    h.alloc.get(&h.d_hints, sizeof(int) * hints.size(), st);
-    h.hints_cap = hints.size();
-  }
-  if (!hints.empty())
-    HS_CUDA(cudaMemcpyAsync(h.d_hints, hints.data(), sizeof(int) * hints.size(), cudaMemcpyHostToDevice, st));
+  for (int w = nw - 1; w >= 0; --w)
+    if (h.waves[w].b_count) steps.push_back(ApplyStepDev{AS_BWD, w});
   h.alloc.put(h.d_apply_steps, st);
   h.alloc.put(h.d_waves, st);
   h.d_apply_steps = nullptr;
@@ -1459,7 +1539,7 @@ FactorHandle::~FactorHandle() {
   alloc.put(d_apply_steps, stream);
   alloc.put(d_waves, stream);
   alloc.put(d_apply_bar, stream);
-  alloc.put(d_hints, stream);
+  alloc.put(d_items, stream);
   alloc.put(d_dscale, stream);
   alloc.put(d_val_f, stream);
   alloc.put(d_flag, stream);
@@ -1469,7 +1549,6 @@ FactorHandle::~FactorHandle() {
   alloc.put(d_perm, stream);
   alloc.put(d_nodes, stream);
   alloc.put(d_nbrs, stream);
-  alloc.put(d_targets, stream);
   alloc.put(d_contribs, stream);
   alloc.put(d_ws, stream);
   alloc.put(d_t, stream);
