@@ -505,14 +505,14 @@ __global__ void k_convert(const A *__restrict__ a, B *__restrict__ b, int64_t n,
 // to a power of two <= 32).  Every reduction visits the rows of one right-hand
 // side in an order that depends on n alone: thread t of block b takes rows
 // b*PT + t + k*gridDim*PT in turn, blocks reduce in a fixed tree, and the last
-// block to finish adds the block partials in block order.  So a right-hand
+// block to finish adds the block partials in a fixed order.  So a right-hand
 // side gets the same bits whether it is solved alone or batched with others
 // (the apply and the SpMV are column-wise already).
 // ---------------------------------------------------------------------------
 constexpr int PT = 256;
 
 struct PcgScal {       // per-rhs scalars, each an array of NP doubles
-  double *bnorm2, *rz, *alpha, *beta, *pq, *rr;
+  double *bnorm2, *rz, *alpha, *beta, *pq, *rr, *tol2;   // tol2: rtol^2 ||b||^2
 };
 struct PcgFlags {
   int *active, *iters, *counter, *done;
@@ -538,7 +538,15 @@ __device__ void block_partial(const double (&v)[NP], double *part) {
   }
 }
 
-// returns true in the last block to finish; sums[j] = ordered total
+// Returns true in the last block to finish; sums[j] = the total of the block
+// partials.  Warp j (then j + 8, ...) adds right-hand side j's: lane l takes
+// blocks l, l + 32, ... in turn, then the lanes in the butterfly's order (an
+// order that depends on the grid alone, so on n alone).  One thread per
+// right-hand side adding the partials one after another made this the longest
+// part of each of the three vector kernels at n = 262144: 57 to 66 us a kernel,
+// of which the vectors themselves need about 2 us; the 512 x 512 FP32 solve is
+// 1.19 times faster with the sums spread over the lanes (and the vector passes
+// around an application fused into these kernels).
 template <int NP>
 __device__ bool finish_sum(const double *part, int *counter, double *sums) {
   __shared__ bool last;
@@ -548,21 +556,24 @@ __device__ bool finish_sum(const double *part, int *counter, double *sums) {
   __syncthreads();
   if (!last) return false;
   __threadfence();
-  if (threadIdx.x < NP) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nb = (int)gridDim.x;
+  for (int j = warp; j < NP; j += PT / 32) {
     double s = 0.0;
-    for (int b = 0; b < (int)gridDim.x; ++b) s += ((volatile const double *)part)[b * NP + threadIdx.x];
-    sums[threadIdx.x] = s;
+#pragma unroll 8
+    for (int b = lane; b < nb; b += 32) s += __ldcg(part + (int64_t)b * NP + j);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) sums[j] = s;
   }
   __syncthreads();
   if (threadIdx.x == 0) *counter = 0;
   return true;
 }
 
-enum { DOT_BNORM = 0, DOT_RZ_FIRST = 1, DOT_RZ = 2, DOT_PLAIN = 3 };
-
+// out[j] = u_j . w_j
 template <int NP>
 __global__ void __launch_bounds__(PT) k_dot(const double *__restrict__ u, const double *__restrict__ w, int64_t n,
-                                            double *part, PcgScal sc, PcgFlags fl, int mode, double *plain_out) {
+                                            double *part, PcgFlags fl, double *out) {
   __shared__ double sums[NP];
   double v[NP];
 #pragma unroll
@@ -572,22 +583,74 @@ __global__ void __launch_bounds__(PT) k_dot(const double *__restrict__ u, const 
     for (int j = 0; j < NP; ++j) v[j] = fma(u[i * NP + j], w[i * NP + j], v[j]);
   block_partial<NP>(v, part);
   if (!finish_sum<NP>(part, fl.counter, sums)) return;
+  if (threadIdx.x < NP) out[threadIdx.x] = sums[threadIdx.x];
+}
+
+// The start of a solve in one pass: the right-hand sides from the caller's
+// layout (cluster order, padded to NP), r = b, x = p = 0, the apply's workspace
+// from r (factor precision, times ds when scaling), ||b||^2 and the counters
+template <typename T, int NP>
+__global__ void __launch_bounds__(PT) k_start(const double *__restrict__ b, int64_t ld,
+                                              const int32_t *__restrict__ perm, int64_t n, int nrhs,
+                                              const double *__restrict__ ds, double *__restrict__ B,
+                                              double *__restrict__ R, double *__restrict__ X, double *__restrict__ P,
+                                              T *__restrict__ ws, double *part, PcgScal sc, PcgFlags fl, double rtol2) {
+  __shared__ double sums[NP];
+  double v[NP];
+#pragma unroll
+  for (int j = 0; j < NP; ++j) v[j] = 0.0;
+  for (int64_t i = blockIdx.x * (int64_t)PT + threadIdx.x; i < n; i += (int64_t)gridDim.x * PT) {
+    const int64_t src = perm[i];
+    const double d = ds ? ds[i] : 1.0;
+#pragma unroll
+    for (int j = 0; j < NP; ++j) {
+      const double r = j < nrhs ? b[src + j * ld] : 0.0;
+      B[i * NP + j] = r;
+      R[i * NP + j] = r;
+      X[i * NP + j] = 0.0;
+      P[i * NP + j] = 0.0;
+      ws[i * NP + j] = (T)(ds ? r * d : r);
+      v[j] = fma(r, r, v[j]);
+    }
+  }
+  block_partial<NP>(v, part);
+  if (!finish_sum<NP>(part, fl.counter, sums)) return;
   const int j = threadIdx.x;
   if (j < NP) {
-    const double s = sums[j];
-    if (mode == DOT_BNORM) {
-      sc.bnorm2[j] = s;
-      fl.active[j] = s > 0.0 ? 1 : 0;
-      fl.iters[j] = 0;
-    } else if (mode == DOT_RZ_FIRST) {
-      sc.beta[j] = 0.0;
-      sc.rz[j] = s;
-    } else if (mode == DOT_RZ) {
-      sc.beta[j] = (fl.active[j] && sc.rz[j] != 0.0) ? s / sc.rz[j] : 0.0;
-      sc.rz[j] = s;
-    } else {
-      plain_out[j] = s;
+    sc.bnorm2[j] = sums[j];
+    sc.tol2[j] = rtol2 * sums[j];
+    sc.rz[j] = 0.0;   // beta = 0 in the first iteration
+    fl.active[j] = sums[j] > 0.0 ? 1 : 0;
+    fl.iters[j] = 0;
+  }
+}
+
+// z from the apply's workspace (factor precision, times ds when scaling),
+// r . z and beta in one pass
+template <typename T, int NP>
+__global__ void __launch_bounds__(PT) k_zdot(const T *__restrict__ ws, const double *__restrict__ ds,
+                                             const double *__restrict__ r, int64_t n, double *__restrict__ z,
+                                             double *part, PcgScal sc, PcgFlags fl) {
+  __shared__ double sums[NP];
+  double v[NP];
+#pragma unroll
+  for (int j = 0; j < NP; ++j) v[j] = 0.0;
+  for (int64_t i = blockIdx.x * (int64_t)PT + threadIdx.x; i < n; i += (int64_t)gridDim.x * PT) {
+    const double d = ds ? ds[i] : 1.0;
+#pragma unroll
+    for (int j = 0; j < NP; ++j) {
+      const double w = (double)ws[i * NP + j];
+      const double zv = ds ? w * d : w;
+      z[i * NP + j] = zv;
+      v[j] = fma(r[i * NP + j], zv, v[j]);
     }
+  }
+  block_partial<NP>(v, part);
+  if (!finish_sum<NP>(part, fl.counter, sums)) return;
+  const int j = threadIdx.x;
+  if (j < NP) {
+    sc.beta[j] = (fl.active[j] && sc.rz[j] != 0.0) ? sums[j] / sc.rz[j] : 0.0;
+    sc.rz[j] = sums[j];
   }
 }
 
@@ -632,11 +695,13 @@ __global__ void __launch_bounds__(PT) k_spmv_p(const int32_t *__restrict__ rp, c
   }
 }
 
-// x += alpha p ; r -= alpha q ; partial ||r||^2 ; convergence per rhs
-template <int NP>
+// x += alpha p ; r -= alpha q, also into the apply's workspace (factor
+// precision, times ds when scaling) ; partial ||r||^2 ; convergence per rhs
+template <typename T, int NP>
 __global__ void __launch_bounds__(PT) k_update(double *__restrict__ x, double *__restrict__ r,
                                                const double *__restrict__ p, const double *__restrict__ q, int64_t n,
-                                               double *part, PcgScal sc, PcgFlags fl, double rtol2) {
+                                               const double *__restrict__ ds, T *__restrict__ ws, double *part,
+                                               PcgScal sc, PcgFlags fl) {
   __shared__ double sums[NP];
   double alpha[NP], v[NP];
 #pragma unroll
@@ -644,7 +709,8 @@ __global__ void __launch_bounds__(PT) k_update(double *__restrict__ x, double *_
     alpha[j] = sc.alpha[j];
     v[j] = 0.0;
   }
-  for (int64_t i = blockIdx.x * (int64_t)PT + threadIdx.x; i < n; i += (int64_t)gridDim.x * PT)
+  for (int64_t i = blockIdx.x * (int64_t)PT + threadIdx.x; i < n; i += (int64_t)gridDim.x * PT) {
+    const double d = ds ? ds[i] : 1.0;
 #pragma unroll
     for (int j = 0; j < NP; ++j) {
       const int64_t e = i * NP + j;
@@ -652,8 +718,10 @@ __global__ void __launch_bounds__(PT) k_update(double *__restrict__ x, double *_
       const double rv = fma(-alpha[j], q[e], r[e]);
       x[e] = xv;
       r[e] = rv;
+      ws[e] = (T)(ds ? rv * d : rv);
       v[j] = fma(rv, rv, v[j]);
     }
+  }
   block_partial<NP>(v, part);
   if (!finish_sum<NP>(part, fl.counter, sums)) return;
   const int j = threadIdx.x;
@@ -661,7 +729,7 @@ __global__ void __launch_bounds__(PT) k_update(double *__restrict__ x, double *_
     sc.rr[j] = sums[j];
     if (fl.active[j]) {
       fl.iters[j] += 1;
-      if (sums[j] <= rtol2 * sc.bnorm2[j]) fl.active[j] = 0;
+      if (sums[j] <= sc.tol2[j]) fl.active[j] = 0;
     }
   }
   __syncthreads();
@@ -707,7 +775,7 @@ int grid_for(int64_t total) {
 }
 
 // grid of the PCG reduction kernels: a function of n only (see above)
-int rgrid_for(int64_t n) { return grid_for(n); }
+int rgrid_for(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>((n + PT - 1) / PT, 152 * 4)); }
 
 // One pass of Algorithm 2 over right-hand sides [j0, j0 + NR) of the
 // workspace ws (layout [unknown][nrhs]); tb0 and tb1 are the scratch of even and
@@ -956,7 +1024,7 @@ void ensure_buffers(FactorHandle &h, int nrhs_cap, cudaStream_t st) {
   h.alloc.get(&h.d_pcg, sizeof(double) * 7 * n * nrhs_cap, st);
   h.part_blocks = 152 * 8;
   h.alloc.get(&h.d_part, sizeof(double) * h.part_blocks * 32, st);
-  h.alloc.get(&h.d_scal, sizeof(double) * 6 * 32, st);
+  h.alloc.get(&h.d_scal, sizeof(double) * 7 * 32, st);
   h.alloc.get(&h.d_iflags, sizeof(int) * (2 * 32 + 2), st);
   HS_CUDA(cudaMemset(h.d_iflags, 0, sizeof(int) * (2 * 32 + 2)));
   if (!h.h_done) HS_CUDA(cudaMallocHost(&h.h_done, sizeof(int)));
@@ -1143,50 +1211,47 @@ int pcg_solve(FactorHandle &h, const double *b, double *x, int nrhs, int64_t ld,
   const int64_t n = h.plan.n;
   const int64_t tot = n * np;
   double *X = h.d_pcg, *R = X + tot, *P0 = R + tot, *P1 = P0 + tot, *Q = P1 + tot, *B = Q + tot, *Z = B + tot;
-  PcgScal sc{h.d_scal, h.d_scal + 32, h.d_scal + 64, h.d_scal + 96, h.d_scal + 128, h.d_scal + 160};
+  PcgScal sc{h.d_scal,      h.d_scal + 32,  h.d_scal + 64, h.d_scal + 96,
+             h.d_scal + 128, h.d_scal + 160, h.d_scal + 192};
   PcgFlags fl{h.d_iflags, h.d_iflags + 32, h.d_iflags + 64, h.d_iflags + 65};
   const int g = rgrid_for(n);
   const double rtol2 = rtol * rtol;
-  k_gather_in<double><<<grid_for(tot), 256, 0, st>>>(b, ld, h.d_perm, n, nrhs, np, B, nullptr);
-  count_launch();
-  HS_CUDA(cudaMemcpyAsync(R, B, sizeof(double) * tot, cudaMemcpyDeviceToDevice, st));
-  HS_CUDA(cudaMemsetAsync(X, 0, sizeof(double) * tot, st));
-  HS_CUDA(cudaMemsetAsync(P0, 0, sizeof(double) * tot, st));
-  with_np(np, [&](auto c) {
-    constexpr int NP = decltype(c)::value;
-    k_dot<NP><<<g, PT, 0, st>>>(B, B, n, h.d_part, sc, fl, DOT_BNORM, nullptr);
-  });
-  count_launch();
-  // z = A_H^-1 r ; first direction p = z (beta = 0)
-  apply_pcg(h, R, Z, np, st, !graphs_enabled());
-  with_np(np, [&](auto c) {
-    constexpr int NP = decltype(c)::value;
-    k_dot<NP><<<g, PT, 0, st>>>(R, Z, n, h.d_part, sc, fl, DOT_RZ_FIRST, nullptr);
-    k_spmv_p<NP><<<g, PT, 0, st>>>(h.d_rowptr, h.d_col, h.d_val, n, Z, P0, P1, Q, h.d_part, sc, fl);
-    k_update<NP><<<g, PT, 0, st>>>(X, R, P1, Q, n, h.d_part, sc, fl, rtol2);
-  });
-  count_launch(3);
-  HS_CUDA(cudaGetLastError());
-  // One iteration after the first: z = A_H^-1 r, beta, p_new = z + beta p_old,
-  // q = A p_new, alpha, x and r updates.  Right-hand sides that have converged
-  // get alpha = beta = 0 and stay as they are.  Recorded as a graph per
-  // direction buffer pair.
-  auto body = [&, np](cudaStream_t cs, double *pold, double *pnew) {
-    apply_pcg(h, R, Z, np, cs, true);
+  auto with_t = [&](auto &&f) {
+    if (h.prec == HS_PREC_F64)
+      f((double *)h.d_ws);
+    else
+      f((float *)h.d_ws);
+  };
+  with_t([&](auto *ws) {
+    using T = std::remove_pointer_t<decltype(ws)>;
     with_np(np, [&](auto c) {
       constexpr int NP = decltype(c)::value;
-      k_dot<NP><<<g, PT, 0, cs>>>(R, Z, n, h.d_part, sc, fl, DOT_RZ, nullptr);
-      k_spmv_p<NP><<<g, PT, 0, cs>>>(h.d_rowptr, h.d_col, h.d_val, n, Z, pold, pnew, Q, h.d_part, sc, fl);
-      k_update<NP><<<g, PT, 0, cs>>>(X, R, pnew, Q, n, h.d_part, sc, fl, rtol2);
+      k_start<T, NP><<<g, PT, 0, st>>>(b, ld, h.d_perm, n, nrhs, h.d_dscale, B, R, X, P0, ws, h.d_part, sc, fl,
+                                       rtol2);
+    });
+  });
+  count_launch();
+  HS_CUDA(cudaGetLastError());
+  // One iteration: z = A_H^-1 r (r is in the workspace already), beta, p_new =
+  // z + beta p_old, q = A p_new, alpha, x and r updates.  Right-hand sides that
+  // have converged get alpha = beta = 0 and stay as they are.  Recorded as a
+  // graph per direction buffer pair; nothing of one call (its tolerance,
+  // buffers or iteration limit) is in it.
+  auto body = [&, np](cudaStream_t cs, double *pold, double *pnew) {
+    apply_ws_direct(h, np, cs);
+    with_t([&](auto *ws) {
+      using T = std::remove_pointer_t<decltype(ws)>;
+      with_np(np, [&](auto c) {
+        constexpr int NP = decltype(c)::value;
+        k_zdot<T, NP><<<g, PT, 0, cs>>>(ws, h.d_dscale, R, n, Z, h.d_part, sc, fl);
+        k_spmv_p<NP><<<g, PT, 0, cs>>>(h.d_rowptr, h.d_col, h.d_val, n, Z, pold, pnew, Q, h.d_part, sc, fl);
+        k_update<T, NP><<<g, PT, 0, cs>>>(X, R, pnew, Q, n, h.d_dscale, ws, h.d_part, sc, fl);
+      });
     });
     count_launch(3);
     HS_CUDA(cudaGetLastError());
   };
-  int it = 1;
-  while (true) {
-    HS_CUDA(cudaMemcpyAsync(h.h_done, fl.done, sizeof(int), cudaMemcpyDeviceToHost, st));
-    HS_CUDA(cudaStreamSynchronize(st));
-    if (*h.h_done || it >= maxit) break;
+  for (int it = 0;;) {
     // after an odd number of iterations the latest direction is in P1
     double *pold = (it & 1) ? P1 : P0, *pnew = (it & 1) ? P0 : P1;
     if (graphs_enabled()) {
@@ -1196,6 +1261,9 @@ int pcg_solve(FactorHandle &h, const double *b, double *x, int nrhs, int64_t ld,
       body(st, pold, pnew);
     }
     ++it;
+    HS_CUDA(cudaMemcpyAsync(h.h_done, fl.done, sizeof(int), cudaMemcpyDeviceToHost, st));
+    HS_CUDA(cudaStreamSynchronize(st));
+    if (*h.h_done || it >= maxit) break;
   }
   // true relative residual
   k_residual<<<grid_for(tot), 256, 0, st>>>(h.d_rowptr, h.d_col, h.d_val, n, np, X, B, Q);
@@ -1203,7 +1271,7 @@ int pcg_solve(FactorHandle &h, const double *b, double *x, int nrhs, int64_t ld,
   double *rr_d = h.d_scal + 5 * 32;
   with_np(np, [&](auto c) {
     constexpr int NP = decltype(c)::value;
-    k_dot<NP><<<g, PT, 0, st>>>(Q, Q, n, h.d_part, sc, fl, DOT_PLAIN, rr_d);
+    k_dot<NP><<<g, PT, 0, st>>>(Q, Q, n, h.d_part, fl, rr_d);
   });
   count_launch();
   k_scatter_out<double><<<grid_for(n * nrhs), 256, 0, st>>>(X, h.d_perm, n, nrhs, np, x, ld, nullptr);
