@@ -355,7 +355,7 @@ int eig_small_max() {
     const int cap = std::min(32, jacobi_cap<T>());
     if (!e) return cap;
     const int x = std::atoi(e);
-    return x < 0 ? cap : std::min(x, cap);
+    return x < 0 ? cap : std::min(std::max(x, 8), cap);   // the tridiagonal path needs m > 8
   }();
   return v;
 }
@@ -369,20 +369,6 @@ inline bool tri_cluster_enabled() {
   static const bool v = [] {
     const char *e = std::getenv("HS_TRI_CLUSTER");
     return !(e && e[0] == '0');
-  }();
-  return v;
-}
-
-// Smallest super node whose truncation takes the multi-CTA path (cluster or
-// step-kernel tridiagonalisation, eigenvectors of T for the whole wave,
-// reflector products by batches of columns); below it one CTA per node does
-// everything (default 64).  HS_GRID_TRIDIAG_MIN (environment) moves the
-// limit, which lets small test problems exercise the path.
-inline int grid_tridiag_min() {
-  static const int v = [] {
-    const char *e = std::getenv("HS_GRID_TRIDIAG_MIN");
-    const int x = e ? std::atoi(e) : 0;
-    return x > 3 ? x : 64;
   }();
   return v;
 }
@@ -1621,26 +1607,50 @@ void Run<T>::finish() {
   h_.info.alg_flops = alg_flops_;
 }
 
-// Truncation of very large nodes across the whole GPU: k_trunc_big up to J
-// (TB_PREP), the tridiagonal steps (two launches per step over all the nodes'
-// CTAs), Z = Q^T [U1, X] (GC), k_trunc_big from T to its eigenvectors
-// (TB_POST), then U_2 = Q Y by batches of columns.
+// A list of tasks, each owning consecutive CTAs from its blk0 on, uploaded.
+template <typename X>
+const X *upload_list(Exec &ex, const std::vector<X> &v) {
+  Uploader u;
+  const size_t o = u.add(v);
+  char *d = u.upload(ex.scr, ex.sg, ex.st);
+  return (const X *)(d + o);
+}
+
+// Truncation of a wave's nodes above the Jacobi limit (kernels_eig.cu): U_1 and
+// J, the tridiagonalisation, Z = Q^T X (GC), the ranks, the eigenvalues and
+// eigenvectors of T, and U_2 = Q Y.  eps = 0 ends after the first (complete
+// bases).
 template <typename T>
-void trunc_grid(Exec &ex, const std::vector<TruncTask<T>> &tasks, const TruncTask<T> *d_tasks, int *d_k,
-                double eps, int variant, int max_m) {
-  const int n = (int)tasks.size();
+void trunc_big(Exec &ex, const std::vector<TruncTask<T>> &all, int *d_k, int variant) {
+  std::vector<TruncTask<T>> prep[2], tasks;
+  int pmax[2] = {0, 0}, max_m = 0, max_np = 1;
+  for (const TruncTask<T> &t : all) {
+    const int c = t.m <= kTruncPrepMid ? 0 : 1;
+    prep[c].push_back(t);
+    pmax[c] = std::max(pmax[c], t.m);
+    if (t.eps > 0.0) {
+      tasks.push_back(t);
+      max_m = std::max(max_m, t.m);
+      max_np = std::max(max_np, t.np);
+    }
+  }
   // nested spans (phases 10-14) inside the large-truncation span (5)
   ex.begin(10);
-  launch_trunc_big_mode<T>(d_tasks, n, d_k, eps, variant, max_m, 1 /* TB_PREP */, ex.st);
+  for (int c = 0; c < 2; ++c)
+    if (!prep[c].empty())
+      launch_trunc_prep<T>(upload_list(ex, prep[c]), (int)prep[c].size(), d_k, variant, pmax[c], ex.st);
   ex.end();
-  std::vector<GridTri<T>> gt(n);
-  int blocks = 0;
-  for (int q = 0; q < n; ++q) {
-    const TruncTask<T> &t = tasks[q];
+  const int n = (int)tasks.size();
+  if (n == 0) return;
+  // nodes that fit a thread-block cluster's shared memory are tridiagonalised
+  // there in one launch per cluster size; the others by the step kernels
+  std::vector<GridTri<T>> by_c[4], steps;
+  int cmax[4] = {0, 0, 0, 0}, smax = 0, sblocks = 0;
+  for (const TruncTask<T> &t : tasks) {
     const BigLayout<T> L = big_layout<T>(t.work, t.m);
-    GridTri<T> &g = gt[q];
+    GridTri<T> g;
     g.A = L.A;
-    g.X = L.Y;                 // the step vectors live in Y until TB_POST
+    g.X = L.Y;                 // the step vectors live in Y until the eigenvectors go there
     g.P = L.Y + t.m;
     g.V = L.Y + 2 * (size_t)t.m;
     g.px = L.Y + 3 * (size_t)t.m;
@@ -1650,30 +1660,18 @@ void trunc_grid(Exec &ex, const std::vector<TruncTask<T>> &tasks, const TruncTas
     g.tau = L.tau;
     g.m = t.m;
     g.nblk = (t.m + kTriRows - 1) / kTriRows;
-    g.blk0 = blocks;
-    blocks += g.nblk;
-  }
-  // nodes that fit a thread-block cluster's shared memory are tridiagonalised
-  // there in one launch per cluster size; the others by the step kernels
-  std::vector<GridTri<T>> by_c[4], steps;
-  int cmax[4] = {0, 0, 0, 0}, smax = 0;
-  for (const GridTri<T> &g : gt) {
+    g.blk0 = 0;
     const int c = tri_cluster_enabled() ? tri_cluster_size<T>(g.m) : 0;
     if (c > 0) {
       const int q = c == 1 ? 0 : c == 2 ? 1 : c == 4 ? 2 : 3;
       by_c[q].push_back(g);
       cmax[q] = std::max(cmax[q], g.m);
     } else {
-      GridTri<T> h = g;
-      h.blk0 = 0;
-      steps.push_back(h);
+      g.blk0 = sblocks;
+      sblocks += g.nblk;
+      steps.push_back(g);
       smax = std::max(smax, g.m);
     }
-  }
-  int sblocks = 0;
-  for (GridTri<T> &g : steps) {
-    g.blk0 = sblocks;
-    sblocks += g.nblk;
   }
   Uploader u;
   const size_t og = u.add(steps);
@@ -1700,62 +1698,55 @@ void trunc_grid(Exec &ex, const std::vector<TruncTask<T>> &tasks, const TruncTas
     HS_CUDA(cudaStreamWaitEvent(ex.st, ex.join_ev, 0));
   }
   ex.end();
-  (void)blocks;
-  const int nb = refl_batch<T>(max_m);
-  if (variant != HS_LORASP) {
-    // Z = Q^T [U_1, G U_1] has 2 k1 <= 4 np columns, in batches of up to 4
-    const int nbz = std::min(nb, 4);
-    std::vector<ReflTask<T>> zf;
+  // products with Q: by warps up to kQmulMax, by CTAs above
+  auto products = [&](bool fwd) {
+    std::vector<QmulTask<T>> qm;
+    std::vector<ReflTask<T>> rf;
+    int blocks = 0, qmax = 0;
+    const int nb = fwd ? std::min(refl_batch<T>(max_m), 4) : refl_batch<T>(max_m);
     for (const TruncTask<T> &t : tasks) {
       const BigLayout<T> L = big_layout<T>(t.work, t.m);
-      for (int j0 = 0; j0 < 4 * std::max(t.np, 1); j0 += nbz)
-        zf.push_back(ReflTask<T>{L.A, L.tau, L.LS, t.U, L.sc_int, t.m, j0, 1});
+      const int ncol = fwd ? std::min(2 * std::max(t.np, 1), t.m) : t.m;   // at most; the kernels know k1 and k2
+      T *cols = fwd ? L.LS : L.Y;
+      if (t.m <= kQmulMax) {
+        qm.push_back(QmulTask<T>{L.A, L.tau, cols, t.U, L.sc_int, t.m, fwd ? 1 : 0, blocks});
+        blocks += qmul_blocks<T>(t.m, ncol);
+        qmax = std::max(qmax, t.m);
+      } else {
+        for (int j0 = 0; j0 < ncol; j0 += nb)
+          rf.push_back(ReflTask<T>{L.A, L.tau, cols, t.U, L.sc_int, t.m, j0, fwd ? 1 : 0});
+      }
     }
-    Uploader uz;
-    const size_t oz = uz.add(zf);
-    char *dz = uz.upload(ex.scr, ex.sg, ex.st);
+    if (!qm.empty()) launch_qmul<T>(upload_list(ex, qm), (int)qm.size(), blocks, qmax, fwd, ex.st);
+    if (!rf.empty()) launch_refl<T>(upload_list(ex, rf), (int)rf.size(), nb, max_m, ex.st);
+  };
+  if (variant != HS_LORASP) {
     ex.begin(12);
-    launch_refl<T>((const ReflTask<T> *)(dz + oz), (int)zf.size(), nbz, max_m, ex.st);
+    products(true);   // Z = Q^T X
     ex.end();
   }
   ex.begin(13);
-  launch_trunc_big_mode<T>(d_tasks, n, d_k, eps, variant, max_m, 2 /* TB_POST */, ex.st);
+  launch_rank<T>(upload_list(ex, tasks), n, d_k, variant, max_m, max_np, ex.st);
   {
-    // eigenvectors of T: clusters spread over many CTAs (at most m per node)
+    // eigenvalues and eigenvectors of T (at most m per node)
     const int spc = invit_slots<T>(max_m);
-    std::vector<InvitTask<T>> it;
-    int iblocks = 0;
+    std::vector<EigTask<T>> ev, it;
+    int eblocks = 0, iblocks = 0;
     for (const TruncTask<T> &t : tasks) {
       const BigLayout<T> L = big_layout<T>(t.work, t.m);
-      InvitTask<T> x;
-      x.dt = L.dt;
-      x.et = L.et;
-      x.lam = L.lam;
-      x.starts = (const int *)L.pw;
-      x.sc = L.sc_int;
-      x.tnorm = L.sc_tnorm;
-      x.Y = L.Y;
-      x.m = t.m;
+      EigTask<T> x{L.dt, L.et, L.lam, L.sc_int, L.sc_b, L.sc_tnorm, L.Y, t.m, eblocks};
+      ev.push_back(x);
+      eblocks += eigval_blocks<T>(t.m);
       x.blk0 = iblocks;
-      iblocks += (t.m + spc - 1) / spc;
       it.push_back(x);
+      iblocks += (t.m + spc - 1) / spc;
     }
-    Uploader ui;
-    const size_t oi = ui.add(it);
-    char *di = ui.upload(ex.scr, ex.sg, ex.st);
-    launch_invit<T>((const InvitTask<T> *)(di + oi), (int)it.size(), iblocks, spc, max_m, ex.st);
+    launch_eigval<T>(upload_list(ex, ev), n, eblocks, max_m, ex.st);
+    launch_invit<T>(upload_list(ex, it), n, iblocks, spc, max_m, ex.st);
   }
   ex.end();
-  std::vector<ReflTask<T>> yb;
-  for (const TruncTask<T> &t : tasks) {
-    const BigLayout<T> L = big_layout<T>(t.work, t.m);
-    for (int j0 = 0; j0 < t.m; j0 += nb) yb.push_back(ReflTask<T>{L.A, L.tau, L.Y, t.U, L.sc_int, t.m, j0, 0});
-  }
-  Uploader uy;
-  const size_t oy = uy.add(yb);
-  char *dy = uy.upload(ex.scr, ex.sg, ex.st);
   ex.begin(14);
-  launch_refl<T>((const ReflTask<T> *)(dy + oy), (int)yb.size(), nb, max_m, ex.st);
+  products(false);   // U_2 = Q Y
   ex.end();
 }
 
@@ -1791,33 +1782,6 @@ struct HostClock {
 // Runs the factorizations of `runs` in lock step: at every step (level counted
 // from the leaves, wave index) the work of all problems that have that step
 // goes into one launch per kernel kind, with one read of the new ranks.
-// The large-node truncation tasks of a wave split by class (256 or 1024
-// threads per node, or the multi-CTA path), uploaded, then launched.
-template <typename U>
-struct BigClasses {
-  std::vector<TruncTask<U>> cls[3];
-  int cmax[3] = {0, 0, 0};
-  size_t o[3] = {0, 0, 0};
-  char *d = nullptr;
-  void prepare(Exec &ex, const std::vector<TruncTask<U>> &tasks) {
-    for (const TruncTask<U> &t : tasks) {
-      const int c = (t.eps > 0.0 && t.m >= grid_tridiag_min()) ? 2 : t.m <= kTruncBigMidMax ? 0 : 1;
-      cls[c].push_back(t);
-      cmax[c] = std::max(cmax[c], t.m);
-    }
-    Uploader u;
-    o[0] = u.add(cls[0]);
-    o[1] = u.add(cls[1]);
-    o[2] = u.add(cls[2]);
-    d = u.upload(ex.scr, ex.sg, ex.st);
-  }
-  void launch(Exec &ex, int *d_k, double eps, int variant) {
-    launch_trunc_big<U>((const TruncTask<U> *)(d + o[0]), (int)cls[0].size(), d_k, eps, variant, cmax[0], ex.st);
-    launch_trunc_big<U>((const TruncTask<U> *)(d + o[1]), (int)cls[1].size(), d_k, eps, variant, cmax[1], ex.st);
-    if (!cls[2].empty()) trunc_grid<U>(ex, cls[2], (const TruncTask<U> *)(d + o[2]), d_k, eps, variant, cmax[2]);
-  }
-};
-
 template <typename T>
 void execute(Exec &ex, std::vector<std::unique_ptr<Run<T>>> &runs) {
   const auto t_start = std::chrono::steady_clock::now();
@@ -1911,16 +1875,10 @@ void execute(Exec &ex, std::vector<std::unique_ptr<Run<T>>> &runs) {
         ex.end();
       }
       if (nbig || nb64) {
-        // one launch per class (k_idx keeps each rank's slot): 256 or 1024
-        // threads per node, or the multi-CTA path for very large nodes
-        BigClasses<T> bc;
-        BigClasses<double> bc64;
-        if (nbig) bc.prepare(ex, B.trunc_big);
-        if (nb64) bc64.prepare(ex, B.trunc_big64);
         ex.begin(5);
         HS_CUDA(cudaEventRecord(ex.ev_big[0], ex.st));
-        if (nbig) bc.launch(ex, d_k, eps, variant);
-        if (nb64) bc64.launch(ex, d_k, eps, variant);
+        if (nbig) trunc_big<T>(ex, B.trunc_big, d_k, variant);
+        if (nb64) trunc_big<double>(ex, B.trunc_big64, d_k, variant);
         HS_CUDA(cudaEventRecord(ex.ev_big[1], ex.st));
         ex.end();
       }

@@ -188,53 +188,48 @@ void launch_chol_inv(const CholTask<T> *d_tasks, int ntasks, int *d_status, int 
 template <typename T>
 void launch_trunc(const TruncTask<T> *d_tasks, int ntasks, int *d_k, double eps, int variant,
                   int max_m, cudaStream_t st);
-// large super nodes (kernels_eig.cu): tridiagonalisation / bisection / inverse iteration
-// Global work area of one large-truncation node (offsets from TruncTask::work;
-// the host computes the same addresses for the multi-CTA kernels):
+// super nodes above the Jacobi limit (kernels_eig.cu): tridiagonalisation /
+// multisection / inverse iteration.
+// Global work area of one such node (offsets from TruncTask::work; the host
+// computes the same addresses):
 //   A (m^2 T)   Gram / J, then the Householder reflectors in its rows
-//   Y (m^2 T)   eigenvectors of T; before that the multi-CTA tridiagonalisation
-//               keeps its step vectors here
-//   LU (4 m^2 T), LS (164 m T), FL (m^2 bytes): inverse iteration and Z
-//   VG          the per-node vectors (d, e, pw in FP64; dt, et, lam, v, tau, wt,
-//               redt in T) when they are not in shared memory
-//   SC          persistent scalars between the kernels of the multi-CTA path:
-//               k1, k2, cluster count (ints), the norm bound of T, then
-//               c = U1^T G U1 (kMaxK1 x kMaxK1 doubles)
+//   Y (m^2 T)   eigenvectors of T; before that G U_1 and the step kernels' vectors
+//   LS (32 m T) X, then Z = Q^T X (k1 columns); before that scratch of U_1
+//   VG          the per-node vectors (d, e in FP64; dt, et, lam, tau in T)
+//   SC          scalars passed between the kernels: k1, k2 (ints), the norm
+//               bound of T, C = U1^T G U1 (kMaxK1 x kMaxK1 doubles), and
+//               eps^2 lambda_max, the Gershgorin bound of T, max e^2
 template <typename T>
 struct BigLayout {
-  T *A, *Y, *LU, *LS;
-  unsigned char *FL, *VG;
-  double *d, *e, *pw;
-  T *dt, *et, *lam, *v, *tau, *wt, *redt;
-  int *sc_int;        // k1, k2, number of eigenvalue clusters
-  double *sc_c;       // c = U1^T G U1 (kMaxK1 x kMaxK1 doubles, ld kMaxK1)
+  T *A, *Y, *LS;
+  double *d, *e;
+  T *dt, *et, *lam, *tau;
+  int *sc_int;        // k1, k2
+  double *sc_c;       // C (kMaxK1 x kMaxK1 doubles, ld kMaxK1)
+  double *sc_b;       // eps^2 lambda_max, upper bound of the spectrum of T, max e^2
   double *sc_tnorm;   // norm bound of T (inverse-iteration tolerance)
 };
 
 template <typename T>
 __host__ __device__ inline size_t big_vec_bytes(int m) {
-  return 3 * sizeof(double) * (size_t)m + 6 * sizeof(T) * (size_t)((m + 1) & ~1) + 34 * sizeof(T) + 16;
+  return 2 * sizeof(double) * (size_t)m + 4 * sizeof(T) * (size_t)((m + 1) & ~1);
 }
 
 // bytes of the SC area (after its 16-byte alignment)
-constexpr size_t kBigScBytes = 24 + sizeof(double) * kMaxK1 * kMaxK1;
+constexpr size_t kBigScBytes = 24 + sizeof(double) * (kMaxK1 * kMaxK1 + 3);
 
 template <typename T>
 __host__ __device__ inline BigLayout<T> big_layout(T *work, int m) {
   BigLayout<T> L;
   L.A = work;
   L.Y = work + (size_t)m * m;
-  L.LU = L.Y + (size_t)m * m;
-  L.LS = L.LU + 4 * (size_t)m * m;
-  L.FL = (unsigned char *)(L.LS + 164 * (size_t)m);
-  L.VG = (unsigned char *)(((uintptr_t)(L.FL + (size_t)m * m) + 15) & ~(uintptr_t)15);
+  // also read as doubles
+  L.LS = (T *)(((uintptr_t)(L.Y + (size_t)m * m) + 15) & ~(uintptr_t)15);
+  unsigned char *p = (unsigned char *)(L.LS + 32 * (size_t)m);
   const size_t me = (size_t)((m + 1) & ~1);
-  unsigned char *p = L.VG;
   L.d = (double *)p;
   p += sizeof(double) * m;
   L.e = (double *)p;
-  p += sizeof(double) * m;
-  L.pw = (double *)p;
   p += sizeof(double) * m;
   L.dt = (T *)p;
   p += sizeof(T) * me;
@@ -242,17 +237,13 @@ __host__ __device__ inline BigLayout<T> big_layout(T *work, int m) {
   p += sizeof(T) * me;
   L.lam = (T *)p;
   p += sizeof(T) * me;
-  L.v = (T *)p;
-  p += sizeof(T) * me;
   L.tau = (T *)p;
   p += sizeof(T) * me;
-  L.wt = (T *)p;
-  p += sizeof(T) * me;
-  L.redt = (T *)p;
-  unsigned char *sc = (unsigned char *)(((uintptr_t)(L.VG + big_vec_bytes<T>(m)) + 15) & ~(uintptr_t)15);
+  unsigned char *sc = (unsigned char *)(((uintptr_t)p + 15) & ~(uintptr_t)15);
   L.sc_int = (int *)sc;
   L.sc_tnorm = (double *)(sc + 16);
   L.sc_c = (double *)(sc + 24);
+  L.sc_b = L.sc_c + kMaxK1 * kMaxK1;
   return L;
 }
 
@@ -271,21 +262,34 @@ struct GridTri {
   int m, nblk, blk0;
 };
 
-// Inverse iteration of a node's selected eigenvalues (multi-CTA path): the
-// clusters of close eigenvalues (starts, count in sc[2]) are spread one per
-// thread over many CTAs, each thread's LU and vector in shared memory.
+// Eigenvalues of a node's T and their inverse iteration: T in the factor
+// precision, the eigenvalues, the node's scalars (SC), the eigenvectors (column
+// q at Y + q m), and the node's first CTA in the launch
 template <typename T>
-struct InvitTask {
-  const T *dt, *et, *lam;
-  const int *starts;
+struct EigTask {
+  const T *dt, *et;
+  T *lam;
   const int *sc;
+  const double *sb;
   const double *tnorm;
-  T *Y;              // eigenvectors of T, column q at Y + q m
+  T *Y;
   int m, blk0;
 };
 
-// Products with Q = H_0 ... H_{m-3} of a node's reflectors: forward (Q^T, the
-// 2 k1 columns of Z, in place) or backward (Q Y into U columns k1..).  A task is
+// Products with Q by warps (m <= kQmulMax): the columns (column-major, ld m),
+// for the backward product U (row-major m x m), the node's first CTA
+constexpr int kQmulMax = 1024;
+template <typename T>
+struct QmulTask {
+  const T *A;
+  const T *tau;
+  T *cols;
+  T *U;
+  const int *sc;
+  int m, fwd, blk0;
+};
+
+// The same for larger nodes: forward (Q^T, the k1 columns of Z, in place) or backward (Q Y into U columns k1..).  A task is
 // one batch of columns [j0, j0 + nb) of one node; k1, k2 come from the node's
 // scalar area (sc).
 template <typename T>
@@ -298,19 +302,29 @@ struct ReflTask {
   int m, j0, fwd;
 };
 
-// Large-node truncations of m <= kTruncBigMidMax run 256 threads per node,
-// larger ones 1024; launch_trunc_big takes tasks of one class at a time.
-constexpr int kTruncBigMidMax = 128;
+// k_trunc_prep runs 256 threads per node up to this m, 1024 above; a launch
+// takes tasks of one class
+constexpr int kTruncPrepMid = 256;
 
 template <typename T>
 size_t trunc_big_work_elems(int m);
+// U_1, J and X of each node; for eps = 0 the complete basis and its rank instead
 template <typename T>
-void launch_trunc_big(const TruncTask<T> *d_tasks, int ntasks, int *d_k, double eps, int variant,
-                      int max_m, cudaStream_t st);
-// the multi-CTA path: k_trunc_big in one of its modes (TB_PREP = 1, TB_POST = 2)
+void launch_trunc_prep(const TruncTask<T> *d_tasks, int ntasks, int *d_k, int variant, int max_m, cudaStream_t st);
+// ranks from the tridiagonals (max_np: most preserved vectors of the tasks)
 template <typename T>
-void launch_trunc_big_mode(const TruncTask<T> *d_tasks, int ntasks, int *d_k, double eps, int variant, int max_m,
-                           int mode, cudaStream_t st);
+void launch_rank(const TruncTask<T> *d_tasks, int ntasks, int *d_k, int variant, int max_m, int max_np,
+                 cudaStream_t st);
+// CTAs of launch_eigval for a node of size m
+template <typename T>
+int eigval_blocks(int m);
+template <typename T>
+void launch_eigval(const EigTask<T> *d_tasks, int ntasks, int total_blocks, int m_max, cudaStream_t st);
+// CTAs of launch_qmul for ncol columns of a node of size m <= kQmulMax
+template <typename T>
+int qmul_blocks(int m, int ncol);
+template <typename T>
+void launch_qmul(const QmulTask<T> *d_tasks, int ntasks, int total_blocks, int m_max, bool fwd, cudaStream_t st);
 // one step k of the multi-CTA tridiagonalisation over `total_blocks` CTAs
 // (phase 0: apply step k-1's update and take column k; phase 1: reflector
 // and p = tau A v)
@@ -326,7 +340,7 @@ template <typename T>
 void launch_tri_cluster(const GridTri<T> *d_tasks, int ntasks, int C, int m_max, cudaStream_t st);
 // inverse iteration over total_blocks CTAs of `spc` slots each
 template <typename T>
-void launch_invit(const InvitTask<T> *d_tasks, int ntasks, int total_blocks, int spc, int m_max, cudaStream_t st);
+void launch_invit(const EigTask<T> *d_tasks, int ntasks, int total_blocks, int spc, int m_max, cudaStream_t st);
 // slots per CTA of launch_invit for nodes of size up to m
 template <typename T>
 int invit_slots(int m);

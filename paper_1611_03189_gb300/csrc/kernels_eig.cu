@@ -1,29 +1,36 @@
-// Truncation of large super nodes (m above the shared-memory Jacobi limit):
-// symmetric eigen-decomposition of the Gram matrix by Householder
-// tridiagonalisation, Sturm-sequence bisection and inverse iteration.
-//
-// One CTA per super node: 256 threads for m <= 128, 1024 above (a function of
-// m alone, so a node gets the same arithmetic in any batch):
-//   1. GC basis U_1 = orth[phi_s, A_sw phi_w] (Sec. 6; Appendix B: its dominant
-//      left singular vectors), as in the Jacobi path.
-//   2. ||A_sw||_2^2 = lambda_max(G).  LoRaSp: top eigenvalue of T below.  GC:
-//      G = J + (rank <= 2 k1 terms in span{U_1, G U_1}), so lambda_max(G) follows
-//      from the tridiagonal T of J by a warp multisection on the Haynsworth
-//      inertia count of the low-rank correction (no second tridiagonalisation).
-//   3. J = G (LoRaSp), (I - U1 U1^T) G (I - U1 U1^T) (GC) or I - U1 U1^T (GC,
-//      eps = 0).  Tridiagonalise J = Q T Q^T; k2 = #{lambda(T) > thr} by one
-//      Sturm count (FP64), thr = eps^2 lambda_max(G) (Sec. 3.2, strict).
-//   4. The k2 largest eigenvalues of T by bisection (FP64), their eigenvectors
-//      by inverse iteration on T (tridiagonal LU with partial pivoting, three
-//      steps, modified Gram-Schmidt inside clusters of eigenvalues closer than
-//      10 u ||T||), then U_2 = Q Y by the stored Householder reflectors.
+// Truncation of super nodes above the shared-memory Jacobi limit: symmetric
+// eigen-decomposition of the Gram matrix by Householder tridiagonalisation,
+// Sturm-sequence multisection and inverse iteration.  Per wave, one launch of
+// each kernel for all its nodes:
+//   1. k_trunc_prep (one CTA per node): GC basis U_1 = orth[phi_s, A_sw phi_w]
+//      (Sec. 6; Appendix B: its dominant left singular vectors), J = G (LoRaSp)
+//      or (I - U1 U1^T) G (I - U1 U1^T) (GC), and with C = U1^T G U1 the
+//      coupling X = (I - U1 U1^T) G U1 of the two blocks of G.
+//   2. J = Q T Q^T (kernels_cluster.cu, or the step kernels below), and
+//      Z = Q^T X (k_qmul).
+//   3. k_rank (one CTA per node): ||A_sw||_2^2 = lambda_max(G), from T (LoRaSp)
+//      or from the inertia of G - sigma I in the basis [U_1, its complement]
+//      (GC); the rank k2 = #{lambda(T) > eps^2 lambda_max(G)} by one Sturm count
+//      in FP64 (Sec. 3.2, strict).
+//   4. k_eigval: the k2 largest eigenvalues of T, 8 or 32 lanes each.
+//   5. k_invit: their eigenvectors by inverse iteration on T (tridiagonal LU
+//      with partial pivoting, three steps, modified Gram-Schmidt inside
+//      clusters of eigenvalues closer than 10 u ||T||), one lane each.
+//   6. k_qmul: U_2 = Q Y by the stored reflectors, a few columns per warp.
 // The host re-orthonormalises [U_1, U_2] afterwards (CholQR2), which keeps its
-// span.  The tridiagonalisation works in global memory until the trailing
-// block fits in shared memory, then finishes there.
+// span.  What a kernel does for a node depends on the node alone, so it gets
+// the same bits in any batch.
+//
+// All of it is bound by chains of dependent steps (a division per row of T, a
+// reduction per reflector), not by arithmetic or bandwidth, so the kernels cut
+// the number of steps (many points of a section at once), spread the
+// eigenvalues over the SMs, and keep the chains in registers and shared
+// memory.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
 #include <algorithm>
+#include <cstdlib>
 
 #include "hs_internal.h"
 #include "trunc_common.cuh"
@@ -31,24 +38,6 @@
 namespace hs {
 
 namespace {
-
-
-__device__ double bsum(double v, double *red) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();
-  if (l == 0) red[w] = v;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double s = (threadIdx.x < (blockDim.x >> 5)) ? red[threadIdx.x] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (threadIdx.x == 0) red[32] = s;
-  }
-  __syncthreads();
-  const double s = red[32];
-  __syncthreads();
-  return s;
-}
 
 // Block-wide sum in T (red: 33 T of shared memory); every thread gets the total.
 // Reductions inside the per-step loops stay in the factor precision: on this
@@ -71,238 +60,12 @@ __device__ T bsum_t(T v, T *red) {
   return r;
 }
 
-// Shared scratch of the large-truncation kernel (sizes in elements).
-template <typename T>
-struct Big {
-  double *d, *e, *pw, *red;   // tridiagonal in FP64 (rank decision), work vector
-  T *dt, *et, *lam;           // tridiagonal and selected eigenvalues in T
-  T *v;          // Householder vector of the current step
-  T *wt;         // p, then w = p - K v of the current step
-  T *redt;       // 33 T of reduction scratch
-  T *tau;        // reflector coefficients
-  T *tile;       // trailing block once it fits in shared memory
-  int tile_cap;  // max trailing size held in shared memory
-};
-
-// Householder tridiagonalisation of the symmetric m x m matrix A (global, ld m,
-// full storage; destroyed).  On exit d (diagonal) and e (sub-diagonal) hold
-// T, reflector k is I - tau[k] v v^T with v[0] = 1 on rows k+1.. and v[1..]
-// stored in A[k][k+2..].
-template <typename T>
-__device__ void tridiag(T *A, int m, Big<T> &b) {
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const int warp = tid >> 5, lane = tid & 31, nw = nt >> 5;
-  // element (i, j) of the working matrix is W[(i - off) * ld + (j - off)]
-  T *W = A;
-  int off = 0, ld = m;
-  bool in_smem = false;
-  for (int k = 0; k + 2 < m; ++k) {
-    const int n1 = m - k - 1;
-    if (!in_smem && n1 + 1 <= b.tile_cap) {
-      // move the trailing block rows/cols k.. into shared memory
-      const int ls = m - k;
-      for (int64_t q = tid; q < (int64_t)ls * ls; q += nt) {
-        const int i = (int)(q / ls), j = (int)(q % ls);
-        b.tile[q] = A[(int64_t)(k + i) * m + k + j];
-      }
-      W = b.tile;
-      off = k;
-      ld = ls;
-      in_smem = true;
-      __syncthreads();
-    }
-    const T *rowk = W + (int64_t)(k - off) * ld + (k - off);   // rowk[j] = A[k][k + j]
-    T s2t = T(0);
-    for (int i = 1 + tid; i <= n1; i += nt) s2t = fma(rowk[i], rowk[i], s2t);
-    const double xn2 = (double)bsum_t<T>(s2t, b.redt);
-    const double alpha = (double)rowk[1];
-    const double sig = xn2 - alpha * alpha;
-    double tau = 0.0, beta = alpha, scale = 0.0;
-    if (sig > 0.0) {
-      beta = -copysign(sqrt(xn2), alpha);
-      tau = (beta - alpha) / beta;
-      scale = 1.0 / (alpha - beta);
-    }
-    const T scale_t = (T)scale, tau_t = (T)tau;
-    for (int i = tid; i < n1; i += nt) {
-      const T vi = (i == 0) ? T(1) : rowk[1 + i] * scale_t;
-      b.v[i] = vi;
-      if (i >= 1) A[(int64_t)k * m + k + 1 + i] = vi;  // keep the reflector in global row k
-    }
-    if (tid == 0) {
-      b.d[k] = (double)rowk[0];
-      b.e[k] = beta;
-      b.tau[k] = tau_t;
-    }
-    __syncthreads();
-    if (tau != 0.0 && in_smem) {
-      // trailing block in shared memory: by its symmetry p_i = tau sum_j
-      // A22_ji v_j and the rank-2 update are column walks, thread i on column
-      // i, consecutive threads on consecutive words (no per-row reductions)
-      T *A22 = W + (int64_t)(k + 1 - off) * ld + (k + 1 - off);
-      T pvt = T(0);
-      for (int i = tid; i < n1; i += nt) {
-        const T *col = A22 + i;
-        T a0 = T(0), a1 = T(0), a2 = T(0), a3 = T(0);
-        int j = 0;
-        for (; j + 3 < n1; j += 4) {
-          a0 = fma(col[(int64_t)j * ld], b.v[j], a0);
-          a1 = fma(col[(int64_t)(j + 1) * ld], b.v[j + 1], a1);
-          a2 = fma(col[(int64_t)(j + 2) * ld], b.v[j + 2], a2);
-          a3 = fma(col[(int64_t)(j + 3) * ld], b.v[j + 3], a3);
-        }
-        for (; j < n1; ++j) a0 = fma(col[(int64_t)j * ld], b.v[j], a0);
-        const T pi = tau_t * ((a0 + a1) + (a2 + a3));
-        b.wt[i] = pi;
-        pvt = fma(pi, b.v[i], pvt);
-      }
-      const T K = T(0.5) * tau_t * bsum_t<T>(pvt, b.redt);
-      for (int i = tid; i < n1; i += nt) b.wt[i] = fma(-K, b.v[i], b.wt[i]);  // w
-      __syncthreads();
-      for (int i = tid; i < n1; i += nt) {
-        T *col = A22 + i;
-        const T vi = b.v[i], wi = b.wt[i];
-        for (int j = 0; j < n1; ++j) {
-          T &a = col[(int64_t)j * ld];
-          a = fma(-b.v[j], wi, fma(-b.wt[j], vi, a));
-        }
-      }
-      __syncthreads();
-    } else if (tau != 0.0) {
-      T *A22 = W + (int64_t)(k + 1 - off) * ld + (k + 1 - off);
-      // p = tau * A22 v, one warp per row, four independent partial sums
-      for (int i = warp; i < n1; i += nw) {
-        const T *row = A22 + (int64_t)i * ld;
-        T a0 = T(0), a1 = T(0), a2 = T(0), a3 = T(0);
-        int j = lane;
-        for (; j + 96 < n1; j += 128) {
-          a0 = fma(row[j], b.v[j], a0);
-          a1 = fma(row[j + 32], b.v[j + 32], a1);
-          a2 = fma(row[j + 64], b.v[j + 64], a2);
-          a3 = fma(row[j + 96], b.v[j + 96], a3);
-        }
-        for (; j < n1; j += 32) a0 = fma(row[j], b.v[j], a0);
-        T acc = (a0 + a1) + (a2 + a3);
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (lane == 0) b.wt[i] = tau_t * acc;
-      }
-      __syncthreads();
-      T pvt = T(0);
-      for (int i = tid; i < n1; i += nt) pvt = fma(b.wt[i], b.v[i], pvt);
-      const T K = T(0.5) * tau_t * bsum_t<T>(pvt, b.redt);
-      for (int i = tid; i < n1; i += nt) b.wt[i] = fma(-K, b.v[i], b.wt[i]);  // w
-      __syncthreads();
-      // A22 -= v w^T + w v^T, one warp per row
-      for (int i = warp; i < n1; i += nw) {
-        T *row = A22 + (int64_t)i * ld;
-        const T vi = b.v[i], wi = b.wt[i];
-#pragma unroll 4
-        for (int j = lane; j < n1; j += 32) row[j] = fma(-vi, b.wt[j], fma(-wi, b.v[j], row[j]));
-      }
-      __syncthreads();
-    }
-  }
-  if (tid == 0) {
-    auto at = [&](int i, int j) { return (double)W[(int64_t)(i - off) * ld + (j - off)]; };
-    if (m >= 2) {
-      b.d[m - 2] = at(m - 2, m - 2);
-      b.e[m - 2] = at(m - 1, m - 2);
-      b.tau[m - 2] = T(0);
-    }
-    b.d[m - 1] = at(m - 1, m - 1);
-    b.e[m - 1] = 0.0;
-    b.tau[m - 1] = T(0);
-  }
-  __syncthreads();
-  for (int i = tid; i < m; i += nt) {
-    b.dt[i] = (T)b.d[i];
-    b.et[i] = (T)b.e[i];
-  }
-  __syncthreads();
-}
-
 template <typename R>
 __device__ __forceinline__ R unit_round();
 template <>
 __device__ __forceinline__ double unit_round<double>() { return 2.220446049250313e-16; }
 template <>
 __device__ __forceinline__ float unit_round<float>() { return 1.1920929e-07f; }
-
-// number of eigenvalues of the tridiagonal (d, e) below sigma (Sturm sequence)
-template <typename R>
-__device__ int sturm_below(const R *d, const R *e, int m, R sigma, R pivmin) {
-  int c = 0;
-  R q = d[0] - sigma;
-  if (fabs(q) < pivmin) q = -pivmin;
-  if (q < R(0)) ++c;
-  for (int i = 1; i < m; ++i) {
-    q = d[i] - sigma - e[i - 1] * e[i - 1] / q;
-    if (fabs(q) < pivmin) q = -pivmin;
-    if (q < R(0)) ++c;
-  }
-  return c;
-}
-
-template <typename R>
-struct Gersh {
-  R lo, hi, pivmin, tnorm;
-};
-
-// Gershgorin interval of the tridiagonal (every thread computes the same)
-template <typename R>
-__device__ Gersh<R> gershgorin(const R *d, const R *e, int m) {
-  Gersh<R> g;
-  R lo = d[0], hi = d[0], emax = R(0);
-  for (int i = 0; i < m; ++i) {
-    const R r = (i > 0 ? fabs(e[i - 1]) : R(0)) + (i + 1 < m ? fabs(e[i]) : R(0));
-    lo = fmin(lo, d[i] - r);
-    hi = fmax(hi, d[i] + r);
-    emax = fmax(emax, e[i] * e[i]);
-  }
-  g.tnorm = fmax(fabs(lo), fabs(hi));
-  const R pad = unit_round<R>() * g.tnorm * R(2 * m) + R(1e-30);
-  g.lo = lo - pad;
-  g.hi = hi + pad;
-  g.pivmin = fmax(R(1e-30) * fmax(R(1), emax), R(1e-35));
-  return g;
-}
-
-// idx-th smallest eigenvalue (0-based) by bisection
-template <typename R>
-__device__ R bisect_eig(const R *d, const R *e, int m, int idx, const Gersh<R> &g) {
-  R lo = g.lo, hi = g.hi;
-  const R tol = R(4) * unit_round<R>() * g.tnorm;
-  for (int it = 0; it < 200 && hi - lo > tol; ++it) {
-    const R mid = R(0.5) * (lo + hi);
-    if (mid <= lo || mid >= hi) break;
-    if (sturm_below<R>(d, e, m, mid, g.pivmin) <= idx)
-      lo = mid;
-    else
-      hi = mid;
-  }
-  return R(0.5) * (lo + hi);
-}
-
-// idx-th smallest eigenvalue by multisection with one warp (33 sub-intervals per
-// round; called by all 32 lanes of a warp, every lane returns the result)
-template <typename R>
-__device__ R multisect_eig(const R *d, const R *e, int m, int idx, const Gersh<R> &g) {
-  const int lane = threadIdx.x & 31;
-  R lo = g.lo, hi = g.hi;
-  const R tol = R(4) * unit_round<R>() * g.tnorm;
-  for (int round = 0; round < 40 && hi - lo > tol; ++round) {
-    const R sig = lo + (hi - lo) * R(lane + 1) / R(33);
-    const bool below = sturm_below<R>(d, e, m, sig, g.pivmin) <= idx;   // eigenvalue idx >= sig
-    const unsigned mask = __ballot_sync(0xffffffffu, below);
-    const int l = mask ? 31 - __clz(mask) : -1;
-    const R nlo = l >= 0 ? lo + (hi - lo) * R(l + 1) / R(33) : lo;
-    const R nhi = lo + (hi - lo) * R(l + 2) / R(33);
-    if (!(nhi > nlo)) break;
-    lo = nlo;
-    hi = nhi;
-  }
-  return R(0.5) * (lo + hi);
-}
 
 __device__ __forceinline__ float hash_unit(uint32_t a, uint32_t b) {
   uint32_t x = a * 0x9E3779B9u ^ (b + 0x7F4A7C15u);
@@ -314,159 +77,164 @@ __device__ __forceinline__ float hash_unit(uint32_t a, uint32_t b) {
   return (float)(x >> 8) * (2.0f / 16777216.0f) - 1.0f;
 }
 
-// Inverse iteration for eigenvalue lam of the tridiagonal (d, e): LU of
-// T - lam I with partial pivoting (rows i, i+1 interchanged when the
-// sub-diagonal dominates), three solves from a fixed pseudo-random start,
-// modified Gram-Schmidt against `nprev` previous vectors of the same cluster
-// of close eigenvalues.  y: output (length m); lu: 4 m of scratch; flags: m
-// bytes; element i of y, lu's four arrays and flags sits at index i * st (st >
-// 1 interleaves the scratch of several threads, so that their accesses to
-// global memory coalesce).
+
+// Quotients of the Sturm recurrences that only place eigenvalues (shifts of
+// the inverse iteration, lambda_max): approximate division (2 ulp), which
+// moves a computed count no more than the rounding of the recurrence itself
+// does.  The rank count divides exactly, in FP64.
+__device__ __forceinline__ float place_div(float a, float b) { return __fdividef(a, b); }
+// FP64: the hardware's reciprocal seed (20 bits) and two Newton steps
+// y <- y + y (1 - b y), good to the last place or two, at 6 of the FP64
+// instructions whose rate bounds these loops, against about twice that for
+// the exactly rounded quotient
+__device__ __forceinline__ double place_div(double a, double b) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
+  y = fma(y, fma(-b, y, 1.0), y);
+  y = fma(y, fma(-b, y, 1.0), y);
+  return a * y;
+}
+
+// number of eigenvalues above sigma of the tridiagonal with diagonal d and
+// squared sub-diagonal e2 (e2[i] couples i - 1 and i; e2[0] unused)
 template <typename R>
-__device__ void inverse_iteration(const R *d, const R *e, int m, R lam, R tnorm, R *y, const R *prev,
-                                  int nprev, R *lu, unsigned char *flags, uint32_t seed, int st = 1) {
-  const size_t sm = (size_t)m * st;
-  R *u0 = lu, *u1 = lu + sm, *u2 = lu + 2 * sm, *l = lu + 3 * sm;
-  auto I = [st](int i) { return (size_t)i * st; };
-  const R small = unit_round<R>() * tnorm + R(1e-30);
-  R a = d[0] - lam, c = (m > 1) ? e[0] : R(0);
-  for (int i = 0; i + 1 < m; ++i) {
-    const R bsub = e[i];
-    const R an = d[i + 1] - lam;
-    const R cn = (i + 2 < m) ? e[i + 1] : R(0);
-    if (fabs(a) >= fabs(bsub)) {
-      const R piv = (a == R(0)) ? small : a;
-      const R mult = bsub / piv;
-      u0[I(i)] = piv;
-      u1[I(i)] = c;
-      u2[I(i)] = R(0);
-      l[I(i)] = mult;
-      flags[I(i)] = 0;
-      a = an - mult * c;
-      c = cn;
-    } else {
-      const R mult = a / bsub;
-      u0[I(i)] = bsub;
-      u1[I(i)] = an;
-      u2[I(i)] = cn;
-      l[I(i)] = mult;
-      flags[I(i)] = 1;
-      a = c - mult * an;
-      c = -mult * cn;
-    }
+__device__ __forceinline__ int count_above(const R *d, const R *e2, int m, R sigma, R pivmin) {
+  R q = d[0] - sigma;
+  if (fabs(q) < pivmin) q = -pivmin;
+  int c = q > R(0);
+#pragma unroll 4
+  for (int i = 1; i < m; ++i) {
+    q = (d[i] - sigma) - place_div(e2[i], q);
+    if (fabs(q) < pivmin) q = -pivmin;
+    c += q > R(0);
   }
-  u0[I(m - 1)] = a;
-  for (int i = 0; i < m; ++i)
-    if (fabs(u0[I(i)]) < small) u0[I(i)] = copysign(small, u0[I(i)]);
-  for (int i = 0; i < m; ++i) y[I(i)] = (R)hash_unit(seed, (uint32_t)i);
-  for (int it = 0; it < 3; ++it) {
-    for (int i = 0; i + 1 < m; ++i) {
-      if (flags[I(i)]) {
-        const R t = y[I(i)];
-        y[I(i)] = y[I(i + 1)];
-        y[I(i + 1)] = t - l[I(i)] * y[I(i)];
-      } else {
-        y[I(i + 1)] -= l[I(i)] * y[I(i)];
-      }
-    }
-    for (int i = m - 1; i >= 0; --i) {
-      R s = y[I(i)];
-      if (i + 1 < m) s -= u1[I(i)] * y[I(i + 1)];
-      if (i + 2 < m) s -= u2[I(i)] * y[I(i + 2)];
-      y[I(i)] = s / u0[I(i)];
-    }
-    for (int pass = 0; pass < 2; ++pass)
-      for (int p = 0; p < nprev; ++p) {
-        const R *q = prev + (size_t)p * m;
-        R dot = R(0);
-        for (int i = 0; i < m; ++i) dot += q[i] * y[I(i)];
-        for (int i = 0; i < m; ++i) y[I(i)] -= dot * q[i];
-      }
-    // normalise, scaling by the largest entry first to keep the sum in range
-    R big = R(0);
-    for (int i = 0; i < m; ++i) big = fmax(big, fabs(y[I(i)]));
-    const R sc = big > R(0) ? R(1) / big : R(0);
-    R nrm = R(0);
-    for (int i = 0; i < m; ++i) nrm += (y[I(i)] * sc) * (y[I(i)] * sc);
-    nrm = sqrt(nrm);
-    const R inv = nrm > R(0) ? sc / nrm : R(0);
-    for (int i = 0; i < m; ++i) y[I(i)] *= inv;
+  return c;
+}
+
+// positive eigenvalues of the symmetric k x k matrix S (ld N)
+template <typename R, int N>
+__device__ __forceinline__ int count_positive(R (&S)[N][N], int k) {
+  if constexpr (N <= 2) {
+    if (k == 0) return 0;
+    if (k == 1) return S[0][0] > R(0);
+    const R det = S[0][0] * S[1][1] - S[1][0] * S[1][0];
+    if (det < R(0)) return 1;
+    return S[0][0] + S[1][1] > R(0) ? 2 : 0;
+  } else {
+    // cyclic Jacobi
+    for (int sweep = 0; sweep < 16; ++sweep)
+      for (int p = 0; p < k; ++p)
+        for (int q = p + 1; q < k; ++q) {
+          const R apq = S[q][p];
+          if (fabs(apq) <= R(1e-30)) continue;
+          const R th = (S[q][q] - S[p][p]) / (R(2) * apq);
+          R tt = R(1) / (fabs(th) + sqrt(R(1) + th * th));
+          if (th < R(0)) tt = -tt;
+          const R c = R(1) / sqrt(R(1) + tt * tt), sn = tt * c;
+          for (int l = 0; l < k; ++l) {
+            const R slp = S[l][p], slq = S[l][q];
+            S[l][p] = c * slp - sn * slq;
+            S[l][q] = sn * slp + c * slq;
+          }
+          for (int l = 0; l < k; ++l) {
+            const R spl = S[p][l], sql = S[q][l];
+            S[p][l] = c * spl - sn * sql;
+            S[q][l] = sn * spl + c * sql;
+          }
+        }
+    int pos = 0;
+    for (int p = 0; p < k; ++p) pos += S[p][p] > R(0);
+    return pos;
   }
 }
 
-
-// Eigenvalues of G above sigma, for sigma > lambda_max(T), where Q^T G Q = T + Z M Z^T,
-// T = tridiag(d, e) (the tridiagonal of the projected Gram J = P G P), Z = Q^T [U_1, G U_1]
-// (m x 2 k1, column j at Z + j*m) and M = [[-C, I], [I, 0]], C = U_1^T G U_1 (k1 x k1,
-// ld kMaxK1).  NZ >= 2 k1 bounds the small dense parts held per thread.
-// Haynsworth inertia of [[T - sigma I, Z], [Z^T, -M^-1]] gives
-//   #eig(G) > sigma = n_+(-M^-1 - Z^T (T - sigma I)^-1 Z) - n_+(-M^-1),  n_+(-M^-1) = k1,
-// since T - sigma I is negative definite.  With T - sigma I = L D L^T (L unit
-// lower bidiagonal) and W = L^-1 Z, Z^T (T - sigma I)^-1 Z = W^T D^-1 W: one
-// forward sweep with register accumulators, no storage.
-template <typename R, int NZ>
-__device__ int count_above_lowrank(const R *d, const R *e, int m, const R *Z, int k1, const R *C, R sigma) {
-  const int nz = 2 * k1;
-  R w[NZ];
-  R g[NZ][NZ];
-  for (int a = 0; a < NZ; ++a) {
+// Eigenvalues above sigma > 0 of G = [[C, X^T], [X, J]] (basis [U_1, its
+// complement]), J = Q T Q^T, Z = Q^T X (column a at Z + a ldz).  Haynsworth
+// inertia of [[T - sigma I, Z], [Z^T, C - sigma I]]: those of T - sigma I, plus
+// those of C - sigma I - Z^T (T - sigma I)^-1 Z.  (T carries k1 more zero
+// eigenvalues than the complement's block, which no sigma > 0 counts.)  With
+// T - sigma I = L D L^T and W = L^-1 Z, the product is W^T D^-1 W: one forward
+// sweep with register accumulators.  The FP32 sweep and the FP64 one differ
+// in precision only.
+template <typename R, int KB>
+__device__ __forceinline__ int count_above_gc(const R *d, const R *e, const R *e2, int m, const R *Z, int ldz, int k1,
+                                              const R *C, R sigma, R pivmin) {
+  R w[KB], g[KB][KB];
+#pragma unroll
+  for (int a = 0; a < KB; ++a) {
     w[a] = R(0);
-    for (int b2 = 0; b2 < NZ; ++b2) g[a][b2] = R(0);
+#pragma unroll
+    for (int b = 0; b < KB; ++b) g[a][b] = R(0);
   }
-  R dd = R(1), lprev = R(0);
+  int c = 0;
+  R l = R(0), inv = R(0);
+#pragma unroll 2
   for (int i = 0; i < m; ++i) {
-    dd = (i == 0) ? d[0] - sigma : d[i] - sigma - lprev * e[i - 1];
-    const R inv = R(1) / dd;
+    R q = (d[i] - sigma) - e2[i] * inv;   // e2[0] = 0
+    if (fabs(q) < pivmin) q = -pivmin;
+    c += q > R(0);
+    inv = place_div(R(1), q);
 #pragma unroll
-    for (int a = 0; a < NZ; ++a)
-      if (a < nz) w[a] = Z[(size_t)a * m + i] - (i == 0 ? R(0) : lprev * w[a]);
+    for (int a = 0; a < KB; ++a)
+      if (KB <= 2 || a < k1) w[a] = (a < k1 ? Z[(size_t)a * ldz + i] : R(0)) - l * w[a];
 #pragma unroll
-    for (int a = 0; a < NZ; ++a)
+    for (int a = 0; a < KB; ++a)
 #pragma unroll
-      for (int b2 = 0; b2 < NZ; ++b2)
-        if (a < nz && b2 <= a) g[a][b2] = fma(w[a] * inv, w[b2], g[a][b2]);
-    lprev = (i + 1 < m) ? e[i] * inv : R(0);
+      for (int b = 0; b <= a; ++b)
+        if (KB <= 2 || a < k1) g[a][b] = fma(w[a] * inv, w[b], g[a][b]);
+    l = e[i] * inv;                        // e[m - 1] = 0
   }
-  R S[NZ][NZ];
-  for (int a = 0; a < nz; ++a)
-    for (int b = 0; b < nz; ++b) {
-      R v = R(0);
-      if (a < k1 && b >= k1 && b - k1 == a) v = R(-1);
-      if (b < k1 && a >= k1 && a - k1 == b) v = R(-1);
-      if (a >= k1 && b >= k1) v = -C[(a - k1) * kMaxK1 + (b - k1)];
-      S[a][b] = v - (b <= a ? g[a][b] : g[b][a]);
-    }
-  // symmetrise and count positive eigenvalues by cyclic Jacobi on the small matrix
-  for (int a = 0; a < nz; ++a)
-    for (int b = a + 1; b < nz; ++b) {
-      const R v = R(0.5) * (S[a][b] + S[b][a]);
+  R S[KB][KB];
+#pragma unroll
+  for (int a = 0; a < KB; ++a)
+#pragma unroll
+    for (int b = 0; b <= a; ++b) {
+      const R v = (a < k1 && b < k1 ? R(0.5) * (C[a * kMaxK1 + b] + C[b * kMaxK1 + a]) : R(0)) - g[a][b] -
+                  (a == b ? sigma : R(0));
       S[a][b] = v;
       S[b][a] = v;
     }
-  for (int sweep = 0; sweep < (NZ > 4 ? 16 : 12); ++sweep)
-    for (int p = 0; p < nz; ++p)
-      for (int q = p + 1; q < nz; ++q) {
-        const R apq = S[p][q];
-        if (fabs(apq) <= R(1e-30)) continue;
-        const R th = (S[q][q] - S[p][p]) / (R(2) * apq);
-        R tt = R(1) / (fabs(th) + sqrt(R(1) + th * th));
-        if (th < R(0)) tt = -tt;
-        const R c = R(1) / sqrt(R(1) + tt * tt), sn = tt * c;
-        for (int k = 0; k < nz; ++k) {
-          const R skp = S[k][p], skq = S[k][q];
-          S[k][p] = c * skp - sn * skq;
-          S[k][q] = sn * skp + c * skq;
-        }
-        for (int k = 0; k < nz; ++k) {
-          const R spk = S[p][k], sqk = S[q][k];
-          S[p][k] = c * spk - sn * sqk;
-          S[q][k] = sn * spk + c * sqk;
-        }
-      }
-  int pos = 0;
-  for (int a = 0; a < nz; ++a)
-    if (S[a][a] > R(0)) ++pos;
-  return pos - k1;
+  return c + count_positive<R, KB>(S, k1);
+}
+
+// several preserved vectors (k1 > 2) in a call of its own, off the register
+// allocation of the one-vector path
+template <typename R>
+__device__ __noinline__ int count_above_gc_wide(const R *d, const R *e, const R *e2, int m, const R *Z, int ldz,
+                                                int k1, const R *C, R sigma, R pivmin) {
+  return count_above_gc<R, kMaxK1>(d, e, e2, m, Z, ldz, k1, C, sigma, pivmin);
+}
+
+template <typename R>
+__device__ __forceinline__ R sturm_pivmin(R emax2) {
+  return fmax(R(1e-30) * fmax(R(1), emax2), R(1e-35));
+}
+
+// The multisection of one value by the lanes of a warp group: `above(sigma)`
+// is true below the wanted eigenvalue and false above it.  With closed ends
+// the L points include lo and hi, whose counts confirm the bracket (returns -1
+// when the value lies below lo, 1 above hi); else they divide (lo, hi) into
+// L + 1 parts.
+template <typename R, int L, typename F>
+__device__ __forceinline__ int section(R &lo, R &hi, int lane, bool closed, F &&above) {
+  const int l = lane % L;
+  const R h = hi - lo;
+  const R p0 = closed ? lo + h * R(l) / R(L - 1) : lo + h * R(l + 1) / R(L + 1);
+  const unsigned ball = __ballot_sync(0xffffffffu, above(p0));
+  const unsigned mine = L == 32 ? ball : (ball >> (lane / L * L)) & ((1u << (L & 31)) - 1u);
+  const int n = __popc(mine);   // points below the value
+  if (closed) {
+    if (n == 0) return -1;
+    if (n == L) return 1;
+    const R a = lo + h * R(n - 1) / R(L - 1), b = lo + h * R(n) / R(L - 1);
+    lo = a;
+    hi = b;
+  } else {
+    const R a = n > 0 ? lo + h * R(n) / R(L + 1) : lo, b = n < L ? lo + h * R(n + 1) / R(L + 1) : hi;
+    lo = a;
+    hi = b;
+  }
+  return 0;
 }
 
 // J = G - U1 X^T - X U1^T + U1 c U1^T (the Gram matrix projected off span U_1),
@@ -512,366 +280,678 @@ __device__ __noinline__ void build_projected_gram_wide(const T *G, const T *U, c
   build_projected_gram<T, kMaxK1>(G, U, Y, s_c, A, m, k1);
 }
 
-// The count for k1 > 2 (several preserved vectors) in a call of its own, so
-// that its 16 x 16 local arrays stay out of the kernel's register allocation.
-template <typename R>
-__device__ __noinline__ int count_above_lowrank_wide(const R *d, const R *e, int m, const R *Z, int k1,
-                                                     const R *C, R sigma) {
-  return count_above_lowrank<R, 2 * kMaxK1>(d, e, m, Z, k1, C, sigma);
-}
-
-// mode: TB_FULL does all steps in this CTA.  The multi-CTA path for very large
-// nodes splits it: TB_PREP stops before the tridiagonalisation (A = J, Z saved,
-// k1 and c stored in SC); the step kernels tridiagonalise; TB_POST takes d, e
-// and the reflectors from global memory and stops after the eigenvectors of T
-// (Y, k2 in SC) -- the reflector kernels do the two products with Q.
-enum { TB_FULL = 0, TB_PREP = 1, TB_POST = 2 };
-
+// U_1, J, X and C of one node, or the complete basis (eps = 0)
 template <typename T, int NT>
-__global__ void __launch_bounds__(NT) k_trunc_big(const TruncTask<T> *__restrict__ tasks, int *__restrict__ kout,
-                                                 int variant, int tile_cap, int vec_smem, int mode) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+__global__ void __launch_bounds__(NT) k_trunc_prep(const TruncTask<T> *__restrict__ tasks, int *__restrict__ kout,
+                                                  int variant) {
   __shared__ double red[33];
-  __shared__ int s_k2;
   __shared__ double s_gR[kMaxK1 * 2 * kMaxPhi], s_gW[kMaxK1 * kMaxK1 + kMaxK1];
   __shared__ int s_gk;
-  __shared__ T s_c[kMaxK1 * kMaxK1];   // c = U1^T G U1, ld kMaxK1
+  __shared__ T s_c[kMaxK1 * kMaxK1];   // C = U1^T G U1, ld kMaxK1
+  __shared__ T redt[34];
   const TruncTask<T> t = tasks[blockIdx.x];
-  const double eps = t.eps;
   const int m = t.m;
   const int tid = threadIdx.x, nt = blockDim.x;
-  // global work, all T: A (m^2), Y (m^2), LU (4 m^2), LS (164 m: Z = Q^T [U1, X] in
-  // 4 m, then per-thread inverse-iteration slots when the shared tile is too
-  // small); then flags (m^2 bytes); then the per-node vectors when they do not
-  // fit in shared memory (vec_smem == 0)
   const BigLayout<T> L = big_layout<T>(t.work, m);
-  T *A = L.A;
-  T *Y = L.Y;
-  T *LU = L.LU;
-  T *LS = L.LS;
-  unsigned char *FL = L.FL;
-  unsigned char *VG = L.VG;
-  // vector layout (shared memory, or global at VG), then the shared tile
-  Big<T> b;
-  unsigned char *p = vec_smem ? smem_raw : VG;
-  b.d = (double *)p;
-  p += sizeof(double) * m;
-  b.e = (double *)p;
-  p += sizeof(double) * m;
-  b.pw = (double *)p;
-  p += sizeof(double) * m;
-  const int me = (m + 1) & ~1;
-  b.dt = (T *)p;
-  p += sizeof(T) * me;
-  b.et = (T *)p;
-  p += sizeof(T) * me;
-  b.lam = (T *)p;
-  p += sizeof(T) * me;
-  b.v = (T *)p;
-  p += sizeof(T) * me;
-  b.tau = (T *)p;
-  p += sizeof(T) * me;
-  b.wt = (T *)p;
-  p += sizeof(T) * me;
-  b.redt = (T *)p;
-  p += sizeof(T) * 34;
-  p = (unsigned char *)(((uintptr_t)p + 15) & ~(uintptr_t)15);
-  b.tile = (T *)(vec_smem ? p : smem_raw);
-  b.tile_cap = tile_cap;
-  b.red = red;
-  if (m == 0) {
-    if (tid == 0) kout[t.k_idx] = 0;
+  T *A = L.A, *Y = L.Y;
+  const bool gc = variant != HS_LORASP;
+  if (!gc) {
+    if (t.eps == 0.0) {
+      // no truncation: the complete basis U = I
+      for (int64_t q = tid; q < (int64_t)m * m; q += nt) t.U[q] = (q / m == q % m) ? T(1) : T(0);
+      if (tid == 0) kout[t.k_idx] = m;
+      return;
+    }
+    for (int64_t q = tid; q < (int64_t)m * m; q += nt) A[q] = t.G[q];
+    if (tid == 0) L.sc_int[0] = 0;
     return;
   }
-  // ---- GC basis U_1 (same rule as the Jacobi path; scratch b.pw, m doubles)
-  int k1 = 0;
-  if (variant != HS_LORASP)
-    k1 = gc_basis_dev<T>(t.phi, t.a, t.np, m, variant == HS_GC_PROJ, t.eps1, t.U, b.pw, red, s_gR, s_gW, &s_gk);
-  const bool gc = variant != HS_LORASP;
-  if (gc && eps == 0.0) {
+  // GC basis (scratch: m doubles in LS)
+  const int k1 = gc_basis_dev<T>(t.phi, t.a, t.np, m, variant == HS_GC_PROJ, t.eps1, t.U, (double *)L.LS, red, s_gR,
+                                 s_gW, &s_gk);
+  if (t.eps == 0.0) {
     // no truncation: complete the GC basis to all of R^m (Householder QR of
-    // U_1; scratch k1 m doubles in Y and LU, 5 m^2 T)
-    // (nothing to complete when U_1 already spans R^m)
+    // U_1; scratch k1 m doubles); nothing to complete when it spans R^m
     if (k1 < m) {
       if (k1 <= 2)
-        gc_complete<T>(t.U, m, k1, (double *)Y, red);
+        gc_complete<T>(t.U, m, k1, (double *)L.LS, red);
       else
-        gc_complete_n<T>(t.U, m, k1, (double *)Y, s_gW, red);
+        gc_complete_n<T>(t.U, m, k1, (double *)L.LS, s_gW, red);
     }
     if (tid == 0) kout[t.k_idx] = m;
     return;
   }
-  // ---- lambda_max(G) (GC) follows from the tridiagonal of the projected Gram below
-  double lmax = 0.0;
-  // ---- J
-  if (mode == TB_POST) {
-    // J, Z and c were made by TB_PREP; Z is already Q^T [U1, X]
-    for (int q = tid; q < kMaxK1 * kMaxK1; q += nt) s_c[q] = (T)L.sc_c[q];
-    __syncthreads();
-  } else if (!gc) {
-    for (int64_t q = tid; q < (int64_t)m * m; q += nt) A[q] = t.G[q];
-  } else if (eps > 0.0) {
-    // X = G U1 in Y's first columns, c = U1^T X; one warp per row of G
-    {
-      const int warp = tid >> 5, lane = tid & 31, nw = nt >> 5;
-      for (int i = warp; i < m; i += nw)
-        for (int a = 0; a < k1; ++a) {
-          T s = T(0);
-          for (int j = lane; j < m; j += 32) s = fma(t.G[(int64_t)i * m + j], t.U[(int64_t)j * m + a], s);
-          for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-          if (lane == 0) Y[(size_t)a * m + i] = s;
-        }
-    }
-    __syncthreads();
-    for (int q = tid; q < kMaxK1 * kMaxK1; q += nt) s_c[q] = T(0);
-    __syncthreads();
-    for (int a = 0; a < k1; ++a)
-      for (int bb = 0; bb < k1; ++bb) {
-        T s = T(0);
-        for (int i = tid; i < m; i += nt) s = fma(t.U[(int64_t)i * m + a], Y[(size_t)bb * m + i], s);
-        const T cab = bsum_t<T>(s, b.redt);
-        if (tid == 0) s_c[a * kMaxK1 + bb] = cab;
-      }
-    __syncthreads();
-    // J = G - U1 X^T - X U1^T + U1 c U1^T, one warp per row
-    if (k1 <= 2)
-      build_projected_gram<T, 2>(t.G, t.U, Y, s_c, A, m, k1);
-    else
-      build_projected_gram_wide<T>(t.G, t.U, Y, s_c, A, m, k1);
-  } else {
-    for (int64_t q = tid; q < (int64_t)m * m; q += nt) {
-      const int i = (int)(q / m), j = (int)(q % m);
-      double v = (i == j) ? 1.0 : 0.0;
-      for (int a = 0; a < k1; ++a) v -= (double)t.U[(int64_t)i * m + a] * (double)t.U[(int64_t)j * m + a];
-      A[q] = (T)v;
-    }
-  }
-  __syncthreads();
-  // X = G U1 (Y columns 0..k1-1) is needed again below: move it next to U1 first
-  T *Zb = LS;  // Z = Q^T [U1, X], 2 k1 <= 2 kMaxK1 columns of m
-  if (gc && eps > 0.0 && mode != TB_POST) {
-    for (int64_t q = tid; q < (int64_t)m * k1; q += nt) {
-      const int a = (int)(q / m), i = (int)(q % m);
-      Zb[(size_t)a * m + i] = t.U[(int64_t)i * m + a];
-      Zb[(size_t)(k1 + a) * m + i] = Y[(size_t)a * m + i];
-    }
-  }
-  __syncthreads();
-  if (mode == TB_PREP) {
-    if (tid == 0) L.sc_int[0] = k1;
-    for (int q = tid; q < kMaxK1 * kMaxK1; q += nt) L.sc_c[q] = (double)s_c[q];
-    return;
-  }
-  if (mode == TB_POST) {
-    // the step kernels left d, e, tau for k < m - 2 and the updated trailing 2 x 2 block
-    if (tid == 0) {
-      if (m >= 2) {
-        b.d[m - 2] = (double)A[(int64_t)(m - 2) * m + m - 2];
-        b.e[m - 2] = (double)A[(int64_t)(m - 1) * m + m - 2];
-        b.tau[m - 2] = T(0);
-      }
-      b.d[m - 1] = (double)A[(int64_t)(m - 1) * m + m - 1];
-      b.e[m - 1] = 0.0;
-      b.tau[m - 1] = T(0);
-    }
-    __syncthreads();
-    for (int i = tid; i < m; i += nt) {
-      b.dt[i] = (T)b.d[i];
-      b.et[i] = (T)b.e[i];
-    }
-    __syncthreads();
-  } else {
-    tridiag<T>(A, m, b);
-  }
-  const Gersh<T> g = gershgorin<T>(b.dt, b.et, m);
-  double thr;
-  __shared__ double s_lmax;
-  if (!gc) {
-    if (tid < 32) {
-      const T lt = multisect_eig<T>(b.dt, b.et, m, m - 1, g);
-      if (tid == 0) s_lmax = (double)lt;
-    }
-    __syncthreads();
-    lmax = s_lmax;
-    thr = eps * eps * lmax;
-  } else if (eps > 0.0) {
-    // Z = Q^T [U1, X]: reflectors in forward order, one warp per column
-    if (mode != TB_POST) {
-      const int warp = tid >> 5, lane = tid & 31, nw = nt >> 5;
-      for (int j = warp; j < 2 * k1; j += nw) {
-        T *z = Zb + (size_t)j * m;
-        for (int k = 0; k + 2 < m; ++k) {
-          const T tk = b.tau[k];
-          if (tk == T(0)) continue;
-          const int n1 = m - k - 1;
-          const T *vrow = A + (int64_t)k * m + k + 1;
-          T sdot = T(0);
-          for (int i = lane; i < n1; i += 32) sdot = fma(i == 0 ? T(1) : vrow[i], z[k + 1 + i], sdot);
-          for (int o = 16; o > 0; o >>= 1) sdot += __shfl_xor_sync(0xffffffffu, sdot, o);
-          sdot *= tk;
-          for (int i = lane; i < n1; i += 32) z[k + 1 + i] -= sdot * (i == 0 ? T(1) : vrow[i]);
-          __syncwarp();
-        }
-      }
-    }
-    __syncthreads();
-    // lambda_max(G) by multisection on the low-rank count, one warp
-    if (tid < 32) {
-      const T lmaxT = multisect_eig<T>(b.dt, b.et, m, m - 1, g);
-      T trace = T(0);
-      for (int i = 0; i < m; ++i) trace += t.G[(int64_t)i * m + i];
-      T lo = lmaxT, hi = fmax(trace, lmaxT) * T(1.0001) + T(1e-30);
-      for (int round = 0; round < 40 && hi - lo > T(4) * unit_round<T>() * hi; ++round) {
-        const T sig = lo + (hi - lo) * T(tid + 1) / T(33);
-        const int c = k1 == 0 ? 0
-                      : k1 <= 2 ? count_above_lowrank<T, 4>(b.dt, b.et, m, Zb, k1, s_c, sig)
-                                : count_above_lowrank_wide<T>(b.dt, b.et, m, Zb, k1, s_c, sig);
-        const unsigned above = __ballot_sync(0xffffffffu, c >= 1);
-        const int l = above ? 31 - __clz(above) : -1;   // highest sigma with an eigenvalue above it
-        const T nlo = l >= 0 ? lo + (hi - lo) * T(l + 1) / T(33) : lo;
-        const T nhi = lo + (hi - lo) * T(l + 2) / T(33);
-        lo = nlo;
-        hi = nhi;
-      }
-      if (tid == 0) s_lmax = (double)(T(0.5) * (lo + hi));
-    }
-    __syncthreads();
-    lmax = s_lmax;
-    thr = eps * eps * lmax;
-  } else {
-    thr = 0.5;
-  }
-  // ---- rank: eigenvalues strictly above thr, one Sturm count in FP64
-  if (tid == 0) {
-    const Gersh<double> gd = gershgorin<double>(b.d, b.e, m);
-    int k2 = m - sturm_below<double>(b.d, b.e, m, thr, gd.pivmin);
-    if (k2 > m - k1) k2 = m - k1;
-    if (k2 > t.cap - k1) k2 = t.cap - k1;   // max_rank_ratio: the largest eigenvalues are kept
-    if (k2 < 0) k2 = 0;
-    s_k2 = k2;
-  }
-  __syncthreads();
-  const int k2 = s_k2;
-  // ---- the k2 largest eigenvalues, descending (shifts for inverse iteration)
-  for (int j = tid; j < k2; j += nt) b.lam[j] = bisect_eig<T>(b.dt, b.et, m, m - 1 - j, g);
-  __syncthreads();
-  // ---- eigenvectors of T by inverse iteration.  Only the span of the selected
-  // vectors matters and the host re-orthonormalises them (CholQR2), which
-  // tolerates the overlap u ||T|| / gap that inverse iteration leaves between
-  // vectors of distinct eigenvalues.  Vectors are orthogonalised against each
-  // other only inside clusters closer than 10 u ||T||, where they could come
-  // out nearly parallel; a cluster is handled by one thread in order.
-  const T ortol = T(10) * unit_round<T>() * g.tnorm;
-  // cluster starts (thread 0 scans; b.pw reused as an int list)
-  int *starts = (int *)b.pw;
-  __shared__ int s_nc;
-  if (tid == 0) {
-    int nc = 0;
-    for (int j = 0; j < k2; ++j)
-      if (j == 0 || b.lam[j - 1] - b.lam[j] >= ortol) starts[nc++] = j;
-    starts[nc] = k2;
-    s_nc = nc;
-  }
-  __syncthreads();
-  const int nc = s_nc;
-  if (mode == TB_POST) {
-    // the eigenvectors of T come from k_invit, spread over many CTAs
-    if (tid == 0) {
-      L.sc_int[2] = nc;
-      *L.sc_tnorm = (double)g.tnorm;
-    }
-  } else {
-    // each worker thread owns a slot: u0,u1,u2,l,y (5 m T) + m flags, in the
-    // shared tile (see below for the global fallback)
-    const size_t tile_bytes = (size_t)b.tile_cap * b.tile_cap * sizeof(T);
-    const size_t slot_bytes = ((5 * (size_t)m * sizeof(T) + (size_t)m + 15) / 16) * 16;
-    int nslot = (int)(tile_bytes / slot_bytes);
-    // fewer than 8 slots in the tile: up to one per thread in the (otherwise unused)
-    // LU and FL regions of global memory, interleaved so that the threads'
-    // accesses coalesce (5 m T per slot in LU's 4 m^2, m flags in FL's m^2)
-    const bool glob = nslot < 8;
-    int ns_g = 0;
-    if (glob) {
-      ns_g = (int)((4 * (size_t)m * m) / (5 * (size_t)m));
-      if (ns_g > nt) ns_g = nt;
-      if (ns_g < 1) ns_g = 1;
-      nslot = ns_g;
-    }
-    if (nslot > nt) nslot = nt;
-    if (tid < nslot) {
-      T *lu, *ys;
-      unsigned char *fl;
-      int st = 1;
-      if (glob) {
-        lu = LU + tid;
-        ys = LU + 4 * (size_t)m * ns_g + tid;
-        fl = FL + tid;
-        st = ns_g;
-      } else {
-        unsigned char *slot = (unsigned char *)b.tile + (size_t)tid * slot_bytes;
-        lu = (T *)slot;
-        ys = lu + 4 * (size_t)m;
-        fl = (unsigned char *)(ys + m);
-      }
-      for (int c = tid; c < nc; c += nslot) {
-        const int j0 = starts[c], j1 = starts[c + 1];
-        for (int q = j0; q < j1; ++q) {
-          inverse_iteration<T>(b.dt, b.et, m, b.lam[q], g.tnorm, ys, Y + (size_t)j0 * m, q - j0, lu, fl,
-                               (uint32_t)(q * 7919 + 17), st);
-          for (int i = 0; i < m; ++i) Y[(size_t)q * m + i] = ys[(size_t)i * st];
-        }
-      }
-    }
-  }
-  __syncthreads();
-  if (mode == TB_POST) {
-    // U_2 = Q Y is left to the reflector kernel
-    if (tid == 0) {
-      L.sc_int[0] = k1;
-      L.sc_int[1] = k2;
-      kout[t.k_idx] = k1 + k2;
-    }
-    return;
-  }
-  // ---- back-transformation U_2 = Q Y (reflectors in reverse order): columns
-  // staged in shared memory in batches, one warp per column
+  // G U1 in Y's first columns, C = U1^T G U1; one warp per row of G
   {
     const int warp = tid >> 5, lane = tid & 31, nw = nt >> 5;
-    const size_t tile_elems = (size_t)b.tile_cap * b.tile_cap;
-    // columns staged in the shared tile, or transformed in place in Y when
-    // the tile cannot hold one column
-    const bool in_place = tile_elems < (size_t)m;
-    int batch = in_place ? max(k2, 1) : (int)(tile_elems / (size_t)m);
-    for (int jb = 0; jb < k2; jb += batch) {
-      const int nb = min(batch, k2 - jb);
-      T *ysm = in_place ? Y + (size_t)jb * m : b.tile;
-      if (!in_place)
-        for (int64_t q = tid; q < (int64_t)nb * m; q += nt) ysm[q] = Y[(size_t)jb * m + q];
-      __syncthreads();
-      for (int j = warp; j < nb; j += nw) {
-        T *y = ysm + (size_t)j * m;
-        for (int k = m - 3; k >= 0; --k) {
-          const T tk = b.tau[k];
-          if (tk == T(0)) continue;
-          const int n1 = m - k - 1;
-          const T *vrow = A + (int64_t)k * m + k + 1;  // v[0] = 1 implicit, v[i] at vrow[i] for i >= 1
-          T s = T(0);
-          for (int i = lane; i < n1; i += 32) s = fma(i == 0 ? T(1) : vrow[i], y[k + 1 + i], s);
-          for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-          s *= tk;
-          for (int i = lane; i < n1; i += 32) y[k + 1 + i] -= s * (i == 0 ? T(1) : vrow[i]);
-          __syncwarp();
+    for (int i = warp; i < m; i += nw)
+      for (int a = 0; a < k1; ++a) {
+        T s = T(0);
+        for (int j = lane; j < m; j += 32) s = fma(t.G[(int64_t)i * m + j], t.U[(int64_t)j * m + a], s);
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) Y[(size_t)a * m + i] = s;
+      }
+  }
+  __syncthreads();
+  for (int q = tid; q < kMaxK1 * kMaxK1; q += nt) s_c[q] = T(0);
+  __syncthreads();
+  for (int a = 0; a < k1; ++a)
+    for (int bb = 0; bb < k1; ++bb) {
+      T s = T(0);
+      for (int i = tid; i < m; i += nt) s = fma(t.U[(int64_t)i * m + a], Y[(size_t)bb * m + i], s);
+      const T cab = bsum_t<T>(s, redt);
+      if (tid == 0) s_c[a * kMaxK1 + bb] = cab;
+    }
+  __syncthreads();
+  if (k1 <= 2)
+    build_projected_gram<T, 2>(t.G, t.U, Y, s_c, A, m, k1);
+  else
+    build_projected_gram_wide<T>(t.G, t.U, Y, s_c, A, m, k1);
+  // X = G U1 - U1 C (the scratch in LS is no longer in use)
+  T *X = L.LS;
+  for (int64_t q = tid; q < (int64_t)m * k1; q += nt) {
+    const int a = (int)(q / m), i = (int)(q % m);
+    T x = Y[(size_t)a * m + i];
+    for (int b = 0; b < k1; ++b) x = fma(-t.U[(int64_t)i * m + b], s_c[b * kMaxK1 + a], x);
+    X[(size_t)a * m + i] = x;
+  }
+  if (tid == 0) L.sc_int[0] = k1;
+  for (int q = tid; q < kMaxK1 * kMaxK1; q += nt) L.sc_c[q] = (double)s_c[q];
+}
+
+// ---------------------------------------------------------------------------
+// lambda_max(G) and the rank of one node per CTA.
+// lambda_max: FP32 factors section its bracket by 256 points a round (three
+// rounds to 4 u); the FP64 factor starts from such an FP32 value and confirms
+// and refines it by one warp's sections in FP64, whose rate (1/64 of FP32's)
+// makes more points a round cost more than they save.  The bracket is
+// [largest diagonal entry, Gershgorin bound of T + trace C].
+// Rank: the FP64 Sturm count at eps^2 lambda_max runs from both ends of T at
+// once (two threads) and meets in the middle row, whose pivot takes both
+// neighbours' quotients: the same inertia in half the dependent divisions.
+// ---------------------------------------------------------------------------
+constexpr int kRankThreads = 256;
+
+// dynamic shared memory: d, e2 (FP64), d, e, e2, Z in T, and for the FP64
+// factor also in FP32; Z stays in global memory when it does not fit
+template <typename T>
+__host__ __device__ inline size_t rank_smem_bytes(int m, int zcols) {
+  const size_t mm = (size_t)m + 1;
+  size_t b = 2 * sizeof(double) * mm + (3 + (size_t)zcols) * sizeof(float) * mm;
+  if (sizeof(T) == 8) b += (1 + (size_t)zcols) * sizeof(double) * mm;
+  return b + 64;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kRankThreads) k_rank(const TruncTask<T> *__restrict__ tasks, int *__restrict__ kout,
+                                                      int variant, int zcols, int in_smem) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ double s_red[3 * kRankThreads / 32];
+  __shared__ float s_cf[kMaxK1 * kMaxK1];
+  __shared__ T s_ct[kMaxK1 * kMaxK1];
+  __shared__ double s_half[2], s_lmax;
+  __shared__ int s_cnt[2];
+  const TruncTask<T> t = tasks[blockIdx.x];
+  const int m = t.m;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const BigLayout<T> L = big_layout<T>(t.work, m);
+  const bool gc = variant != HS_LORASP;
+  const int k1 = gc ? L.sc_int[0] : 0;
+  const size_t mm = (size_t)m + 1;
+  // (nodes beyond shared memory keep these vectors in Y, which is free until
+  // the eigenvectors go there)
+  double *d = in_smem ? (double *)smem_raw : (double *)(((uintptr_t)L.Y + 15) & ~(uintptr_t)15), *e2 = d + mm;
+  unsigned char *p = (unsigned char *)(e2 + mm);
+  double *ed = nullptr, *zd = nullptr;   // FP64 factor: e and Z
+  if constexpr (sizeof(T) == 8) {
+    ed = (double *)p;
+    zd = ed + mm;
+    p = (unsigned char *)(zd + (size_t)zcols * mm);
+  }
+  float *df = (float *)p, *ef = df + mm, *e2f = ef + mm, *zf = e2f + mm;
+  const bool zs = zcols >= k1;           // Z in shared memory
+  // T: the tridiagonalisation left d, e for k < m - 2 and the trailing 2 x 2 block in A
+  double dmax = -1e300, emax = 0.0, glo = 1e300, ghi = -1e300;
+  auto dat = [&](int i) {
+    return i + 2 < m ? L.d[i] : (double)L.A[(int64_t)i * m + i];
+  };
+  auto eat = [&](int i) {   // e_i couples i and i + 1
+    return i + 2 < m ? L.e[i] : i + 2 == m ? (double)L.A[(int64_t)(m - 1) * m + m - 2] : 0.0;
+  };
+  for (int i = tid; i < m; i += kRankThreads) {
+    // FP32 factors work on the FP32 rounding of T throughout, the count in FP64
+    const double di = dat(i), ei = eat(i), em = i > 0 ? eat(i - 1) : 0.0;
+    d[i] = di;
+    e2[i] = em * em;
+    const double r = fabs(em) + fabs(ei);
+    glo = fmin(glo, di - r);
+    ghi = fmax(ghi, di + r);
+    dmax = fmax(dmax, di);
+    emax = fmax(emax, em * em);
+    L.dt[i] = (T)di;
+    L.et[i] = (T)ei;
+    if (sizeof(T) == 8) ed[i] = ei;
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    glo = fmin(glo, __shfl_xor_sync(0xffffffffu, glo, o));
+    ghi = fmax(ghi, __shfl_xor_sync(0xffffffffu, ghi, o));
+    dmax = fmax(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
+    emax = fmax(emax, __shfl_xor_sync(0xffffffffu, emax, o));
+  }
+  constexpr int NW = kRankThreads / 32;
+  __shared__ double s_emax[NW];
+  if (lane == 0) {
+    s_red[warp] = glo;
+    s_red[NW + warp] = ghi;
+    s_red[2 * NW + warp] = dmax;
+    s_emax[warp] = emax;
+  }
+  __syncthreads();
+  for (int q = 0; q < NW; ++q) {
+    glo = fmin(glo, s_red[q]);
+    ghi = fmax(ghi, s_red[NW + q]);
+    dmax = fmax(dmax, s_red[2 * NW + q]);
+    emax = fmax(emax, s_emax[q]);
+  }
+  const double tnorm = fmax(fabs(glo), fabs(ghi));
+  // the bracket of lambda_max(G): C's diagonal bounds it below, its trace above
+  double ctr = 0.0, cmax = 0.0;
+  for (int a = 0; a < k1; ++a) {
+    const double c = L.sc_c[a * kMaxK1 + a];
+    ctr += fmax(c, 0.0);
+    cmax = fmax(cmax, c);
+  }
+  const double hi_u = (fmax(ghi, 0.0) + ctr) * (1.0 + 1e-4) + (sizeof(T) == 8 ? 1e-290 : 1e-30);
+  // The FP64 factor's T, Z and C times a power of two that brings the
+  // bracket's end near 1 (the values may lie outside the FP32 range, and a
+  // weakly coupled node's far below any absolute floor)
+  const double sc = sizeof(T) == 8 ? exp2(-(double)ilogb(hi_u)) : 1.0;
+  const double hi0 = hi_u * sc, lo0 = fmax(fmax(dmax, cmax), 0.0) * (1.0 - 1e-4) * sc;
+  const double emax_u = emax;
+  emax *= sc * sc;
+  if (sizeof(T) == 8)
+    for (int i = tid; i < m; i += kRankThreads) {
+      const double em = i > 0 ? eat(i - 1) * sc : 0.0;
+      d[i] *= sc;
+      e2[i] = em * em;
+      ed[i] *= sc;
+    }
+  for (int i = tid; i < m; i += kRankThreads) {
+    const float e1 = (float)(eat(i) * sc), e0 = i > 0 ? (float)(eat(i - 1) * sc) : 0.f;
+    df[i] = (float)d[i];
+    ef[i] = e1;
+    e2f[i] = e0 * e0;
+    if (zs)
+      for (int a = 0; a < k1; ++a) {
+        const T z = L.LS[(size_t)a * m + i];
+        zf[(size_t)a * mm + i] = (float)((double)z * sc);
+        if (sizeof(T) == 8) zd[(size_t)a * mm + i] = (double)z * sc;
+      }
+  }
+  if (!zs && sizeof(T) == 8)   // Z is not used after this kernel
+    for (int64_t q = tid; q < (int64_t)m * k1; q += kRankThreads) L.LS[q] = (T)((double)L.LS[q] * sc);
+  for (int q = tid; q < kMaxK1 * kMaxK1; q += kRankThreads) {
+    s_cf[q] = (float)(L.sc_c[q] * sc);
+    s_ct[q] = (T)(L.sc_c[q] * sc);
+  }
+  __syncthreads();
+  const float pivf = sturm_pivmin<float>((float)emax);
+  double lmax;   // of the scaled G
+  const bool wide_global = gc && !zs;   // many preserved vectors on a huge node
+  {
+    float lo = (float)lo0, hi = (float)hi0 * 1.000001f + 1e-37f;
+    if (!wide_global || sizeof(T) == 4) {
+      for (int round = 0; round < 8 && hi - lo > 4.f * unit_round<float>() * hi; ++round) {
+        const float h = hi - lo;
+        const float sig = lo + h * (float)(tid + 1) * (1.f / (kRankThreads + 1));
+        int c;
+        if (k1 == 0)
+          c = count_above<float>(df, e2f, m, sig, pivf);
+        else if (wide_global)
+          c = count_above_gc_wide<float>(df, ef, e2f, m, (const float *)(const void *)L.LS, m, k1, s_cf, sig, pivf);
+        else if (k1 <= 2)
+          c = count_above_gc<float, 2>(df, ef, e2f, m, zf, (int)mm, k1, s_cf, sig, pivf);
+        else
+          c = count_above_gc_wide<float>(df, ef, e2f, m, zf, (int)mm, k1, s_cf, sig, pivf);
+        const int n = __syncthreads_count(c >= 1);
+        const float a = n > 0 ? lo + h * (float)n * (1.f / (kRankThreads + 1)) : lo;
+        const float b = n < kRankThreads ? lo + h * (float)(n + 1) * (1.f / (kRankThreads + 1)) : hi;
+        lo = a;
+        hi = b;
+      }
+    }
+    lmax = (double)(0.5f * (lo + hi));
+    if constexpr (sizeof(T) == 8) {
+      if (warp == 0) {
+        const double piv = sturm_pivmin<double>(emax);
+        auto above = [&](double sig) {
+          if (k1 == 0) return count_above<double>(d, e2, m, sig, piv) >= 1;
+          const double *z = zs ? zd : (const double *)L.LS;   // (beyond shared memory: scaled in place below)
+          const int ldz = zs ? (int)mm : m;
+          return (k1 <= 2 ? count_above_gc<double, 2>(d, ed, e2, m, z, ldz, k1, s_ct, sig, piv)
+                          : count_above_gc_wide<double>(d, ed, e2, m, z, ldz, k1, s_ct, sig, piv)) >= 1;
+        };
+        double l = lmax * (1.0 - 7.6e-6), h = lmax * (1.0 + 7.6e-6);   // 64 u of FP32
+        const int miss = wide_global ? 2 : section<double, 32>(l, h, lane, true, above);
+        if (miss != 0) {
+          const double was_l = lmax * (1.0 - 7.6e-6), was_h = lmax * (1.0 + 7.6e-6);
+          l = miss == 1 ? was_h : lo0;
+          h = miss == -1 ? was_l : hi0;
         }
+        for (int round = 0; round < 40 && h - l > 4.0 * unit_round<double>() * h; ++round) {
+          const double pl = l, ph = h;
+          section<double, 32>(l, h, lane, false, above);
+          if (!(l > pl || h < ph)) break;
+        }
+        if (lane == 0) s_lmax = 0.5 * (l + h);
       }
       __syncthreads();
-      for (int64_t q = tid; q < (int64_t)m * nb; q += nt) {
-        const int i = (int)(q / nb), j = (int)(q % nb);
-        t.U[(int64_t)i * m + k1 + jb + j] = ysm[(size_t)j * m + i];
-      }
-      __syncthreads();
+      lmax = s_lmax;
     }
   }
-  if (tid == 0) kout[t.k_idx] = k1 + k2;
+  const double thr = t.eps * t.eps * lmax;
+  // the Sturm count in FP64 from both ends, middle row h
+  const double piv = sturm_pivmin<double>(emax);
+  const int h = m / 2;
+  if (tid == 0) {
+    int c = 0;
+    double q = 0.0;
+    for (int i = 0; i < h; ++i) {
+      q = d[i] - thr - (i > 0 ? e2[i] / q : 0.0);
+      if (fabs(q) < piv) q = -piv;
+      c += q < 0.0;
+    }
+    s_half[0] = h > 0 ? e2[h] / q : 0.0;
+    s_cnt[0] = c;
+  } else if (tid == 32) {
+    int c = 0;
+    double q = 0.0;
+    for (int i = m - 1; i > h; --i) {
+      q = d[i] - thr - (i + 1 < m ? e2[i + 1] / q : 0.0);
+      if (fabs(q) < piv) q = -piv;
+      c += q < 0.0;
+    }
+    s_half[1] = h + 1 < m ? e2[h + 1] / q : 0.0;
+    s_cnt[1] = c;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    double q = d[h] - thr - s_half[0] - s_half[1];
+    if (fabs(q) < piv) q = -piv;
+    int k2 = m - (s_cnt[0] + s_cnt[1] + (q < 0.0 ? 1 : 0));
+    k2 = max(0, min(k2, min(m - k1, t.cap - k1)));   // max_rank_ratio: the largest eigenvalues are kept
+    // a block whose Gram matrix has left the FP64 range has nothing to keep
+    if (sizeof(T) == 8 && hi_u < 1e-280) k2 = 0;
+    L.sc_int[1] = k2;
+    L.sc_b[0] = thr / sc;
+    L.sc_b[1] = ghi + unit_round<T>() * tnorm * 2.0 * m + (sizeof(T) == 8 ? 1e-290 : 1e-30);
+    L.sc_b[2] = emax_u;
+    *L.sc_tnorm = tnorm;
+    kout[t.k_idx] = k1 + k2;
+  }
+}
+
+// ---------------------------------------------------------------------------
+// The k2 largest eigenvalues of T (shifts of the inverse iteration), `lanes`
+// of a warp sectioning each: 8 below m = 128, where a wave has many nodes and
+// the work counts, 32 from there on, where the rounds do.  The bracket is
+// (eps^2 lambda_max, Gershgorin bound).  The FP64 factor places them in FP32
+// first and confirms and refines that bracket in FP64.
+// ---------------------------------------------------------------------------
+constexpr int kEigThreads = 128;
+__host__ __device__ inline int eig_lanes(int m) { return m < 128 ? 8 : 32; }
+
+template <typename T>
+__host__ __device__ inline size_t eigval_smem_bytes(int m) {
+  return 2 * sizeof(float) * (size_t)m + (sizeof(T) == 8 ? 2 * sizeof(double) * (size_t)m : 0) + 16;
+}
+
+template <typename Task>
+__device__ __forceinline__ int task_of(const Task *tasks, int ntasks, int b) {
+  int lo = 0, hi = ntasks - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (tasks[mid].blk0 <= b)
+      lo = mid;
+    else
+      hi = mid - 1;
+  }
+  return lo;
+}
+
+template <typename T, int LN>
+__device__ void eigvals(const EigTask<T> &t, int first, const double *d, const double *e2, const float *df,
+                        const float *e2f, double scf) {
+  const int m = t.m, k2 = t.sc[1];
+  const int lane = threadIdx.x & 31;
+  const int jj = first + (int)threadIdx.x / LN;
+  const int j = min(jj, k2 - 1);
+  // scaled as the arrays are
+  const double thr = t.sb[0] * scf, hi0 = t.sb[1] * scf, emax = t.sb[2] * scf * scf, tnorm = *t.tnorm * scf;
+  const float pivf = sturm_pivmin<float>((float)emax);
+  float lo = (float)thr, hi = (float)hi0;
+  const float tol = 4.f * unit_round<float>() * (float)tnorm;
+  for (int round = 0; round < 12 && __any_sync(0xffffffffu, hi - lo > tol); ++round)
+    section<float, LN>(lo, hi, lane, false,
+                       [&](float s) { return count_above<float>(df, e2f, m, s, pivf) > j; });
+  if constexpr (sizeof(T) == 4) {
+    if (jj < k2 && lane % LN == 0) t.lam[jj] = 0.5f * (lo + hi);
+  } else {
+    const double piv = sturm_pivmin<double>(emax);
+    auto above = [&](double s) { return count_above<double>(d, e2, m, s, piv) > j; };
+    const double mid = 0.5 * ((double)lo + (double)hi), w = 64.0 * 1.2e-7 * tnorm;
+    double l = mid - w, h = mid + w;
+    const int miss = section<double, LN>(l, h, lane, true, above);
+    if (miss != 0) {
+      l = miss == 1 ? mid + w : fmin(thr, mid - 2.0 * w);
+      h = miss == -1 ? mid - w : hi0;
+    }
+    const double told = 4.0 * unit_round<double>() * tnorm;
+    for (int round = 0; round < 40 && __any_sync(0xffffffffu, h - l > told); ++round)
+      section<double, LN>(l, h, lane, false, above);
+    if (jj < k2 && lane % LN == 0) t.lam[jj] = 0.5 * (l + h) / scf;
+  }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kEigThreads) k_eigval(const EigTask<T> *__restrict__ tasks, int ntasks) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const EigTask<T> t = tasks[task_of(tasks, ntasks, blockIdx.x)];
+  const int m = t.m;
+  const int lanes = eig_lanes(m);
+  const int first = (blockIdx.x - t.blk0) * (kEigThreads / lanes);
+  if (first >= t.sc[1]) return;
+  double *d = (double *)smem_raw, *e2 = d + m;
+  float *df = sizeof(T) == 8 ? (float *)(e2 + m) : (float *)smem_raw;
+  float *e2f = df + m;
+  // as in k_rank: the FP64 factor's T scaled near 1
+  const double scf = sizeof(T) == 8 ? exp2(-(double)ilogb(fmax(t.sb[1], 1e-290))) : 1.0;
+  for (int i = threadIdx.x; i < m; i += kEigThreads) {
+    const T di = t.dt[i], ei = i > 0 ? t.et[i - 1] : T(0);
+    df[i] = sizeof(T) == 8 ? (float)(di * scf) : (float)di;
+    const float es = sizeof(T) == 8 ? (float)(ei * scf) : (float)ei;
+    e2f[i] = es * es;
+    if (sizeof(T) == 8) {
+      d[i] = (double)di * scf;
+      e2[i] = ((double)ei * scf) * ((double)ei * scf);
+    }
+  }
+  __syncthreads();
+  if (lanes == 8)
+    eigvals<T, 8>(t, first, d, e2, df, e2f, scf);
+  else
+    eigvals<T, 32>(t, first, d, e2, df, e2f, scf);
+}
+
+// ---------------------------------------------------------------------------
+// Inverse iteration for the selected eigenvalues, one lane each: LU of
+// T - lam I with partial pivoting (rows i, i+1 interchanged when the
+// sub-diagonal dominates), three solves from a fixed pseudo-random start,
+// modified Gram-Schmidt against the vectors already found of the same cluster
+// of eigenvalues closer than 10 u ||T|| (those could come out nearly
+// parallel; the lane of a cluster's first eigenvalue takes them all in turn).
+// Only the span of the selected vectors matters and the host
+// re-orthonormalises them, which tolerates the overlap u ||T|| / gap that
+// inverse iteration leaves between vectors of distinct eigenvalues.
+// One warp per CTA; a lane's LU (inverse pivots, two super-diagonals,
+// multipliers), vector and interchange flags sit in shared memory, element i
+// of lane s at i * st + s with st odd, so that neither the lanes' sweeps nor
+// the write-out of whole vectors conflict.  A sweep carries its two last
+// values in registers: one fused multiply-add (forward) or two and a product
+// (backward) per row on the dependent chain.
+// ---------------------------------------------------------------------------
+template <typename T>
+__host__ __device__ inline size_t invit_smem_bytes(int m, int slots, bool with_t) {
+  return ((5 * sizeof(T) + 1) * (size_t)(slots | 1) + (with_t ? 2 * sizeof(T) : 0)) * (size_t)m + 16;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(32) k_invit(const EigTask<T> *__restrict__ tasks, int ntasks, int spc,
+                                              int with_t) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const EigTask<T> t = tasks[task_of(tasks, ntasks, blockIdx.x)];
+  const int m = t.m, k2 = t.sc[1];
+  const int lane = threadIdx.x;
+  const int q0 = (blockIdx.x - t.blk0) * spc;
+  if (q0 >= k2) return;
+  const int st = spc | 1;
+  const size_t sm = (size_t)m * st;
+  T *iu = (T *)smem_raw + (with_t ? 2 * (size_t)m : 0), *u1 = iu + sm, *u2 = u1 + sm, *lm = u2 + sm, *y = lm + sm;
+  unsigned char *fl = (unsigned char *)(y + sm);
+  const T *dt = t.dt, *et = t.et;   // staged when they fit beside the slots
+  if (with_t) {
+    T *ds = (T *)smem_raw, *es = ds + m;
+    for (int i = lane; i < m; i += 32) {
+      ds[i] = t.dt[i];
+      es[i] = t.et[i];
+    }
+    dt = ds;
+    et = es;
+  }
+  __syncwarp();
+  const T tnorm = (T)*t.tnorm;
+  const T ortol = T(10) * unit_round<T>() * tnorm;
+  const T small = unit_round<T>() * tnorm + T(sizeof(T) == 8 ? 1e-290 : 1e-30);
+  const int q = q0 + lane;
+  // lane of a cluster's first eigenvalue: vectors q .. q + nrun - 1
+  int nrun = 0;
+  if (lane < spc && q < k2 && (q == 0 || t.lam[q - 1] - t.lam[q] >= ortol)) {
+    nrun = 1;
+    while (q + nrun < k2 && t.lam[q + nrun - 1] - t.lam[q + nrun] < ortol) ++nrun;
+  }
+  for (int run = 0; __any_sync(0xffffffffu, run < nrun); ++run) {
+    const bool on = run < nrun;
+    if (on) {
+      const T lam = t.lam[q + run];
+      const T *prev = t.Y + (size_t)q * m;
+      const uint32_t seed = (uint32_t)((q + run) * 7919 + 17);
+      T a = dt[0] - lam, c = m > 1 ? et[0] : T(0);
+      for (int i = 0; i + 1 < m; ++i) {
+        const T b = et[i];
+        const T an = dt[i + 1] - lam;
+        const T cn = i + 2 < m ? et[i + 1] : T(0);
+        const size_t o = (size_t)i * st + lane;
+        const bool swap = fabs(a) < fabs(b);
+        T piv = swap ? b : (a == T(0) ? small : a);
+        const T inv = T(1) / piv;
+        const T mult = (swap ? a : b) * inv;
+        iu[o] = fabs(piv) < small ? T(1) / copysign(small, piv) : inv;
+        u1[o] = swap ? an : c;
+        u2[o] = swap ? cn : T(0);
+        lm[o] = mult;
+        fl[o] = swap;
+        const T na = swap ? c - mult * an : an - mult * c;
+        c = swap ? -mult * cn : cn;
+        a = na;
+      }
+      iu[(size_t)(m - 1) * st + lane] = T(1) / (fabs(a) < small ? copysign(small, a) : a);
+      for (int i = 0; i < m; ++i) y[(size_t)i * st + lane] = (T)hash_unit(seed, (uint32_t)i);
+      T scale = T(1);
+      for (int it = 0; it < 3; ++it) {
+        T cur = y[lane] * scale;
+#pragma unroll 4
+        for (int i = 0; i + 1 < m; ++i) {
+          const size_t o = (size_t)i * st + lane;
+          const T yn = y[o + st] * scale;
+          const T l = lm[o];
+          const bool swap = fl[o];
+          y[o] = swap ? yn : cur;
+          cur = swap ? fma(-l, yn, cur) : fma(-l, cur, yn);
+        }
+        T y1 = cur * iu[(size_t)(m - 1) * st + lane], y2 = T(0);
+        y[(size_t)(m - 1) * st + lane] = y1;
+        T big = fabs(y1);
+#pragma unroll 4
+        for (int i = m - 2; i >= 0; --i) {
+          const size_t o = (size_t)i * st + lane;
+          const T s = fma(-u1[o], y1, fma(-u2[o], y2, y[o])) * iu[o];
+          y[o] = s;
+          y2 = y1;
+          y1 = s;
+          big = fmax(big, fabs(s));
+        }
+        if (run > 0) {
+          for (int pass = 0; pass < 2; ++pass)
+            for (int p = 0; p < run; ++p) {
+              const T *v = prev + (size_t)p * m;
+              T dot = T(0);
+              for (int i = 0; i < m; ++i) dot += v[i] * y[(size_t)i * st + lane];
+              for (int i = 0; i < m; ++i) y[(size_t)i * st + lane] -= dot * v[i];
+            }
+          big = T(0);
+          for (int i = 0; i < m; ++i) big = fmax(big, fabs(y[(size_t)i * st + lane]));
+        }
+        // norm, scaling by the largest entry first to keep the sum in range;
+        // the next sweep applies the factor as it reads
+        const T sc = big > T(0) ? T(1) / big : T(0);
+        T n0 = T(0), n1 = T(0);
+#pragma unroll 2
+        for (int i = 0; i + 1 < m; i += 2) {
+          const T v0 = y[(size_t)i * st + lane] * sc, v1 = y[(size_t)(i + 1) * st + lane] * sc;
+          n0 = fma(v0, v0, n0);
+          n1 = fma(v1, v1, n1);
+        }
+        if (m & 1) {
+          const T v0 = y[(size_t)(m - 1) * st + lane] * sc;
+          n0 = fma(v0, v0, n0);
+        }
+        const T nrm = sqrt(n0 + n1);
+        scale = nrm > T(0) ? sc / nrm : T(0);
+      }
+      for (int i = 0; i < m; ++i) y[(size_t)i * st + lane] *= scale;
+    }
+    __syncwarp();
+    // whole vectors, consecutive lanes on consecutive entries
+    for (int s = 0; s < spc; ++s) {
+      if (!__shfl_sync(0xffffffffu, (int)on, s)) continue;
+      T *out = t.Y + (size_t)(q0 + s + run) * m;
+      for (int i = lane; i < m; i += 32) out[i] = y[(size_t)i * st + s];
+    }
+    __syncwarp();   // the vectors are read back by the next of a cluster
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Products with Q = H_0 ... H_{m-3} (I - tau_k v_k v_k^T, v_k = 1 at row k + 1,
+// its tail in row k of A): forward (Z = Q^T X, in place) or backward (U_2 = Q Y,
+// into U's columns from k1 on).  A warp keeps its columns in registers (row
+// lane + 32 e in register e, e < E) and applies the reflectors one after the
+// other: products over the rows above, one warp sum for all its columns, one
+// update, no barrier; the next reflector's row is loaded meanwhile.  Four warps
+// per CTA.  A node's E, columns per warp and sums depend on m alone.
+// (One CTA per 16 columns with block sums took three barriers a reflector.)
+// ---------------------------------------------------------------------------
+constexpr int kQmWarps = 4;
+__host__ __device__ inline int qmul_e(int m) { return m <= 64 ? 2 : m <= 128 ? 4 : m <= 256 ? 8 : m <= 512 ? 16 : 32; }
+template <typename T>
+__host__ __device__ constexpr int qmul_cols(int E) {
+  return sizeof(T) == 4 ? (E <= 8 ? 4 : E == 16 ? 2 : 1) : (E <= 4 ? 4 : E == 8 ? 2 : 1);
+}
+
+template <typename T, int E, int C>
+__device__ void qmul_warp(const QmulTask<T> &t, int j0, int nc, T *stage, int sld) {
+  const int m = t.m, lane = threadIdx.x & 31;
+  T yv[C][E];
+#pragma unroll
+  for (int c = 0; c < C; ++c)
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const int i = lane + 32 * e;
+      yv[c][e] = i < m && c < nc ? t.cols[(size_t)(j0 + c) * m + i] : T(0);
+    }
+  const int steps = m - 2;
+  auto load = [&](int s, T (&v)[E], T &tau) {
+    const int k = t.fwd ? s : m - 3 - s;
+    tau = t.tau[k];
+    const T *row = t.A + (size_t)k * m;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const int i = lane + 32 * e;
+      v[e] = i > k + 1 && i < m ? __ldg(row + i) : (i == k + 1 ? T(1) : T(0));
+    }
+  };
+  T v[E], tau;
+  if (steps > 0) load(0, v, tau);
+  for (int s = 0; s < steps; ++s) {
+    T vn[E], taun = T(0);
+    if (s + 1 < steps) load(s + 1, vn, taun);
+    T dot[C];
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+      dot[c] = T(0);
+#pragma unroll
+      for (int e = 0; e < E; ++e) dot[c] = fma(v[e], yv[c][e], dot[c]);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int c = 0; c < C; ++c) dot[c] += __shfl_xor_sync(0xffffffffu, dot[c], o);
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+      const T f = tau * dot[c];
+#pragma unroll
+      for (int e = 0; e < E; ++e) yv[c][e] = fma(-f, v[e], yv[c][e]);
+    }
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[e] = vn[e];
+    tau = taun;
+  }
+  if (t.fwd) {
+#pragma unroll
+    for (int c = 0; c < C; ++c)
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const int i = lane + 32 * e;
+        if (i < m && c < nc) t.cols[(size_t)(j0 + c) * m + i] = yv[c][e];
+      }
+  } else {
+    // through shared memory: U's rows take the CTA's adjacent columns together
+    const int c0 = (threadIdx.x >> 5) * C;
+#pragma unroll
+    for (int c = 0; c < C; ++c)
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const int i = lane + 32 * e;
+        if (i < m && c < nc) stage[(size_t)i * sld + c0 + c] = yv[c][e];
+      }
+  }
+}
+
+// EM: the largest E of the launch (its registers); a node runs its own E
+template <typename T, int EM>
+__global__ void __launch_bounds__(kQmWarps * 32) k_qmul(const QmulTask<T> *__restrict__ tasks, int ntasks) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const QmulTask<T> t = tasks[task_of(tasks, ntasks, blockIdx.x)];
+  const int m = t.m, E = qmul_e(m);
+  const int k1 = t.sc[0];
+  const int ncol = t.fwd ? k1 : t.sc[1];
+  const int C = qmul_cols<T>(E);
+  const int per = kQmWarps * C;
+  const int jc = (blockIdx.x - t.blk0) * per;   // the CTA's first column
+  if (jc >= ncol) return;
+  T *stage = (T *)smem_raw;
+  const int sld = per + 1;
+  const int j0 = jc + (threadIdx.x >> 5) * C;
+  const int nc = min(C, ncol - j0);
+  if (nc > 0) {
+    if (E == 2)
+      qmul_warp<T, 2, qmul_cols<T>(2)>(t, j0, nc, stage, sld);
+    if constexpr (EM >= 4)
+      if (E == 4) qmul_warp<T, 4, qmul_cols<T>(4)>(t, j0, nc, stage, sld);
+    if constexpr (EM >= 8)
+      if (E == 8) qmul_warp<T, 8, qmul_cols<T>(8)>(t, j0, nc, stage, sld);
+    if constexpr (EM >= 16)
+      if (E == 16) qmul_warp<T, 16, qmul_cols<T>(16)>(t, j0, nc, stage, sld);
+    if constexpr (EM >= 32)
+      if (E == 32) qmul_warp<T, 32, qmul_cols<T>(32)>(t, j0, nc, stage, sld);
+  }
+  if (t.fwd) return;
+  __syncthreads();
+  const int w = min(per, ncol - jc);
+  for (int q = threadIdx.x; q < m * w; q += kQmWarps * 32) {
+    const int i = q / w, c = q % w;
+    t.U[(int64_t)i * m + k1 + jc + c] = stage[(size_t)i * sld + c];
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -983,7 +1063,7 @@ __global__ void __launch_bounds__(kTriRows * 32) k_tri_symv(const GridTri<T> *__
   const int rb = blockIdx.x - t.blk0;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (warp == 0) {
-    // the reflector of x = A[k+1.., k] (as in the one-CTA tridiagonalisation)
+    // the reflector of x = A[k+1.., k] (as in the cluster tridiagonalisation)
     const double xn2 = (double)warp_sum_parts<T>(t.px, t.nblk, lane);
     if (lane == 0) {
       const double alpha = (double)t.X[k + 1];
@@ -1042,49 +1122,8 @@ __global__ void __launch_bounds__(kTriRows * 32) k_tri_symv(const GridTri<T> *__
   }
 }
 
-// Inverse iteration of the multi-CTA path: one warp per CTA, `spc` of its
-// threads active, each with a slot (LU of T - lam I and the vector: 5 m T and m
-// flags) in shared memory, taking one cluster of close eigenvalues.  Same
-// arithmetic as the one-CTA kernel; each step of the recurrence stays on chip.
-template <typename T>
-__device__ __forceinline__ int invit_task(const InvitTask<T> *tasks, int ntasks, int b) {
-  int lo = 0, hi = ntasks - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (tasks[mid].blk0 <= b)
-      lo = mid;
-    else
-      hi = mid - 1;
-  }
-  return lo;
-}
-
-template <typename T>
-__host__ __device__ inline size_t invit_slot_bytes(int m) {
-  return ((5 * (size_t)m * sizeof(T) + (size_t)m + 15) / 16) * 16;
-}
-
-template <typename T>
-__global__ void __launch_bounds__(32) k_invit(const InvitTask<T> *__restrict__ tasks, int ntasks, int spc) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const InvitTask<T> t = tasks[invit_task(tasks, ntasks, blockIdx.x)];
-  const int m = t.m;
-  const int c = (blockIdx.x - t.blk0) * spc + threadIdx.x;
-  if ((int)threadIdx.x >= spc || c >= t.sc[2]) return;
-  unsigned char *slot = smem_raw + (size_t)threadIdx.x * invit_slot_bytes<T>(m);
-  T *lu = (T *)slot;
-  T *ys = lu + 4 * (size_t)m;
-  unsigned char *fl = (unsigned char *)(ys + m);
-  const T tnorm = (T)*t.tnorm;
-  const int j0 = t.starts[c], j1 = t.starts[c + 1];
-  for (int q = j0; q < j1; ++q) {
-    inverse_iteration<T>(t.dt, t.et, m, t.lam[q], tnorm, ys, t.Y + (size_t)j0 * m, q - j0, lu, fl,
-                         (uint32_t)(q * 7919 + 17));
-    for (int i = 0; i < m; ++i) t.Y[(size_t)q * m + i] = ys[i];
-  }
-}
-
-// Products with the reflectors of a node, one CTA per batch of columns held in
+// The same products for nodes too large for a warp's registers (m > 1024), one CTA
+// per batch of columns held in
 // shared memory: for each reflector the block forms all the batch's dot
 // products (fixed-order reduction), then updates the columns.
 constexpr int RT = 256;
@@ -1098,7 +1137,7 @@ __global__ void __launch_bounds__(RT) k_refl(const ReflTask<T> *__restrict__ tas
   const ReflTask<T> t = tasks[blockIdx.x];
   const int m = t.m;
   const int k1 = t.sc[0];
-  const int ncol = t.fwd ? 2 * k1 : t.sc[1];
+  const int ncol = t.fwd ? k1 : t.sc[1];
   if (t.j0 >= ncol) return;
   const int nc = min(nb, ncol - t.j0);
   T *Ys = (T *)smem_raw;
@@ -1151,64 +1190,104 @@ __global__ void __launch_bounds__(RT) k_refl(const ReflTask<T> *__restrict__ tas
 
 }  // namespace
 
-// bytes of the per-node vectors of k_trunc_big (d, e, pw in FP64; six m-vectors
-// and 34 reduction slots in T), 16-byte aligned
-template <typename T>
-size_t trunc_big_vec_bytes(int m) {
-  return big_vec_bytes<T>(m);
-}
-
 template <typename T>
 size_t trunc_big_work_elems(int m) {
-  // A, Y, LU (6 m^2 T) + LS (164 m T) + flags (m^2 bytes) + the vectors (when
-  // they do not fit in shared memory) + SC; Y and LU also hold k1 m doubles
-  // of scratch
-  const size_t bytes = sizeof(T) * (6 * (size_t)m * m + 164 * (size_t)m) + (size_t)m * m + 16 +
-                       trunc_big_vec_bytes<T>(m) + 16 + kBigScBytes + 64;
+  // A, Y (2 m^2 T), LS (32 m T), the vectors and SC
+  const size_t bytes = sizeof(T) * (2 * (size_t)m * m + 32 * (size_t)m) + 16 + big_vec_bytes<T>(m) + 16 + kBigScBytes + 64;
   return (bytes + sizeof(T) - 1) / sizeof(T);
 }
 
-template <typename T, int NT>
-void launch_trunc_big_nt(const TruncTask<T> *d_tasks, int ntasks, int *d_k, double eps, int variant, int max_m,
-                         cudaStream_t st) {
+// 256 threads per node up to m = 256, 1024 above (a function of m alone)
+template <typename T>
+void launch_trunc_prep(const TruncTask<T> *d_tasks, int ntasks, int *d_k, int variant, int max_m, cudaStream_t st) {
   if (ntasks == 0) return;
-  // the per-node vectors go to shared memory while they leave room for a
-  // tile of at least 64 x 64; the rest of the budget is the tile, no larger
-  // than the largest node needs
-  const size_t budget = 200 * 1024;
-  size_t fixed = trunc_big_vec_bytes<T>(max_m) + 32;
-  const int vec_smem = fixed + 64 * 64 * sizeof(T) <= budget ? 1 : 0;
-  if (!vec_smem) fixed = 32;
-  int cap = 0;
-  while (cap < max_m && (size_t)(cap + 1) * (cap + 1) * sizeof(T) + fixed <= budget) ++cap;
-  const size_t sm = fixed + (size_t)cap * cap * sizeof(T);
-  check_dynamic_smem(sm, allow_max_dynamic_smem<&k_trunc_big<T, NT>>(), "k_trunc_big");
-  k_trunc_big<T, NT><<<ntasks, NT, sm, st>>>(d_tasks, d_k, variant, cap, vec_smem, TB_FULL);
+  if (max_m <= kTruncPrepMid)
+    k_trunc_prep<T, 256><<<ntasks, 256, 0, st>>>(d_tasks, d_k, variant);
+  else
+    k_trunc_prep<T, 1024><<<ntasks, 1024, 0, st>>>(d_tasks, d_k, variant);
   count_launch();
   HS_CUDA(cudaGetLastError());
 }
 
 template <typename T>
-void launch_trunc_big(const TruncTask<T> *d_tasks, int ntasks, int *d_k, double eps, int variant, int max_m,
-                      cudaStream_t st) {
-  if (max_m <= kTruncBigMidMax)
-    launch_trunc_big_nt<T, 256>(d_tasks, ntasks, d_k, eps, variant, max_m, st);
-  else
-    launch_trunc_big_nt<T, 1024>(d_tasks, ntasks, d_k, eps, variant, max_m, st);
+void launch_rank(const TruncTask<T> *d_tasks, int ntasks, int *d_k, int variant, int max_m, int max_np,
+                 cudaStream_t st) {
+  if (ntasks == 0) return;
+  const int limit = allow_max_dynamic_smem<&k_rank<T>>();
+  int zcols = variant == HS_LORASP ? 0 : 2 * max_np;
+  if (rank_smem_bytes<T>(max_m, zcols) > (size_t)limit) zcols = 0;
+  size_t sm = rank_smem_bytes<T>(max_m, zcols);
+  const int in_smem = sm <= (size_t)limit;
+  if (!in_smem) sm = 0;
+  k_rank<T><<<ntasks, kRankThreads, sm, st>>>(d_tasks, d_k, variant, zcols, in_smem);
+  count_launch();
+  HS_CUDA(cudaGetLastError());
 }
 
 template <typename T>
-void launch_trunc_big_mode(const TruncTask<T> *d_tasks, int ntasks, int *d_k, double eps, int variant, int max_m,
-                           int mode, cudaStream_t st) {
-  if (ntasks == 0) return;
-  // per-node vectors in global memory (the step kernels write d, e, tau there);
-  // the whole budget is the tile
+int eigval_blocks(int m) {
+  const int per = kEigThreads / eig_lanes(m);
+  return (m + per - 1) / per;
+}
+
+template <typename T>
+void launch_eigval(const EigTask<T> *d_tasks, int ntasks, int total_blocks, int m_max, cudaStream_t st) {
+  if (ntasks == 0 || total_blocks == 0) return;
+  const size_t sm = eigval_smem_bytes<T>(m_max);
+  check_dynamic_smem(sm, allow_max_dynamic_smem<&k_eigval<T>>(), "k_eigval");
+  k_eigval<T><<<total_blocks, kEigThreads, sm, st>>>(d_tasks, ntasks);
+  count_launch();
+  HS_CUDA(cudaGetLastError());
+}
+
+template <typename T>
+int invit_slots(int m) {
   const size_t budget = 200 * 1024;
-  int cap = 0;
-  while (cap < max_m && (size_t)(cap + 1) * (cap + 1) * sizeof(T) + 32 <= budget) ++cap;
-  const size_t sm = 32 + (size_t)cap * cap * sizeof(T);
-  check_dynamic_smem(sm, allow_max_dynamic_smem<&k_trunc_big<T, 1024>>(), "k_trunc_big");
-  k_trunc_big<T, 1024><<<ntasks, 1024, sm, st>>>(d_tasks, d_k, variant, cap, 0, mode);
+  int spc = 32;
+  while (spc > 1 && invit_smem_bytes<T>(std::max(m, 1), spc, true) > budget) --spc;
+  return spc;
+}
+
+template <typename T>
+void launch_invit(const EigTask<T> *d_tasks, int ntasks, int total_blocks, int spc, int m_max, cudaStream_t st) {
+  if (ntasks == 0 || total_blocks == 0) return;
+  const int limit = allow_max_dynamic_smem<&k_invit<T>>();
+  const bool with_t = invit_smem_bytes<T>(m_max, spc, true) <= (size_t)limit;
+  const size_t sm = invit_smem_bytes<T>(m_max, spc, with_t);
+  check_dynamic_smem(sm, limit, "k_invit");
+  k_invit<T><<<total_blocks, 32, sm, st>>>(d_tasks, ntasks, spc, with_t ? 1 : 0);
+  count_launch();
+  HS_CUDA(cudaGetLastError());
+}
+
+template <typename T>
+int qmul_blocks(int m, int ncol) {
+  const int per = kQmWarps * qmul_cols<T>(qmul_e(m));
+  return (ncol + per - 1) / per;
+}
+
+template <typename T, int EM>
+static void launch_qmul_e(const QmulTask<T> *d_tasks, int ntasks, int total_blocks, size_t sm, cudaStream_t st) {
+  check_dynamic_smem(sm, allow_max_dynamic_smem<&k_qmul<T, EM>>(), "k_qmul");
+  k_qmul<T, EM><<<total_blocks, kQmWarps * 32, sm, st>>>(d_tasks, ntasks);
+}
+
+template <typename T>
+void launch_qmul(const QmulTask<T> *d_tasks, int ntasks, int total_blocks, int m_max, bool fwd, cudaStream_t st) {
+  if (ntasks == 0 || total_blocks == 0) return;
+  const int E = qmul_e(m_max);
+  // the staged columns: the larger of m (4 C(E) + 1) over the classes up to E
+  size_t sm = 0;
+  if (!fwd)
+    for (int e = 2; e <= E; e *= 2)
+      sm = std::max(sm, sizeof(T) * (size_t)std::min(m_max, 32 * e) * (kQmWarps * qmul_cols<T>(e) + 1));
+  switch (E) {
+    case 2: launch_qmul_e<T, 2>(d_tasks, ntasks, total_blocks, sm, st); break;
+    case 4: launch_qmul_e<T, 4>(d_tasks, ntasks, total_blocks, sm, st); break;
+    case 8: launch_qmul_e<T, 8>(d_tasks, ntasks, total_blocks, sm, st); break;
+    case 16: launch_qmul_e<T, 16>(d_tasks, ntasks, total_blocks, sm, st); break;
+    default: launch_qmul_e<T, 32>(d_tasks, ntasks, total_blocks, sm, st); break;
+  }
   count_launch();
   HS_CUDA(cudaGetLastError());
 }
@@ -1241,40 +1320,22 @@ void launch_refl(const ReflTask<T> *d_tasks, int ntasks, int nb, int m_max, cuda
   HS_CUDA(cudaGetLastError());
 }
 
-template <typename T>
-int invit_slots(int m) {
-  const size_t budget = 200 * 1024;
-  const int spc = (int)(budget / invit_slot_bytes<T>(std::max(m, 1)));
-  return std::max(1, std::min(spc, 32));
-}
 
-template <typename T>
-void launch_invit(const InvitTask<T> *d_tasks, int ntasks, int total_blocks, int spc, int m_max, cudaStream_t st) {
-  if (ntasks == 0 || total_blocks == 0) return;
-  const size_t sm = (size_t)spc * invit_slot_bytes<T>(m_max);
-  check_dynamic_smem(sm, allow_max_dynamic_smem<&k_invit<T>>(), "k_invit");
-  k_invit<T><<<total_blocks, 32, sm, st>>>(d_tasks, ntasks, spc);
-  count_launch();
-  HS_CUDA(cudaGetLastError());
-}
-
-template int invit_slots<double>(int);
-template int invit_slots<float>(int);
-template void launch_invit<double>(const InvitTask<double> *, int, int, int, int, cudaStream_t);
-template void launch_invit<float>(const InvitTask<float> *, int, int, int, int, cudaStream_t);
-template void launch_trunc_big_mode<double>(const TruncTask<double> *, int, int *, double, int, int, int,
-                                            cudaStream_t);
-template void launch_trunc_big_mode<float>(const TruncTask<float> *, int, int *, double, int, int, int,
-                                           cudaStream_t);
-template void launch_tri_step<double>(const GridTri<double> *, int, int, int, int, cudaStream_t);
-template void launch_tri_step<float>(const GridTri<float> *, int, int, int, int, cudaStream_t);
-template int refl_batch<double>(int);
-template int refl_batch<float>(int);
-template void launch_refl<double>(const ReflTask<double> *, int, int, int, cudaStream_t);
-template void launch_refl<float>(const ReflTask<float> *, int, int, int, cudaStream_t);
-template size_t trunc_big_work_elems<double>(int);
-template size_t trunc_big_work_elems<float>(int);
-template void launch_trunc_big<double>(const TruncTask<double> *, int, int *, double, int, int, cudaStream_t);
-template void launch_trunc_big<float>(const TruncTask<float> *, int, int *, double, int, int, cudaStream_t);
+#define HS_INST(T)                                                                                             \
+  template void launch_trunc_prep<T>(const TruncTask<T> *, int, int *, int, int, cudaStream_t);                \
+  template void launch_rank<T>(const TruncTask<T> *, int, int *, int, int, int, cudaStream_t);                 \
+  template int eigval_blocks<T>(int);                                                                          \
+  template void launch_eigval<T>(const EigTask<T> *, int, int, int, cudaStream_t);                             \
+  template int invit_slots<T>(int);                                                                            \
+  template void launch_invit<T>(const EigTask<T> *, int, int, int, int, cudaStream_t);                         \
+  template int qmul_blocks<T>(int, int);                                                                       \
+  template void launch_qmul<T>(const QmulTask<T> *, int, int, int, bool, cudaStream_t);                        \
+  template void launch_tri_step<T>(const GridTri<T> *, int, int, int, int, cudaStream_t);                      \
+  template int refl_batch<T>(int);                                                                             \
+  template void launch_refl<T>(const ReflTask<T> *, int, int, int, cudaStream_t);                              \
+  template size_t trunc_big_work_elems<T>(int);
+HS_INST(double)
+HS_INST(float)
+#undef HS_INST
 
 }  // namespace hs
