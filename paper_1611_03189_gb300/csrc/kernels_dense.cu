@@ -186,109 +186,268 @@ __global__ void __launch_bounds__(256) k_sum(const SumTask<T> *__restrict__ task
 }
 
 // ---------------------------------------------------------------------------
-// Cholesky and inverse of the factor, one CTA per matrix
-// ---------------------------------------------------------------------------
-constexpr int CHOL_THREADS = 512;
-
-// W (ld m) holds A on entry; on exit the lower triangle holds L^-1 and the
-// strict upper triangle is zero.  Returns 0 or (failing pivot + 1).  tmp holds
-// 3m values.
+// Cholesky and inverse of the factor, one CTA per matrix, in shared memory.
 //
-// Right-looking Cholesky fused with the rows of X = L^-1 by forward
-// substitution: step j forms column j of L and, in the same phase as the
-// trailing update, row j of X,
-//   X_jc = (delta_jc - sum_{p=c..j-1} L_jp X_pc) / L_jj   (c <= j),
-// thread c owning column c of X.  Row j of L is needed only in step j, so row
-// j - 1 of X (kept in tmp until then) replaces it during step j.  Two
-// barriers per step.
+// Block columns of 16.  Step b, with j0 = 16 b, D_b = L_bb^-1:
+//   panel   P_i = L_ib = W_ib D_b^T for the rows i below, and the finished block
+//           row X_b,0:j0 = -D_b R_b of the inverse, one thread per row or column;
+//   update  W_i,c -= P_i P_c^T (c > b, the trailing block) and
+//           R_i,c += P_i X_b,c (c <= b, X_bb = D_b): the sums R_i = sum_p L_ip X_p
+//           of the inverse's rows grow in place of the columns of L that are no
+//           longer needed, so both halves are one rank-16 update of whole rows,
+//           in 32 x 16 tiles per warp, 4 x 4 outputs a lane, 16-byte loads along
+//           k (P) or along the row (X).
+// The only serial chain is the 16 x 16 diagonal block: one warp factors it in
+// registers, lane = row, and forms D_b with the same shuffles.  Warp 0 updates
+// the next diagonal block first and factors it while the other warps finish
+// the update.  Three barriers per 16 columns.
+// What bounds it: the diagonal chain up to m of about 100, the CUDA cores' FMA
+// rate above (FP64: throughout).  (The form before, column by column with two
+// barriers a column and a forward substitution down each column, was bound by
+// shared-memory latency.)
+// ---------------------------------------------------------------------------
+constexpr int kCholNb = 16;
+
+// row strides in elements: odd multiples of 16 bytes, so that 8 consecutive
+// rows' 16-byte pieces fall into different banks
 template <typename T>
-__device__ int chol_inv_inplace(T *W, int m, T *tmp, int *flag) {
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const int warp0 = tid >> 5, lane0 = tid & 31, nw0 = nt >> 5;
-  T *col = tmp;                  // scaled column j of L
-  T *xr0 = tmp + m, *xr1 = xr0 + m;   // rows j (j even: xr0) and j - 1 of X
-  (void)flag;
-  for (int j = 0; j < m; ++j) {
-    // every thread reads the pivot (the previous step's update is complete)
-    const T d = W[(size_t)j * m + j];
-    if (!(d > T(0)) || !isfinite(d)) return j + 1;
-    const T djj = sqrt(d);
-    for (int i = j + 1 + tid; i < m; i += nt) {
-      const T l = W[(size_t)i * m + j] / djj;
-      W[(size_t)i * m + j] = l;
-      col[i] = l;
-    }
-    __syncthreads();
-    // trailing update, one warp per row (lanes over columns, coalesced)
-    for (int i = j + 1 + warp0; i < m; i += nw0) {
-      const T li = col[i];
-      T *row = W + (size_t)i * m;
-      for (int c = j + 1 + lane0; c <= i; c += 32) row[c] -= li * col[c];
-    }
-    // row j of X; row j - 1 of X retires into row j - 1 of W
-    T *xj = (j & 1) ? xr1 : xr0;
-    const T *xprev = (j & 1) ? xr0 : xr1;
-    const T *Lj = W + (size_t)j * m;
-    for (int c = tid; c <= j; c += nt) {
-      T s0 = (c == j) ? T(1) : T(0), s1 = T(0);
-      int p = c;
-      for (; p + 2 < j; p += 2) {
-        s0 = fma(-Lj[p], W[(size_t)p * m + c], s0);
-        s1 = fma(-Lj[p + 1], W[(size_t)(p + 1) * m + c], s1);
-      }
-      if (p + 1 < j) s0 = fma(-Lj[p], W[(size_t)p * m + c], s0);
-      if (c + 1 <= j) s1 = fma(-Lj[j - 1], xprev[c], s1);
-      xj[c] = (s0 + s1) / djj;
-      if (c + 1 <= j) W[(size_t)(j - 1) * m + c] = xprev[c];
-    }
-    __syncthreads();
-  }
-  // the last row of X, and zeros above the diagonal
-  const T *xlast = ((m - 1) & 1) ? xr1 : xr0;
-  for (int c = tid; c < m; c += nt) W[(size_t)(m - 1) * m + c] = xlast[c];
-  __syncthreads();
-  for (int64_t e = tid; e < (int64_t)m * m; e += nt) {
-    const int i = (int)(e / m), c = (int)(e % m);
-    if (c > i) W[e] = T(0);
-  }
-  __syncthreads();
-  return 0;
+__host__ __device__ constexpr int chol_ps() {
+  return kCholNb + 16 / (int)sizeof(T);
+}
+template <typename T>
+__host__ __device__ inline int chol_ld(int m) {
+  constexpr int v = 16 / (int)sizeof(T);
+  const int q = (m + v - 1) / v;
+  return v * (q | 1);
+}
+template <typename T>
+__host__ __device__ inline size_t chol_smem_bytes(int m) {
+  return sizeof(T) * (size_t)m * (chol_ld<T>(m) + chol_ps<T>());
 }
 
-template <typename T, bool SMEM>
-__global__ void __launch_bounds__(CHOL_THREADS) k_chol_inv(const CholTask<T> *__restrict__ tasks,
-                                                           int *__restrict__ status) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int flag;
-  const CholTask<T> t = tasks[blockIdx.x];
-  const int m = t.m;
-  if (threadIdx.x == 0) flag = 0;
-  if (m == 0) {
-    if (threadIdx.x == 0) status[t.status_idx] = 0;
-    return;
+// v[0 .. 16 / sizeof(T)) = 16 bytes at p
+__device__ __forceinline__ void ld16(const float *p, float *v) {
+  const float4 q = *reinterpret_cast<const float4 *>(p);
+  v[0] = q.x;
+  v[1] = q.y;
+  v[2] = q.z;
+  v[3] = q.w;
+}
+__device__ __forceinline__ void ld16(const double *p, double *v) {
+  const double2 q = *reinterpret_cast<const double2 *>(p);
+  v[0] = q.x;
+  v[1] = q.y;
+}
+__device__ __forceinline__ void st16(float *p, const float *v) {
+  *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void st16(double *p, const double *v) {
+  *reinterpret_cast<double2 *>(p) = make_double2(v[0], v[1]);
+}
+// d^-1/2 to about one unit in the last place
+__device__ __forceinline__ float inv_sqrt(float d) {
+  const float y = rsqrtf(d);
+  return y * fmaf(-0.5f * d * y, y, 1.5f);
+}
+__device__ __forceinline__ double inv_sqrt(double d) { return rsqrt(d); }
+
+// One warp: D = L^-1 of the diagonal block at j0 (jb <= 16 columns), in its
+// place with zeros above the diagonal; *fail = first failing pivot + 1.
+template <typename T>
+__device__ __forceinline__ void chol_diag(T *W, int ld, int j0, int jb, int *fail) {
+  const int lane = threadIdx.x & 31, i = lane & 15;   // row of A, then column of D (lanes 16.. repeat)
+  T r[kCholNb], x[kCholNb];
+#pragma unroll
+  for (int c = 0; c < kCholNb; ++c) {
+    r[c] = (i < jb && c <= i) ? W[(size_t)(j0 + i) * ld + j0 + c] : (c == i ? T(1) : T(0));
+    x[c] = c == i ? T(1) : T(0);
   }
-  T *W;
-  T *tmp;
-  if (SMEM) {
-    W = reinterpret_cast<T *>(smem_raw);
-    tmp = W + (size_t)m * m;
-  } else {
-    W = t.Linv;  // requires ldl == m
-    tmp = reinterpret_cast<T *>(smem_raw);
-  }
-  for (int64_t e = threadIdx.x; e < (int64_t)m * m; e += blockDim.x) {
-    const int i = (int)(e / m), c = (int)(e % m);
-    W[e] = (c <= i) ? t.A[(int64_t)i * t.lda + c] : T(0);
-  }
-  __syncthreads();
-  const int st = chol_inv_inplace(W, m, tmp, &flag);
-  if (SMEM && st == 0) {
-    for (int64_t e = threadIdx.x; e < (int64_t)m * m; e += blockDim.x) {
-      const int i = (int)(e / m), c = (int)(e % m);
-      t.Linv[(int64_t)i * t.ldl + c] = W[e];
+  int bad = 0;
+#pragma unroll
+  for (int j = 0; j < kCholNb; ++j) {
+    T d = __shfl_sync(0xffffffffu, r[j], j);
+    if (!(d > T(0)) || !isfinite(d)) {
+      if (!bad) bad = j0 + j + 1;
+      d = T(1);
+    }
+    const T inv = inv_sqrt(d);
+    const T l = r[j] * inv;   // L_ij
+    x[j] *= inv;              // D_ji
+#pragma unroll
+    for (int c = j + 1; c < kCholNb; ++c) {
+      const T lc = __shfl_sync(0xffffffffu, l, c);
+      r[c] = fma(-l, lc, r[c]);
+      x[c] = fma(-lc, x[j], x[c]);
     }
   }
-  if (threadIdx.x == 0) status[t.status_idx] = st;
+  __syncwarp();
+  if (lane < jb) {
+#pragma unroll
+    for (int c = 0; c < kCholNb; ++c)
+      if (c < jb) W[(size_t)(j0 + c) * ld + j0 + lane] = x[c];
+  }
+  if (bad && lane == 0) *fail = bad;
+  __syncwarp();
+}
+
+// Rank-16 update of the tile at rows i0 .. i0 + 31, columns c0 .. c0 + 15.
+// kind 0: W -= P_i P_c^T; 1: W += P_i X_b; 2: W = P_i X_b (X_b: rows j0 ..)
+template <typename T>
+__device__ __forceinline__ void chol_tile(T *W, int ld, const T *P, int i0, int c0, int j0, int m, int kind) {
+  constexpr int V = 16 / (int)sizeof(T), PS = chol_ps<T>();
+  const int lane = threadIdx.x & 31;
+  const int ib = i0 + (lane & 7), cb = c0 + 4 * (lane >> 3);
+  T acc[4][4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[r][c] = T(0);
+  const T *pa[4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) pa[r] = P + (size_t)min(ib + 8 * r, m - 1) * PS;
+  if (kind == 0) {
+    const T *pb[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) pb[c] = P + (size_t)min(cb + c, m - 1) * PS;
+#pragma unroll
+    for (int k = 0; k < kCholNb; k += V) {
+      T a[4][V], b[4][V];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) ld16(pa[r] + k, a[r]);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) ld16(pb[c] + k, b[c]);
+#pragma unroll
+      for (int u = 0; u < V; ++u)
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) acc[r][c] = fma(-a[r][u], b[c][u], acc[r][c]);
+    }
+  } else {
+    const T *xb = W + (size_t)j0 * ld + cb;
+#pragma unroll
+    for (int k = 0; k < kCholNb; k += V) {
+      T a[4][V], b[V][4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) ld16(pa[r] + k, a[r]);
+#pragma unroll
+      for (int u = 0; u < V; ++u)
+#pragma unroll
+        for (int c = 0; c < 4; c += V) ld16(xb + (size_t)(k + u) * ld + c, &b[u][c]);
+#pragma unroll
+      for (int u = 0; u < V; ++u)
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) acc[r][c] = fma(a[r][u], b[u][c], acc[r][c]);
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const int i = ib + 8 * r;
+    if (i >= m) continue;
+#pragma unroll
+    for (int c = 0; c < 4; c += V) {
+      if (cb + c >= ld) continue;   // the last trailing columns; ld is a multiple of V
+      T *p = W + (size_t)i * ld + cb + c;
+      if (kind != 2) {
+        T w[V];
+        ld16(p, w);
+#pragma unroll
+        for (int u = 0; u < V; ++u) acc[r][c + u] += w[u];
+      }
+      st16(p, &acc[r][c]);
+    }
+  }
+}
+
+template <typename T, int NT>
+__global__ void __launch_bounds__(NT) k_chol_inv(const CholTask<T> *__restrict__ tasks, int *__restrict__ status) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int s_fail;
+  constexpr int V = 16 / (int)sizeof(T), PS = chol_ps<T>(), NW = NT / 32;
+  const CholTask<T> t = tasks[blockIdx.x];
+  const int m = t.m, ld = chol_ld<T>(m);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (m == 0) {
+    if (tid == 0) status[t.status_idx] = 0;
+    return;
+  }
+  T *W = reinterpret_cast<T *>(smem_raw);
+  T *P = W + (size_t)m * ld;
+  if (tid == 0) s_fail = 0;
+  for (int i = warp; i < m; i += NW)
+    for (int c = lane; c < ld; c += 32) W[(size_t)i * ld + c] = c <= i ? t.A[(int64_t)i * t.lda + c] : T(0);
+  __syncthreads();
+  if (warp == 0) chol_diag<T>(W, ld, 0, min(kCholNb, m), &s_fail);
+  for (int j0 = 0; j0 < m; j0 += kCholNb) {
+    __syncthreads();   // D_b and the update of the step before are complete
+    if (s_fail) break;
+    const int j1 = min(j0 + kCholNb, m), jb = j1 - j0, rest = m - j1;
+    const T *D = W + (size_t)j0 * ld + j0;
+    for (int q = tid; q < rest + j0; q += NT) {
+      T v[kCholNb], o[kCholNb];
+      if (q < rest) {
+        // row j1 + q of the panel (a full block: jb = 16)
+        const T *w = W + (size_t)(j1 + q) * ld + j0;
+#pragma unroll
+        for (int k = 0; k < kCholNb; k += V) ld16(w + k, v + k);
+      } else {
+        // column q - rest of the inverse's block row
+        const T *w = W + (size_t)j0 * ld + (q - rest);
+#pragma unroll
+        for (int k = 0; k < kCholNb; ++k) v[k] = k < jb ? -w[(size_t)k * ld] : T(0);
+      }
+#pragma unroll
+      for (int k = 0; k < kCholNb; ++k) {
+        T s = T(0);
+        if (k < jb) {
+#pragma unroll
+          for (int p = 0; p <= k; ++p) s = fma(D[(size_t)k * ld + p], v[p], s);
+        }
+        o[k] = s;
+      }
+      if (q < rest) {
+#pragma unroll
+        for (int k = 0; k < kCholNb; k += V) st16(P + (size_t)(j1 + q) * PS + k, o + k);
+      } else {
+        T *w = W + (size_t)j0 * ld + (q - rest);
+#pragma unroll
+        for (int k = 0; k < kCholNb; ++k)
+          if (k < jb) w[(size_t)k * ld] = o[k];
+      }
+    }
+    __syncthreads();
+    if (rest == 0) break;
+    if (warp == 0) {
+      chol_tile<T>(W, ld, P, j1, j1, j0, m, 0);
+      __syncwarp();
+      chol_diag<T>(W, ld, j1, min(kCholNb, m - j1), &s_fail);
+    } else {
+      // all other tiles, dealt out to the other warps in turn
+      const int nic = j1 / kCholNb, nct = (rest + kCholNb - 1) / kCholNb;
+      int turn = 1;
+      for (int rt = 0; rt * 32 < rest; ++rt) {
+        const int ntr = min(2 * (rt + 1), nct);
+        for (int ct = 0; ct < nic + ntr; ++ct) {
+          if (rt == 0 && ct == nic) continue;   // warp 0's
+          if (turn == warp) {
+            if (ct < nic)
+              chol_tile<T>(W, ld, P, j1 + 32 * rt, kCholNb * ct, j0, m, ct == nic - 1 ? 2 : 1);
+            else
+              chol_tile<T>(W, ld, P, j1 + 32 * rt, j1 + kCholNb * (ct - nic), j0, m, 0);
+          }
+          turn = turn + 1 == NW ? 1 : turn + 1;
+        }
+      }
+    }
+  }
+  __syncthreads();
+  const int st = s_fail;
+  if (st == 0)
+    for (int i = warp; i < m; i += NW)
+      for (int c = lane; c < m; c += 32) t.Linv[(int64_t)i * t.ldl + c] = c <= i ? W[(size_t)i * ld + c] : T(0);
+  if (tid == 0) status[t.status_idx] = st;
 }
 
 // ---------------------------------------------------------------------------
@@ -669,19 +828,26 @@ int chol_smem_cap() {
   return sizeof(T) == 8 ? 160 : 224;
 }
 
+template <typename T, int NT>
+static void launch_chol_nt(const CholTask<T> *d_tasks, int ntasks, int *d_status, int max_m, cudaStream_t st) {
+  const size_t sm = chol_smem_bytes<T>(max_m);
+  check_dynamic_smem(sm, allow_max_dynamic_smem<&k_chol_inv<T, NT>>(), "k_chol_inv");
+  k_chol_inv<T, NT><<<ntasks, NT, sm, st>>>(d_tasks, d_status);
+}
+
+// Threads by the largest matrix of the launch: the update's tiles (about
+// m^2 / 1024 a step) keep that many warps busy; a matrix's arithmetic does not
+// depend on them.
 template <typename T>
 void launch_chol_inv(const CholTask<T> *d_tasks, int ntasks, int *d_status, int max_m,
                      cudaStream_t st) {
   if (ntasks == 0) return;
-  if (max_m <= chol_smem_cap<T>()) {
-    const size_t sm = sizeof(T) * ((size_t)max_m * max_m + 3 * (size_t)max_m + 8);
-    check_dynamic_smem(sm, allow_max_dynamic_smem<&k_chol_inv<T, true>>(), "k_chol_inv");
-    k_chol_inv<T, true><<<ntasks, CHOL_THREADS, sm, st>>>(d_tasks, d_status);
-  } else {
-    const size_t sm = sizeof(T) * (3 * (size_t)max_m + 8);
-    check_dynamic_smem(sm, allow_max_dynamic_smem<&k_chol_inv<T, false>>(), "k_chol_inv");
-    k_chol_inv<T, false><<<ntasks, CHOL_THREADS, sm, st>>>(d_tasks, d_status);
-  }
+  if (max_m <= 48)
+    launch_chol_nt<T, 128>(d_tasks, ntasks, d_status, max_m, st);
+  else if (max_m <= 112)
+    launch_chol_nt<T, 256>(d_tasks, ntasks, d_status, max_m, st);
+  else
+    launch_chol_nt<T, 512>(d_tasks, ntasks, d_status, max_m, st);
   count_launch();
   HS_CUDA(cudaGetLastError());
 }
