@@ -445,17 +445,25 @@ struct Exec : TcTimer {
       if (cudaEventElapsedTime(&t, sp.e0, sp.e1) == cudaSuccess && sp.phase < nphase) ms[sp.phase] += t;
     }
   }
-  // a second stream for work that runs beside the factor stream (joined
-  // back by an event before anything depends on it)
-  cudaStream_t side = nullptr;
-  cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
-  cudaStream_t side_stream() {
-    if (!side) {
-      HS_CUDA(cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking));
-      HS_CUDA(cudaEventCreateWithFlags(&fork_ev, cudaEventDisableTiming));
-      HS_CUDA(cudaEventCreateWithFlags(&join_ev, cudaEventDisableTiming));
+  // Streams for work that runs beside the factor stream: fork(q) returns aux
+  // stream q, ordered after what the factor stream holds so far, and join(q)
+  // orders the factor stream after it.
+  static constexpr int kAux = 6;
+  cudaStream_t aux[kAux] = {};
+  cudaEvent_t fork_ev[kAux] = {}, join_ev[kAux] = {};
+  cudaStream_t fork(int q) {
+    if (!aux[q]) {
+      HS_CUDA(cudaStreamCreateWithFlags(&aux[q], cudaStreamNonBlocking));
+      HS_CUDA(cudaEventCreateWithFlags(&fork_ev[q], cudaEventDisableTiming));
+      HS_CUDA(cudaEventCreateWithFlags(&join_ev[q], cudaEventDisableTiming));
     }
-    return side;
+    HS_CUDA(cudaEventRecord(fork_ev[q], st));
+    HS_CUDA(cudaStreamWaitEvent(aux[q], fork_ev[q], 0));
+    return aux[q];
+  }
+  void join(int q) {
+    HS_CUDA(cudaEventRecord(join_ev[q], aux[q]));
+    HS_CUDA(cudaStreamWaitEvent(st, join_ev[q], 0));
   }
   explicit Exec(cudaStream_t s) : st(s) {
     HS_CUDA(cudaEventCreate(&ev_big[0]));
@@ -472,11 +480,12 @@ struct Exec : TcTimer {
   ~Exec() {
     // copies from the pinned staging buffers may still be in flight after an error
     cudaStreamSynchronize(st);
-    if (side) {
-      cudaStreamSynchronize(side);
-      cudaStreamDestroy(side);
-      cudaEventDestroy(fork_ev);
-      cudaEventDestroy(join_ev);
+    for (int q = 0; q < kAux; ++q) {
+      if (!aux[q]) continue;
+      cudaStreamSynchronize(aux[q]);
+      cudaStreamDestroy(aux[q]);
+      if (fork_ev[q]) cudaEventDestroy(fork_ev[q]);
+      if (join_ev[q]) cudaEventDestroy(join_ev[q]);
     }
     al.put(d_err, st);
     for (auto &e : tc_ev) {
@@ -1642,10 +1651,11 @@ void trunc_big(Exec &ex, const std::vector<TruncTask<T>> &all, int *d_k, int var
   ex.end();
   const int n = (int)tasks.size();
   if (n == 0) return;
-  // nodes that fit a thread-block cluster's shared memory are tridiagonalised
-  // there in one launch per cluster size; the others by the step kernels
-  std::vector<GridTri<T>> by_c[4], steps;
-  int cmax[4] = {0, 0, 0, 0}, smax = 0, sblocks = 0;
+  // Nodes that fit on chip are tridiagonalised there, one launch per class
+  // (one CTA, or a cluster of 2 to 16); larger ones go by the step kernels (two
+  // launches a step) until the trailing block fits, and finish there.
+  std::vector<GridTri<T>> by_c[kTriClasses], tail[kTriClasses], steps;
+  int cmax[kTriClasses] = {}, tmax[kTriClasses] = {}, kmax = 0, sblocks = 0;
   for (const TruncTask<T> &t : tasks) {
     const BigLayout<T> L = big_layout<T>(t.work, t.m);
     GridTri<T> g;
@@ -1658,45 +1668,58 @@ void trunc_big(Exec &ex, const std::vector<TruncTask<T>> &all, int *d_k, int var
     g.d = L.d;
     g.e = L.e;
     g.tau = L.tau;
-    g.m = t.m;
+    g.m = g.ld = t.m;
     g.nblk = (t.m + kTriRows - 1) / kTriRows;
     g.blk0 = 0;
-    const int c = tri_cluster_enabled() ? tri_cluster_size<T>(g.m) : 0;
-    if (c > 0) {
-      const int q = c == 1 ? 0 : c == 2 ? 1 : c == 4 ? 2 : 3;
+    g.kend = t.m - 2;
+    const int q = tri_cluster_enabled() ? tri_class<T>(g.m) : -1;
+    if (q >= 0) {
       by_c[q].push_back(g);
       cmax[q] = std::max(cmax[q], g.m);
-    } else {
-      g.blk0 = sblocks;
-      sblocks += g.nblk;
-      steps.push_back(g);
-      smax = std::max(smax, g.m);
+      continue;
     }
+    if (tri_cluster_enabled()) {
+      const int n2 = tri_onchip_max<T>(), k0 = t.m - n2, qt = tri_class<T>(n2);
+      g.kend = k0;
+      GridTri<T> x = g;
+      x.A += (size_t)k0 * g.ld + k0;
+      x.d += k0;
+      x.e += k0;
+      x.tau += k0;
+      x.m = n2;
+      tail[qt].push_back(x);
+      tmax[qt] = std::max(tmax[qt], n2);
+    }
+    g.blk0 = sblocks;
+    sblocks += g.nblk;
+    kmax = std::max(kmax, g.kend);
+    steps.push_back(g);
   }
-  Uploader u;
-  const size_t og = u.add(steps);
-  size_t oc[4];
-  for (int q = 0; q < 4; ++q) oc[q] = u.add(by_c[q]);
-  char *dg = u.upload(ex.scr, ex.sg, ex.st);
-  const GridTri<T> *d_gt = (const GridTri<T> *)(dg + og);
   ex.begin(11);
-  // the cluster launches run on a side stream, beside the step kernels
-  const bool fork = !steps.empty() && (by_c[0].size() + by_c[1].size() + by_c[2].size() + by_c[3].size()) > 0;
-  cudaStream_t cs = fork ? ex.side_stream() : ex.st;
-  if (fork) {
-    HS_CUDA(cudaEventRecord(ex.fork_ev, ex.st));
-    HS_CUDA(cudaStreamWaitEvent(cs, ex.fork_ev, 0));
+  // the classes are independent: the step kernels, or else the largest class,
+  // stay on the factor stream and the others run beside them
+  int home = -1, used = 0;
+  if (steps.empty())
+    for (int q = 0; q < kTriClasses; ++q)
+      if (!by_c[q].empty()) home = q;
+  for (int q = 0; q < kTriClasses; ++q) {
+    if (by_c[q].empty() || q == home) continue;
+    const GridTri<T> *d = upload_list(ex, by_c[q]);
+    launch_tri_onchip<T>(d, (int)by_c[q].size(), q, cmax[q], ex.fork(used++));
   }
-  for (int q = 0; q < 4; ++q)
-    launch_tri_cluster<T>((const GridTri<T> *)(dg + oc[q]), (int)by_c[q].size(), 1 << q, cmax[q], cs);
-  for (int k = 0; k + 2 <= smax; ++k) {
-    launch_tri_step<T>(d_gt, (int)steps.size(), sblocks, k, 0, ex.st);
-    if (k + 3 <= smax) launch_tri_step<T>(d_gt, (int)steps.size(), sblocks, k, 1, ex.st);
+  if (home >= 0)
+    launch_tri_onchip<T>(upload_list(ex, by_c[home]), (int)by_c[home].size(), home, cmax[home], ex.st);
+  if (!steps.empty()) {
+    const GridTri<T> *d_gt = upload_list(ex, steps);
+    for (int k = 0; k <= kmax; ++k) {
+      launch_tri_step<T>(d_gt, (int)steps.size(), sblocks, k, 0, ex.st);
+      if (k < kmax) launch_tri_step<T>(d_gt, (int)steps.size(), sblocks, k, 1, ex.st);
+    }
+    for (int q = 0; q < kTriClasses; ++q)
+      if (!tail[q].empty())
+        launch_tri_onchip<T>(upload_list(ex, tail[q]), (int)tail[q].size(), q, tmax[q], ex.st);
   }
-  if (fork) {
-    HS_CUDA(cudaEventRecord(ex.join_ev, cs));
-    HS_CUDA(cudaStreamWaitEvent(ex.st, ex.join_ev, 0));
-  }
+  for (int q = 0; q < used; ++q) ex.join(q);
   ex.end();
   // products with Q: by warps up to kQmulMax, by CTAs above
   auto products = [&](bool fwd) {

@@ -260,6 +260,8 @@ struct GridTri {
   double *d, *e;
   T *tau;
   int m, nblk, blk0;
+  int ld;            // row stride of A (m, or the whole matrix's for a trailing block)
+  int kend;          // step kernels: steps 0 .. kend - 1, then the update of step kend - 1
 };
 
 // Eigenvalues of a node's T and their inverse iteration: T in the factor
@@ -330,14 +332,17 @@ void launch_qmul(const QmulTask<T> *d_tasks, int ntasks, int total_blocks, int m
 // and p = tau A v)
 template <typename T>
 void launch_tri_step(const GridTri<T> *d_tasks, int ntasks, int total_blocks, int k, int phase, cudaStream_t st);
-// the whole tridiagonalisation of each node by one thread-block cluster
-// (kernels_cluster.cu): the cluster size (1, 2, 4 or 8 CTAs) that holds a node
-// of size m in shared memory, 0 when none does; all tasks of a launch use
-// cluster size C
+// the whole tridiagonalisation of each node (or trailing block) on chip
+// (kernels_cluster.cu): class 0 in one CTA, class q in a cluster of 2^q; -1 when
+// none holds a block of size m.  All tasks of a launch are of one class.
+constexpr int kTriClasses = 5;
 template <typename T>
-int tri_cluster_size(int m);
+int tri_class(int m);
+// the largest block any class holds
 template <typename T>
-void launch_tri_cluster(const GridTri<T> *d_tasks, int ntasks, int C, int m_max, cudaStream_t st);
+int tri_onchip_max();
+template <typename T>
+void launch_tri_onchip(const GridTri<T> *d_tasks, int ntasks, int q, int m_max, cudaStream_t st);
 // inverse iteration over total_blocks CTAs of `spc` slots each
 template <typename T>
 void launch_invit(const EigTask<T> *d_tasks, int ntasks, int total_blocks, int spc, int m_max, cudaStream_t st);

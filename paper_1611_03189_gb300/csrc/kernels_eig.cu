@@ -997,7 +997,7 @@ __global__ void __launch_bounds__(kTriRows * 32) k_tri_update(const GridTri<T> *
   __shared__ T wpart[kTriRows];
   const GridTri<T> t = tasks[tri_task(tasks, ntasks, blockIdx.x)];
   const int m = t.m;
-  if (k > m - 2) return;
+  if (k > t.kend) return;
   const int rb = blockIdx.x - t.blk0;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = rb * kTriRows + warp;
@@ -1059,7 +1059,7 @@ __global__ void __launch_bounds__(kTriRows * 32) k_tri_symv(const GridTri<T> *__
   __shared__ T wpart[kTriRows];
   const GridTri<T> t = tasks[tri_task(tasks, ntasks, blockIdx.x)];
   const int m = t.m;
-  if (k > m - 3) return;
+  if (k >= t.kend) return;
   const int rb = blockIdx.x - t.blk0;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (warp == 0) {
