@@ -179,7 +179,7 @@ struct GemmBatch {
   double flops = 0.0;
   int tc = HS_TC_NONE;   // float batches: run on the tensor cores in this precision
   void add(const T *A, int lda, int ta, const T *B, int ldb, int tb, T *C, int ldc, int M, int N,
-           int K, T alpha, T beta) {
+           int K, T alpha, T beta, int sym = 0, int kmode = 0) {
     if (M <= 0 || N <= 0) return;
     if (K <= 0 && beta == T(1)) return;
     GemmTask<T> t;
@@ -196,6 +196,8 @@ struct GemmBatch {
     t.tb = tb;
     t.alpha = alpha;
     t.beta = beta;
+    t.sym = sym;
+    t.kmode = kmode;
     tasks.push_back(t);
     flops += 2.0 * M * N * (double)std::max(K, 0);
   }
@@ -217,21 +219,22 @@ struct GemmBatch {
       part[0].swap(tasks);
     }
     tasks.clear();
-    const int tms[3] = {GEMM_TM, TC_TILE_M, TC_TILE_M}, tns[3] = {GEMM_TN, 64, 128};
     for (int v = 0; v < 3; ++v) {
       if (part[v].empty()) continue;
+      const int cls = v == 0 ? gemm_tile_class<T>(part[v].data(), (int)part[v].size()) : 0;
+      const int tm = v == 0 ? gemm_tile<T>(cls) : TC_TILE_M, tn = v == 0 ? tm : v == 1 ? 64 : 128;
       std::vector<int> tile_start;
       int tiles = 0;
       for (const GemmTask<T> &t : part[v]) {
         tile_start.push_back(tiles);
-        tiles += ((t.M + tms[v] - 1) / tms[v]) * ((t.N + tns[v] - 1) / tns[v]);
+        tiles += v == 0 ? gemm_tiles(t, tm) : ((t.M + tm - 1) / tm) * ((t.N + tn - 1) / tn);
       }
       Uploader u;
       const size_t ot = u.add(part[v]);
       const size_t os = u.add(tile_start);
       char *d = u.upload(scr, sg, st);
       if (v == 0) {
-        launch_gemm<T>((const GemmTask<T> *)(d + ot), (const int *)(d + os), (int)part[v].size(), tiles, st);
+        launch_gemm<T>((const GemmTask<T> *)(d + ot), (const int *)(d + os), (int)part[v].size(), tiles, cls, st);
         continue;
       }
       if constexpr (std::is_same<T, float>::value) {
@@ -239,7 +242,7 @@ struct GemmBatch {
         double f = 0.0;
         for (const GemmTask<T> &t : part[v]) f += 2.0 * t.M * t.N * (double)std::max(t.K, 0);
         if (timer) timer->before(st);
-        launch_gemm_tc(tc, tns[v], (const GemmTask<float> *)(d + ot), (const int *)(d + os), (int)part[v].size(),
+        launch_gemm_tc(tc, tn, (const GemmTask<float> *)(d + ot), (const int *)(d + os), (int)part[v].size(),
                        tiles, d_err, st, wait_cycles);
         if (timer) timer->after(st, f);
       }
@@ -674,8 +677,8 @@ struct Exec : TcTimer {
         dc.push_back(c);
         if (rest > 0) {
           T *Lp = x.Lf + (size_t)(j0 + jb) * m + j0;
-          pan.add(x.W + (size_t)(j0 + jb) * m + j0, m, 0, Db, jb, 1, Lp, m, rest, jb, jb, T(1), T(0));
-          trl.add(Lp, m, 0, Lp, m, 1, x.W + (size_t)(j0 + jb) * m + j0 + jb, m, rest, rest, jb, T(-1), T(1));
+          pan.add(x.W + (size_t)(j0 + jb) * m + j0, m, 0, Db, jb, 1, Lp, m, rest, jb, jb, T(1), T(0), 0, GEMM_B_UP);
+          trl.add(Lp, m, 0, Lp, m, 1, x.W + (size_t)(j0 + jb) * m + j0 + jb, m, rest, rest, jb, T(-1), T(1), 1);
         }
       }
       Uploader u;
@@ -693,8 +696,8 @@ struct Exec : TcTimer {
         const int m = x.t.m, i0 = b * nb, jb = std::min(nb, m - i0);
         const T *Db = x.D + (size_t)b * nb * nb;
         if (b > 0) {
-          g1.add(x.Lf + (size_t)i0 * m, m, 0, x.t.Linv, m, 0, x.Tb, m, jb, i0, i0, T(1), T(0));
-          g2.add(Db, jb, 0, x.Tb, m, 0, x.t.Linv + (size_t)i0 * m, m, jb, i0, jb, T(-1), T(0));
+          g1.add(x.Lf + (size_t)i0 * m, m, 0, x.t.Linv, m, 0, x.Tb, m, jb, i0, i0, T(1), T(0), 0, GEMM_B_LOW);
+          g2.add(Db, jb, 0, x.Tb, m, 0, x.t.Linv + (size_t)i0 * m, m, jb, i0, jb, T(-1), T(0), 0, GEMM_A_LOW);
         }
         dg.copy(x.t.Linv + (size_t)i0 * m + i0, m, jb, jb, Db, jb, 0);
       }
@@ -1094,7 +1097,7 @@ void Run<T>::wave_a(int li, int widx, WaveBatches<T> &B) {
         tt.a = a64;
         tt.phi = phi64;
       }
-      B.gram64.add(AsW64, x.dW, 0, AsW64, x.dW, 1, const_cast<double *>(tt.G), m, m, m, x.dW, 1.0, 0.0);
+      B.gram64.add(AsW64, x.dW, 0, AsW64, x.dW, 1, const_cast<double *>(tt.G), m, m, m, x.dW, 1.0, 0.0, 1);
       tt.np = np;
       tt.eps1 = h_.eps1;
       double *U64 = talloc<double>(scr, (size_t)m * m);
@@ -1118,7 +1121,7 @@ void Run<T>::wave_a(int li, int widx, WaveBatches<T> &B) {
       }
       B.narrow.push_back(ConvTask{U64, x.U, (int64_t)m * m, 0});
     } else if (x.red && m > 0) {
-      B.gram.add(x.AsW, x.dW, 0, x.AsW, x.dW, 1, x.G, m, m, m, x.dW, T(1), T(0));
+      B.gram.add(x.AsW, x.dW, 0, x.AsW, x.dW, 1, x.G, m, m, m, x.dW, T(1), T(0), 1);
       if (use_phi_) B.gram.add(x.AsW, x.dW, 0, x.phiW, h_.nphi, 0, x.a, h_.nphi, m, h_.nphi, x.dW, T(1), T(0));
       TruncTask<T> tt;
       tt.G = x.G;
@@ -1190,12 +1193,12 @@ void Run<T>::wave_b(const int *hb, size_t nchol, size_t ntrunc, double big_ms, W
       T *Sg2 = talloc<T>(scr, (size_t)k * k), *Lg2 = talloc<T>(scr, (size_t)k * k);
       U1s[q] = talloc<T>(scr, (size_t)m * m);
       U2s[q] = talloc<T>(scr, (size_t)m * m);
-      B.o1.add(x.U, m, 1, x.U, m, 0, Sg, k, k, k, m, T(1), T(0));
+      B.o1.add(x.U, m, 1, x.U, m, 0, Sg, k, k, k, m, T(1), T(0), 1);
       B.oc1.add(Sg, k, Lg, k, tag(3, lv_->level, x.s));
-      B.o2.add(x.U, m, 0, Lg, k, 1, U1s[q], m, m, k, k, T(1), T(0));
-      B.o3.add(U1s[q], m, 1, U1s[q], m, 0, Sg2, k, k, k, m, T(1), T(0));
+      B.o2.add(x.U, m, 0, Lg, k, 1, U1s[q], m, m, k, k, T(1), T(0), 0, GEMM_B_UP);
+      B.o3.add(U1s[q], m, 1, U1s[q], m, 0, Sg2, k, k, k, m, T(1), T(0), 1);
       B.oc2.add(Sg2, k, Lg2, k, tag(3, lv_->level, x.s));
-      B.o4.add(U1s[q], m, 0, Lg2, k, 1, U2s[q], m, m, k, k, T(1), T(0));
+      B.o4.add(U1s[q], m, 0, Lg2, k, 1, U2s[q], m, m, k, k, T(1), T(0), 0, GEMM_B_UP);
     }
     for (int q : big_sup_)
       if (U2s[q]) S[q].U = U2s[q];
@@ -1241,31 +1244,33 @@ bool Run<T>::wave_c(WaveBatches<T> &B, size_t count) {
       x.phir = use_phi_ ? talloc<T>(per, (size_t)k * h_.nphi) : nullptr;
     }
     // L^-1 U and its CholQR2
-    B.g1.add(x.Linv, m, 0, x.U, m, 0, x.Ut, k, m, k, m, T(1), T(0));
-    B.g2.add(x.Ut, k, 1, x.Ut, k, 0, x.S1, k, k, k, m, T(1), T(0));
+    B.g1.add(x.Linv, m, 0, x.U, m, 0, x.Ut, k, m, k, m, T(1), T(0), 0, GEMM_A_LOW);
+    B.g2.add(x.Ut, k, 1, x.Ut, k, 0, x.S1, k, k, k, m, T(1), T(0), 1);
     B.c1.add(x.S1, k, x.L1, k, tag(1, lv_->level, x.s));
-    B.g3.add(x.Ut, k, 0, x.L1, k, 1, x.Q1, k, m, k, k, T(1), T(0));
-    B.g4.add(x.Q1, k, 1, x.Q1, k, 0, x.S2, k, k, k, m, T(1), T(0));
+    B.g3.add(x.Ut, k, 0, x.L1, k, 1, x.Q1, k, m, k, k, T(1), T(0), 0, GEMM_B_UP);
+    B.g4.add(x.Q1, k, 1, x.Q1, k, 0, x.S2, k, k, k, m, T(1), T(0), 1);
     B.c2.add(x.S2, k, x.L2, k, tag(2, lv_->level, x.s));
-    B.g5.add(x.Q1, k, 0, x.L2, k, 1, x.Q, k, m, k, k, T(1), T(0));
-    B.g5.add(x.L1, k, 1, x.L2, k, 1, x.Rinv, k, k, k, k, T(1), T(0));
+    B.g5.add(x.Q1, k, 0, x.L2, k, 1, x.Q, k, m, k, k, T(1), T(0), 0, GEMM_B_UP);
+    B.g5.add(x.L1, k, 1, x.L2, k, 1, x.Rinv, k, k, k, k, T(1), T(0), 0, GEMM_A_UP | GEMM_B_UP);
     // quantities needing Q / L^-1
-    B.g6.add(x.Linv, m, 1, x.Q, k, 0, x.Wt, k, m, k, m, T(1), T(0));          // L^-T Q
-    B.g6.add(x.Linv, m, 0, x.AsN, dN, 0, x.Gt, dN, m, dN, m, T(1), T(0));       // L^-1 A_sN
-    B.g6.add(x.Linv, m, 1, x.Linv, m, 0, x.M, m, m, m, m, T(1), T(0));          // L^-T L^-1
+    B.g6.add(x.Linv, m, 1, x.Q, k, 0, x.Wt, k, m, k, m, T(1), T(0), 0, GEMM_A_UP);   // L^-T Q
+    B.g6.add(x.Linv, m, 0, x.AsN, dN, 0, x.Gt, dN, m, dN, m, T(1), T(0), 0, GEMM_A_LOW);   // L^-1 A_sN
+    B.g6.add(x.Linv, m, 1, x.Linv, m, 0, x.M, m, m, m, m, T(1), T(0), 1,
+             GEMM_A_UP | GEMM_B_LOW);                                                 // L^-T L^-1
     if (x.red) {
       B.g6.add(x.U, m, 1, x.AsW, x.dW, 0, x.ArW, x.dW, k, x.dW, m, T(1), T(0));  // U^T A_sW
       if (use_phi_) B.g6.add(x.U, m, 1, phi_[x.s], h_.nphi, 0, x.phir, h_.nphi, k, h_.nphi, m, T(1), T(0));
     }
-    B.g7.add(x.Rinv, k, 0, x.Wt, k, 1, x.Pm, m, k, m, k, T(1), T(0));           // P_ss = R^-1 (L^-T Q)^T
-    B.g7.add(x.Wt, k, 0, x.Wt, k, 1, x.M, m, m, m, k, T(-1), T(1));             // M_ss -= W W^T
+    B.g7.add(x.Rinv, k, 0, x.Wt, k, 1, x.Pm, m, k, m, k, T(1), T(0), 0, GEMM_A_UP);   // P_ss = R^-1 (L^-T Q)^T
+    B.g7.add(x.Wt, k, 0, x.Wt, k, 1, x.M, m, m, m, k, T(-1), T(1), 1);          // M_ss -= W W^T
     B.g7.add(x.Q, k, 1, x.Gt, dN, 0, x.Tm, dN, k, dN, m, T(1), T(0));           // Q^T L^-1 A_sN
-    B.g7.add(x.Gt, dN, 1, x.Gt, dN, 0, x.Z, dN, dN, dN, m, T(1), T(0));         // (L^-1 A_sN)^T (L^-1 A_sN)
+    B.g7.add(x.Gt, dN, 1, x.Gt, dN, 0, x.Z, dN, dN, dN, m, T(1), T(0), 1);      // (L^-1 A_sN)^T (L^-1 A_sN)
     B.gb.add(x.M, m, 0, x.AsN, dN, 0, x.B, dN, m, dN, m, T(1), T(0));           // B_s = M_ss A_sN
-    B.g8.add(x.Tm, dN, 1, x.Tm, dN, 0, x.Z, dN, dN, dN, k, T(-1), T(1));        // - T^T T
+    B.g8.add(x.Tm, dN, 1, x.Tm, dN, 0, x.Z, dN, dN, dN, k, T(-1), T(1), 1);     // - T^T T
     if (x.red) {
-      B.g8.add(x.Tm, dN, 1, x.Rinv, k, 1, x.ANr, k, dN, k, k, T(1), T(0));      // A_Nr = T^T R^-T
-      B.g8.add(x.Rinv, k, 0, x.Rinv, k, 1, x.Arr, k, k, k, k, T(1), T(0));      // A_rr = R^-1 R^-T
+      B.g8.add(x.Tm, dN, 1, x.Rinv, k, 1, x.ANr, k, dN, k, k, T(1), T(0), 0, GEMM_B_LOW);   // A_Nr = T^T R^-T
+      B.g8.add(x.Rinv, k, 0, x.Rinv, k, 1, x.Arr, k, k, k, k, T(1), T(0), 1,
+               GEMM_A_UP | GEMM_B_LOW);                                               // A_rr = R^-1 R^-T
     }
   }
   flops_ += B.c1.flops + B.c2.flops + B.g1.flops + B.g2.flops + B.g3.flops + B.g4.flops + B.g5.flops +
@@ -1600,7 +1605,7 @@ void Run<T>::root_b(CholBatch<T> &cb, GemmBatch<T> &g) {
   const double f0 = cb.flops + g.flops;
   cb.add(b.ptr, b.ld, root_linv_, m, tag(4, 0, 0));
   alg_flops_ += (double)m * m * m / 3;
-  g.add(root_linv_, m, 1, root_linv_, m, 0, root_ainv_, m, m, m, m, T(1), T(0));
+  g.add(root_linv_, m, 1, root_linv_, m, 0, root_ainv_, m, m, m, m, T(1), T(0), 1, GEMM_A_UP | GEMM_B_LOW);
   flops_ += cb.flops + g.flops - f0;
   h_.root_inv = root_ainv_;
   h_.info.root_size = m;

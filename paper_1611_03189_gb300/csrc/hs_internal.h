@@ -84,6 +84,11 @@ inline void check_dynamic_smem(size_t bytes, int limit, const char *what) {
 // C = alpha * op(A) * op(B) + beta * C, all row-major.
 // op(A) is M x K: A[i*lda + k] (ta = 0) or A[k*lda + i] (ta = 1).
 // op(B) is K x N: B[k*ldb + j] (tb = 0) or B[j*ldb + k] (tb = 1).
+// sym: the result (and C, when beta is not 0) is symmetric, M = N.
+// kmode: triangles of zeros in the operands -- op(A)[i][k] = 0 for k > i
+// (A_LOW) or k < i (A_UP), op(B)[k][j] = 0 for k > j (B_UP) or k < j (B_LOW).
+// Both are hints: the tensor-core kernel computes the whole product.
+enum { GEMM_A_LOW = 1, GEMM_A_UP = 2, GEMM_B_UP = 4, GEMM_B_LOW = 8 };
 template <typename T>
 struct GemmTask {
   const T *A;
@@ -93,6 +98,7 @@ struct GemmTask {
   int lda, ldb, ldc;
   int ta, tb;
   T alpha, beta;
+  int sym = 0, kmode = 0;
 };
 
 // dst = beta * dst + alpha * sum_s op(src_s), rows x cols; sources listed in
@@ -153,8 +159,21 @@ struct TruncTask {
 // ---------------------------------------------------------------------------
 // kernel launchers (kernels_dense.cu)
 // ---------------------------------------------------------------------------
+// CUDA-core GEMM: tiles of gemm_tile<T>(class) squared, the class chosen for a
+// whole batch (HOST tasks) by gemm_tile_class
 template <typename T>
-void launch_gemm(const GemmTask<T> *d_tasks, const int *d_tile_start, int ntasks, int total_tiles,
+constexpr int gemm_tile(int cls) {
+  return sizeof(T) == 4 ? (cls == 0 ? 64 : 32) : (cls == 0 ? 32 : 16);
+}
+template <typename T>
+inline int gemm_tiles(const GemmTask<T> &t, int tm) {
+  const int r = (t.M + tm - 1) / tm, c = (t.N + tm - 1) / tm;
+  return t.sym ? r * (r + 1) / 2 : r * c;
+}
+template <typename T>
+int gemm_tile_class(const GemmTask<T> *tasks, int n);
+template <typename T>
+void launch_gemm(const GemmTask<T> *d_tasks, const int *d_tile_start, int ntasks, int total_tiles, int tile_class,
                  cudaStream_t st);
 template <typename T>
 void launch_sum(const SumTask<T> *d_tasks, const SumSrc<T> *d_srcs, const int *d_tile_start,
@@ -374,9 +393,7 @@ void launch_diag_scale(const int32_t *rp, const int32_t *ci, const double *val, 
 template <typename T>
 void launch_phi_scale(const T *raw, const double *ds, int64_t n, int np, T *out, cudaStream_t st);
 
-// tile bookkeeping for the batched GEMM / sum kernels
-constexpr int GEMM_TM = 64;
-constexpr int GEMM_TN = 64;
+// tile bookkeeping of the batched sum kernel
 constexpr int SUM_TILE = 32;
 
 // Tensor-core GEMM (kernels_tc.cu): operand precision of the tcgen05 path.

@@ -1,7 +1,7 @@
 // Batched variable-size dense kernels of the factorization.
 //
-//   k_gemm       C = alpha op(A) op(B) + beta C over a list of tasks (tiles of
-//                64 x 64, 16 x 16 threads, 4 x 4 outputs per thread).
+//   k_gemm       C = alpha op(A) op(B) + beta C over a list of tasks, one tile
+//                per CTA.
 //   k_sum        dst = beta dst + alpha sum_s op(src_s), sources summed in list
 //                order: block gathers, merges and the deterministic Schur
 //                scatter of Sec. 3.2 (several super nodes of one wave updating
@@ -36,101 +36,146 @@ struct Lim<float> {
   static __device__ __forceinline__ float tiny() { return 1e-35f; }
 };
 
+// the task of CTA b: the last one whose first tile is <= b.  A warp probes 32
+// places at a time (4096 tasks: three dependent loads instead of twelve)
 __device__ __forceinline__ int find_task(const int *tile_start, int ntasks, int b) {
-  int lo = 0, hi = ntasks - 1;
-  while (lo < hi) {
-    int mid = (lo + hi + 1) >> 1;
-    if (tile_start[mid] <= b)
-      lo = mid;
-    else
-      hi = mid - 1;
+  const int lane = threadIdx.x & 31;
+  int lo = 0, len = ntasks;
+  while (len > 1) {
+    const int step = (len + 31) / 32;
+    const int at = lane * step;
+    const unsigned below = __ballot_sync(0xffffffffu, at < len && tile_start[lo + min(at, len - 1)] <= b);
+    const int c = __popc(below) - 1;   // tile_start[lo] <= b
+    lo += c * step;
+    len = min(step, len - c * step);
   }
   return lo;
 }
 
 // ---------------------------------------------------------------------------
-// batched GEMM
+// batched GEMM: one tile of TM x TN outputs per CTA, RM x RN adjacent ones per
+// thread, operands staged through shared memory GK rows at a time, the next
+// rows loaded while the current ones are used.  An output is the sum over k in
+// order, whatever the tile, so a task gets the same bits in any launch.
+//
+// Symmetric products (task.sym) run the tiles on and below the diagonal and
+// write each value to both places; operands with a triangle of zeros
+// (task.kmode) limit a tile's k to the part that is not zero.  Both leave the
+// results as they are and take about half of the factorization's products'
+// work away.
+//
+// Tile sizes.  FP32: 64 x 64, 4 x 4 a thread (bound by the FMA rate when the
+// tiles fill the GPU); 32 x 32 when they do not, or when most of a 64 x 64
+// tile would be padding.  FP64: its rate (1/64 of FP32's) bounds any tile, so
+// the tiles are small to spread a wave's few large products over the SMs:
+// 32 x 32, or 16 x 16 below 8 tiles an SM (a 320^3 product: 25 tiles of 64 x 64
+// keep 25 SMs busy for 330 us; 400 of 16 x 16 take about 60).
 // ---------------------------------------------------------------------------
-constexpr int GK = 16;
-
-template <typename T>
-__global__ void __launch_bounds__(256) k_gemm(const GemmTask<T> *__restrict__ tasks,
-                                              const int *__restrict__ tile_start, int ntasks) {
-  __shared__ T As[GK][GEMM_TM + 1];
-  __shared__ T Bs[GK][GEMM_TN + 1];
+template <typename T, int TM, int RM, int GK>
+__global__ void __launch_bounds__((TM / RM) * (TM / RM)) k_gemm(const GemmTask<T> *__restrict__ tasks,
+                                                                const int *__restrict__ tile_start, int ntasks) {
+  constexpr int TX = TM / RM, NT = TX * TX, E = TM * GK / NT;
+  constexpr int LD = TM + 16 / (int)sizeof(T);
+  __shared__ __align__(16) T As[2][GK][LD];
+  __shared__ __align__(16) T Bs[2][GK][LD];
   const int ti = find_task(tile_start, ntasks, blockIdx.x);
   const GemmTask<T> t = tasks[ti];
   const int local = blockIdx.x - tile_start[ti];
-  const int tiles_n = (t.N + GEMM_TN - 1) / GEMM_TN;
-  const int row0 = (local / tiles_n) * GEMM_TM;
-  const int col0 = (local % tiles_n) * GEMM_TN;
+  int tr, tc;
+  if (t.sym) {
+    tr = (int)((sqrtf(8.f * (float)local + 1.f) - 1.f) * 0.5f);
+    while (tr * (tr + 1) / 2 > local) --tr;
+    while ((tr + 1) * (tr + 2) / 2 <= local) ++tr;
+    tc = local - tr * (tr + 1) / 2;
+  } else {
+    const int tiles_n = (t.N + TM - 1) / TM;
+    tr = local / tiles_n;
+    tc = local % tiles_n;
+  }
+  const int row0 = tr * TM, col0 = tc * TM;
+  int k_lo = 0, k_hi = t.K;
+  if (t.kmode & GEMM_A_LOW) k_hi = min(k_hi, row0 + TM);
+  if (t.kmode & GEMM_A_UP) k_lo = max(k_lo, row0);
+  if (t.kmode & GEMM_B_UP) k_hi = min(k_hi, col0 + TM);
+  if (t.kmode & GEMM_B_LOW) k_lo = max(k_lo, col0);
   const int tid = threadIdx.x;
-  const int tx = tid & 15, ty = tid >> 4;
-  T acc[4][4];
+  const int tx = tid % TX, ty = tid / TX;
+  T acc[RM][RM];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < RM; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = T(0);
-
-  for (int k0 = 0; k0 < t.K; k0 += GK) {
+    for (int j = 0; j < RM; ++j) acc[i][j] = T(0);
+  T ra[E], rb[E];
+  auto load = [&](int k0) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int e = tid + 256 * q;
-      int i, k;
-      if (t.ta == 0) {
-        i = e / GK;
-        k = e % GK;
-      } else {
-        k = e / GEMM_TM;
-        i = e % GEMM_TM;
+    for (int q = 0; q < E; ++q) {
+      const int e = tid + NT * q;
+      {
+        const int i = t.ta == 0 ? e / GK : e % TM, k = t.ta == 0 ? e % GK : e / TM;
+        const int gi = row0 + i, gk = k0 + k;
+        ra[q] = gi < t.M && gk < k_hi ? (t.ta == 0 ? t.A[(int64_t)gi * t.lda + gk] : t.A[(int64_t)gk * t.lda + gi])
+                                      : T(0);
       }
-      const int gi = row0 + i, gk = k0 + k;
-      T v = T(0);
-      if (gi < t.M && gk < t.K)
-        v = (t.ta == 0) ? t.A[(int64_t)gi * t.lda + gk] : t.A[(int64_t)gk * t.lda + gi];
-      As[k][i] = v;
-      int j;
-      if (t.tb == 0) {
-        k = e / GEMM_TN;
-        j = e % GEMM_TN;
-      } else {
-        j = e / GK;
-        k = e % GK;
+      {
+        const int j = t.tb == 0 ? e % TM : e / GK, k = t.tb == 0 ? e / TM : e % GK;
+        const int gj = col0 + j, gk = k0 + k;
+        rb[q] = gj < t.N && gk < k_hi ? (t.tb == 0 ? t.B[(int64_t)gk * t.ldb + gj] : t.B[(int64_t)gj * t.ldb + gk])
+                                      : T(0);
       }
-      const int gj = col0 + j;
-      const int gk2 = k0 + k;
-      T w = T(0);
-      if (gj < t.N && gk2 < t.K)
-        w = (t.tb == 0) ? t.B[(int64_t)gk2 * t.ldb + gj] : t.B[(int64_t)gj * t.ldb + gk2];
-      Bs[k][j] = w;
     }
-    __syncthreads();
+  };
+  auto store = [&](int buf) {
+#pragma unroll
+    for (int q = 0; q < E; ++q) {
+      const int e = tid + NT * q;
+      if (t.ta == 0)
+        As[buf][e % GK][e / GK] = ra[q];
+      else
+        As[buf][e / TM][e % TM] = ra[q];
+      if (t.tb == 0)
+        Bs[buf][e / TM][e % TM] = rb[q];
+      else
+        Bs[buf][e % GK][e / GK] = rb[q];
+    }
+  };
+  if (k_lo < k_hi) {
+    load(k_lo);
+    store(0);
+  }
+  __syncthreads();
+  int buf = 0;
+  for (int k0 = k_lo; k0 < k_hi; k0 += GK) {
+    const bool more = k0 + GK < k_hi;
+    if (more) load(k0 + GK);
 #pragma unroll
     for (int kk = 0; kk < GK; ++kk) {
-      T a[4], b[4];
+      T a[RM], b[RM];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
+      for (int i = 0; i < RM; ++i) a[i] = As[buf][kk][ty * RM + i];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
+      for (int j = 0; j < RM; ++j) b[j] = Bs[buf][kk][tx * RM + j];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < RM; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+        for (int j = 0; j < RM; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
     }
+    if (more) store(buf ^ 1);   // (read last before the barrier of the pass before)
     __syncthreads();
+    buf ^= 1;
   }
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int r = row0 + ty + 16 * i;
+  for (int i = 0; i < RM; ++i) {
+    const int r = row0 + ty * RM + i;
     if (r >= t.M) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int c = col0 + tx + 16 * j;
+    for (int j = 0; j < RM; ++j) {
+      const int c = col0 + tx * RM + j;
       if (c >= t.N) continue;
       T *p = t.C + (int64_t)r * t.ldc + c;
       T v = t.alpha * acc[i][j];
       if (t.beta != T(0)) v = fma(t.beta, *p, v);
       *p = v;
+      if (t.sym && tr != tc) t.C[(int64_t)c * t.ldc + r] = v;
     }
   }
 }
@@ -796,10 +841,34 @@ size_t trunc_small_arrays(int m) {
 // launchers
 // ---------------------------------------------------------------------------
 template <typename T>
-void launch_gemm(const GemmTask<T> *d_tasks, const int *d_tile_start, int ntasks, int total_tiles,
+int gemm_tile_class(const GemmTask<T> *tasks, int n) {
+  double tiles = 0, work[2] = {0, 0};
+  for (int q = 0; q < n; ++q)
+    for (int c = 0; c < 2; ++c) {
+      const int tm = gemm_tile<T>(c);
+      const double w = gemm_tiles(tasks[q], tm);
+      if (c == 0) tiles += w;
+      work[c] += w * tm * tm * (tasks[q].K + 16.0);
+    }
+  if (sizeof(T) == 8) return tiles < 152 * 8 ? 1 : 0;
+  return tiles < 152 * 2 || work[1] * 1.5 < work[0] ? 1 : 0;
+}
+
+template <typename T>
+void launch_gemm(const GemmTask<T> *d_tasks, const int *d_tile_start, int ntasks, int total_tiles, int tile_class,
                  cudaStream_t st) {
   if (ntasks == 0 || total_tiles == 0) return;
-  k_gemm<T><<<total_tiles, 256, 0, st>>>(d_tasks, d_tile_start, ntasks);
+  if constexpr (sizeof(T) == 4) {
+    if (tile_class == 0)
+      k_gemm<T, 64, 4, 16><<<total_tiles, 256, 0, st>>>(d_tasks, d_tile_start, ntasks);
+    else
+      k_gemm<T, 32, 2, 32><<<total_tiles, 256, 0, st>>>(d_tasks, d_tile_start, ntasks);
+  } else {
+    if (tile_class == 0)
+      k_gemm<T, 32, 2, 16><<<total_tiles, 256, 0, st>>>(d_tasks, d_tile_start, ntasks);
+    else
+      k_gemm<T, 16, 1, 32><<<total_tiles, 256, 0, st>>>(d_tasks, d_tile_start, ntasks);
+  }
   count_launch();
   HS_CUDA(cudaGetLastError());
 }
@@ -978,7 +1047,8 @@ void launch_status_merge(const StatusMerge *d_tasks, int ntasks, cudaStream_t st
 }
 
 #define HS_INST(T)                                                                            \
-  template void launch_gemm<T>(const GemmTask<T> *, const int *, int, int, cudaStream_t);     \
+  template int gemm_tile_class<T>(const GemmTask<T> *, int);                                  \
+  template void launch_gemm<T>(const GemmTask<T> *, const int *, int, int, int, cudaStream_t); \
   template void launch_sum<T>(const SumTask<T> *, const SumSrc<T> *, const int *, int, int,   \
                               cudaStream_t);                                                  \
   template void launch_chol_inv<T>(const CholTask<T> *, int, int *, int, cudaStream_t);       \

@@ -563,7 +563,7 @@ void launch_tc_bn(const GemmTask<float> *d_tasks, const int *d_tile_start, int n
 // ---------------------------------------------------------------------------
 // Autotuner of the batched GEMM.  For each class of task shapes (the larger of
 // M and N, and K, each bucketed by powers of four) it times three variants on
-// a synthetic batch of that class -- the CUDA-core kernel with 64 x 64 tiles
+// a synthetic batch of that class -- the CUDA-core kernel with its own tiles
 // and the tensor-core kernel with 128 x 64 and 128 x 128 tiles -- and keeps
 // the fastest (a tensor-core variant must win by 15%).  Small tasks favour the
 // CUDA-core kernel (more CTAs per SM, no TMEM set-up); large ones the tensor
@@ -675,7 +675,8 @@ void tune_device(int kind, TuneTable &tt) {
         t.alpha = 1.f;
         t.beta = 0.f;
       }
-      const int tms[3] = {GEMM_TM, TC_TILE_M, TC_TILE_M}, tns[3] = {GEMM_TN, 64, 128};
+      const int cls = gemm_tile_class<float>(tasks.data(), T);
+      const int tms[3] = {gemm_tile<float>(cls), TC_TILE_M, TC_TILE_M}, tns[3] = {gemm_tile<float>(cls), 64, 128};
       std::vector<int> starts(3 * (T + 1));
       int tiles[3];
       for (int v = 0; v < 3; ++v) {
@@ -697,7 +698,7 @@ void tune_device(int kind, TuneTable &tt) {
         for (int rep = 0; rep < 4; ++rep) {
           HS_CUDA(cudaEventRecord(e0, st));
           if (v == 0)
-            launch_gemm<float>(d_t, d_s, T, tiles[0], st);
+            launch_gemm<float>(d_t, d_s, T, tiles[0], cls, st);
           else if (v == 1)
             launch_gemm_tc(kind, 64, d_t, d_s + (T + 1), T, tiles[1], d_err, st);
           else
