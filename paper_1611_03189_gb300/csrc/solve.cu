@@ -1026,7 +1026,7 @@ void ensure_buffers(FactorHandle &h, int nrhs_cap, cudaStream_t st) {
   h.alloc.get(&h.d_part, sizeof(double) * h.part_blocks * 32, st);
   h.alloc.get(&h.d_scal, sizeof(double) * 7 * 32, st);
   h.alloc.get(&h.d_iflags, sizeof(int) * (2 * 32 + 2), st);
-  HS_CUDA(cudaMemset(h.d_iflags, 0, sizeof(int) * (2 * 32 + 2)));
+  HS_CUDA(cudaMemsetAsync(h.d_iflags, 0, sizeof(int) * (2 * 32 + 2), st));
   if (!h.h_done) HS_CUDA(cudaMallocHost(&h.h_done, sizeof(int)));
   h.nrhs_cap = nrhs_cap;
 }
