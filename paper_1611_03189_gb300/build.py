@@ -64,14 +64,17 @@ def build(verbose: bool = False, force: bool = False) -> str:
             if log:
                 print(log)
     if force or not os.path.exists(LIB) or os.path.getmtime(LIB) < max(os.path.getmtime(o) for o in objs):
-        tmp = LIB + ".tmp"
+        tmp = LIB + f".tmp{os.getpid()}"
         cmd = [nvcc, "-shared", "-o", tmp] + objs + ARCH + ["-lcudart"]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"link failed:\n{r.stdout}\n{r.stderr}")
         os.replace(tmp, LIB)
-    with open(stamp, "w") as f:
-        f.write(machine + "\n")
+    if force or not os.path.exists(stamp):
+        tmp = stamp + f".{os.getpid()}"
+        with open(tmp, "w") as f:
+            f.write(machine + "\n")
+        os.replace(tmp, stamp)
     return LIB
 
 
