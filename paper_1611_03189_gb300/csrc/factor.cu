@@ -345,17 +345,19 @@ struct CholBatch {
   }
 };
 
-// Largest super node whose truncation uses the shared-memory Jacobi kernel
-// (default 32: above that the tridiagonal path needs fewer operations than
-// the ~10 Jacobi sweeps, and on the 512 x 512 workload it took less time);
-// larger ones use the tridiagonal path.
+// Largest super node whose truncation uses the Jacobi kernel; larger ones take
+// the tridiagonal path.  Its ~10 sweeps of m - 1 rounds with two barriers each
+// lose to the tridiagonal path's 2 m steps from the smallest sizes on: with the
+// limit at 32 the small truncations of a 512 x 512 factorization took 11.8 ms
+// (FP32) and those of a 331 x 198 one 33.9 ms (FP64), with it at 16 they take
+// 1.3 and 2.6 and the rest grows by 4 and 7; 8 gives the same again.
 // HS_EIG_SMALL_MAX (environment) lowers the limit, which lets small test
 // problems exercise the tridiagonal path.
 template <typename T>
 int eig_small_max() {
   static const int v = [] {
     const char *e = std::getenv("HS_EIG_SMALL_MAX");
-    const int cap = std::min(32, jacobi_cap<T>());
+    const int cap = 16;
     if (!e) return cap;
     const int x = std::atoi(e);
     return x < 0 ? cap : std::min(std::max(x, 8), cap);   // the tridiagonal path needs m > 8
@@ -1883,14 +1885,13 @@ void execute(Exec &ex, std::vector<std::unique_ptr<Run<T>>> &runs) {
         ex.gemm(B.gram64, false);
       }
       ex.end();
-      const double eps = wp[0]->handle().eps;
       const int variant = wp[0]->handle().variant;
       if (ntrunc) {
         Uploader u;
         const size_t o = u.add(B.trunc);
         char *d = u.upload(ex.scr, ex.sg, ex.st);
         ex.begin(4);
-        launch_trunc<T>((const TruncTask<T> *)(d + o), (int)ntrunc, d_k, eps, variant, B.max_trunc_m, ex.st);
+        launch_trunc<T>((const TruncTask<T> *)(d + o), (int)ntrunc, d_k, variant, B.max_trunc_m, ex.st);
         ex.end();
       }
       if (nt64) {
@@ -1898,8 +1899,7 @@ void execute(Exec &ex, std::vector<std::unique_ptr<Run<T>>> &runs) {
         const size_t o = u.add(B.trunc64);
         char *d = u.upload(ex.scr, ex.sg, ex.st);
         ex.begin(4);
-        launch_trunc<double>((const TruncTask<double> *)(d + o), (int)nt64, d_k, eps, variant, B.max_trunc64_m,
-                             ex.st);
+        launch_trunc<double>((const TruncTask<double> *)(d + o), (int)nt64, d_k, variant, B.max_trunc64_m, ex.st);
         ex.end();
       }
       if (nbig || nb64) {

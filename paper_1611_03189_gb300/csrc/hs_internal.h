@@ -205,8 +205,7 @@ template <typename T>
 void launch_chol_inv(const CholTask<T> *d_tasks, int ntasks, int *d_status, int max_m,
                      cudaStream_t st);
 template <typename T>
-void launch_trunc(const TruncTask<T> *d_tasks, int ntasks, int *d_k, double eps, int variant,
-                  int max_m, cudaStream_t st);
+void launch_trunc(const TruncTask<T> *d_tasks, int ntasks, int *d_k, int variant, int max_m, cudaStream_t st);
 // super nodes above the Jacobi limit (kernels_eig.cu): tridiagonalisation /
 // multisection / inverse iteration.
 // Global work area of one such node (offsets from TruncTask::work; the host
@@ -374,11 +373,6 @@ void launch_refl(const ReflTask<T> *d_tasks, int ntasks, int nb, int m_max, cuda
 // columns per reflector task that fit the shared-memory budget for nodes of size m
 template <typename T>
 int refl_batch(int m);
-// largest m handled by the shared-memory Jacobi truncation
-template <typename T>
-constexpr int jacobi_cap() {
-  return sizeof(T) == 8 ? 110 : 156;
-}
 template <typename T>
 void launch_scatter_values(const double *val, const int64_t *dest, int64_t nnz, T *pool,
                            cudaStream_t st);

@@ -658,7 +658,7 @@ __device__ int select_columns(const T *A, const T *V, int m, double thr, T *U, i
   return k;
 }
 
-template <typename T, bool SMEM>
+template <typename T>
 __global__ void __launch_bounds__(TRUNC_THREADS) k_trunc(const TruncTask<T> *__restrict__ tasks,
                                                         int *__restrict__ kout, int variant) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -673,17 +673,10 @@ __global__ void __launch_bounds__(TRUNC_THREADS) k_trunc(const TruncTask<T> *__r
   const int mp = m + (m & 1);
   const int np = mp / 2 > 0 ? mp / 2 : 1;
   unsigned char *p = smem_raw;
-  T *A;
-  T *V;
-  if (SMEM) {
-    A = reinterpret_cast<T *>(p);
-    p += sizeof(T) * (size_t)m * m;
-    V = reinterpret_cast<T *>(p);
-    p += sizeof(T) * (size_t)m * m;
-  } else {
-    A = t.work;
-    V = t.work + (size_t)m * m;
-  }
+  T *A = reinterpret_cast<T *>(p);
+  p += sizeof(T) * (size_t)m * m;
+  T *V = reinterpret_cast<T *>(p);
+  p += sizeof(T) * (size_t)m * m;
   JacobiShared<T> sh;
   sh.cs = reinterpret_cast<T *>(p);
   p += sizeof(T) * np;
@@ -922,23 +915,11 @@ void launch_chol_inv(const CholTask<T> *d_tasks, int ntasks, int *d_status, int 
 }
 
 template <typename T>
-int trunc_smem_cap() {
-  return sizeof(T) == 8 ? 110 : 156;
-}
-
-template <typename T>
-void launch_trunc(const TruncTask<T> *d_tasks, int ntasks, int *d_k, double eps, int variant,
-                  int max_m, cudaStream_t st) {
+void launch_trunc(const TruncTask<T> *d_tasks, int ntasks, int *d_k, int variant, int max_m, cudaStream_t st) {
   if (ntasks == 0) return;
-  if (max_m <= trunc_smem_cap<T>()) {
-    const size_t sm = 2 * sizeof(T) * (size_t)max_m * max_m + trunc_small_arrays<T>(max_m);
-    check_dynamic_smem(sm, allow_max_dynamic_smem<&k_trunc<T, true>>(), "k_trunc");
-    k_trunc<T, true><<<ntasks, TRUNC_THREADS, sm, st>>>(d_tasks, d_k, variant);
-  } else {
-    const size_t sm = trunc_small_arrays<T>(max_m);
-    check_dynamic_smem(sm, allow_max_dynamic_smem<&k_trunc<T, false>>(), "k_trunc");
-    k_trunc<T, false><<<ntasks, TRUNC_THREADS, sm, st>>>(d_tasks, d_k, variant);
-  }
+  const size_t sm = 2 * sizeof(T) * (size_t)max_m * max_m + trunc_small_arrays<T>(max_m);
+  check_dynamic_smem(sm, allow_max_dynamic_smem<&k_trunc<T>>(), "k_trunc");
+  k_trunc<T><<<ntasks, TRUNC_THREADS, sm, st>>>(d_tasks, d_k, variant);
   count_launch();
   HS_CUDA(cudaGetLastError());
 }
@@ -1053,8 +1034,7 @@ void launch_status_merge(const StatusMerge *d_tasks, int ntasks, cudaStream_t st
                               cudaStream_t);                                                  \
   template void launch_chol_inv<T>(const CholTask<T> *, int, int *, int, cudaStream_t);       \
   template int chol_smem_cap<T>();                                                            \
-  template void launch_trunc<T>(const TruncTask<T> *, int, int *, double, int, int,           \
-                                cudaStream_t);                                                \
+  template void launch_trunc<T>(const TruncTask<T> *, int, int *, int, int, cudaStream_t);    \
   template void launch_phi_scale<T>(const T *, const double *, int64_t, int, T *, cudaStream_t); \
   template void launch_scatter_values<T>(const double *, const int64_t *, int64_t, T *,       \
                                          cudaStream_t);
