@@ -2045,8 +2045,15 @@ void factorize_t(const std::vector<FactorHandle *> &hs, const std::vector<const 
   std::vector<std::unique_ptr<Run<T>>> runs;
   for (size_t p = 0; p < hs.size(); ++p) {
     FactorHandle &h = *hs[p];
-    if (!h.pers) h.pers.reset(new DevArena(256ull << 20, h.alloc));
-    if (!h.scratch) h.scratch.reset(new DevArena(64ull << 20, h.alloc));
+    // chunks by the problem's size (records and live blocks take 1 to 8 KB an
+    // unknown), so that a small factorization neither allocates nor holds much
+    // more than it uses: 320 MB a handle of 1000 to 4096 unknowns before, 16 to
+    // 50 MB now
+    auto chunk = [&](size_t per, size_t lo, size_t hi) {
+      return std::min(hi, std::max(lo, ((size_t)h.plan.n * per + (lo - 1)) & ~(lo - 1)));
+    };
+    if (!h.pers) h.pers.reset(new DevArena(chunk(8192, 8ull << 20, 256ull << 20), h.alloc));
+    if (!h.scratch) h.scratch.reset(new DevArena(chunk(4096, 8ull << 20, 64ull << 20), h.alloc));
     h.pers->set_alloc(h.alloc, st);
     h.scratch->set_alloc(h.alloc, st);
     h.pers->reset();     // a refactorization reuses the previous factor's memory
