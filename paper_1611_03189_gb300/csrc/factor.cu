@@ -29,6 +29,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <functional>
 #include <memory>
 #include <string>
 #include <type_traits>
@@ -114,54 +115,90 @@ struct BlockRef {
   int rowkey;  // key whose unknowns index the rows of the stored matrix
 };
 
-// Pinned host staging for descriptor uploads, two buffers used in alternate
-// waves: a wave's host->device copies have completed by the next wave's
-// synchronisation, so a buffer is rewritten only two waves later.  Callers
+// Pinned host staging for descriptor uploads, two sets of blocks used in
+// alternate waves: a wave's host->device copies have completed by the next
+// wave's synchronisation, so a block is rewritten only two waves later.  Callers
 // flip (next_wave) once per synchronised step and never twice between two
 // synchronisations.
 struct Staging {
-  char *buf[2] = {nullptr, nullptr};
-  size_t cap[2] = {0, 0};
-  size_t off = 0;
+  struct Block {
+    char *p;
+    size_t cap;
+  };
+  std::vector<Block> set[2];
+  size_t next[2] = {0, 0};
   int cur = 0;
-  std::vector<char *> retired;  // outgrown buffers, freed after the final synchronisation
   ~Staging() {
-    for (int i = 0; i < 2; ++i) cudaFreeHost(buf[i]);
-    for (char *p : retired) cudaFreeHost(p);
+    for (auto &v : set)
+      for (Block &b : v) cudaFreeHost(b.p);
   }
   void next_wave() {
     cur ^= 1;
-    off = 0;
+    next[cur] = 0;
   }
-  char *put(const char *src, size_t n) {
-    size_t o = (off + 255) & ~(size_t)255;
-    if (o + n > cap[cur]) {
-      if (buf[cur]) retired.push_back(buf[cur]);
-      cap[cur] = std::max<size_t>(std::max<size_t>(2 * cap[cur], n + 256), (size_t)4 << 20);
-      HS_CUDA(cudaMallocHost(&buf[cur], cap[cur]));
-      o = 0;
-    }
-    std::memcpy(buf[cur] + o, src, n);
-    off = o + n;
-    return buf[cur] + o;
+  // a block of at least n bytes of the current set
+  Block get(size_t n) {
+    std::vector<Block> &v = set[cur];
+    for (; next[cur] < v.size(); ++next[cur])
+      if (v[next[cur]].cap >= n) return v[next[cur]++];
+    Block b{nullptr, std::max(n, (size_t)1 << 20)};
+    HS_CUDA(cudaMallocHost(&b.p, b.cap));
+    v.push_back(b);
+    next[cur] = v.size();
+    return b;
   }
 };
 
-struct Uploader {
-  std::vector<char> buf;
-  template <typename X>
-  size_t add(const std::vector<X> &v) {
-    const size_t off = (buf.size() + 15) & ~(size_t)15;
-    buf.resize(off + v.size() * sizeof(X));
-    if (!v.empty()) std::memcpy(buf.data() + off, v.data(), v.size() * sizeof(X));
-    return off;
+// The launches of a step, queued while the host builds their task lists and
+// then run together: the lists are laid out in one block on both sides and go up
+// in one copy (a copy of its own per launch was some 2000 copies a factorization
+// at 512 x 512, each a gap of a few microseconds in the stream).  What is queued
+// runs in order, on the stream that was `on` when it was queued.
+struct Queue {
+  cudaStream_t st = nullptr;    // the factor stream
+  cudaStream_t on = nullptr;    // stream of the launches being queued
+  cudaStream_t up = nullptr;    // stream the lists go up on: what is queued must run on it or be ordered after it
+  DevArena scr{16ull << 20};    // device side of the lists and other per-wave scratch
+  Staging sg;
+  std::vector<std::function<void()>> ops;
+  char *hp = nullptr, *dp = nullptr;   // the block being filled
+  size_t cap = 0, off = 0, sent = 0;
+  void next_wave() {
+    scr.reset();
+    sg.next_wave();
+    hp = dp = nullptr;
+    cap = off = sent = 0;
   }
-  char *upload(DevArena &a, Staging &sg, cudaStream_t st) {
-    if (buf.empty()) return nullptr;
-    char *d = (char *)a.alloc(buf.size());
-    const char *h = sg.put(buf.data(), buf.size());
-    HS_CUDA(cudaMemcpyAsync(d, h, buf.size(), cudaMemcpyHostToDevice, st));
-    return d;
+  // device address of a copy of v, valid once the queue has run
+  template <typename X>
+  const X *list(const std::vector<X> &v) {
+    const size_t n = sizeof(X) * std::max<size_t>(v.size(), 1);
+    size_t o = (off + 255) & ~(size_t)255;
+    if (!hp || o + n > cap) {
+      send();
+      const Staging::Block b = sg.get(n);
+      hp = b.p;
+      cap = b.cap;
+      dp = (char *)scr.alloc(cap);
+      off = sent = o = 0;
+    }
+    if (!v.empty()) std::memcpy(hp + o, v.data(), sizeof(X) * v.size());
+    off = o + n;
+    return (const X *)(dp + o);
+  }
+  // copies what has been listed since the last copy
+  void send() {
+    if (off > sent) HS_CUDA(cudaMemcpyAsync(dp + sent, hp + sent, off - sent, cudaMemcpyHostToDevice, up));
+    sent = off;
+  }
+  template <typename F>
+  void op(F &&f) {
+    ops.emplace_back(std::forward<F>(f));
+  }
+  void run() {
+    send();
+    for (auto &f : ops) f();
+    ops.clear();
   }
 };
 
@@ -205,8 +242,7 @@ struct GemmBatch {
   // set, each task goes to the variant the autotuner picked for its shape
   // (CUDA-core kernel, or tensor-core kernel with 64- or 128-wide tiles): up
   // to three launches, whose tasks are independent of each other.
-  void launch(DevArena &scr, Staging &sg, cudaStream_t st, int *d_err = nullptr, TcTimer *timer = nullptr,
-              long long wait_cycles = 0) {
+  void queue(Queue &q, int *d_err = nullptr, TcTimer *timer = nullptr, long long wait_cycles = 0) {
     if (tasks.empty()) return;
     const bool on_tc = std::is_same<T, float>::value && tc != HS_TC_NONE;
     std::vector<GemmTask<T>> part[3];
@@ -219,6 +255,7 @@ struct GemmBatch {
       part[0].swap(tasks);
     }
     tasks.clear();
+    const cudaStream_t on = q.on;
     for (int v = 0; v < 3; ++v) {
       if (part[v].empty()) continue;
       const int cls = v == 0 ? gemm_tile_class<T>(part[v].data(), (int)part[v].size()) : 0;
@@ -229,22 +266,23 @@ struct GemmBatch {
         tile_start.push_back(tiles);
         tiles += v == 0 ? gemm_tiles(t, tm) : ((t.M + tm - 1) / tm) * ((t.N + tn - 1) / tn);
       }
-      Uploader u;
-      const size_t ot = u.add(part[v]);
-      const size_t os = u.add(tile_start);
-      char *d = u.upload(scr, sg, st);
+      const GemmTask<T> *d_t = q.list(part[v]);
+      const int *d_s = q.list(tile_start);
+      const int n = (int)part[v].size();
       if (v == 0) {
-        launch_gemm<T>((const GemmTask<T> *)(d + ot), (const int *)(d + os), (int)part[v].size(), tiles, cls, st);
+        q.op([=] { launch_gemm<T>(d_t, d_s, n, tiles, cls, on); });
         continue;
       }
       if constexpr (std::is_same<T, float>::value) {
         if (!d_err) fail(HS_ERR_INVALID, "internal: tensor-core GEMM launched without an error word");
         double f = 0.0;
         for (const GemmTask<T> &t : part[v]) f += 2.0 * t.M * t.N * (double)std::max(t.K, 0);
-        if (timer) timer->before(st);
-        launch_gemm_tc(tc, tn, (const GemmTask<float> *)(d + ot), (const int *)(d + os), (int)part[v].size(),
-                       tiles, d_err, st, wait_cycles);
-        if (timer) timer->after(st, f);
+        const int kind = tc;
+        q.op([=] {
+          if (timer) timer->before(on);
+          launch_gemm_tc(kind, tn, d_t, d_s, n, tiles, d_err, on, wait_cycles);
+          if (timer) timer->after(on, f);
+        });
       }
     }
   }
@@ -292,15 +330,14 @@ struct SumBatch {
     src(s, sld, trans);
     end();
   }
-  void launch(DevArena &scr, Staging &sg, cudaStream_t st) {
+  void queue(Queue &q) {
     if (tasks.empty()) return;
-    Uploader u;
-    const size_t ot = u.add(tasks);
-    const size_t os = u.add(srcs);
-    const size_t ol = u.add(tile_start);
-    char *d = u.upload(scr, sg, st);
-    launch_sum<T>((const SumTask<T> *)(d + ot), (const SumSrc<T> *)(d + os), (const int *)(d + ol),
-                  (int)tasks.size(), tiles, st);
+    const SumTask<T> *d_t = q.list(tasks);
+    const SumSrc<T> *d_r = q.list(srcs);
+    const int *d_s = q.list(tile_start);
+    const int n = (int)tasks.size(), nt = tiles;
+    const cudaStream_t on = q.on;
+    q.op([=] { launch_sum<T>(d_t, d_r, d_s, n, nt, on); });
     tasks.clear();
     srcs.clear();
     tile_start.clear();
@@ -383,24 +420,42 @@ T *talloc(DevArena &a, size_t n) {
   return (T *)a.alloc(sizeof(T) * std::max<size_t>(n, 1));
 }
 
-// Pending device status words checked at the next synchronisation point.
+// Device status words of a Cholesky batch, checked at the next synchronisation.
 struct PendingStatus {
-  int *d = nullptr;
+  size_t chunk, off;   // place in Exec's words
   std::vector<Tag> what;
 };
 
-// What the launches of one factorization step share: the stream, an arena for
-// task descriptors, the pinned staging buffers, the status words to check and
-// the host buffer of the per-wave rank read.  One Exec drives one problem, or
+// What the launches of one factorization step share: the stream and the queue,
+// the status words and ranks read back, events.  One Exec drives one problem, or
 // many independent problems whose steps are batched into the same launches.
-struct Exec : TcTimer {
-  cudaStream_t st = nullptr;
-  DevArena scr{16ull << 20};
-  Staging sg;
+struct Exec : Queue, TcTimer {
   std::vector<PendingStatus> pending;
-  DevArena stat{1ull << 20};   // status words: kept until the sync_check that reads them
-  int *hbuf = nullptr;
-  size_t hbuf_cap = 0;
+  // Words the host reads at the next sync_check (statuses, ranks; the first
+  // word of the first chunk is the tensor-core kernel's error word): device
+  // chunks and their pinned copies, copied up to the words in use.
+  struct Words {
+    int *d, *h;
+    size_t cap, used;
+  };
+  std::vector<Words> words;
+  // n words; the place of the first in (chunk, off)
+  int *get_words(size_t n, size_t &chunk, size_t &off) {
+    for (size_t c = 0; c < words.size(); ++c)
+      if (words[c].used + n <= words[c].cap && (c + 1 == words.size() || words[c + 1].used == 0)) {
+        chunk = c;
+        off = words[c].used;
+        words[c].used += n;
+        return words[c].d + off;
+      }
+    Words w{nullptr, nullptr, std::max(n, (size_t)1 << 16), n};
+    al.get(&w.d, sizeof(int) * w.cap, st);
+    words.push_back(w);
+    HS_CUDA(cudaMallocHost(&words.back().h, sizeof(int) * w.cap));
+    chunk = words.size() - 1;
+    off = 0;
+    return w.d;
+  }
   cudaEvent_t ev_big[2] = {nullptr, nullptr};
   // batched: a problem whose pivot fails is marked here and leaves the lock
   // step; the others go on (single: the failure is an error of the call)
@@ -412,7 +467,7 @@ struct Exec : TcTimer {
   // the FP64 and FP32 factors) and the error word of that kernel's bounded
   // waits, read at every sync_check after a tensor-core launch
   int tc = HS_TC_NONE;
-  int *d_err = nullptr;
+  int *d_err = nullptr;        // (the first word)
   bool tc_pending = false;
   long long wait_cycles = 0;   // bound of the kernels' waits (hs_opts.timeout_cycles; 0 = default)
   // device time of the tensor-core launches: an event pair around each,
@@ -432,17 +487,23 @@ struct Exec : TcTimer {
   std::vector<size_t> open;     // spans begun and not yet ended (nesting)
   void begin(int phase) {
     if (!prof) return;
-    Span sp{phase, nullptr, nullptr};
-    HS_CUDA(cudaEventCreate(&sp.e0));
-    HS_CUDA(cudaEventCreate(&sp.e1));
-    HS_CUDA(cudaEventRecord(sp.e0, st));
-    open.push_back(spans.size());
-    spans.push_back(sp);
+    const cudaStream_t o = on;
+    op([=] {
+      Span sp{phase, nullptr, nullptr};
+      HS_CUDA(cudaEventCreate(&sp.e0));
+      HS_CUDA(cudaEventCreate(&sp.e1));
+      HS_CUDA(cudaEventRecord(sp.e0, o));
+      open.push_back(spans.size());
+      spans.push_back(sp);
+    });
   }
   void end() {
-    if (!prof || open.empty()) return;
-    HS_CUDA(cudaEventRecord(spans[open.back()].e1, st));
-    open.pop_back();
+    if (!prof) return;
+    const cudaStream_t o = on;
+    op([=] {
+      HS_CUDA(cudaEventRecord(spans[open.back()].e1, o));
+      open.pop_back();
+    });
   }
   void phase_times(double *ms, int nphase) {
     for (Span &sp : spans) {
@@ -450,10 +511,10 @@ struct Exec : TcTimer {
       if (cudaEventElapsedTime(&t, sp.e0, sp.e1) == cudaSuccess && sp.phase < nphase) ms[sp.phase] += t;
     }
   }
-  // Streams for work that runs beside the factor stream: fork(q) returns aux
-  // stream q, ordered after what the factor stream holds so far, and join(q)
-  // orders the factor stream after it.
-  static constexpr int kAux = 6;
+  // Streams for work that runs beside the factor stream.  Queued: fork(q)
+  // returns aux stream q, ordered after what the stream `on` holds by then, and
+  // join(q) orders `on` after it.
+  static constexpr int kAux = 8;
   cudaStream_t aux[kAux] = {};
   cudaEvent_t fork_ev[kAux] = {}, join_ev[kAux] = {};
   cudaStream_t fork(int q) {
@@ -462,15 +523,24 @@ struct Exec : TcTimer {
       HS_CUDA(cudaEventCreateWithFlags(&fork_ev[q], cudaEventDisableTiming));
       HS_CUDA(cudaEventCreateWithFlags(&join_ev[q], cudaEventDisableTiming));
     }
-    HS_CUDA(cudaEventRecord(fork_ev[q], st));
-    HS_CUDA(cudaStreamWaitEvent(aux[q], fork_ev[q], 0));
-    return aux[q];
+    const cudaStream_t o = on, x = aux[q];
+    const cudaEvent_t e = fork_ev[q];
+    op([=] {
+      HS_CUDA(cudaEventRecord(e, o));
+      HS_CUDA(cudaStreamWaitEvent(x, e, 0));
+    });
+    return x;
   }
   void join(int q) {
-    HS_CUDA(cudaEventRecord(join_ev[q], aux[q]));
-    HS_CUDA(cudaStreamWaitEvent(st, join_ev[q], 0));
+    const cudaStream_t o = on, x = aux[q];
+    const cudaEvent_t e = join_ev[q];
+    op([=] {
+      HS_CUDA(cudaEventRecord(e, x));
+      HS_CUDA(cudaStreamWaitEvent(o, e, 0));
+    });
   }
-  explicit Exec(cudaStream_t s) : st(s) {
+  explicit Exec(cudaStream_t s) {
+    st = on = up = s;
     HS_CUDA(cudaEventCreate(&ev_big[0]));
     HS_CUDA(cudaEventCreate(&ev_big[1]));
   }
@@ -480,7 +550,9 @@ struct Exec : TcTimer {
   void use_alloc(const DevAlloc &a) {
     al = a;
     scr.set_alloc(a, st);
-    stat.set_alloc(a, st);
+    size_t c, o;
+    d_err = get_words(1, c, o);
+    HS_CUDA(cudaMemsetAsync(d_err, 0, sizeof(int), st));
   }
   ~Exec() {
     // copies from the pinned staging buffers may still be in flight after an error
@@ -492,7 +564,10 @@ struct Exec : TcTimer {
       if (fork_ev[q]) cudaEventDestroy(fork_ev[q]);
       if (join_ev[q]) cudaEventDestroy(join_ev[q]);
     }
-    al.put(d_err, st);
+    for (Words &w : words) {
+      al.put(w.d, st);
+      cudaFreeHost(w.h);
+    }
     for (auto &e : tc_ev) {
       cudaEventDestroy(e.first);
       cudaEventDestroy(e.second);
@@ -501,18 +576,8 @@ struct Exec : TcTimer {
       cudaEventDestroy(sp.e0);
       cudaEventDestroy(sp.e1);
     }
-    cudaFreeHost(hbuf);
     cudaEventDestroy(ev_big[0]);
     cudaEventDestroy(ev_big[1]);
-  }
-  int *host_ints(size_t n) {
-    if (n > hbuf_cap) {
-      cudaFreeHost(hbuf);
-      hbuf = nullptr;
-      hbuf_cap = std::max(n, (size_t)1 << 16);
-      HS_CUDA(cudaMallocHost(&hbuf, hbuf_cap * sizeof(int)));
-    }
-    return hbuf;
   }
   bool mark_failed(const Tag &t, int pivot) {
     const std::string msg = describe(t) + " is not positive definite (pivot " + std::to_string(pivot) + ")";
@@ -531,15 +596,11 @@ struct Exec : TcTimer {
     if (g.tasks.empty()) return;
     g.tc = (tensor_cores && std::is_same<T, float>::value) ? tc : HS_TC_NONE;
     if (g.tc != HS_TC_NONE) {
-      if (!d_err) {
-        al.get(&d_err, 256, st);
-        HS_CUDA(cudaMemsetAsync(d_err, 0, sizeof(int), st));
-      }
       tc_pending = true;
-      g.launch(scr, sg, st, d_err, this, wait_cycles);
+      g.queue(*this, d_err, this, wait_cycles);
       return;
     }
-    g.launch(scr, sg, st, d_err);
+    g.queue(*this);
   }
   void before(cudaStream_t s) override {
     if (tc_ev_used == tc_ev.size()) {
@@ -555,15 +616,16 @@ struct Exec : TcTimer {
     ++tc_ev_used;
     tc_flops += flops;
   }
-  // waits for the stream, then checks the pending status words
+  // copies the words in use, waits for the stream, then checks the pending
+  // statuses; the words read stay in the host copies until the next get_words
   void sync_check() {
+    for (Words &w : words)
+      if (w.used) HS_CUDA(cudaMemcpyAsync(w.h, w.d, sizeof(int) * w.used, cudaMemcpyDeviceToHost, st));
     const auto t0 = std::chrono::steady_clock::now();
     HS_CUDA(cudaStreamSynchronize(st));
     wait_ms += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
     if (tc_pending) {
-      int e = 0;
-      HS_CUDA(cudaMemcpy(&e, d_err, sizeof(int), cudaMemcpyDeviceToHost));
-      if (e) fail(HS_ERR_TIMEOUT, "a bounded wait of the tensor-core GEMM ran out");
+      if (words[0].h[0]) fail(HS_ERR_TIMEOUT, "a bounded wait of the tensor-core GEMM ran out");
       tc_pending = false;
       for (size_t i = 0; i < tc_ev_used; ++i) {
         float t = 0.f;
@@ -573,22 +635,21 @@ struct Exec : TcTimer {
       tc_ev_used = 0;
     }
     for (auto &ps : pending) {
-      std::vector<int> hv(ps.what.size());
-      HS_CUDA(cudaMemcpy(hv.data(), ps.d, ps.what.size() * sizeof(int), cudaMemcpyDeviceToHost));
+      const int *h = words[ps.chunk].h + ps.off;
       for (size_t i = 0; i < ps.what.size(); ++i)
-        if (hv[i] != 0) mark_failed(ps.what[i], hv[i] - 1);
+        if (h[i] != 0) mark_failed(ps.what[i], h[i] - 1);
     }
     pending.clear();
-    stat.reset();
+    for (size_t c = 0; c < words.size(); ++c) words[c].used = c == 0 ? 1 : 0;   // (the error word stays)
   }
   // Cholesky-inverse batch whose statuses are checked at the next sync_check
   template <typename T>
   void chol_checked(CholBatch<T> &cb) {
     if (cb.tasks.empty()) return;
     PendingStatus ps;
-    ps.d = (int *)stat.alloc(sizeof(int) * cb.tasks.size());
+    int *d = get_words(cb.tasks.size(), ps.chunk, ps.off);
     ps.what = cb.what;
-    chol_inv_any<T>(cb.tasks, ps.d);
+    chol_inv_any<T>(cb.tasks, d);
     pending.push_back(ps);
   }
 
@@ -608,10 +669,10 @@ struct Exec : TcTimer {
       }
     }
     if (!small.empty()) {
-      Uploader u;
-      const size_t o = u.add(small);
-      char *d = u.upload(scr, sg, st);
-      launch_chol_inv<T>((const CholTask<T> *)(d + o), (int)small.size(), status, small_max, st);
+      const CholTask<T> *d = list(small);
+      const int n = (int)small.size();
+      const cudaStream_t o = on;
+      op([=] { launch_chol_inv<T>(d, n, status, small_max, o); });
     }
     if (!large.empty()) chol_inv_blocked<T>(large, status);
   }
@@ -649,7 +710,8 @@ struct Exec : TcTimer {
       maxblk = std::max(maxblk, x.nblk);
       w.push_back(x);
     }
-    int *bs = (int *)stat.alloc(sizeof(int) * nbs);
+    int *bs = (int *)scr.alloc(sizeof(int) * nbs);
+    const cudaStream_t o = on;
     {
       int off = 0;
       SumBatch<T> cp;
@@ -658,9 +720,11 @@ struct Exec : TcTimer {
         off += x.nblk;
         cp.copy(x.W, x.t.m, x.t.m, x.t.m, x.t.A, x.t.lda, 0);
         // the inverse is lower triangular with a zero strict upper part
-        HS_CUDA(cudaMemsetAsync(x.t.Linv, 0, sizeof(T) * (size_t)x.t.m * x.t.m, st));
+        T *Li = x.t.Linv;
+        const size_t bytes = sizeof(T) * (size_t)x.t.m * x.t.m;
+        op([=] { HS_CUDA(cudaMemsetAsync(Li, 0, bytes, o)); });
       }
-      cp.launch(scr, sg, st);
+      cp.queue(*this);
     }
     for (int b = 0; b < maxblk; ++b) {
       std::vector<CholTask<T>> dc;
@@ -683,10 +747,9 @@ struct Exec : TcTimer {
           trl.add(Lp, m, 0, Lp, m, 1, x.W + (size_t)(j0 + jb) * m + j0 + jb, m, rest, rest, jb, T(-1), T(1), 1);
         }
       }
-      Uploader u;
-      const size_t o = u.add(dc);
-      char *d = u.upload(scr, sg, st);
-      launch_chol_inv<T>((const CholTask<T> *)(d + o), (int)dc.size(), bs, nb, st);
+      const CholTask<T> *d = list(dc);
+      const int n = (int)dc.size();
+      op([=] { launch_chol_inv<T>(d, n, bs, nb, o); });
       gemm(pan, false);   // the Cholesky of A_ss stays in FP32 on every path
       gemm(trl, false);
     }
@@ -705,14 +768,13 @@ struct Exec : TcTimer {
       }
       gemm(g1, false);
       gemm(g2, false);
-      dg.launch(scr, sg, st);
+      dg.queue(*this);
     }
     std::vector<StatusMerge> sm;
     for (Work &x : w) sm.push_back(StatusMerge{x.bs, x.nblk, nb, status + x.t.status_idx});
-    Uploader u;
-    const size_t o = u.add(sm);
-    char *d = u.upload(scr, sg, st);
-    launch_status_merge((const StatusMerge *)(d + o), (int)sm.size(), st);
+    const StatusMerge *d = list(sm);
+    const int n = (int)sm.size();
+    op([=] { launch_status_merge(d, n, o); });
   }
 };
 
@@ -737,6 +799,7 @@ struct WaveBatches {
   GemmBatch<T> o1, o2, o3, o4;
   CholBatch<T> oc1, oc2;
   // phase B and the Schur update
+  GemmBatch<T> ga, gz;                             // L^-1 A_sN, L^-T L^-1, their Schur product
   GemmBatch<T> g1, g2, g3, g4, g5, g6, g7, g8, gb;
   CholBatch<T> c1, c2;
   SumBatch<T> schur;
@@ -760,6 +823,7 @@ class Run {
   void begin();                                  // outputs cleared, leaf blocks
   void level_begin(int li, SumBatch<T> &sb);     // merge into the level's super nodes
   void wave_a(int li, int widx, WaveBatches<T> &B);
+  void wave_l(WaveBatches<T> &B);               // the elimination's products that need no rank
   void wave_b(const int *hb, size_t nchol, size_t ntrunc, double big_ms, WaveBatches<T> &B);
   // the elimination's GEMM tasks of super nodes [c_next_, c_next_ + count)
   // of the wave; returns whether nodes remain
@@ -1156,6 +1220,23 @@ void Run<T>::wave_a(int li, int widx, WaveBatches<T> &B) {
 }
 
 template <typename T>
+void Run<T>::wave_l(WaveBatches<T> &B) {
+  DevArena &scr = *h_.scratch;
+  const double f0 = B.ga.flops + B.gz.flops;
+  for (Sup &x : cur_) {
+    const int m = x.m, dN = x.dN;
+    x.Gt = talloc<T>(scr, (size_t)m * dN);
+    x.Z = talloc<T>(scr, (size_t)dN * dN);
+    x.M = talloc<T>(*h_.pers, (size_t)m * m);
+    B.ga.add(x.Linv, m, 0, x.AsN, dN, 0, x.Gt, dN, m, dN, m, T(1), T(0), 0, GEMM_A_LOW);   // L^-1 A_sN
+    B.ga.add(x.Linv, m, 1, x.Linv, m, 0, x.M, m, m, m, m, T(1), T(0), 1,
+             GEMM_A_UP | GEMM_B_LOW);                                                 // L^-T L^-1
+    B.gz.add(x.Gt, dN, 1, x.Gt, dN, 0, x.Z, dN, dN, dN, m, T(1), T(0), 1);            // (L^-1 A_sN)^T (L^-1 A_sN)
+  }
+  flops_ += B.ga.flops + B.gz.flops - f0;
+}
+
+template <typename T>
 void Run<T>::wave_b(const int *hb, size_t nchol, size_t ntrunc, double big_ms, WaveBatches<T> &B) {
   DevArena &scr = *h_.scratch;
   // this run's slices of the statuses and ranks read after phase A
@@ -1234,9 +1315,6 @@ bool Run<T>::wave_c(WaveBatches<T> &B, size_t count) {
       x.Wt = talloc<T>(scr, (size_t)m * k);
       x.Tm = talloc<T>(scr, (size_t)k * dN);
     }
-    x.Gt = talloc<T>(scr, (size_t)m * dN);
-    x.Z = talloc<T>(scr, (size_t)dN * dN);
-    x.M = talloc<T>(per, (size_t)m * m);
     x.Pm = talloc<T>(per, (size_t)k * m);
     x.B = talloc<T>(per, (size_t)m * dN);
     if (x.red) {
@@ -1254,11 +1332,8 @@ bool Run<T>::wave_c(WaveBatches<T> &B, size_t count) {
     B.c2.add(x.S2, k, x.L2, k, tag(2, lv_->level, x.s));
     B.g5.add(x.Q1, k, 0, x.L2, k, 1, x.Q, k, m, k, k, T(1), T(0), 0, GEMM_B_UP);
     B.g5.add(x.L1, k, 1, x.L2, k, 1, x.Rinv, k, k, k, k, T(1), T(0), 0, GEMM_A_UP | GEMM_B_UP);
-    // quantities needing Q / L^-1
+    // quantities needing Q
     B.g6.add(x.Linv, m, 1, x.Q, k, 0, x.Wt, k, m, k, m, T(1), T(0), 0, GEMM_A_UP);   // L^-T Q
-    B.g6.add(x.Linv, m, 0, x.AsN, dN, 0, x.Gt, dN, m, dN, m, T(1), T(0), 0, GEMM_A_LOW);   // L^-1 A_sN
-    B.g6.add(x.Linv, m, 1, x.Linv, m, 0, x.M, m, m, m, m, T(1), T(0), 1,
-             GEMM_A_UP | GEMM_B_LOW);                                                 // L^-T L^-1
     if (x.red) {
       B.g6.add(x.U, m, 1, x.AsW, x.dW, 0, x.ArW, x.dW, k, x.dW, m, T(1), T(0));  // U^T A_sW
       if (use_phi_) B.g6.add(x.U, m, 1, phi_[x.s], h_.nphi, 0, x.phir, h_.nphi, k, h_.nphi, m, T(1), T(0));
@@ -1266,7 +1341,6 @@ bool Run<T>::wave_c(WaveBatches<T> &B, size_t count) {
     B.g7.add(x.Rinv, k, 0, x.Wt, k, 1, x.Pm, m, k, m, k, T(1), T(0), 0, GEMM_A_UP);   // P_ss = R^-1 (L^-T Q)^T
     B.g7.add(x.Wt, k, 0, x.Wt, k, 1, x.M, m, m, m, k, T(-1), T(1), 1);          // M_ss -= W W^T
     B.g7.add(x.Q, k, 1, x.Gt, dN, 0, x.Tm, dN, k, dN, m, T(1), T(0));           // Q^T L^-1 A_sN
-    B.g7.add(x.Gt, dN, 1, x.Gt, dN, 0, x.Z, dN, dN, dN, m, T(1), T(0), 1);      // (L^-1 A_sN)^T (L^-1 A_sN)
     B.gb.add(x.M, m, 0, x.AsN, dN, 0, x.B, dN, m, dN, m, T(1), T(0));           // B_s = M_ss A_sN
     B.g8.add(x.Tm, dN, 1, x.Tm, dN, 0, x.Z, dN, dN, dN, k, T(-1), T(1), 1);     // - T^T T
     if (x.red) {
@@ -1623,19 +1697,14 @@ void Run<T>::finish() {
   h_.info.alg_flops = alg_flops_;
 }
 
-// A list of tasks, each owning consecutive CTAs from its blk0 on, uploaded.
-template <typename X>
-const X *upload_list(Exec &ex, const std::vector<X> &v) {
-  Uploader u;
-  const size_t o = u.add(v);
-  char *d = u.upload(ex.scr, ex.sg, ex.st);
-  return (const X *)(d + o);
-}
-
 // Truncation of a wave's nodes above the Jacobi limit (kernels_eig.cu): U_1 and
 // J, the tridiagonalisation, Z = Q^T X (GC), the ranks, the eigenvalues and
 // eigenvectors of T, and U_2 = Q Y.  eps = 0 ends after the first (complete
 // bases).
+// aux streams: the rank-independent products, the Jacobi truncations, then the
+// tridiagonalisation's classes
+constexpr int kAuxL = 0, kAuxJacobi = 1, kAuxTri = 2;
+
 template <typename T>
 void trunc_big(Exec &ex, const std::vector<TruncTask<T>> &all, int *d_k, int variant) {
   std::vector<TruncTask<T>> prep[2], tasks;
@@ -1652,9 +1721,13 @@ void trunc_big(Exec &ex, const std::vector<TruncTask<T>> &all, int *d_k, int var
   }
   // nested spans (phases 10-14) inside the large-truncation span (5)
   ex.begin(10);
+  const cudaStream_t o = ex.on;
   for (int c = 0; c < 2; ++c)
-    if (!prep[c].empty())
-      launch_trunc_prep<T>(upload_list(ex, prep[c]), (int)prep[c].size(), d_k, variant, pmax[c], ex.st);
+    if (!prep[c].empty()) {
+      const TruncTask<T> *d = ex.list(prep[c]);
+      const int np = (int)prep[c].size(), pm = pmax[c];
+      ex.op([=] { launch_trunc_prep<T>(d, np, d_k, variant, pm, o); });
+    }
   ex.end();
   const int n = (int)tasks.size();
   if (n == 0) return;
@@ -1709,24 +1782,27 @@ void trunc_big(Exec &ex, const std::vector<TruncTask<T>> &all, int *d_k, int var
   if (steps.empty())
     for (int q = 0; q < kTriClasses; ++q)
       if (!by_c[q].empty()) home = q;
-  for (int q = 0; q < kTriClasses; ++q) {
-    if (by_c[q].empty() || q == home) continue;
-    const GridTri<T> *d = upload_list(ex, by_c[q]);
-    launch_tri_onchip<T>(d, (int)by_c[q].size(), q, cmax[q], ex.fork(used++));
-  }
-  if (home >= 0)
-    launch_tri_onchip<T>(upload_list(ex, by_c[home]), (int)by_c[home].size(), home, cmax[home], ex.st);
+  auto onchip = [&](const std::vector<GridTri<T>> &v, int q, int mx, cudaStream_t x) {
+    const GridTri<T> *d = ex.list(v);
+    const int nv = (int)v.size();
+    ex.op([=] { launch_tri_onchip<T>(d, nv, q, mx, x); });
+  };
+  for (int q = 0; q < kTriClasses; ++q)
+    if (!by_c[q].empty() && q != home) onchip(by_c[q], q, cmax[q], ex.fork(kAuxTri + used++));
+  if (home >= 0) onchip(by_c[home], home, cmax[home], o);
   if (!steps.empty()) {
-    const GridTri<T> *d_gt = upload_list(ex, steps);
-    for (int k = 0; k <= kmax; ++k) {
-      launch_tri_step<T>(d_gt, (int)steps.size(), sblocks, k, 0, ex.st);
-      if (k < kmax) launch_tri_step<T>(d_gt, (int)steps.size(), sblocks, k, 1, ex.st);
-    }
+    const GridTri<T> *d_gt = ex.list(steps);
+    const int ns = (int)steps.size();
+    ex.op([=] {
+      for (int k = 0; k <= kmax; ++k) {
+        launch_tri_step<T>(d_gt, ns, sblocks, k, 0, o);
+        if (k < kmax) launch_tri_step<T>(d_gt, ns, sblocks, k, 1, o);
+      }
+    });
     for (int q = 0; q < kTriClasses; ++q)
-      if (!tail[q].empty())
-        launch_tri_onchip<T>(upload_list(ex, tail[q]), (int)tail[q].size(), q, tmax[q], ex.st);
+      if (!tail[q].empty()) onchip(tail[q], q, tmax[q], o);
   }
-  for (int q = 0; q < used; ++q) ex.join(q);
+  for (int q = 0; q < used; ++q) ex.join(kAuxTri + q);
   ex.end();
   // products with Q: by warps up to kQmulMax, by CTAs above
   auto products = [&](bool fwd) {
@@ -1747,8 +1823,15 @@ void trunc_big(Exec &ex, const std::vector<TruncTask<T>> &all, int *d_k, int var
           rf.push_back(ReflTask<T>{L.A, L.tau, cols, t.U, L.sc_int, t.m, j0, fwd ? 1 : 0});
       }
     }
-    if (!qm.empty()) launch_qmul<T>(upload_list(ex, qm), (int)qm.size(), blocks, qmax, fwd, ex.st);
-    if (!rf.empty()) launch_refl<T>(upload_list(ex, rf), (int)rf.size(), nb, max_m, ex.st);
+    const int nq = (int)qm.size(), nr = (int)rf.size();
+    if (nq) {
+      const QmulTask<T> *d = ex.list(qm);
+      ex.op([=] { launch_qmul<T>(d, nq, blocks, qmax, fwd, o); });
+    }
+    if (nr) {
+      const ReflTask<T> *d = ex.list(rf);
+      ex.op([=] { launch_refl<T>(d, nr, nb, max_m, o); });
+    }
   };
   if (variant != HS_LORASP) {
     ex.begin(12);
@@ -1756,7 +1839,10 @@ void trunc_big(Exec &ex, const std::vector<TruncTask<T>> &all, int *d_k, int var
     ex.end();
   }
   ex.begin(13);
-  launch_rank<T>(upload_list(ex, tasks), n, d_k, variant, max_m, max_np, ex.st);
+  {
+    const TruncTask<T> *d = ex.list(tasks);
+    ex.op([=] { launch_rank<T>(d, n, d_k, variant, max_m, max_np, o); });
+  }
   {
     // eigenvalues and eigenvectors of T (at most m per node)
     const int spc = invit_slots<T>(max_m);
@@ -1771,8 +1857,11 @@ void trunc_big(Exec &ex, const std::vector<TruncTask<T>> &all, int *d_k, int var
       it.push_back(x);
       iblocks += (t.m + spc - 1) / spc;
     }
-    launch_eigval<T>(upload_list(ex, ev), n, eblocks, max_m, ex.st);
-    launch_invit<T>(upload_list(ex, it), n, iblocks, spc, max_m, ex.st);
+    const EigTask<T> *de = ex.list(ev), *di = ex.list(it);
+    ex.op([=] {
+      launch_eigval<T>(de, n, eblocks, max_m, o);
+      launch_invit<T>(di, n, iblocks, spc, max_m, o);
+    });
   }
   ex.end();
   ex.begin(14);
@@ -1827,18 +1916,18 @@ void execute(Exec &ex, std::vector<std::unique_ptr<Run<T>>> &runs) {
     for (auto &r : runs)
       if (li < r->levels() && r->ok()) part.push_back(r.get());
     {
-      // the merge's descriptors go into the staging buffer in use: flipping
-      // to the other one here would make the next wave step flip back to a
-      // buffer whose copies may still be pending (no synchronisation between)
-      ex.scr.reset();
+      // the merge's lists go into the staging set in use: flipping to the
+      // other one here would make the next wave step flip back to a set whose
+      // copies may still be pending (no synchronisation between)
       SumBatch<T> sb;
       for (Run<T> *r : part) {
         r->handle().scratch->reset();
         r->level_begin(li, sb);
       }
       ex.begin(0);
-      sb.launch(ex.scr, ex.sg, ex.st);
+      sb.queue(ex);
       ex.end();
+      ex.run();
       hc.tick(0);
     }
     int nw = 0;
@@ -1848,10 +1937,9 @@ void execute(Exec &ex, std::vector<std::unique_ptr<Run<T>>> &runs) {
       for (Run<T> *r : part)
         if (w < r->waves(li) && r->ok()) wp.push_back(r);
       if (wp.empty()) continue;
-      // one flip of the staging buffers per wave step: the other buffer's
-      // copies were enqueued before the previous step's synchronisation
-      ex.scr.reset();
-      ex.sg.next_wave();
+      // one flip of the staging sets per wave step: the other set's copies
+      // were enqueued before the previous step's synchronisation
+      ex.next_wave();
       for (Run<T> *r : wp) r->handle().scratch->reset();
       WaveBatches<T> B;
       // phase A
@@ -1865,69 +1953,84 @@ void execute(Exec &ex, std::vector<std::unique_ptr<Run<T>>> &runs) {
       for (size_t i = 0; i < nt64; ++i) B.trunc64[i].k_idx = (int)(B.k_off64 + i);
       for (size_t i = 0; i < nb64; ++i) B.trunc_big64[i].k_idx = (int)(B.k_off64 + nt64 + i);
       ex.begin(1);
-      B.gather.launch(ex.scr, ex.sg, ex.st);
+      B.gather.queue(ex);
       ex.end();
-      int *d_stat = (int *)ex.scr.alloc(sizeof(int) * (nchol + ntrunc + nbig + nt64 + nb64 + 1));
+      size_t rchunk = 0, roff = 0;
+      int *d_stat = ex.get_words(nchol + ntrunc + nbig + nt64 + nb64 + 1, rchunk, roff);
       int *d_k = d_stat + nchol;
+      // the Cholesky of A_ss and what needs no rank run beside the truncation
+      const cudaStream_t side = ex.fork(kAuxL);
+      ex.on = side;
       if (nchol) {
         ex.begin(2);
         ex.chol_inv_any<T>(B.chol.tasks, d_stat);
         ex.end();
       }
+      ex.on = ex.st;
       ex.begin(3);
       ex.gemm(B.gram, false);   // the Gram feeds the rank decision
       if (!B.widen.empty()) {
         // FP64 truncation of an FP32 factor: FP64 copies, then their Gram
-        Uploader u;
-        const size_t o = u.add(B.widen);
-        char *d = u.upload(ex.scr, ex.sg, ex.st);
-        launch_convert_list((const ConvTask *)(d + o), (int)B.widen.size(), ex.st);
+        const ConvTask *d = ex.list(B.widen);
+        const int n = (int)B.widen.size();
+        ex.op([=, &ex] { launch_convert_list(d, n, ex.st); });
         ex.gemm(B.gram64, false);
       }
       ex.end();
       const int variant = wp[0]->handle().variant;
-      if (ntrunc) {
-        Uploader u;
-        const size_t o = u.add(B.trunc);
-        char *d = u.upload(ex.scr, ex.sg, ex.st);
+      const bool jac = ntrunc || nt64;
+      if (jac) {
+        const cudaStream_t js = nbig || nb64 ? ex.fork(kAuxJacobi) : ex.st;
+        ex.on = js;
         ex.begin(4);
-        launch_trunc<T>((const TruncTask<T> *)(d + o), (int)ntrunc, d_k, variant, B.max_trunc_m, ex.st);
+        if (ntrunc) {
+          const TruncTask<T> *d = ex.list(B.trunc);
+          const int mx = B.max_trunc_m;
+          ex.op([=] { launch_trunc<T>(d, (int)ntrunc, d_k, variant, mx, js); });
+        }
+        if (nt64) {
+          const TruncTask<double> *d = ex.list(B.trunc64);
+          const int mx = B.max_trunc64_m;
+          ex.op([=] { launch_trunc<double>(d, (int)nt64, d_k, variant, mx, js); });
+        }
         ex.end();
-      }
-      if (nt64) {
-        Uploader u;
-        const size_t o = u.add(B.trunc64);
-        char *d = u.upload(ex.scr, ex.sg, ex.st);
-        ex.begin(4);
-        launch_trunc<double>((const TruncTask<double> *)(d + o), (int)nt64, d_k, variant, B.max_trunc64_m, ex.st);
-        ex.end();
+        ex.on = ex.st;
       }
       if (nbig || nb64) {
         ex.begin(5);
-        HS_CUDA(cudaEventRecord(ex.ev_big[0], ex.st));
+        ex.op([&ex] { HS_CUDA(cudaEventRecord(ex.ev_big[0], ex.st)); });
         if (nbig) trunc_big<T>(ex, B.trunc_big, d_k, variant);
         if (nb64) trunc_big<double>(ex, B.trunc_big64, d_k, variant);
-        HS_CUDA(cudaEventRecord(ex.ev_big[1], ex.st));
+        ex.op([&ex] { HS_CUDA(cudaEventRecord(ex.ev_big[1], ex.st)); });
         ex.end();
+        if (jac) ex.join(kAuxJacobi);
       }
       if (!B.narrow.empty()) {
         // the FP64 bases back to the factor precision
-        Uploader u;
-        const size_t o = u.add(B.narrow);
-        char *d = u.upload(ex.scr, ex.sg, ex.st);
-        launch_convert_list((const ConvTask *)(d + o), (int)B.narrow.size(), ex.st);
+        const ConvTask *d = ex.list(B.narrow);
+        const int n = (int)B.narrow.size();
+        ex.op([=, &ex] { launch_convert_list(d, n, ex.st); });
       }
+      ex.run();
+      // built while the GPU works on the truncation
+      for (Run<T> *r : wp) r->wave_l(B);
+      ex.on = ex.up = side;
+      ex.begin(7);
+      ex.gemm(B.ga);
+      ex.gemm(B.gz);
+      ex.end();
+      ex.on = ex.st;
+      ex.join(kAuxL);
+      ex.run();
+      ex.up = ex.st;
       // one read of the statuses and ranks
-      const size_t nread = nchol + ntrunc + nbig + nt64 + nb64;
-      int *hb = ex.host_ints(nread + 1);
-      if (nread) HS_CUDA(cudaMemcpyAsync(hb, d_stat, sizeof(int) * nread, cudaMemcpyDeviceToHost, ex.st));
       hc.tick(2);
       ex.sync_check();
       hc.tick(3);
       float big_ms = 0.f;
       if (nbig || nb64) HS_CUDA(cudaEventElapsedTime(&big_ms, ex.ev_big[0], ex.ev_big[1]));
       for (Run<T> *r : wp)
-        if (r->ok()) r->wave_b(hb, nchol, ntrunc, big_ms, B);
+        if (r->ok()) r->wave_b(ex.words[rchunk].h + roff, nchol, ntrunc, big_ms, B);
       hc.tick(4);
       // U of the large path: CholQR2
       ex.begin(6);
@@ -1938,6 +2041,7 @@ void execute(Exec &ex, std::vector<std::unique_ptr<Run<T>>> &runs) {
       ex.chol_checked(B.oc2);
       ex.gemm(B.o4);
       ex.end();
+      ex.run();
       hc.tick(5);
       // phase B and the Schur update.  The GEMM tasks are built and launched
       // in chunks of super nodes, so that the GPU starts on the first chunk
@@ -1968,6 +2072,7 @@ void execute(Exec &ex, std::vector<std::unique_ptr<Run<T>>> &runs) {
         ex.gemm(B.g8);
         ex.gemm(B.gb, false);   // read by the solves: in FP32 on every mixed path
         ex.end();
+        ex.run();
         B.c1.tasks.clear();
         B.c1.what.clear();
         B.c2.tasks.clear();
@@ -1978,8 +2083,9 @@ void execute(Exec &ex, std::vector<std::unique_ptr<Run<T>>> &runs) {
         if (r->ok()) r->wave_d(B);
       hc.tick(8);
       ex.begin(8);
-      B.schur.launch(ex.scr, ex.sg, ex.st);
+      B.schur.queue(ex);
       ex.end();
+      ex.run();
       hc.tick(9);
     }
     for (Run<T> *r : part)
@@ -1987,9 +2093,8 @@ void execute(Exec &ex, std::vector<std::unique_ptr<Run<T>>> &runs) {
     hc.tick(10);
   }
   // the roots (one flip: the last wave step synchronised after the other
-  // buffer's copies)
-  ex.scr.reset();
-  ex.sg.next_wave();
+  // set's copies)
+  ex.next_wave();
   {
     SumBatch<T> sb;
     for (auto &r : runs)
@@ -1998,7 +2103,7 @@ void execute(Exec &ex, std::vector<std::unique_ptr<Run<T>>> &runs) {
         r->root_a(sb);
       }
     ex.begin(9);
-    sb.launch(ex.scr, ex.sg, ex.st);
+    sb.queue(ex);
     CholBatch<T> cb;
     GemmBatch<T> g;
     for (auto &r : runs)
@@ -2006,6 +2111,7 @@ void execute(Exec &ex, std::vector<std::unique_ptr<Run<T>>> &runs) {
     ex.chol_checked(cb);
     ex.gemm(g);
     ex.end();
+    ex.run();
   }
   ex.sync_check();
   hc.tick(11);
