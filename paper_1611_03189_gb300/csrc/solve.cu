@@ -77,19 +77,46 @@ __device__ __forceinline__ void load_x(const T *x, int nr, T (&v)[NR]) {
   }
 }
 
+// Programmatic dependent launch.  Each wave's launch may start while the one
+// before it still runs: it reads its item and its first record entries, asks for
+// the rest of them to come to L2 (none of which any launch of the solve writes),
+// and only then waits for the launch before.  That takes the two longest loads
+// of a step, descriptor and records from HBM, off the chain of dependent
+// launches: 692 -> 591 us an iteration at 512 x 512 (FP32, one right-hand side),
+// the 64 x 64 FP64 solve 829 -> 725 us, GMRES at 256 x 256 5.00 -> 4.62 ms.  FP64
+// passes of 8 or more right-hand sides keep to plain launches (300 x 217, five:
+// 1.59 ms against 1.66: they are bound by the FP64 rate, and CTAs that wait take
+// slots).  DEP is false there and inside the persistent kernel.
+template <typename T, int NR>
+__host__ __device__ constexpr bool early_start() {
+  return sizeof(T) == 4 || NR < 8;
+}
+__device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.launch_dependents;"); }
+template <bool DEP>
+__device__ __forceinline__ void dep_wait() {
+  if constexpr (DEP) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
+// av[u][r] = a[r][c0 + 32 u + lane] (0 from len on)
+template <typename T, int R>
+__device__ __forceinline__ void load_chunk(const T *const (&a)[R], int c0, int len, int lane, T (&av)[4][R]) {
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int c = c0 + 32 * u + lane;
+#pragma unroll
+    for (int r = 0; r < R; ++r) av[u][r] = c < len ? __ldg(a[r] + c) : T(0);
+  }
+}
+
 // acc[r][j] += sum_c a[r][c] x[c*stride + j] for c = lane, lane + 32, ... < len:
-// R rows share every load of x, and 4 R row elements per lane are in flight
+// R rows share every load of x, and 4 R row elements per lane are in flight;
+// av holds the first chunk
 template <typename T, int NR, int R, bool VEC>
 __device__ __forceinline__ void rows_dot(const T *const (&a)[R], const T *x, int len, int64_t stride, int nr,
-                                         int lane, T (&acc)[R][NR]) {
+                                         int lane, T (&av)[4][R], T (&acc)[R][NR]) {
   for (int c0 = 0; c0 < len; c0 += 128) {
-    T av[4][R];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int c = c0 + 32 * u + lane;
-#pragma unroll
-      for (int r = 0; r < R; ++r) av[u][r] = c < len ? __ldg(a[r] + c) : T(0);
-    }
+    if (c0 > 0) load_chunk<T, R>(a, c0, len, lane, av);
 #pragma unroll
     for (int u = 0; u < 4; ++u)
       if (c0 + 32 * u < len) {
@@ -145,18 +172,24 @@ __device__ __forceinline__ bool warp_sum_writer(int lane) {
   return V >= 32 || lane % (32 / (V >= 32 ? 32 : V)) == 0;
 }
 
+// av[u] = A[q*ld] for q = q0 + AW u (0 from len on)
+template <typename T>
+__device__ __forceinline__ void load_cols(const T *A, int64_t ld, int q0, int len, bool active, T (&av)[4]) {
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int q = q0 + AW * u;
+    av[u] = active && q < len ? __ldg(A + q * ld) : T(0);
+  }
+}
+
 // acc[j] += sum_q A[q*ld] x[q*stride + j] over q = warp, warp + AW, ... < len:
-// a CTA's warps share the walk down 32 adjacent columns (lane: one column)
+// a CTA's warps share the walk down 32 adjacent columns (lane: one column);
+// av holds the first entries
 template <typename T, int NR, bool VEC>
 __device__ __forceinline__ void cols_dot(const T *A, int64_t ld, const T *x, int len, int64_t stride, int nr, int warp,
-                                         bool active, T (&acc)[NR]) {
+                                         bool active, T (&av)[4], T (&acc)[NR]) {
   for (int q0 = warp; q0 < len; q0 += 4 * AW) {
-    T av[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int q = q0 + AW * u;
-      av[u] = active && q < len ? __ldg(A + q * ld) : T(0);
-    }
+    if (q0 > warp) load_cols<T>(A, ld, q0, len, active, av);
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int q = q0 + AW * u;
@@ -185,7 +218,7 @@ __host__ __device__ constexpr int rows_per_pass() {
 }
 
 // One item of the forward step of a wave.
-template <typename T, int NR, bool VEC>
+template <typename T, int NR, bool VEC, bool DEP>
 __device__ __forceinline__ void fwd_item(const ApplyItem &it, const ApplyNode *__restrict__ nodes,
                                          const ApplyContrib *__restrict__ cb, T *ws, T *tcur, const T *tprev, int nrhs,
                                          int j0, ItemSmem<T, NR> &sm) {
@@ -196,18 +229,38 @@ __device__ __forceinline__ void fwd_item(const ApplyItem &it, const ApplyNode *_
     constexpr int R = rows_per_pass<T, NR>();
     const int total = it.m + it.k;
     const T *x = ws + it.x * nrhs + j0;
-#pragma unroll 1
-    for (int r0 = it.i0 + warp * AR; r0 < min(it.i0 + (warp + 1) * AR, total); r0 += R) {
-      const T *a[R];
-      T acc[R][NR];
+    const int w0 = it.i0 + warp * AR, w1 = min(w0 + AR, total);
+    auto row_ptr = [&](int row) {
+      row = min(row, total - 1);
+      return row < it.m ? (const T *)it.A + (int64_t)row * it.m : (const T *)it.P + (int64_t)(row - it.m) * it.m;
+    };
+    const T *a[R];
+    T av[4][R];
 #pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const int row = min(r0 + r, total - 1);
-        a[r] = row < it.m ? (const T *)it.A + (int64_t)row * it.m : (const T *)it.P + (int64_t)(row - it.m) * it.m;
+    for (int r = 0; r < R; ++r) a[r] = row_ptr(w0 + r);
+    if (w0 < w1) {
+      load_chunk<T, R>(a, 0, it.m, lane, av);
+      if constexpr (DEP) {
+        // the rest of the rows, one line (128 bytes) per lane and turn
+        constexpr int LE = 128 / (int)sizeof(T);
+        const int lines = it.m > 128 ? (it.m - 128 + LE - 1) / LE : 0;
+        for (int q = lane; q < AR * lines; q += 32) prefetch_l2(row_ptr(w0 + q % AR) + 128 + (q / AR) * LE);
+      }
+    }
+    dep_wait<DEP>();
+#pragma unroll 1
+    for (int r0 = w0; r0 < w1; r0 += R) {
+      T acc[R][NR];
+      if (r0 > w0) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) a[r] = row_ptr(r0 + r);
+        load_chunk<T, R>(a, 0, it.m, lane, av);
+      }
+#pragma unroll
+      for (int r = 0; r < R; ++r)
 #pragma unroll
         for (int j = 0; j < NR; ++j) acc[r][j] = T(0);
-      }
-      rows_dot<T, NR, R, VEC>(a, x, it.m, nrhs, nr, lane, acc);
+      rows_dot<T, NR, R, VEC>(a, x, it.m, nrhs, nr, lane, av, acc);
       constexpr int V = R * NR;
       T(&v)[V] = reinterpret_cast<T(&)[V]>(acc);
       warp_sums<T, V>(v, lane);
@@ -230,9 +283,16 @@ __device__ __forceinline__ void fwd_item(const ApplyItem &it, const ApplyNode *_
     T acc[NR];
 #pragma unroll
     for (int j = 0; j < NR; ++j) acc[j] = T(0);
+    ApplyContrib ac = cb[it.first];
+    T av[4];
+    load_cols<T>((const T *)ac.A + i, ac.ld, warp, ac.m, active, av);
+    dep_wait<DEP>();
     for (int c = 0; c < it.count; ++c) {
-      const ApplyContrib ac = cb[it.first + c];
-      cols_dot<T, NR, VEC>((const T *)ac.A + i, ac.ld, ws + ac.x * nrhs + j0, ac.m, nrhs, nr, warp, active, acc);
+      if (c > 0) {
+        ac = cb[it.first + c];
+        load_cols<T>((const T *)ac.A + i, ac.ld, warp, ac.m, active, av);
+      }
+      cols_dot<T, NR, VEC>((const T *)ac.A + i, ac.ld, ws + ac.x * nrhs + j0, ac.m, nrhs, nr, warp, active, av, acc);
     }
 #pragma unroll
     for (int j = 0; j < NR; ++j) sm.part[warp][j][lane] = acc[j];
@@ -247,6 +307,7 @@ __device__ __forceinline__ void fwd_item(const ApplyItem &it, const ApplyNode *_
     __syncthreads();
   } else {
     // t_s of the previous wave into the place of its phi_s, one node per warp
+    dep_wait<DEP>();
     if (warp < it.count) {
       const ApplyNode &nd = nodes[it.first + warp];
       const int64_t src = nd.toff * nrhs, dst = nd.xs * nrhs;
@@ -261,7 +322,7 @@ __device__ __forceinline__ void fwd_item(const ApplyItem &it, const ApplyNode *_
 
 // One item of the backward step: x_s = t_s + P_ss^T x_r - B_s x_N for the
 // unknowns i0 .. i0 + 31 of s, in place of t_s (tsrc: the last wave's t_s)
-template <typename T, int NR, bool VEC>
+template <typename T, int NR, bool VEC, bool DEP>
 __device__ __forceinline__ void bwd_item(const ApplyItem &it, const ApplyNbr *__restrict__ nb, T *ws, const T *tsrc,
                                          int nrhs, int j0, ItemSmem<T, NR> &sm) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -270,8 +331,22 @@ __device__ __forceinline__ void bwd_item(const ApplyItem &it, const ApplyNbr *__
   T acc[NR];
 #pragma unroll
   for (int j = 0; j < NR; ++j) acc[j] = T(0);
-  if (it.k > 0)
-    cols_dot<T, NR, VEC>((const T *)it.P + i, it.m, ws + it.r * nrhs + j0, it.k, nrhs, nr, warp, i < it.m, acc);
+  const T *P = (const T *)it.P + i;
+  T av[4];
+  load_cols<T>(P, it.m, warp, it.k, i < it.m, av);
+  if constexpr (DEP) {
+    // what the first loads leave: lines of P_ss's rows, and of the rows of B_s
+    for (int q = 4 * AW + (int)threadIdx.x; q < it.k; q += AT)
+      prefetch_l2((const T *)it.P + (int64_t)q * it.m + it.i0);
+    constexpr int LE = 128 / (int)sizeof(T);
+    if (it.count > 0) {
+      const int lines = (it.dN + LE - 1) / LE, rows = min(kApplyRows, it.m - it.i0);
+      for (int q = threadIdx.x; q < rows * lines; q += AT)
+        prefetch_l2((const T *)it.A + (int64_t)(it.i0 + q / lines) * it.dN + (q % lines) * LE);
+    }
+  }
+  dep_wait<DEP>();
+  if (it.k > 0) cols_dot<T, NR, VEC>(P, it.m, ws + it.r * nrhs + j0, it.k, nrhs, nr, warp, i < it.m, av, acc);
 #pragma unroll
   for (int j = 0; j < NR; ++j) sm.part[warp][j][lane] = acc[j];
   if (it.count > 0) {
@@ -290,7 +365,9 @@ __device__ __forceinline__ void bwd_item(const ApplyItem &it, const ApplyNbr *__
 #pragma unroll
         for (int r = 0; r < R; ++r)
           a[r] = (const T *)it.A + (int64_t)min(it.i0 + r0 + r, it.m - 1) * it.dN + n.col;
-        rows_dot<T, NR, R, VEC>(a, ws + n.x * nrhs + j0, n.size, nrhs, nr, lane, ra);
+        T bv[4][R];
+        load_chunk<T, R>(a, 0, n.size, lane, bv);
+        rows_dot<T, NR, R, VEC>(a, ws + n.x * nrhs + j0, n.size, nrhs, nr, lane, bv, ra);
       }
       constexpr int V = R * NR;
       T(&v)[V] = reinterpret_cast<T(&)[V]>(ra);
@@ -325,14 +402,16 @@ __global__ void __launch_bounds__(AT) k_fwd(const ApplyItem *__restrict__ items,
                                             const ApplyContrib *__restrict__ cb, T *ws, T *tcur, const T *tprev,
                                             int nrhs, int j0) {
   __shared__ ItemSmem<T, NR> sm;
-  fwd_item<T, NR, VEC>(items[blockIdx.x], nodes, cb, ws, tcur, tprev, nrhs, j0, sm);
+  if constexpr (early_start<T, NR>()) dep_launch();
+  fwd_item<T, NR, VEC, early_start<T, NR>()>(items[blockIdx.x], nodes, cb, ws, tcur, tprev, nrhs, j0, sm);
 }
 
 template <typename T, int NR, bool VEC>
 __global__ void __launch_bounds__(AT) k_bwd(const ApplyItem *__restrict__ items, const ApplyNbr *__restrict__ nb,
                                             T *ws, const T *tsrc, int nrhs, int j0) {
   __shared__ ItemSmem<T, NR> sm;
-  bwd_item<T, NR, VEC>(items[blockIdx.x], nb, ws, tsrc, nrhs, j0, sm);
+  if constexpr (early_start<T, NR>()) dep_launch();
+  bwd_item<T, NR, VEC, early_start<T, NR>()>(items[blockIdx.x], nb, ws, tsrc, nrhs, j0, sm);
 }
 
 template <typename T>
@@ -350,7 +429,9 @@ __device__ __forceinline__ void root_warp(const T *__restrict__ Ainv, int m, int
   T acc[1][NR];
 #pragma unroll
   for (int j = 0; j < NR; ++j) acc[0][j] = T(0);
-  rows_dot<T, NR, 1, VEC>(a, tb + j0, m, nrhs, nr, lane, acc);
+  T av[4][1];
+  load_chunk<T, 1>(a, 0, m, lane, av);
+  rows_dot<T, NR, 1, VEC>(a, tb + j0, m, nrhs, nr, lane, av, acc);
   warp_sums<T, NR>(acc[0], lane);
   if (warp_sum_writer<NR>(lane)) {
     const int j = warp_sum_first<NR>(lane);
@@ -451,11 +532,11 @@ __global__ void __launch_bounds__(AT) k_apply_persistent(
       T *tc = (st.wave & 1) ? tb1 : tb0, *tp = (st.wave & 1) ? tb0 : tb1;
       if (st.kind == AS_FWD) {
         for (int i = blockIdx.x; i < wa.f_count; i += gridDim.x)
-          fwd_item<T, NR, VEC>(items[wa.f_first + i], nodes, cb, ws, tc, tp, nrhs, j0, sm);
+          fwd_item<T, NR, VEC, false>(items[wa.f_first + i], nodes, cb, ws, tc, tp, nrhs, j0, sm);
       } else {
         const T *ts = st.wave == nwaves - 1 ? tc : nullptr;
         for (int i = blockIdx.x; i < wa.b_count; i += gridDim.x)
-          bwd_item<T, NR, VEC>(items[wa.b_first + i], nbrs, ws, ts, nrhs, j0, sm);
+          bwd_item<T, NR, VEC, false>(items[wa.b_first + i], nbrs, ws, ts, nrhs, j0, sm);
       }
     }
     if (si + 1 < nsteps && !grid_barrier(bar, (unsigned)si, err, limit)) return;
@@ -777,6 +858,23 @@ int grid_for(int64_t total) {
 // grid of the PCG reduction kernels: a function of n only (see above)
 int rgrid_for(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>((n + PT - 1) / PT, 152 * 4)); }
 
+// A launch of k_fwd or k_bwd, which with `early` may start before the one
+// before it ends (dep_wait)
+template <typename... P, typename... A>
+void launch_step(bool early, void (*kernel)(P...), int grid, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid, 1, 1);
+  cfg.blockDim = dim3(AT, 1, 1);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = early ? 1 : 0;
+  HS_CUDA(cudaLaunchKernelEx(&cfg, kernel, args...));
+  count_launch();
+}
+
 // One pass of Algorithm 2 over right-hand sides [j0, j0 + NR) of the
 // workspace ws (layout [unknown][nrhs]); tb0 and tb1 are the scratch of even and
 // odd waves.
@@ -787,9 +885,9 @@ void apply_waves_nr(const FactorHandle &h, T *ws, T *tb0, T *tb1, int nrhs, int 
   for (int w = 0; w < nw; ++w) {
     const WaveApply &wa = h.waves[w];
     if (!wa.f_count) continue;
-    k_fwd<T, NR, VEC><<<wa.f_count, AT, 0, st>>>(h.d_items + wa.f_first, h.d_nodes, h.d_contribs, ws, buf(w),
-                                                 buf(w + 1), nrhs, j0);
-    count_launch();
+    launch_step(early_start<T, NR>(), k_fwd<T, NR, VEC>, wa.f_count, st, (const ApplyItem *)(h.d_items + wa.f_first),
+                 (const ApplyNode *)h.d_nodes, (const ApplyContrib *)h.d_contribs, ws, buf(w), (const T *)buf(w + 1),
+                 nrhs, j0);
   }
   if (h.root_m > 0) {
     const int64_t cnt = (int64_t)h.root_m * nrhs;
@@ -802,9 +900,8 @@ void apply_waves_nr(const FactorHandle &h, T *ws, T *tb0, T *tb1, int nrhs, int 
   for (int w = nw - 1; w >= 0; --w) {
     const WaveApply &wa = h.waves[w];
     if (!wa.b_count) continue;
-    k_bwd<T, NR, VEC><<<wa.b_count, AT, 0, st>>>(h.d_items + wa.b_first, h.d_nbrs, ws,
-                                                 w == nw - 1 ? (const T *)buf(w) : nullptr, nrhs, j0);
-    count_launch();
+    launch_step(early_start<T, NR>(), k_bwd<T, NR, VEC>, wa.b_count, st, (const ApplyItem *)(h.d_items + wa.b_first),
+                 (const ApplyNbr *)h.d_nbrs, ws, w == nw - 1 ? (const T *)buf(w) : (const T *)nullptr, nrhs, j0);
   }
   HS_CUDA(cudaGetLastError());
 }
