@@ -208,10 +208,12 @@ struct FactorHandle {
 
   // recorded solve graphs and the private stream they are recorded on
   std::vector<GraphEntry> graphs;
+  int applies = 0, pcg_iters = 0;      // since the graphs were last dropped
   cudaStream_t cap_stream = nullptr;
   void drop_graphs() {
     for (GraphEntry &g : graphs) cudaGraphExecDestroy(g.exec);
     graphs.clear();
+    applies = pcg_iters = 0;
   }
 
   // per-level ranks: ranks[li][s] = k or -1

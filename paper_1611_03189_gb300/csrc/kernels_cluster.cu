@@ -99,10 +99,10 @@ __device__ __forceinline__ T partial_total(const T *red) {
   return r[0];
 }
 
-// threads per owned column in the cluster kernel (1 .. 4)
+// threads per owned column in the cluster kernel (1 .. 8)
 __host__ __device__ inline int cl_tpc(int R, int nt) {
   const int q = R > 0 ? nt / R : 1;
-  return q < 1 ? 1 : q > 4 ? 4 : q;
+  return q < 1 ? 1 : q > 8 ? 8 : q;
 }
 
 // One-CTA kernel: 16 columns per warp, two threads (lanes l and l + 16) per

@@ -743,7 +743,6 @@ __global__ void __launch_bounds__(32) k_invit(const EigTask<T> *__restrict__ tas
     const bool on = run < nrun;
     if (on) {
       const T lam = t.lam[q + run];
-      const T *prev = t.Y + (size_t)q * m;
       const uint32_t seed = (uint32_t)((q + run) * 7919 + 17);
       T a = dt[0] - lam, c = m > 1 ? et[0] : T(0);
       for (int i = 0; i + 1 < m; ++i) {
@@ -766,8 +765,11 @@ __global__ void __launch_bounds__(32) k_invit(const EigTask<T> *__restrict__ tas
       }
       iu[(size_t)(m - 1) * st + lane] = T(1) / (fabs(a) < small ? copysign(small, a) : a);
       for (int i = 0; i < m; ++i) y[(size_t)i * st + lane] = (T)hash_unit(seed, (uint32_t)i);
-      T scale = T(1);
-      for (int it = 0; it < 3; ++it) {
+    }
+    T scale = T(1);
+    for (int it = 0; it < 3; ++it) {
+      T big = T(0);
+      if (on) {
         T cur = y[lane] * scale;
 #pragma unroll 4
         for (int i = 0; i + 1 < m; ++i) {
@@ -780,7 +782,7 @@ __global__ void __launch_bounds__(32) k_invit(const EigTask<T> *__restrict__ tas
         }
         T y1 = cur * iu[(size_t)(m - 1) * st + lane], y2 = T(0);
         y[(size_t)(m - 1) * st + lane] = y1;
-        T big = fabs(y1);
+        big = fabs(y1);
 #pragma unroll 4
         for (int i = m - 2; i >= 0; --i) {
           const size_t o = (size_t)i * st + lane;
@@ -790,17 +792,31 @@ __global__ void __launch_bounds__(32) k_invit(const EigTask<T> *__restrict__ tas
           y1 = s;
           big = fmax(big, fabs(s));
         }
-        if (run > 0) {
+      }
+      if (run > 0) {
+        // the whole warp orthogonalises one lane's vector after another
+        // against the cluster's vectors so far (a lane alone walks both with
+        // uncoalesced loads: most of the kernel's time at m = 1340)
+        __syncwarp();
+        for (int s = 0; s < spc; ++s) {
+          if (!__shfl_sync(0xffffffffu, (int)on, s)) continue;
+          const T *prev = t.Y + (size_t)(q0 + s) * m;
           for (int pass = 0; pass < 2; ++pass)
             for (int p = 0; p < run; ++p) {
               const T *v = prev + (size_t)p * m;
               T dot = T(0);
-              for (int i = 0; i < m; ++i) dot += v[i] * y[(size_t)i * st + lane];
-              for (int i = 0; i < m; ++i) y[(size_t)i * st + lane] -= dot * v[i];
+              for (int i = lane; i < m; i += 32) dot = fma(v[i], y[(size_t)i * st + s], dot);
+              for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+              for (int i = lane; i < m; i += 32) y[(size_t)i * st + s] = fma(-dot, v[i], y[(size_t)i * st + s]);
             }
-          big = T(0);
-          for (int i = 0; i < m; ++i) big = fmax(big, fabs(y[(size_t)i * st + lane]));
+          T bg = T(0);
+          for (int i = lane; i < m; i += 32) bg = fmax(bg, fabs(y[(size_t)i * st + s]));
+          for (int o = 16; o > 0; o >>= 1) bg = fmax(bg, __shfl_xor_sync(0xffffffffu, bg, o));
+          if (lane == s) big = bg;
         }
+        __syncwarp();
+      }
+      if (on) {
         // norm, scaling by the largest entry first to keep the sum in range;
         // the next sweep applies the factor as it reads
         const T sc = big > T(0) ? T(1) / big : T(0);
@@ -818,8 +834,9 @@ __global__ void __launch_bounds__(32) k_invit(const EigTask<T> *__restrict__ tas
         const T nrm = sqrt(n0 + n1);
         scale = nrm > T(0) ? sc / nrm : T(0);
       }
-      for (int i = 0; i < m; ++i) y[(size_t)i * st + lane] *= scale;
     }
+    if (on)
+      for (int i = 0; i < m; ++i) y[(size_t)i * st + lane] *= scale;
     __syncwarp();
     // whole vectors, consecutive lanes on consecutive entries
     for (int s = 0; s < spc; ++s) {

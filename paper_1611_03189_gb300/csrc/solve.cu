@@ -1049,6 +1049,8 @@ bool graphs_enabled() {
   return on;
 }
 
+constexpr int kDirectIters = 8;
+
 template <typename F>
 const GraphEntry &graph_for(FactorHandle &h, int key, F &&record) {
   for (const GraphEntry &g : h.graphs)
@@ -1088,8 +1090,10 @@ void run_graph(const GraphEntry &g, cudaStream_t st) {
   count_launch(g.kernels);
 }
 
+// The first apply after a factorization is launched directly: recording and
+// instantiating some 120 launches takes longer than issuing them once.
 void apply_ws(FactorHandle &h, int nrhs, cudaStream_t st) {
-  if (!graphs_enabled()) {
+  if (!graphs_enabled() || h.applies++ == 0) {
     apply_ws_direct(h, nrhs, st);
     return;
   }
@@ -1351,7 +1355,10 @@ int pcg_solve(FactorHandle &h, const double *b, double *x, int nrhs, int64_t ld,
   for (int it = 0;;) {
     // after an odd number of iterations the latest direction is in P1
     double *pold = (it & 1) ? P1 : P0, *pnew = (it & 1) ? P0 : P1;
-    if (graphs_enabled()) {
+    // a factorization's first iterations are launched directly: two recordings
+    // of some 120 launches only pay from a few replays on (24 systems factored
+    // and solved once each: 103 ms with graphs from the start, 93 without)
+    if (graphs_enabled() && h.pcg_iters++ >= kDirectIters) {
       const int key = kPcgGraphKey + 2 * np + (it & 1);
       run_graph(graph_for(h, key, [&](cudaStream_t cs) { body(cs, pold, pnew); }), st);
     } else {
