@@ -99,11 +99,12 @@ __device__ __forceinline__ T partial_total(const T *red) {
   return r[0];
 }
 
-// threads per owned column in the cluster kernel (1 .. 8)
-__host__ __device__ inline int cl_tpc(int R, int nt) {
-  const int q = R > 0 ? nt / R : 1;
-  return q < 1 ? 1 : q > 8 ? 8 : q;
-}
+// cluster kernel: neighbouring columns per warp and pass (FP64 is bound by its
+// FMAs, which fewer columns spread better over the warps), and the row stride
+// in words: the slots rounded up to twice an odd number
+template <typename T>
+constexpr int kClSlots = sizeof(T) == 4 ? 4 : 2;
+__host__ __device__ inline int cl_ld(int R) { return R + (6 - R % 4) % 4; }
 
 // One-CTA kernel: 16 columns per warp, two threads (lanes l and l + 16) per
 // column on alternate rows, so a row stride of 16 (mod 32) words keeps the two
@@ -118,7 +119,7 @@ template <typename T>
 __host__ __device__ inline size_t cl_smem_bytes(int m, int C) {
   if (C == 1) return sizeof(T) * ((size_t)m * cta_ld<T>(m) + 4 * (size_t)m + 48) + 64;
   const int R = (m + C - 1) / C;
-  return sizeof(T) * ((size_t)R * m + 4 * (size_t)m + (size_t)R * (2 + cl_tpc(R, kClThreads)) + 48) + 64;
+  return sizeof(T) * ((size_t)cl_ld(R) * m + 3 * (size_t)m + 2 * (size_t)R) + 64;
 }
 
 // (v, w) of the pending update and v of the current step, per row
@@ -242,60 +243,112 @@ __global__ void __launch_bounds__(NT) k_tri_cta(const GridTri<T> *__restrict__ t
       t.A[(int64_t)i * t.ld + j] = fma(-vpi, pk[j].wp, fma(-wpi, pk[j].vp, W[(size_t)i * ld + j]));
 }
 
+template <typename T>
+struct alignas(2 * sizeof(T)) Pair {
+  T x, y;
+};
+
+// Columns are dealt out cyclically (column i is slot i / C of CTA i % C), so
+// every CTA keeps its share of the trailing matrix to the end.  A warp takes
+// kClSlots neighbouring slots at a time and its lanes the rows: one pass
+// applies the pending update and accumulates p = J v, whose sum over the rows
+// stays in the warp.  The loads of the pending update's and v's rows then serve
+// kClSlots columns, and the row stride (twice an odd number) spreads a warp's
+// rows over the banks.
 template <typename T, int C>
 __global__ void __launch_bounds__(kClThreads) k_tri_cluster(const GridTri<T> *__restrict__ tasks) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  constexpr int nt = kClThreads, NW = nt / 32;
+  constexpr int nt = kClThreads, NW = nt / 32, S = kClSlots<T>;
+  __shared__ T red0[NW], red1[NW], s_x[2], s_r[4];
   cg::cluster_group cluster = cg::this_cluster();
   const int crank = (int)cluster.block_rank();
   const GridTri<T> t = tasks[blockIdx.x / C];
   const int m = t.m;
-  const int R = (m + C - 1) / C;
-  const int c0 = crank * R, c1 = min(m, c0 + R);
+  const int R = (m + C - 1) / C, ld = cl_ld(R);
+  const int ns = crank < m ? (m - 1 - crank) / C + 1 : 0;   // own columns
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int tpc = cl_tpc(R, nt);               // threads per column
-  const int ci = tid % R, part = tid / R;      // own column c0 + ci, rows j = part (mod tpc)
-  struct P2 {
-    T vp, wp;
-  };
-  P2 *pend = reinterpret_cast<P2 *>(smem_raw); // pending update of the previous step
-  T *x = reinterpret_cast<T *>(pend + m);      // column k of J, rows k..
-  T *v = x + m;                                // this step's reflector
-  T *pseg = v + m;                             // p on the own columns, two buffers (step parity)
-  T *psum = pseg + 2 * (size_t)R;              // tpc partial sums per own column
-  T *red0 = psum + (size_t)R * tpc;            // two reduction buffers
-  T *red1 = red0 + NW;
-  T *pvpart = red1 + NW;                       // this CTA's share of p.v, two buffers
-  T *s_r = pvpart + 2;                         // FP64: the reflector's scalars
-  T *slab = s_r + 4;                           // columns c0 .. c1-1 of J, all rows: slab[j R + (i - c0)]
+  T *slab = reinterpret_cast<T *>(smem_raw);                // slot s of row j at slab[j ld + s]
+  Pair<T> *pend = reinterpret_cast<Pair<T> *>(slab + (size_t)m * ld);   // (v, w) of the pending update
+  T *v = reinterpret_cast<T *>(pend + m);                   // this step's reflector
+  T *pseg = v + m;                                          // p on the own columns, two buffers (step parity)
 
-  for (int j = warp; j < m; j += NW)
-    for (int q = lane; q < R; q += 32) slab[(size_t)j * R + q] = c0 + q < c1 ? t.A[(int64_t)j * t.ld + c0 + q] : T(0);
-  for (int j = tid; j < m; j += nt) pend[j] = P2{T(0), T(0)};
+  for (int q = warp; q < m; q += NW)
+    for (int s = lane; s < ld; s += 32)
+      slab[(size_t)q * ld + s] = s < ns ? t.A[(int64_t)q * t.ld + s * C + crank] : T(0);
+  for (int j = tid; j < m; j += nt) pend[j] = Pair<T>{T(0), T(0)};
   cluster.sync();
 
-  // One cluster barrier per step: p and the share of p.v are double-buffered, so
-  // a CTA that runs ahead never overwrites what a slower one still reads, and the
-  // column a step reads is not written in that step.
-  for (int k = 0; k + 2 < m; ++k) {
-    const int owner = k / R;
-    const T *ocol = cluster.map_shared_rank(slab, owner) + (k - owner * R);
-    const P2 pk = pend[k];
-    T s2t = T(0);
-    for (int j = k + tid; j < m; j += nt) {
-      const P2 pj = pend[j];
-      const T a = fma(-pj.vp, pk.wp, fma(-pj.wp, pk.vp, ocol[(size_t)j * R]));
-      x[j] = a;
-      if (j > k) s2t = fma(a, a, s2t);
+  // One cluster barrier per step: p is double-buffered, so a CTA that runs ahead
+  // never overwrites what a slower one still reads, and the row a step reads is
+  // not written from that step on.
+  T tau = T(0);
+  for (int k = 0; k + 1 < m; ++k) {
+    // rows j = k + tid (+ nt): the pending update of step k - 1, and column k
+    // with it applied.  p and the column are read from all CTAs together, the
+    // column as row k of J: one CTA holds the column itself, and all C reading
+    // it there word by word took most of a step (8 us at n = 900, C = 16).
+    T col[2], pj[2], vj[2];
+    T pk = T(0);
+    // block sum over the rows (a warp without any has nothing to add up)
+    auto put_rows = [&](T x, T *red) {
+      if (k + warp * 32 < m) put_partial<T>(x, red);
+      else if (lane == 0) red[warp] = T(0);
+    };
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int j = k + tid + u * nt;
+      col[u] = j < m ? cluster.map_shared_rank(slab, j & (C - 1))[(size_t)k * ld + j / C] : T(0);
+      pj[u] = vj[u] = T(0);
+      if (k > 0 && j < m) {
+        pj[u] = cluster.map_shared_rank(pseg, j & (C - 1))[((k - 1) & 1) * R + j / C];
+        vj[u] = v[j];
+      }
     }
-    put_partial<T>(s2t, red0);
+    if (k > 0) {
+      pk = cluster.map_shared_rank(pseg, k & (C - 1))[((k - 1) & 1) * R + k / C];
+      put_rows(fma(pj[0], vj[0], pj[1] * vj[1]), red1);
+      __syncthreads();
+      T K;
+      if constexpr (sizeof(T) == 4) {
+        K = T(0.5) * tau * partial_total<T, NW>(red1);
+      } else {
+        if (warp == 0) {
+          const T tot = partial_total<T, NW>(red1);
+          if (lane == 0) s_r[3] = T(0.5) * tau * tot;
+        }
+        __syncthreads();
+        K = s_r[3];
+      }
+      pk -= K;                                    // w of row k, where v is 1
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int j = k + tid + u * nt;
+        if (j < m) {
+          pj[u] = fma(-K, vj[u], pj[u]);          // w of row j
+          pend[j] = Pair<T>{vj[u], pj[u]};
+          col[u] = fma(-vj[u], pk, col[u] - pj[u]);
+        }
+      }
+    }
+    if (k + 2 >= m) {                             // the trailing 2 x 2 block, lower triangle
+      __syncthreads();
+      for (int j = max(m - 2, 0); j < m; ++j)
+        if ((j & (C - 1)) == crank && j + tid < m) {
+          const int i = j + tid;
+          const Pair<T> f = pend[i], o = pend[j];
+          t.A[(int64_t)i * t.ld + j] = fma(-f.x, o.y, fma(-f.y, o.x, slab[(size_t)i * ld + j / C]));
+        }
+      break;
+    }
+    if (tid < 2) s_x[tid] = col[0];               // entries k and k + 1
+    put_rows(fma(col[1], col[1], tid > 0 ? col[0] * col[0] : T(0)), red0);
     __syncthreads();
-    T scale, tau, beta, lo;
+    T scale, beta, lo;
     if constexpr (sizeof(T) == 4) {
-      reflector(partial_total<T, NW>(red0), x[k + 1], scale, tau, beta, lo);
+      reflector(partial_total<T, NW>(red0), s_x[1], scale, tau, beta, lo);
     } else {
       if (warp == 0) {
-        reflector(partial_total<T, NW>(red0), x[k + 1], scale, tau, beta, lo);
+        reflector(partial_total<T, NW>(red0), s_x[1], scale, tau, beta, lo);
         if (lane == 0) {
           s_r[0] = scale;
           s_r[1] = tau;
@@ -308,88 +361,70 @@ __global__ void __launch_bounds__(kClThreads) k_tri_cluster(const GridTri<T> *__
       beta = s_r[2];
       lo = T(0);
     }
-    for (int j = k + 1 + tid; j < m; j += nt) {
-      const T vj = (j == k + 1) ? T(1) : x[j] * scale;
-      v[j] = vj;
-      if (crank == owner && j >= k + 2) t.A[(int64_t)k * t.ld + j] = vj;   // reflector k in row k
+    const bool owner = (k & (C - 1)) == crank;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int j = k + tid + u * nt;
+      if (j > k && j < m) {
+        const T x = j == k + 1 ? T(1) : col[u] * scale;
+        v[j] = x;
+        if (owner && j >= k + 2) t.A[(int64_t)k * t.ld + j] = x;   // reflector k in row k
+      }
     }
-    if (crank == owner && tid == 0) {
-      t.d[k] = (double)x[k];
+    if (owner && tid == 0) {
+      t.d[k] = (double)col[0];
       t.e[k] = (double)beta + (double)lo;
       t.tau[k] = tau;
     }
     __syncthreads();
-    // the own columns i > k: pending update of rows j > k, then
-    // p_i = tau sum_j J_ji v_j (rows split over tpc threads per column)
+    // the own columns i > k: pending update of rows j > k, then p_i = tau sum_j J_ji v_j
     T *pcur = pseg + (k & 1) * R;
-    const int i = c0 + ci;
-    if (part < tpc && i < c1 && i > k) {
-      const P2 own = pend[i];
-      T s[4] = {T(0), T(0), T(0), T(0)};
-      int j = k + 1 + part;
-      for (; j + 3 * tpc < m; j += 4 * tpc) {
-        T y[4];
-        P2 f[4];
-        T vj[4];
+    const int live = k >= crank ? (k - crank) / C + 1 : 0;         // first slot with i > k
+    for (int g = live / S + warp; g * S < ns; g += NW) {
+      const int s0 = g * S;
+      Pair<T> own[S];
+      bool on[S];
+      T acc[S];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          f[u] = pend[j + u * tpc];
-          vj[u] = v[j + u * tpc];
-          y[u] = slab[(size_t)(j + u * tpc) * R + ci];
-        }
+      for (int u = 0; u < S; ++u) {
+        on[u] = s0 + u >= live && s0 + u < ns;
+        own[u] = on[u] ? pend[(s0 + u) * C + crank] : Pair<T>{T(0), T(0)};
+        acc[u] = T(0);
+      }
+#pragma unroll 4
+      for (int j = k + 1 + lane; j < m; j += 32) {
+        const Pair<T> f = pend[j];
+        const T vv = v[j];
+        Pair<T> *row = reinterpret_cast<Pair<T> *>(slab + (size_t)j * ld + s0);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          y[u] = fma(-f[u].vp, own.wp, fma(-f[u].wp, own.vp, y[u]));
-          slab[(size_t)(j + u * tpc) * R + ci] = y[u];
-          s[u] = fma(y[u], vj[u], s[u]);
+        for (int u = 0; u < S; u += 2) {
+          if (!on[u] && !on[u + 1]) continue;
+          Pair<T> y = row[u / 2];
+          y.x = fma(-f.x, own[u].y, fma(-f.y, own[u].x, y.x));
+          y.y = fma(-f.x, own[u + 1].y, fma(-f.y, own[u + 1].x, y.y));
+          row[u / 2] = y;
+          acc[u] = fma(y.x, vv, acc[u]);
+          acc[u + 1] = fma(y.y, vv, acc[u + 1]);
         }
       }
-      for (; j < m; j += tpc) {
-        const P2 f = pend[j];
-        const T y = fma(-f.vp, own.wp, fma(-f.wp, own.vp, slab[(size_t)j * R + ci]));
-        slab[(size_t)j * R + ci] = y;
-        s[0] = fma(y, v[j], s[0]);
+      // sums over the lanes, half of the columns handed over at each step
+      int mine = 0;
+#pragma unroll
+      for (int w = S / 2, o = 16; w > 0; w /= 2, o /= 2) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int u = 0; u < w; ++u) {
+          const T keep = up ? acc[u + w] : acc[u], give = up ? acc[u] : acc[u + w];
+          acc[u] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+        if (up) mine += w;
       }
-      psum[part * R + ci] = (s[0] + s[1]) + (s[2] + s[3]);
+#pragma unroll
+      for (int o = 16 / S; o > 0; o >>= 1) acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
+      if ((lane & (32 / S - 1)) == 0 && s0 + mine >= live && s0 + mine < ns) pcur[s0 + mine] = tau * acc[0];
     }
-    __syncthreads();
-    T pvt = T(0);
-    if (part == 0 && i < c1 && i > k) {
-      T acc = T(0);
-      for (int q = 0; q < tpc; ++q) acc += psum[q * R + ci];
-      const T p = tau * acc;
-      pcur[ci] = p;
-      pvt = p * v[i];
-    }
-    put_partial<T>(pvt, red1);
-    __syncthreads();
-    if (warp == 0) {
-      const T tot = partial_total<T, NW>(red1);
-      if (lane == 0) pvpart[k & 1] = tot;
-    }
-    cluster.sync();   // every CTA's p and share of p.v are visible; every walk of step k is done
-    T pv = T(0);
-    if (sizeof(T) == 4 || warp == 0)
-      for (int c = 0; c < C; ++c) pv += cluster.map_shared_rank(pvpart, c)[k & 1];
-    T K = T(0.5) * tau * pv;
-    if constexpr (sizeof(T) == 8) {
-      if (tid == 0) s_r[3] = K;
-      __syncthreads();
-      K = s_r[3];
-    }
-    for (int j = k + 1 + tid; j < m; j += nt) {
-      const int oj = j / R;
-      const T pj = cluster.map_shared_rank(pseg, oj)[(k & 1) * R + j - oj * R];
-      pend[j] = P2{v[j], fma(-K, v[j], pj)};   // the next pending update
-    }
-    __syncthreads();
+    cluster.sync();   // every CTA's p is visible; every walk of step k is done
   }
-  // the last pending update on the trailing 2 x 2 block, lower triangle,
-  // written out by the owners of its columns
-  for (int j = max(c0, m - 2) + tid; j < c1; j += nt)
-    for (int i = j; i < m; ++i)
-      t.A[(int64_t)i * t.ld + j] =
-          fma(-pend[i].vp, pend[j].wp, fma(-pend[i].wp, pend[j].vp, slab[(size_t)i * R + (j - c0)]));
   // no CTA may leave while others still read its shared memory
   cluster.sync();
 }
@@ -467,8 +502,8 @@ int tri_max_m(int q) {
     for (int c = 0; c < kTriClasses; ++c) {
       const int C = 1 << c;
       int mm = 0;
-      // (one CTA: 16 columns per warp; a cluster: at most one owned column per thread)
-      while (cl_smem_bytes<T>(mm + 1, C) <= room[c] && (c == 0 ? mm + 1 <= 256 : (mm + C) / C <= kClThreads)) ++mm;
+      // (one CTA: 16 columns per warp; a cluster: two rows per thread)
+      while (cl_smem_bytes<T>(mm + 1, C) <= room[c] && mm + 1 <= (c == 0 ? 256 : 2 * kClThreads)) ++mm;
       table[dev][c] = mm;
     }
     ready[dev] = true;
@@ -498,7 +533,7 @@ int tri_class(int m) {
   int first = 0;
   if (mode == 0) {
     if (sizeof(T) == 8 && m > 112)
-      first = 3;
+      first = m > 160 ? 4 : 3;
     else if (m > tri_max_m<T>(0))
       first = 2;
   }
