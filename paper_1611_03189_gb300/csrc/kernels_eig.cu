@@ -83,30 +83,36 @@ __device__ __forceinline__ float hash_unit(uint32_t a, uint32_t b) {
 // moves a computed count no more than the rounding of the recurrence itself
 // does.  The rank count divides exactly, in FP64.
 __device__ __forceinline__ float place_div(float a, float b) { return __fdividef(a, b); }
-// FP64: the hardware's reciprocal seed (20 bits) and two Newton steps
-// y <- y + y (1 - b y), good to the last place or two, at 6 of the FP64
-// instructions whose rate bounds these loops, against about twice that for
-// the exactly rounded quotient
+// FP64: the hardware's reciprocal seed y (20 bits) and one step of third order,
+// y + y (r + r^2) with r = 1 - b y (the series of 1 / (1 - r)), which leaves
+// r^3 = 2^-60: 3 of the FP64 instructions whose rate bounds these loops
 __device__ __forceinline__ double place_div(double a, double b) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
-  y = fma(y, fma(-b, y, 1.0), y);
-  y = fma(y, fma(-b, y, 1.0), y);
-  return a * y;
+  const double r = fma(-b, y, 1.0);
+  return a * fma(y, fma(r, r, r), y);
 }
+// sign and magnitude tests of the Sturm pivots; in FP64 by the high word
+// (comparisons issue on the FP64 pipe too)
+__device__ __forceinline__ bool pivot_tiny(float q, float pivmin) { return fabs(q) < pivmin; }
+__device__ __forceinline__ bool pivot_tiny(double q, double pivmin) {
+  return (__double2hiint(q) & 0x7fffffff) < __double2hiint(pivmin);
+}
+__device__ __forceinline__ bool pivot_pos(float q) { return q > 0.f; }
+__device__ __forceinline__ bool pivot_pos(double q) { return __double2hiint(q) >= 0; }   // (not zero: not tiny)
 
 // number of eigenvalues above sigma of the tridiagonal with diagonal d and
 // squared sub-diagonal e2 (e2[i] couples i - 1 and i; e2[0] unused)
 template <typename R>
 __device__ __forceinline__ int count_above(const R *d, const R *e2, int m, R sigma, R pivmin) {
   R q = d[0] - sigma;
-  if (fabs(q) < pivmin) q = -pivmin;
-  int c = q > R(0);
+  if (pivot_tiny(q, pivmin)) q = -pivmin;
+  int c = pivot_pos(q);
 #pragma unroll 4
   for (int i = 1; i < m; ++i) {
     q = (d[i] - sigma) - place_div(e2[i], q);
-    if (fabs(q) < pivmin) q = -pivmin;
-    c += q > R(0);
+    if (pivot_tiny(q, pivmin)) q = -pivmin;
+    c += pivot_pos(q);
   }
   return c;
 }
@@ -114,7 +120,9 @@ __device__ __forceinline__ int count_above(const R *d, const R *e2, int m, R sig
 // positive eigenvalues of the symmetric k x k matrix S (ld N)
 template <typename R, int N>
 __device__ __forceinline__ int count_positive(R (&S)[N][N], int k) {
-  if constexpr (N <= 2) {
+  if constexpr (N == 1) {
+    return S[0][0] > R(0);
+  } else if constexpr (N == 2) {
     if (k == 0) return 0;
     if (k == 1) return S[0][0] > R(0);
     const R det = S[0][0] * S[1][1] - S[1][0] * S[1][0];
@@ -171,12 +179,12 @@ __device__ __forceinline__ int count_above_gc(const R *d, const R *e, const R *e
 #pragma unroll 2
   for (int i = 0; i < m; ++i) {
     R q = (d[i] - sigma) - e2[i] * inv;   // e2[0] = 0
-    if (fabs(q) < pivmin) q = -pivmin;
-    c += q > R(0);
+    if (pivot_tiny(q, pivmin)) q = -pivmin;
+    c += pivot_pos(q);
     inv = place_div(R(1), q);
 #pragma unroll
     for (int a = 0; a < KB; ++a)
-      if (KB <= 2 || a < k1) w[a] = (a < k1 ? Z[(size_t)a * ldz + i] : R(0)) - l * w[a];
+      if (KB <= 2 || a < k1) w[a] = (KB == 1 || a < k1 ? Z[(size_t)a * ldz + i] : R(0)) - l * w[a];
 #pragma unroll
     for (int a = 0; a < KB; ++a)
 #pragma unroll
@@ -509,7 +517,9 @@ __global__ void __launch_bounds__(kRankThreads) k_rank(const TruncTask<T> *__res
           c = count_above<float>(df, e2f, m, sig, pivf);
         else if (wide_global)
           c = count_above_gc_wide<float>(df, ef, e2f, m, (const float *)(const void *)L.LS, m, k1, s_cf, sig, pivf);
-        else if (k1 <= 2)
+        else if (k1 == 1)
+          c = count_above_gc<float, 1>(df, ef, e2f, m, zf, (int)mm, k1, s_cf, sig, pivf);
+        else if (k1 == 2)
           c = count_above_gc<float, 2>(df, ef, e2f, m, zf, (int)mm, k1, s_cf, sig, pivf);
         else
           c = count_above_gc_wide<float>(df, ef, e2f, m, zf, (int)mm, k1, s_cf, sig, pivf);
@@ -528,8 +538,9 @@ __global__ void __launch_bounds__(kRankThreads) k_rank(const TruncTask<T> *__res
           if (k1 == 0) return count_above<double>(d, e2, m, sig, piv) >= 1;
           const double *z = zs ? zd : (const double *)L.LS;   // (beyond shared memory: scaled in place below)
           const int ldz = zs ? (int)mm : m;
-          return (k1 <= 2 ? count_above_gc<double, 2>(d, ed, e2, m, z, ldz, k1, s_ct, sig, piv)
-                          : count_above_gc_wide<double>(d, ed, e2, m, z, ldz, k1, s_ct, sig, piv)) >= 1;
+          return (k1 == 1   ? count_above_gc<double, 1>(d, ed, e2, m, z, ldz, k1, s_ct, sig, piv)
+                  : k1 == 2 ? count_above_gc<double, 2>(d, ed, e2, m, z, ldz, k1, s_ct, sig, piv)
+                            : count_above_gc_wide<double>(d, ed, e2, m, z, ldz, k1, s_ct, sig, piv)) >= 1;
         };
         double l = lmax * (1.0 - 7.6e-6), h = lmax * (1.0 + 7.6e-6);   // 64 u of FP32
         const int miss = wide_global ? 2 : section<double, 32>(l, h, lane, true, above);
@@ -599,7 +610,8 @@ __global__ void __launch_bounds__(kRankThreads) k_rank(const TruncTask<T> *__res
 // first and confirms and refines that bracket in FP64.
 // ---------------------------------------------------------------------------
 constexpr int kEigThreads = 128;
-__host__ __device__ inline int eig_lanes(int m) { return m < 128 ? 8 : 32; }
+template <typename T>
+__host__ __device__ inline int eig_lanes(int m) { return sizeof(T) == 8 || m < 128 ? 8 : 32; }
 
 template <typename T>
 __host__ __device__ inline size_t eigval_smem_bytes(int m) {
@@ -658,7 +670,7 @@ __global__ void __launch_bounds__(kEigThreads) k_eigval(const EigTask<T> *__rest
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const EigTask<T> t = tasks[task_of(tasks, ntasks, blockIdx.x)];
   const int m = t.m;
-  const int lanes = eig_lanes(m);
+  const int lanes = eig_lanes<T>(m);
   const int first = (blockIdx.x - t.blk0) * (kEigThreads / lanes);
   if (first >= t.sc[1]) return;
   double *d = (double *)smem_raw, *e2 = d + m;
@@ -1243,7 +1255,7 @@ void launch_rank(const TruncTask<T> *d_tasks, int ntasks, int *d_k, int variant,
 
 template <typename T>
 int eigval_blocks(int m) {
-  const int per = kEigThreads / eig_lanes(m);
+  const int per = kEigThreads / eig_lanes<T>(m);
   return (m + per - 1) / per;
 }
 
