@@ -11,6 +11,7 @@
 //   k_trunc      truncation of the well-separated block (Sec. 3.2 eq.
 //                local_compression, Sec. 6 GC basis), one CTA per super node:
 //                cyclic Jacobi eigen-solves of the Gram matrix A_sw A_sw^T.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -294,19 +295,29 @@ __device__ __forceinline__ float inv_sqrt(float d) {
   const float y = rsqrtf(d);
   return y * fmaf(-0.5f * d * y, y, 1.5f);
 }
-__device__ __forceinline__ double inv_sqrt(double d) { return rsqrt(d); }
+// (FP64: the hardware's seed y, 20 bits, and the series of (1 - r)^-1/2 to r^2,
+// r = 1 - d y^2: five FP64 instructions on the pivots' serial chain)
+__device__ __forceinline__ double inv_sqrt(double d) {
+  if (d < 1e-290) return rsqrt(d);
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+  const double r = fma(-d * y, y, 1.0);
+  return fma(y, r * fma(r, 0.375, 0.5), y);
+}
 
-// One warp: D = L^-1 of the diagonal block at j0 (jb <= 16 columns), in its
-// place with zeros above the diagonal; *fail = first failing pivot + 1.
+// One warp: D = L^-1 of the diagonal block at row j0, column j0c of W (jb <= 16
+// columns, j0 the first in the matrix), in its place with zeros above the diagonal;
+// *fail = first failing pivot + 1.
 template <typename T>
-__device__ __forceinline__ void chol_diag(T *W, int ld, int j0, int jb, int *fail) {
-  const int lane = threadIdx.x & 31, i = lane & 15;   // row of A, then column of D (lanes 16.. repeat)
-  T r[kCholNb], x[kCholNb];
+__device__ __forceinline__ void chol_diag(T *W, int ld, int j0, int j0c, int jb, int *fail) {
+  // lanes 0 .. 15: row i of A, becoming L's; lanes 16 .. 31: column i of D.  Both
+  // are scaled by the pivot's inverse root and updated by L's column j.
+  const int lane = threadIdx.x & 31, i = lane & 15;
+  const bool inverse = lane >= 16;
+  T r[kCholNb];
 #pragma unroll
-  for (int c = 0; c < kCholNb; ++c) {
-    r[c] = (i < jb && c <= i) ? W[(size_t)(j0 + i) * ld + j0 + c] : (c == i ? T(1) : T(0));
-    x[c] = c == i ? T(1) : T(0);
-  }
+  for (int c = 0; c < kCholNb; ++c)
+    r[c] = !inverse && i < jb && c <= i ? W[(size_t)(j0 + i) * ld + j0c + c] : (c == i ? T(1) : T(0));
   int bad = 0;
 #pragma unroll
   for (int j = 0; j < kCholNb; ++j) {
@@ -315,33 +326,33 @@ __device__ __forceinline__ void chol_diag(T *W, int ld, int j0, int jb, int *fai
       if (!bad) bad = j0 + j + 1;
       d = T(1);
     }
-    const T inv = inv_sqrt(d);
-    const T l = r[j] * inv;   // L_ij
-    x[j] *= inv;              // D_ji
+    r[j] *= inv_sqrt(d);   // L_ij, D_ji
 #pragma unroll
-    for (int c = j + 1; c < kCholNb; ++c) {
-      const T lc = __shfl_sync(0xffffffffu, l, c);
-      r[c] = fma(-l, lc, r[c]);
-      x[c] = fma(-lc, x[j], x[c]);
-    }
+    for (int c = j + 1; c < kCholNb; ++c) r[c] = fma(-r[j], __shfl_sync(0xffffffffu, r[j], c), r[c]);
   }
   __syncwarp();
-  if (lane < jb) {
+  if (inverse && i < jb) {
 #pragma unroll
     for (int c = 0; c < kCholNb; ++c)
-      if (c < jb) W[(size_t)(j0 + c) * ld + j0 + lane] = x[c];
+      if (c < jb) W[(size_t)(j0 + c) * ld + j0c + i] = r[c];
   }
   if (bad && lane == 0) *fail = bad;
   __syncwarp();
 }
 
-// Rank-16 update of the tile at rows i0 .. i0 + 31, columns c0 .. c0 + 15.
+struct NoShift {
+  __device__ __forceinline__ operator int() const { return 0; }
+};
+
+// Rank-16 update of the tile at rows i0 .. i0 + 31, columns c0 .. c0 + 15,
+// which W holds from its column c0 + shift on (a constant 0 in one CTA: a
+// variable there costs registers and a tenth of the kernel).
 // kind 0: W -= P_i P_c^T; 1: W += P_i X_b; 2: W = P_i X_b (X_b: rows j0 ..)
-template <typename T>
-__device__ __forceinline__ void chol_tile(T *W, int ld, const T *P, int i0, int c0, int j0, int m, int kind) {
+template <typename T, typename Shift>
+__device__ __forceinline__ void chol_tile(T *W, int ld, const T *P, int i0, int c0, Shift shift, int j0, int m, int kind) {
   constexpr int V = 16 / (int)sizeof(T), PS = chol_ps<T>();
   const int lane = threadIdx.x & 31;
-  const int ib = i0 + (lane & 7), cb = c0 + 4 * (lane >> 3);
+  const int ib = i0 + (lane & 7), cg = c0 + 4 * (lane >> 3), cb = cg + shift;
   T acc[4][4];
 #pragma unroll
   for (int r = 0; r < 4; ++r)
@@ -353,7 +364,7 @@ __device__ __forceinline__ void chol_tile(T *W, int ld, const T *P, int i0, int 
   if (kind == 0) {
     const T *pb[4];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) pb[c] = P + (size_t)min(cb + c, m - 1) * PS;
+    for (int c = 0; c < 4; ++c) pb[c] = P + (size_t)min(cg + c, m - 1) * PS;
 #pragma unroll
     for (int k = 0; k < kCholNb; k += V) {
       T a[4][V], b[4][V];
@@ -424,7 +435,7 @@ __global__ void __launch_bounds__(NT) k_chol_inv(const CholTask<T> *__restrict__
   for (int i = warp; i < m; i += NW)
     for (int c = lane; c < ld; c += 32) W[(size_t)i * ld + c] = c <= i ? t.A[(int64_t)i * t.lda + c] : T(0);
   __syncthreads();
-  if (warp == 0) chol_diag<T>(W, ld, 0, min(kCholNb, m), &s_fail);
+  if (warp == 0) chol_diag<T>(W, ld, 0, 0, min(kCholNb, m), &s_fail);
   for (int j0 = 0; j0 < m; j0 += kCholNb) {
     __syncthreads();   // D_b and the update of the step before are complete
     if (s_fail) break;
@@ -465,9 +476,9 @@ __global__ void __launch_bounds__(NT) k_chol_inv(const CholTask<T> *__restrict__
     __syncthreads();
     if (rest == 0) break;
     if (warp == 0) {
-      chol_tile<T>(W, ld, P, j1, j1, j0, m, 0);
+      chol_tile<T>(W, ld, P, j1, j1, NoShift(), j0, m, 0);
       __syncwarp();
-      chol_diag<T>(W, ld, j1, min(kCholNb, m - j1), &s_fail);
+      chol_diag<T>(W, ld, j1, j1, min(kCholNb, m - j1), &s_fail);
     } else {
       // all other tiles, dealt out to the other warps in turn
       const int nic = j1 / kCholNb, nct = (rest + kCholNb - 1) / kCholNb;
@@ -478,9 +489,9 @@ __global__ void __launch_bounds__(NT) k_chol_inv(const CholTask<T> *__restrict__
           if (rt == 0 && ct == nic) continue;   // warp 0's
           if (turn == warp) {
             if (ct < nic)
-              chol_tile<T>(W, ld, P, j1 + 32 * rt, kCholNb * ct, j0, m, ct == nic - 1 ? 2 : 1);
+              chol_tile<T>(W, ld, P, j1 + 32 * rt, kCholNb * ct, NoShift(), j0, m, ct == nic - 1 ? 2 : 1);
             else
-              chol_tile<T>(W, ld, P, j1 + 32 * rt, j1 + kCholNb * (ct - nic), j0, m, 0);
+              chol_tile<T>(W, ld, P, j1 + 32 * rt, j1 + kCholNb * (ct - nic), NoShift(), j0, m, 0);
           }
           turn = turn + 1 == NW ? 1 : turn + 1;
         }
@@ -493,6 +504,157 @@ __global__ void __launch_bounds__(NT) k_chol_inv(const CholTask<T> *__restrict__
     for (int i = warp; i < m; i += NW)
       for (int c = lane; c < m; c += 32) t.Linv[(int64_t)i * t.ldl + c] = c <= i ? W[(size_t)i * ld + c] : T(0);
   if (tid == 0) status[t.status_idx] = st;
+}
+
+// The same factorization by a cluster of kCholC CTAs, for FP64 matrices from
+// kCholClusterMin on, where one SM's FP64 rate (2 FMAs a cycle) bounds it.
+// Blocks of 16 columns are dealt out cyclically and stay with their CTA, first
+// as trailing columns, then as the inverse's.  A step needs D_b and the panel
+// P_b alone from elsewhere: their owner writes them into every CTA's shared
+// memory, so a step has one cluster barrier.  The owner of block b + 1 updates
+// that block first, and its diagonal block is inverted beside its other tiles.
+// Every element's arithmetic is k_chol_inv's.
+constexpr int kCholC = 4, kCholClusterMin = 96, kCholClThreads = 256;
+
+__host__ __device__ inline int chol_cl_ld(int m) {
+  const int nblk = (m + kCholNb - 1) / kCholNb;
+  return kCholNb * ((nblk + kCholC - 1) / kCholC) + 2;
+}
+template <typename T>
+__host__ __device__ inline size_t chol_cl_smem_bytes(int m) {
+  return sizeof(T) * ((size_t)m * (chol_cl_ld(m) + 2 * chol_ps<T>()) + 2 * kCholNb * kCholNb);
+}
+
+template <typename T>
+__global__ void __cluster_dims__(kCholC, 1, 1) __launch_bounds__(kCholClThreads)
+    k_chol_cluster(const CholTask<T> *__restrict__ tasks, int *__restrict__ status) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int s_fail, s_failed[2];   // found here; published with D_b (step parity)
+  constexpr int V = 16 / (int)sizeof(T), PS = chol_ps<T>(), NT = kCholClThreads, NW = NT / 32;
+  cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+  const int rank = (int)cluster.block_rank();
+  const CholTask<T> t = tasks[blockIdx.x / kCholC];
+  const int m = t.m, ld = chol_cl_ld(m), nblk = (m + kCholNb - 1) / kCholNb;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  T *W = reinterpret_cast<T *>(smem_raw);          // own block q: block rank + kCholC q, from column 16 q on
+  T *Pb = W + (size_t)m * ld, *Db = Pb + 2 * (size_t)m * PS;   // two buffers each (step parity)
+  if (m == 0) {
+    if (tid == 0 && rank == 0) status[t.status_idx] = 0;
+    return;
+  }
+  if (tid == 0) s_fail = 0;
+  for (int i = warp; i < m; i += NW)
+    for (int c = lane; c < ld; c += 32) {
+      const int g = kCholNb * (rank + kCholC * (c / kCholNb)) + c % kCholNb;
+      W[(size_t)i * ld + c] = g <= i ? t.A[(int64_t)i * t.lda + g] : T(0);
+    }
+  cluster.sync();   // (every CTA runs before any writes to it)
+  // D_b (in place in the own block) and its panel to every CTA
+  auto publish = [&](int b) {
+    const int j0 = b * kCholNb, j1 = min(j0 + kCholNb, m), lc = kCholNb * (b / kCholC), par = b & 1;
+    const T *D = W + (size_t)j0 * ld + lc;
+    for (int q = tid; q < kCholNb * kCholNb; q += NT) {
+      const int k = q / kCholNb, c = q % kCholNb;
+      const T x = j0 + k < m ? D[(size_t)k * ld + c] : T(0);
+      for (int r = 0; r < kCholC; ++r) cluster.map_shared_rank(Db, r)[par * kCholNb * kCholNb + q] = x;
+    }
+    // a row's entries 0 .. 10 and 11 .. 15 take about the same FMAs: a warp each
+    auto panel = [&](auto k0, auto k1, int first) {
+      constexpr int K0 = k0.value, K1 = k1.value;
+      for (int i = j1 + first; i < m; i += NT / 2) {
+        const T *w = W + (size_t)i * ld + lc;
+        T v[kCholNb], o[kCholNb];
+#pragma unroll
+        for (int k = 0; k < kCholNb && k < K1; k += V) ld16(w + k, v + k);
+#pragma unroll
+        for (int k = K0; k < K1; ++k) {
+          T s = T(0);
+#pragma unroll
+          for (int p = 0; p <= k; ++p) s = fma(D[(size_t)k * ld + p], v[p], s);
+          o[k] = s;
+        }
+        for (int r = 0; r < kCholC; ++r) {
+          T *P = cluster.map_shared_rank(Pb, r) + ((size_t)par * m + i) * PS;
+#pragma unroll
+          for (int k = K0; k < K1; ++k) P[k] = o[k];
+        }
+      }
+    };
+    const int first = (warp >> 1) * 32 + lane;
+    if (warp & 1)
+      panel(std::integral_constant<int, 11>(), std::integral_constant<int, kCholNb>(), first);
+    else
+      panel(std::integral_constant<int, 0>(), std::integral_constant<int, 11>(), first);
+    if (tid < kCholC) cluster.map_shared_rank(s_failed, tid)[par] = s_fail;
+  };
+  if (rank == 0) {
+    if (warp == 0) chol_diag<T>(W, ld, 0, 0, min(kCholNb, m), &s_fail);
+    __syncthreads();
+    publish(0);
+  }
+  int fail = 0;
+  for (int b = 0; b < nblk; ++b) {
+    cluster.sync();   // D_b, P_b are here; every CTA is done with step b - 1
+    fail = s_failed[b & 1];
+    if (fail) break;
+    const int j0 = b * kCholNb, j1 = min(j0 + kCholNb, m), jb = j1 - j0, rest = m - j1;
+    const T *P = Pb + (size_t)(b & 1) * m * PS, *D = Db + (b & 1) * kCholNb * kCholNb;
+    // row block b of the inverse, own columns (blocks before b)
+    const int nq = b > rank ? (b - rank + kCholC - 1) / kCholC : 0;   // own blocks before b
+    for (int c = tid; c < kCholNb * nq; c += NT) {
+      T *w = W + (size_t)j0 * ld + c;
+      T v[kCholNb];
+#pragma unroll
+      for (int k = 0; k < kCholNb; ++k) v[k] = k < jb ? -w[(size_t)k * ld] : T(0);
+#pragma unroll
+      for (int k = 0; k < kCholNb; ++k) {
+        T s = T(0);
+#pragma unroll
+        for (int p = 0; p <= k; ++p) s = fma(D[k * kCholNb + p], v[p], s);
+        if (k < jb) w[(size_t)k * ld] = s;
+      }
+    }
+    if (rest == 0) break;
+    __syncthreads();
+    const int nrt = (rest + 31) / 32, nown = rank < nblk ? (nblk - rank + kCholC - 1) / kCholC : 0;
+    const bool next = (b + 1) % kCholC == rank;
+    const int qn = next ? (b + 1) / kCholC : -1;
+    if (next) {
+      for (int rt = warp; rt < nrt; rt += NW)
+        chol_tile<T>(W, ld, P, j1 + 32 * rt, j1, kCholNb * qn - j1, j0, m, 0);
+      __syncthreads();
+      if (warp == 0)
+        chol_diag<T>(W, ld, j1, kCholNb * qn, min(kCholNb, m - j1), &s_fail);
+    }
+    // the other own tiles (the owner of the next block's warp 0 has its diagonal block)
+    if (!next || warp != 0) {
+      const int w0 = next ? 1 : 0;
+      int turn = w0;
+      for (int q = 0; q < nown; ++q) {
+        if (q == qn) continue;
+        const int blk = rank + kCholC * q, c0 = kCholNb * blk;
+        for (int rt = 0; rt < nrt; ++rt) {
+          const int i0 = j1 + 32 * rt;
+          if (blk > b && i0 + 31 < c0) continue;   // above the diagonal
+          if (turn == warp)
+            chol_tile<T>(W, ld, P, i0, c0, kCholNb * q - c0, j0, m, blk > b ? 0 : blk == b ? 2 : 1);
+          turn = turn + 1 == NW ? w0 : turn + 1;
+        }
+      }
+    }
+    if (next) {
+      __syncthreads();
+      publish(b + 1);
+    }
+  }
+  __syncthreads();
+  if (fail == 0)
+    for (int i = warp; i < m; i += NW)
+      for (int c = lane; c < ld; c += 32) {
+        const int g = kCholNb * (rank + kCholC * (c / kCholNb)) + c % kCholNb;
+        if (c < ld - 2 && g < m) t.Linv[(int64_t)i * t.ldl + g] = g <= i ? W[(size_t)i * ld + c] : T(0);
+      }
+  if (tid == 0 && rank == 0) status[t.status_idx] = fail;
 }
 
 // ---------------------------------------------------------------------------
@@ -887,7 +1049,7 @@ static __global__ void k_status_merge(const StatusMerge *__restrict__ t, int n) 
 
 template <typename T>
 int chol_smem_cap() {
-  return sizeof(T) == 8 ? 160 : 224;
+  return sizeof(T) == 8 ? 256 : 224;
 }
 
 template <typename T, int NT>
@@ -897,6 +1059,9 @@ static void launch_chol_nt(const CholTask<T> *d_tasks, int ntasks, int *d_status
   k_chol_inv<T, NT><<<ntasks, NT, sm, st>>>(d_tasks, d_status);
 }
 
+// FP64 from kCholClusterMin on: k_chol_cluster (m = 150 to 160: 0.60 ms in one
+// CTA, about 0.28 in four; its limit of 256 also spares nodes up to there the
+// blocked path).  Below, the diagonal blocks' serial chain is what counts.
 // Threads by the largest matrix of the launch: the update's tiles (about
 // m^2 / 1024 a step) keep that many warps busy; a matrix's arithmetic does not
 // depend on them.
@@ -904,12 +1069,23 @@ template <typename T>
 void launch_chol_inv(const CholTask<T> *d_tasks, int ntasks, int *d_status, int max_m,
                      cudaStream_t st) {
   if (ntasks == 0) return;
-  if (max_m <= 48)
+  bool cluster = false;
+  if constexpr (sizeof(T) == 8) {
+    cluster = max_m > kCholClusterMin;
+    if (cluster) {
+      const size_t sm = chol_cl_smem_bytes<T>(max_m);
+      check_dynamic_smem(sm, allow_max_dynamic_smem<&k_chol_cluster<T>>(), "k_chol_cluster");
+      k_chol_cluster<T><<<ntasks * kCholC, kCholClThreads, sm, st>>>(d_tasks, d_status);
+    }
+  }
+  if (cluster) {
+  } else if (max_m <= 48) {
     launch_chol_nt<T, 128>(d_tasks, ntasks, d_status, max_m, st);
-  else if (max_m <= 112)
+  } else if (max_m <= 112) {
     launch_chol_nt<T, 256>(d_tasks, ntasks, d_status, max_m, st);
-  else
+  } else {
     launch_chol_nt<T, 512>(d_tasks, ntasks, d_status, max_m, st);
+  }
   count_launch();
   HS_CUDA(cudaGetLastError());
 }

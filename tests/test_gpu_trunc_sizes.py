@@ -5,8 +5,9 @@ A strip of 4 a x b unknowns in eight leaves has four super nodes of a b unknowns
 at its first level; eliminating two of them couples the other two, so at least
 one node of exactly m = a b unknowns is compressed.  The sizes lie on both
 sides of the limits of the Jacobi path, of the lanes per eigenvalue, of the
-registers per column of the reflector products and of their threads, and of
-the 16-column blocks of the Cholesky.  Bars as in the parity tests: equal
+registers per column of the reflector products and of their threads, of the
+16-column blocks of the Cholesky and of its clusters, and of the clusters of
+the FP64 tridiagonalisation.  Bars as in the parity tests: equal
 ranks and the apply within 1e-10 element-wise in FP64; in FP32 a PCG within
 two iterations of the FP64 factor's, to the same solution.
 """
@@ -21,7 +22,7 @@ from gpu_util import elem, gpu_factor, need_gpu, oracle_factor
 pytestmark = pytest.mark.gpu
 
 SIZES = [(3, 3), (5, 3), (4, 4), (17, 1), (31, 1), (8, 4), (11, 3), (9, 7), (8, 8), (13, 5), (127, 1), (16, 8),
-         (43, 3), (15, 11), (32, 7), (15, 15), (17, 15), (16, 16), (257, 1), (27, 19), (41, 25)]
+         (43, 3), (15, 11), (32, 7), (15, 15), (17, 15), (16, 16), (257, 1), (27, 19), (41, 25), (32, 3), (97, 1), (161, 1)]
 
 
 @pytest.mark.parametrize("ab", SIZES, ids=lambda ab: str(ab[0] * ab[1]))
