@@ -53,11 +53,7 @@ PRECS = {"f64": 0, "f32": 1, "tf32": 2, "bf16": 3, "tf32x3": 4}
 # large-node truncation.  Each figure names the profiles/ summary that holds
 # the capture and its command; a kernel changed since its capture has no
 # entry here (traffic null).
-TRAFFIC = {
-    # profiles/traffic_diffusion2d_512_f32.md: the large-node truncation of one
-    # factorization = 193.5 MB over its 46 launch groups
-    ("diffusion2d_512", "f32"): {"trunc": 193.48e6 / 46},
-}
+TRAFFIC = {}
 
 
 def make_problem(name: str, seed: int):
@@ -923,8 +919,8 @@ def main():
     tb_ms = info_f["trunc_big_ms"]
     tb_launches = max(info_f["trunc_big_launches"], 1)
     tb_ach = info_f["trunc_big_flops"] / (tb_ms / 1000.0) / 1e12 if tb_ms > 0 else 0.0
-    roof_trunc = {"bound": "alu", "kernel": "k_trunc_big (large-node truncation: tridiagonalisation, "
-                  "bisection, inverse iteration, back-transformation)",
+    roof_trunc = {"bound": "alu", "kernel": "truncation of nodes above 16 unknowns (k_tri_cta / k_tri_cluster, k_rank, "
+                  "k_eigval, k_invit, k_qmul)",
                   "achieved": tb_ach, "peak": alu_peak, "unit": "TFLOP/s", "frac": tb_ach / alu_peak,
                   "peak_source": alu_src, "traffic": TRAFFIC.get((args.workload, args.prec), {}).get("trunc"),
                   "algorithmic_flops_per_launch": info_f["trunc_big_flops"] / tb_launches,

@@ -260,11 +260,10 @@ typedef struct {
   double eig_flops;          /* nominal eigen-solve flops, reported apart: per
                                 truncated node 4/3 m^3 + 2 m^2 k                  */
   double factor_ms;          /* device time of the last factorization             */
-  double trunc_big_ms;       /* device time of the large-node truncation launches
-                                (tridiagonal eigen path), CUDA events             */
+  double trunc_big_ms;       /* device time of the truncation of nodes of more than
+                                16 unknowns (tridiagonal eigen path), CUDA events */
   double trunc_big_flops;    /* nominal eigen-solve flops of those nodes          */
-  int32_t trunc_big_launches;/* waves that ran the large-node truncation (one
-                                launch per thread-count class in each)            */
+  int32_t trunc_big_launches;/* waves that ran the tridiagonal eigen path         */
   double host_ms;            /* host wall time of the factorization call          */
   double wait_ms;            /* of which waiting for the device (rank reads)      */
   double phase_ms[16];       /* with hs_profile_phases(1): device time of the
@@ -272,9 +271,9 @@ typedef struct {
                                 A_sN/A_sW, 2 Cholesky of A_ss, 3 Gram, 4 small
                                 truncation, 5 large truncation, 6 CholQR of the
                                 large-path U, 7 extension GEMMs and CholQR, 8
-                                Schur scatter, 9 root; within 5, the multi-CTA
-                                path: 10 prepare, 11 tridiagonal steps, 12 Q^T Z,
-                                13 eigenvectors of T, 14 Q Y; 15 unused;
+                                Schur scatter, 9 root; within 5: 10 prepare, 11
+                                tridiagonal steps, 12 Q^T X, 13 rank, eigenvalues
+                                and eigenvectors of T, 14 Q Y; 15 unused;
                                 otherwise zeros                                 */
   double alg_flops;          /* algorithmic flops of the factorization, counted
                                 per super node from its sizes (m, rank k,

@@ -1814,7 +1814,7 @@ void trunc_big(Exec &ex, const std::vector<TruncTask<T>> &all, int *d_k, int var
       const BigLayout<T> L = big_layout<T>(t.work, t.m);
       const int ncol = fwd ? std::min(2 * std::max(t.np, 1), t.m) : t.m;   // at most; the kernels know k1 and k2
       T *cols = fwd ? L.LS : L.Y;
-      if (t.m <= kQmulMax) {
+      if (t.m <= kQmulMax<T>) {
         qm.push_back(QmulTask<T>{L.A, L.tau, cols, t.U, L.sc_int, t.m, fwd ? 1 : 0, blocks});
         blocks += qmul_blocks<T>(t.m, ncol);
         qmax = std::max(qmax, t.m);

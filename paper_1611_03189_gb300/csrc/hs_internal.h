@@ -298,7 +298,8 @@ struct EigTask {
 
 // Products with Q by warps (m <= kQmulMax): the columns (column-major, ld m),
 // for the backward product U (row-major m x m), the node's first CTA
-constexpr int kQmulMax = 1024;
+template <typename T>
+constexpr int kQmulMax = sizeof(T) == 4 ? 2048 : 1024;
 template <typename T>
 struct QmulTask {
   const T *A;

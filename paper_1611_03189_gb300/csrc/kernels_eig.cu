@@ -246,8 +246,8 @@ __device__ __forceinline__ int section(R &lo, R &hi, int lane, bool closed, F &&
 }
 
 // J = G - U1 X^T - X U1^T + U1 c U1^T (the Gram matrix projected off span U_1),
-// X = G U1 in Y's columns (column a at Y + a m), c in shared memory (ld
-// kMaxK1); one warp per row.  KB >= k1 sizes the per-row registers.
+// X = G U1 in Y's columns and U1 in U's (column a at + a m), c in shared memory
+// (ld kMaxK1); one warp per row.  KB >= k1 sizes the per-row registers.
 template <typename T, int KB>
 __device__ void build_projected_gram(const T *G, const T *U, const T *Y, const T *s_c, T *A, int m, int k1) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
@@ -255,7 +255,7 @@ __device__ void build_projected_gram(const T *G, const T *U, const T *Y, const T
     T ui[KB], xi[KB], cu[KB];
 #pragma unroll
     for (int a = 0; a < KB; ++a) {
-      ui[a] = a < k1 ? U[(int64_t)i * m + a] : T(0);
+      ui[a] = a < k1 ? U[(size_t)a * m + i] : T(0);
       xi[a] = a < k1 ? Y[(size_t)a * m + i] : T(0);
     }
 #pragma unroll
@@ -271,7 +271,7 @@ __device__ void build_projected_gram(const T *G, const T *U, const T *Y, const T
 #pragma unroll
       for (int a = 0; a < KB; ++a)
         if (a < k1) {
-          const T uj = U[(int64_t)j * m + a];
+          const T uj = U[(size_t)a * m + j];
           v = fma(-ui[a], Y[(size_t)a * m + j], fma(-xi[a], uj, v));
           v = fma(cu[a], uj, v);
         }
@@ -329,13 +329,18 @@ __global__ void __launch_bounds__(NT) k_trunc_prep(const TruncTask<T> *__restric
     if (tid == 0) kout[t.k_idx] = m;
     return;
   }
+  // U1's columns side by side (in U they are m apart, a sector a word: each of
+  // the loops over G below reads them once per row)
+  T *Uc = L.LS + (size_t)kMaxK1 * m;   // (X takes the first kMaxK1 columns of LS)
+  for (int64_t q = tid; q < (int64_t)m * k1; q += nt) Uc[q] = t.U[(q % m) * m + q / m];
+  __syncthreads();
   // G U1 in Y's first columns, C = U1^T G U1; one warp per row of G
   {
     const int warp = tid >> 5, lane = tid & 31, nw = nt >> 5;
     for (int i = warp; i < m; i += nw)
       for (int a = 0; a < k1; ++a) {
         T s = T(0);
-        for (int j = lane; j < m; j += 32) s = fma(t.G[(int64_t)i * m + j], t.U[(int64_t)j * m + a], s);
+        for (int j = lane; j < m; j += 32) s = fma(t.G[(int64_t)i * m + j], Uc[(size_t)a * m + j], s);
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         if (lane == 0) Y[(size_t)a * m + i] = s;
       }
@@ -346,21 +351,21 @@ __global__ void __launch_bounds__(NT) k_trunc_prep(const TruncTask<T> *__restric
   for (int a = 0; a < k1; ++a)
     for (int bb = 0; bb < k1; ++bb) {
       T s = T(0);
-      for (int i = tid; i < m; i += nt) s = fma(t.U[(int64_t)i * m + a], Y[(size_t)bb * m + i], s);
+      for (int i = tid; i < m; i += nt) s = fma(Uc[(size_t)a * m + i], Y[(size_t)bb * m + i], s);
       const T cab = bsum_t<T>(s, redt);
       if (tid == 0) s_c[a * kMaxK1 + bb] = cab;
     }
   __syncthreads();
   if (k1 <= 2)
-    build_projected_gram<T, 2>(t.G, t.U, Y, s_c, A, m, k1);
+    build_projected_gram<T, 2>(t.G, Uc, Y, s_c, A, m, k1);
   else
-    build_projected_gram_wide<T>(t.G, t.U, Y, s_c, A, m, k1);
+    build_projected_gram_wide<T>(t.G, Uc, Y, s_c, A, m, k1);
   // X = G U1 - U1 C (the scratch in LS is no longer in use)
   T *X = L.LS;
   for (int64_t q = tid; q < (int64_t)m * k1; q += nt) {
     const int a = (int)(q / m), i = (int)(q % m);
     T x = Y[(size_t)a * m + i];
-    for (int b = 0; b < k1; ++b) x = fma(-t.U[(int64_t)i * m + b], s_c[b * kMaxK1 + a], x);
+    for (int b = 0; b < k1; ++b) x = fma(-Uc[(size_t)b * m + i], s_c[b * kMaxK1 + a], x);
     X[(size_t)a * m + i] = x;
   }
   if (tid == 0) L.sc_int[0] = k1;
@@ -871,7 +876,12 @@ __global__ void __launch_bounds__(32) k_invit(const EigTask<T> *__restrict__ tas
 // (One CTA per 16 columns with block sums took three barriers a reflector.)
 // ---------------------------------------------------------------------------
 constexpr int kQmWarps = 4;
-__host__ __device__ inline int qmul_e(int m) { return m <= 64 ? 2 : m <= 128 ? 4 : m <= 256 ? 8 : m <= 512 ? 16 : 32; }
+// (E = 48, 64: FP32 only, whose three rows of E registers fit; a CTA per 16
+// columns with block sums, which FP64 keeps there, took 3.2 ms for the four
+// largest nodes of a 40^3 grid, m = 1340)
+__host__ __device__ inline int qmul_e(int m) {
+  return m <= 64 ? 2 : m <= 128 ? 4 : m <= 256 ? 8 : m <= 512 ? 16 : m <= 1024 ? 32 : m <= 1536 ? 48 : 64;
+}
 template <typename T>
 __host__ __device__ constexpr int qmul_cols(int E) {
   return sizeof(T) == 4 ? (E <= 8 ? 4 : E == 16 ? 2 : 1) : (E <= 4 ? 4 : E == 8 ? 2 : 1);
@@ -973,6 +983,10 @@ __global__ void __launch_bounds__(kQmWarps * 32) k_qmul(const QmulTask<T> *__res
       if (E == 16) qmul_warp<T, 16, qmul_cols<T>(16)>(t, j0, nc, stage, sld);
     if constexpr (EM >= 32)
       if (E == 32) qmul_warp<T, 32, qmul_cols<T>(32)>(t, j0, nc, stage, sld);
+    if constexpr (EM >= 48)
+      if (E == 48) qmul_warp<T, 48, qmul_cols<T>(48)>(t, j0, nc, stage, sld);
+    if constexpr (EM >= 64)
+      if (E == 64) qmul_warp<T, 64, qmul_cols<T>(64)>(t, j0, nc, stage, sld);
   }
   if (t.fwd) return;
   __syncthreads();
@@ -1151,7 +1165,7 @@ __global__ void __launch_bounds__(kTriRows * 32) k_tri_symv(const GridTri<T> *__
   }
 }
 
-// The same products for nodes too large for a warp's registers (m > 1024), one CTA
+// The same products for nodes too large for a warp's registers (m > qmul_max), one CTA
 // per batch of columns held in
 // shared memory: for each reflector the block forms all the batch's dot
 // products (fixed-order reduction), then updates the columns.
@@ -1308,14 +1322,21 @@ void launch_qmul(const QmulTask<T> *d_tasks, int ntasks, int total_blocks, int m
   // the staged columns: the larger of m (4 C(E) + 1) over the classes up to E
   size_t sm = 0;
   if (!fwd)
-    for (int e = 2; e <= E; e *= 2)
-      sm = std::max(sm, sizeof(T) * (size_t)std::min(m_max, 32 * e) * (kQmWarps * qmul_cols<T>(e) + 1));
+    for (int e : {2, 4, 8, 16, 32, 48, 64})
+      if (e <= E) sm = std::max(sm, sizeof(T) * (size_t)std::min(m_max, 32 * e) * (kQmWarps * qmul_cols<T>(e) + 1));
   switch (E) {
     case 2: launch_qmul_e<T, 2>(d_tasks, ntasks, total_blocks, sm, st); break;
     case 4: launch_qmul_e<T, 4>(d_tasks, ntasks, total_blocks, sm, st); break;
     case 8: launch_qmul_e<T, 8>(d_tasks, ntasks, total_blocks, sm, st); break;
     case 16: launch_qmul_e<T, 16>(d_tasks, ntasks, total_blocks, sm, st); break;
-    default: launch_qmul_e<T, 32>(d_tasks, ntasks, total_blocks, sm, st); break;
+    case 32: launch_qmul_e<T, 32>(d_tasks, ntasks, total_blocks, sm, st); break;
+    default:
+      if constexpr (sizeof(T) == 4) {
+        if (E == 48) launch_qmul_e<T, 48>(d_tasks, ntasks, total_blocks, sm, st);
+        else launch_qmul_e<T, 64>(d_tasks, ntasks, total_blocks, sm, st);
+      } else {
+        fail(HS_ERR_INVALID, "internal: size of the products with Q");
+      }
   }
   count_launch();
   HS_CUDA(cudaGetLastError());

@@ -22,7 +22,7 @@ from gpu_util import elem, gpu_factor, need_gpu, oracle_factor
 pytestmark = pytest.mark.gpu
 
 SIZES = [(3, 3), (5, 3), (4, 4), (17, 1), (31, 1), (8, 4), (11, 3), (9, 7), (8, 8), (13, 5), (127, 1), (16, 8),
-         (43, 3), (15, 11), (32, 7), (15, 15), (17, 15), (16, 16), (257, 1), (27, 19), (41, 25), (32, 3), (97, 1), (161, 1)]
+         (43, 3), (15, 11), (32, 7), (15, 15), (17, 15), (16, 16), (257, 1), (27, 19), (41, 25), (32, 3), (97, 1), (161, 1), (40, 39)]
 
 
 @pytest.mark.parametrize("ab", SIZES, ids=lambda ab: str(ab[0] * ab[1]))
