@@ -294,6 +294,11 @@ struct SumBatch {
   std::vector<SumSrc<T>> srcs;
   std::vector<int> tile_start;
   int tiles = 0;
+  void reserve(size_t more) {
+    tasks.reserve(tasks.size() + more);
+    srcs.reserve(srcs.size() + more);
+    tile_start.reserve(tile_start.size() + more);
+  }
   // begins a task; sources are appended with src() afterwards
   void begin(T *dst, int ld, int rows, int cols, T alpha, T beta) {
     SumTask<T> t;
@@ -1005,50 +1010,60 @@ void Run<T>::merge(int nred, int key_base, SumBatch<T> &sb) {
       }
     ssize[j] = any ? m : -1;
   }
-  // super-block list
-  FlatMap<int64_t> off;
-  off.reserve(blocks_.size());
+  // super-block list: one lookup per block, whose super block (an index in
+  // order of first appearance) is kept for the copies below
+  FlatMap<BlockRef<T>> nb;
+  nb.reserve(blocks_.size());
+  std::vector<uint64_t> keys;
+  std::vector<BlockRef<T>> refs;
+  keys.reserve(blocks_.size());
+  refs.reserve(blocks_.size());
+  for (auto &kv : blocks_) {
+    keys.push_back(kv.first);
+    refs.push_back(kv.second);
+  }
+  std::vector<int> sup_of(keys.size());
   std::vector<std::pair<int, int>> order;
   std::vector<int64_t> order_off;
   int64_t total = 0;
-  for (auto &kv : blocks_) {
-    const int a = (int)(kv.first >> 32) - key_base, b = (int)(kv.first & 0xffffffffu) - key_base;
+  auto super_key = [&](uint64_t key) {
+    return bkey(((int)(key >> 32) - key_base) / 2, ((int)(key & 0xffffffffu) - key_base) / 2);
+  };
+  constexpr size_t kAhead = 8;
+  for (size_t q = 0; q < keys.size(); ++q) {
+    if (q + kAhead < keys.size()) nb.prefetch(super_key(keys[q + kAhead]));
+    const int a = (int)(keys[q] >> 32) - key_base, b = (int)(keys[q] & 0xffffffffu) - key_base;
     if (a < 0 || b < 0 || a >= nred || b >= nred) fail(HS_ERR_INVALID, "internal: stray block at merge");
     const int I = a / 2, J = b / 2;
-    auto ins = off.try_emplace(bkey(I, J));
+    auto ins = nb.try_emplace(bkey(I, J));
     if (ins.second) {
-      *ins.first = total;
+      ins.first->ld = (int)order.size();   // the index, until the storage is known
       order.emplace_back(std::min(I, J), std::max(I, J));
       order_off.push_back(total);
       total += ((int64_t)ssize[I] * ssize[J] + 3) & ~(int64_t)3;
     }
+    sup_of[q] = ins.first->ld;
   }
   T *base = talloc<T>(*h_.pers, total);
   HS_CUDA(cudaMemsetAsync(base, 0, sizeof(T) * std::max<int64_t>(total, 1), st_));
-  FlatMap<BlockRef<T>> nb;
-  nb.reserve(order.size());
-  for (size_t q = 0; q < order.size(); ++q) {
-    const auto &IJ = order[q];
-    BlockRef<T> br;
-    br.ptr = base + order_off[q];
-    br.ld = ssize[IJ.second];
-    br.rowkey = IJ.first;
-    nb[bkey(IJ.first, IJ.second)] = br;
+  for (auto &kv : nb) {
+    const size_t q = kv.second.ld;
+    kv.second.ptr = base + order_off[q];
+    kv.second.ld = ssize[order[q].second];
+    kv.second.rowkey = order[q].first;
   }
-  for (auto &kv : blocks_) {
-    const int a = std::min((int)(kv.first >> 32), (int)(kv.first & 0xffffffffu)) - key_base;
-    const int b = std::max((int)(kv.first >> 32), (int)(kv.first & 0xffffffffu)) - key_base;
-    const BlockRef<T> &rb = kv.second;
-    const int I = a / 2, J = b / 2;
-    auto sit = nb.find(bkey(I, J));
-    if (sit == nb.end()) fail(HS_ERR_INVALID, "internal: missing super block at merge");
-    const BlockRef<T> sbk = sit->second;
+  sb.reserve(keys.size() + (size_t)(use_phi_ ? nred : 0));
+  for (size_t q = 0; q < keys.size(); ++q) {
+    const int a = std::min((int)(keys[q] >> 32), (int)(keys[q] & 0xffffffffu)) - key_base;
+    const int b = std::max((int)(keys[q] >> 32), (int)(keys[q] & 0xffffffffu)) - key_base;
+    const BlockRef<T> &rb = refs[q];
+    const int I = a / 2, J = b / 2, ld = ssize[order[sup_of[q]].second];
+    T *dst = base + order_off[sup_of[q]];
     // rows a, cols b
     const int ta = (rb.rowkey - key_base == a) ? 0 : 1;
-    sb.copy(sbk.ptr + (int64_t)coff[a] * sbk.ld + coff[b], sbk.ld, rsize[a], rsize[b], rb.ptr, rb.ld, ta);
+    sb.copy(dst + (int64_t)coff[a] * ld + coff[b], ld, rsize[a], rsize[b], rb.ptr, rb.ld, ta);
     if (I == J && a != b)  // mirrored sub-block of a diagonal super block
-      sb.copy(sbk.ptr + (int64_t)coff[b] * sbk.ld + coff[a], sbk.ld, rsize[b], rsize[a], rb.ptr, rb.ld,
-              1 - ta);
+      sb.copy(dst + (int64_t)coff[b] * ld + coff[a], ld, rsize[b], rsize[a], rb.ptr, rb.ld, 1 - ta);
   }
   // preserved vectors (m x nphi row-major per node): contiguous per level
   std::vector<T *> nphi(2 * nsup, nullptr);
@@ -1100,11 +1115,21 @@ void Run<T>::wave_a(int li, int widx, WaveBatches<T> &B) {
   trunc64_first_ = B.trunc64.size();
   big64_first_ = B.trunc_big64.size();
   const double f0 = B.chol.flops + B.gram.flops + B.gram64.flops;
+  // the blocks of the next node are on their way while this one's are copied
+  auto prefetch = [&](int s) {
+    const PlanSuper &ps = lv.sup[s];
+    blocks_.prefetch(bkey(s, s));
+    for (int n : ps.N) blocks_.prefetch(bkey(s, n));
+    for (int w : ps.W) blocks_.prefetch(bkey(s, w));
+  };
   for (size_t q = 0; q < wl.size(); ++q) {
     Sup &x = cur_[q];
     const int s = wl[q];
     const PlanSuper &ps = lv.sup[s];
+    if (q + 1 < wl.size()) prefetch(wl[q + 1]);
     x.s = s;
+    x.Noff.reserve(ps.N.size());
+    x.Woff.reserve(ps.W.size());
     x.m = size_[s];
     x.red = !ps.W.empty();
     for (int n : ps.N) {
@@ -1403,12 +1428,15 @@ void Run<T>::wave_d(WaveBatches<T> &B) {
   {
     int64_t total = 0;
     std::vector<std::pair<uint64_t, int64_t>> fresh;
-    for (uint64_t key : tgt_order)
+    for (size_t ti = 0; ti < tgt_order.size(); ++ti) {
+      if (ti + 8 < tgt_order.size()) blocks_.prefetch(tgt_order[ti + 8]);
+      const uint64_t key = tgt_order[ti];
       if (!blocks_.count(key)) {
         const int a = (int)(key >> 32), b = (int)(key & 0xffffffffu);
         fresh.emplace_back(key, total);
         total += ((int64_t)size_[a] * size_[b] + 3) & ~(int64_t)3;
       }
+    }
     if (!fresh.empty()) {
       T *base = talloc<T>(per, total);
       HS_CUDA(cudaMemsetAsync(base, 0, sizeof(T) * total, st_));
@@ -1424,6 +1452,7 @@ void Run<T>::wave_d(WaveBatches<T> &B) {
   }
   for (size_t ti = 0; ti < tgt_order.size(); ++ti) {
     const uint64_t key = tgt_order[ti];
+    if (ti + 8 < tgt_order.size()) blocks_.prefetch(tgt_order[ti + 8]);
     auto dit = blocks_.find(key);
     if (dit == blocks_.end()) fail(HS_ERR_INVALID, "internal: missing Schur target");
     const BlockRef<T> dst = dit->second;
@@ -1445,8 +1474,22 @@ void Run<T>::wave_d(WaveBatches<T> &B) {
   }
 
   // new red nodes, removal of the eliminated super nodes, apply records
-  for (auto &x : S) {
+  for (size_t q = 0; q < S.size(); ++q) {
+    Sup &x = S[q];
     const PlanSuper &ps = lv_->sup[x.s];
+    if (q + 1 < S.size()) {
+      const int s = S[q + 1].s;
+      const PlanSuper &pn = lv_->sup[s];
+      blocks_.prefetch(bkey(s, s));
+      for (int n : pn.N) {
+        blocks_.prefetch(bkey(s, n));
+        blocks_.prefetch(bkey(n, nsup_ + s));
+      }
+      for (int w : pn.W) {
+        blocks_.prefetch(bkey(s, w));
+        blocks_.prefetch(bkey(w, nsup_ + s));
+      }
+    }
     if (x.red) {
       const int r = nsup_ + x.s;
       size_[r] = x.k;

@@ -101,6 +101,14 @@ class FlatMap {
     ++tombs_;
   }
 
+  // starts loading the slot of k, for a lookup some tens of instructions later
+  // (a lookup is two cache misses on a large map)
+  void prefetch(uint64_t k) const {
+    const size_t i = hash(k) & (state_.size() - 1);
+    __builtin_prefetch(&state_[i]);
+    __builtin_prefetch(&slots_[i]);
+  }
+
   void clear() { init(16); }
 
   void swap(FlatMap &o) {
