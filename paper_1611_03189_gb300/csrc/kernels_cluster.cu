@@ -4,21 +4,22 @@
 // matrices beyond one CTA's shared memory, in one thread-block cluster.
 //
 // The whole n x n matrix stays in shared memory for all steps; with C CTAs each
-// holds a slab of ceil(n / C) columns (all rows).  J is symmetric, so every
-// product is a column walk: a few threads own a column, consecutive threads on
-// consecutive words.  Step k:
+// holds every C-th column (all rows).  J is symmetric, so every product is a
+// column walk.  Step k:
 //   1. column k (= row k), with the pending update of step k - 1, and the
 //      reflector I - tau v v^T of x = J[k+1.., k];
 //   2. one walk of the own columns: the pending update of step k - 1 and
 //      p_i = tau sum_j J_ji v_j;
 //   3. K = tau (p.v) / 2, w = p - K v; (v, w) are the next pending update
 //      J -= v w^T + w v^T.
-// What bounds it is the latency of a step: shared-memory loads of the walk and
-// the barriers (three a step in one CTA; in a cluster one cluster barrier and the
-// distributed reads of column k and p besides).  The reflector's scalars are
-// kept off the FP64 pipe in FP32 factors (see reflector() below), and by one
-// warp in FP64 ones: every thread computing them in FP64, at 1/64 of the FP32
-// rate, took more than half of each step.
+// What bounds it is the latency of a step: the walk's shared-memory loads and
+// the barriers (three a step; in a cluster one cluster barrier and the reads of
+// column k and p from the other CTAs besides).  Measured: about 1 us a step in
+// one CTA, 3.4 us in 16 CTAs at n = 900 (8.0 us when every CTA read column k from
+// the CTA that holds it).  The reflector's scalars are kept off the FP64 pipe in
+// FP32 factors (see reflector() below), and computed by one warp in FP64 ones:
+// every thread computing them in FP64, at 1/64 of the FP32 rate, took more than
+// half of each step.
 // Outputs: d, e (FP64) and tau, reflector k in row k of A (v[0] = 1 implicit,
 // v[1..] at A[k][k+2..]), the trailing 2 x 2 block in A.  Where a node is worked
 // on and every reduction order depend on n alone, so a node gets the same bits
@@ -516,7 +517,9 @@ int tri_max_m(int q) {
 // FP32: one CTA while it fits, then 4 CTAs (a step is bound by its barriers and
 // distributed reads, which cost 2 CTAs as much), then 8, then 16.
 // FP64: the arithmetic itself (3 n^2 FMAs a step at 1/64 of the FP32 rate)
-// outgrows the barriers from about n = 112 on, so 8 CTAs share it from there.
+// outgrows the barriers from about n = 112 on, so 8 CTAs share it from there (88:
+// the same) and 16 from n = 161 on (a 331 x 198 factorization 171.6 ms with 8
+// only, 166.3 with 16 from 161, 166.1 from 129, 167.0 from 113).
 // HS_TRI_CLUSTER=1 (environment) keeps to one CTA, =2 takes the smallest
 // cluster that fits.
 static int tri_mode() {

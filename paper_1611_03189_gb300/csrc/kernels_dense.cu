@@ -7,7 +7,8 @@
 //                scatter of Sec. 3.2 (several super nodes of one wave updating
 //                the same neighbour block).
 //   k_chol_inv   A = L L^T and L^-1, one CTA per matrix (pivot blocks A_ss and
-//                the small Gram matrices of the CholQR of L^-1 U).
+//                the small Gram matrices of the CholQR of L^-1 U); FP64 from 97
+//                unknowns on a cluster of four (k_chol_cluster).
 //   k_trunc      truncation of the well-separated block (Sec. 3.2 eq.
 //                local_compression, Sec. 6 GC basis), one CTA per super node:
 //                cyclic Jacobi eigen-solves of the Gram matrix A_sw A_sw^T.
@@ -244,7 +245,7 @@ __global__ void __launch_bounds__(256) k_sum(const SumTask<T> *__restrict__ task
 //           in 32 x 16 tiles per warp, 4 x 4 outputs a lane, 16-byte loads along
 //           k (P) or along the row (X).
 // The only serial chain is the 16 x 16 diagonal block: one warp factors it in
-// registers, lane = row, and forms D_b with the same shuffles.  Warp 0 updates
+// registers, half its lanes the rows, half D_b's columns.  Warp 0 updates
 // the next diagonal block first and factors it while the other warps finish
 // the update.  Three barriers per 16 columns.
 // What bounds it: the diagonal chain up to m of about 100, the CUDA cores' FMA
@@ -506,14 +507,15 @@ __global__ void __launch_bounds__(NT) k_chol_inv(const CholTask<T> *__restrict__
   if (tid == 0) status[t.status_idx] = st;
 }
 
-// The same factorization by a cluster of kCholC CTAs, for FP64 matrices from
-// kCholClusterMin on, where one SM's FP64 rate (2 FMAs a cycle) bounds it.
+// The same factorization by a cluster of kCholC CTAs, for FP64 matrices above
+// kCholClusterMin, where one SM's FP64 rate (2 FMAs a cycle) bounds it.
 // Blocks of 16 columns are dealt out cyclically and stay with their CTA, first
 // as trailing columns, then as the inverse's.  A step needs D_b and the panel
 // P_b alone from elsewhere: their owner writes them into every CTA's shared
 // memory, so a step has one cluster barrier.  The owner of block b + 1 updates
 // that block first, and its diagonal block is inverted beside its other tiles.
-// Every element's arithmetic is k_chol_inv's.
+// Every element's arithmetic is k_chol_inv's, so a smaller matrix in a launch with
+// such a one keeps its bits.
 constexpr int kCholC = 4, kCholClusterMin = 96, kCholClThreads = 256;
 
 __host__ __device__ inline int chol_cl_ld(int m) {
@@ -1059,7 +1061,7 @@ static void launch_chol_nt(const CholTask<T> *d_tasks, int ntasks, int *d_status
   k_chol_inv<T, NT><<<ntasks, NT, sm, st>>>(d_tasks, d_status);
 }
 
-// FP64 from kCholClusterMin on: k_chol_cluster (m = 150 to 160: 0.60 ms in one
+// FP64 above kCholClusterMin: k_chol_cluster (m = 150 to 160: 0.60 ms in one
 // CTA, about 0.28 in four; its limit of 256 also spares nodes up to there the
 // blocked path).  Below, the diagonal blocks' serial chain is what counts.
 // Threads by the largest matrix of the launch: the update's tiles (about

@@ -610,7 +610,9 @@ __global__ void __launch_bounds__(kRankThreads) k_rank(const TruncTask<T> *__res
 // ---------------------------------------------------------------------------
 // The k2 largest eigenvalues of T (shifts of the inverse iteration), `lanes`
 // of a warp sectioning each: 8 below m = 128, where a wave has many nodes and
-// the work counts, 32 from there on, where the rounds do.  The bracket is
+// the work counts, 32 from there on, where the rounds do.  FP64, bound by its
+// issue rate, takes 8 throughout (331 x 198: 20.5 ms in all with 32 and the
+// longer reciprocal, 15.3 so).  The bracket is
 // (eps^2 lambda_max, Gershgorin bound).  The FP64 factor places them in FP32
 // first and confirms and refines that bracket in FP64.
 // ---------------------------------------------------------------------------
@@ -706,7 +708,8 @@ __global__ void __launch_bounds__(kEigThreads) k_eigval(const EigTask<T> *__rest
 // sub-diagonal dominates), three solves from a fixed pseudo-random start,
 // modified Gram-Schmidt against the vectors already found of the same cluster
 // of eigenvalues closer than 10 u ||T|| (those could come out nearly
-// parallel; the lane of a cluster's first eigenvalue takes them all in turn).
+// parallel; the lane of a cluster's first eigenvalue takes them all in turn, and
+// the warp orthogonalises together).
 // Only the span of the selected vectors matters and the host
 // re-orthonormalises them, which tolerates the overlap u ||T|| / gap that
 // inverse iteration leaves between vectors of distinct eigenvalues.
