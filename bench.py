@@ -53,7 +53,10 @@ PRECS = {"f64": 0, "f32": 1, "tf32": 2, "bf16": 3, "tf32x3": 4}
 # large-node truncation.  Each figure names the profiles/ summary that holds
 # the capture and its command; a kernel changed since its capture has no
 # entry here (traffic null).
-TRAFFIC = {}
+TRAFFIC = {
+    # profiles/traffic_diffusion2d_512_f32.md
+    ("diffusion2d_512", "f32"): {"apply": 341.08e6},
+}
 
 
 def make_problem(name: str, seed: int):

@@ -1071,18 +1071,16 @@ template <typename T>
 void launch_chol_inv(const CholTask<T> *d_tasks, int ntasks, int *d_status, int max_m,
                      cudaStream_t st) {
   if (ntasks == 0) return;
-  bool cluster = false;
-  if constexpr (sizeof(T) == 8) {
-    cluster = max_m > kCholClusterMin;
-    if (cluster) {
+  if (max_m <= 48) {
+    launch_chol_nt<T, 128>(d_tasks, ntasks, d_status, max_m, st);
+  } else if constexpr (sizeof(T) == 8) {
+    if (max_m <= kCholClusterMin) {
+      launch_chol_nt<T, 256>(d_tasks, ntasks, d_status, max_m, st);
+    } else {
       const size_t sm = chol_cl_smem_bytes<T>(max_m);
       check_dynamic_smem(sm, allow_max_dynamic_smem<&k_chol_cluster<T>>(), "k_chol_cluster");
       k_chol_cluster<T><<<ntasks * kCholC, kCholClThreads, sm, st>>>(d_tasks, d_status);
     }
-  }
-  if (cluster) {
-  } else if (max_m <= 48) {
-    launch_chol_nt<T, 128>(d_tasks, ntasks, d_status, max_m, st);
   } else if (max_m <= 112) {
     launch_chol_nt<T, 256>(d_tasks, ntasks, d_status, max_m, st);
   } else {
