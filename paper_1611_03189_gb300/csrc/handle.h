@@ -208,12 +208,15 @@ struct FactorHandle {
 
   // recorded solve graphs and the private stream they are recorded on
   std::vector<GraphEntry> graphs;
-  int applies = 0, pcg_iters = 0;      // since the graphs were last dropped
+  // since the graphs were last dropped: an apply ran, PCG iterations launched directly
+  bool applied = false;
+  int pcg_direct = 0;
   cudaStream_t cap_stream = nullptr;
   void drop_graphs() {
     for (GraphEntry &g : graphs) cudaGraphExecDestroy(g.exec);
     graphs.clear();
-    applies = pcg_iters = 0;
+    applied = false;
+    pcg_direct = 0;
   }
 
   // per-level ranks: ranks[li][s] = k or -1

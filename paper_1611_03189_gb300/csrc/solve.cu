@@ -1093,7 +1093,8 @@ void run_graph(const GraphEntry &g, cudaStream_t st) {
 // The first apply after a factorization is launched directly: recording and
 // instantiating some 120 launches takes longer than issuing them once.
 void apply_ws(FactorHandle &h, int nrhs, cudaStream_t st) {
-  if (!graphs_enabled() || h.applies++ == 0) {
+  if (!graphs_enabled() || !h.applied) {
+    h.applied = true;
     apply_ws_direct(h, nrhs, st);
     return;
   }
@@ -1358,7 +1359,9 @@ int pcg_solve(FactorHandle &h, const double *b, double *x, int nrhs, int64_t ld,
     // a factorization's first iterations are launched directly: two recordings
     // of some 120 launches only pay from a few replays on (24 systems factored
     // and solved once each: 103 ms with graphs from the start, 93 without)
-    if (graphs_enabled() && h.pcg_iters++ >= kDirectIters) {
+    const bool direct = h.pcg_direct < kDirectIters;
+    if (direct) ++h.pcg_direct;
+    if (graphs_enabled() && !direct) {
       const int key = kPcgGraphKey + 2 * np + (it & 1);
       run_graph(graph_for(h, key, [&](cudaStream_t cs) { body(cs, pold, pnew); }), st);
     } else {
