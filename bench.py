@@ -49,8 +49,7 @@ METRIC = "solves/s to rel-res 1e-10 (factor + PCG solve; mixed vs FP64 factor)"
 PRECS = {"f64": 0, "f32": 1, "tf32": 2, "bf16": 3, "tf32x3": 4}
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) per launch unit
 # of the roofline entries, from one ncu capture of the same bench command:
-# "apply" per application (all its launches), "trunc" per launch group of the
-# large-node truncation.  Each figure names the profiles/ summary that holds
+# "apply" per application (all its launches).  Each figure names the profiles/ summary that holds
 # the capture and its command; a kernel changed since its capture has no
 # entry here (traffic null).
 TRAFFIC = {
@@ -908,7 +907,7 @@ def main():
         except Exception as ex:  # the baseline must not hide the GPU number
             cpu = {"error": str(ex)[:200]}
 
-    # ---- the large-node truncation (tridiagonal eigen path): plain FP32/FP64 ALU work ----
+    # ---- the truncation of nodes above 16 unknowns (tridiagonal eigen path): plain FP32/FP64 ALU work ----
     # nominal eigen-solve flops (4/3 m^3 + 2 m^2 k per node) over the device time
     # of its launches (CUDA events on the factor stream, inside the library)
     info_f = G.info()

@@ -410,7 +410,7 @@ int eig_small_max() {
 std::atomic<int> g_phase_prof{0};
 bool phase_profiling() { return g_phase_prof.load() != 0; }
 
-// The cluster tridiagonalisation of the multi-CTA path (HS_TRI_CLUSTER=0 in
+// The on-chip tridiagonalisation (HS_TRI_CLUSTER=0 in
 // the environment turns it off: every node then takes the step kernels).
 inline bool tri_cluster_enabled() {
   static const bool v = [] {
