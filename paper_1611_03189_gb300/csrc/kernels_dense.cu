@@ -291,20 +291,9 @@ __device__ __forceinline__ void st16(float *p, const float *v) {
 __device__ __forceinline__ void st16(double *p, const double *v) {
   *reinterpret_cast<double2 *>(p) = make_double2(v[0], v[1]);
 }
-// d^-1/2 to about one unit in the last place
-__device__ __forceinline__ float inv_sqrt(float d) {
-  const float y = rsqrtf(d);
-  return y * fmaf(-0.5f * d * y, y, 1.5f);
-}
-// (FP64: the hardware's seed y, 20 bits, and the series of (1 - r)^-1/2 to r^2,
-// r = 1 - d y^2: five FP64 instructions on the pivots' serial chain)
-__device__ __forceinline__ double inv_sqrt(double d) {
-  if (d < 1e-290) return rsqrt(d);
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-  const double r = fma(-d * y, y, 1.0);
-  return fma(y, r * fma(r, 0.375, 0.5), y);
-}
+// d^-1/2 (CUDA's: rounded correctly, and within one unit in the last place)
+__device__ __forceinline__ float inv_sqrt(float d) { return __frsqrt_rn(d); }
+__device__ __forceinline__ double inv_sqrt(double d) { return rsqrt(d); }
 
 // One warp: D = L^-1 of the diagonal block at row j0, column j0c of W (jb <= 16
 // columns, j0 the first in the matrix), in its place with zeros above the diagonal;

@@ -78,22 +78,9 @@ __device__ __forceinline__ float hash_unit(uint32_t a, uint32_t b) {
 }
 
 
-// Quotients of the Sturm recurrences that only place eigenvalues (shifts of
-// the inverse iteration, lambda_max): approximate division (2 ulp), which
-// moves a computed count no more than the rounding of the recurrence itself
-// does.  The rank count divides exactly, in FP64.
-__device__ __forceinline__ float place_div(float a, float b) { return __fdividef(a, b); }
-// FP64: the hardware's reciprocal seed y (20 bits) and one step of third order,
-// y + y (r + r^2) with r = 1 - b y (the series of 1 / (1 - r)), which leaves
-// r^3 = 2^-60: 3 of the FP64 instructions whose rate bounds these loops
-__device__ __forceinline__ double place_div(double a, double b) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
-  const double r = fma(-b, y, 1.0);
-  return a * fma(y, fma(r, r, r), y);
-}
-// sign and magnitude tests of the Sturm pivots; in FP64 by the high word
-// (comparisons issue on the FP64 pipe too)
+// Sign and magnitude tests of the Sturm pivots, in FP64 by the high word
+// (comparisons issue on the FP64 pipe too): pivmin's low word is zero
+// (sturm_pivmin), so the comparison of the high words is that of the values
 __device__ __forceinline__ bool pivot_tiny(float q, float pivmin) { return fabs(q) < pivmin; }
 __device__ __forceinline__ bool pivot_tiny(double q, double pivmin) {
   return (__double2hiint(q) & 0x7fffffff) < __double2hiint(pivmin);
@@ -110,7 +97,7 @@ __device__ __forceinline__ int count_above(const R *d, const R *e2, int m, R sig
   int c = pivot_pos(q);
 #pragma unroll 4
   for (int i = 1; i < m; ++i) {
-    q = (d[i] - sigma) - place_div(e2[i], q);
+    q = (d[i] - sigma) - e2[i] / q;
     if (pivot_tiny(q, pivmin)) q = -pivmin;
     c += pivot_pos(q);
   }
@@ -181,7 +168,7 @@ __device__ __forceinline__ int count_above_gc(const R *d, const R *e, const R *e
     R q = (d[i] - sigma) - e2[i] * inv;   // e2[0] = 0
     if (pivot_tiny(q, pivmin)) q = -pivmin;
     c += pivot_pos(q);
-    inv = place_div(R(1), q);
+    inv = R(1) / q;
 #pragma unroll
     for (int a = 0; a < KB; ++a)
       if (KB <= 2 || a < k1) w[a] = (KB == 1 || a < k1 ? Z[(size_t)a * ldz + i] : R(0)) - l * w[a];
@@ -213,9 +200,10 @@ __device__ __noinline__ int count_above_gc_wide(const R *d, const R *e, const R 
   return count_above_gc<R, kMaxK1>(d, e, e2, m, Z, ldz, k1, C, sigma, pivmin);
 }
 
-template <typename R>
-__device__ __forceinline__ R sturm_pivmin(R emax2) {
-  return fmax(R(1e-30) * fmax(R(1), emax2), R(1e-35));
+// smallest pivot of a Sturm recurrence (FP64: its low word cleared, for pivot_tiny)
+__device__ __forceinline__ float sturm_pivmin(float emax2) { return fmaxf(1e-30f * fmaxf(1.f, emax2), 1e-35f); }
+__device__ __forceinline__ double sturm_pivmin(double emax2) {
+  return __hiloint2double(__double2hiint(1e-30 * fmax(1.0, emax2)), 0);
 }
 
 // The multisection of one value by the lanes of a warp group: `above(sigma)`
@@ -508,7 +496,7 @@ __global__ void __launch_bounds__(kRankThreads) k_rank(const TruncTask<T> *__res
     s_ct[q] = (T)(L.sc_c[q] * sc);
   }
   __syncthreads();
-  const float pivf = sturm_pivmin<float>((float)emax);
+  const float pivf = sturm_pivmin((float)emax);
   double lmax;   // of the scaled G
   const bool wide_global = gc && !zs;   // many preserved vectors on a huge node
   {
@@ -538,7 +526,7 @@ __global__ void __launch_bounds__(kRankThreads) k_rank(const TruncTask<T> *__res
     lmax = (double)(0.5f * (lo + hi));
     if constexpr (sizeof(T) == 8) {
       if (warp == 0) {
-        const double piv = sturm_pivmin<double>(emax);
+        const double piv = sturm_pivmin(emax);
         auto above = [&](double sig) {
           if (k1 == 0) return count_above<double>(d, e2, m, sig, piv) >= 1;
           const double *z = zs ? zd : (const double *)L.LS;   // (beyond shared memory: scaled in place below)
@@ -567,7 +555,7 @@ __global__ void __launch_bounds__(kRankThreads) k_rank(const TruncTask<T> *__res
   }
   const double thr = t.eps * t.eps * lmax;
   // the Sturm count in FP64 from both ends, middle row h
-  const double piv = sturm_pivmin<double>(emax);
+  const double piv = sturm_pivmin(emax);
   const int h = m / 2;
   if (tid == 0) {
     int c = 0;
@@ -611,8 +599,7 @@ __global__ void __launch_bounds__(kRankThreads) k_rank(const TruncTask<T> *__res
 // The k2 largest eigenvalues of T (shifts of the inverse iteration), `lanes`
 // of a warp sectioning each: 8 below m = 128, where a wave has many nodes and
 // the work counts, 32 from there on, where the rounds do.  FP64, bound by its
-// issue rate, takes 8 throughout (331 x 198: 20.5 ms in all with 32 and the
-// longer reciprocal, 15.3 so).  The bracket is
+// issue rate, takes 8 throughout.  The bracket is
 // (eps^2 lambda_max, Gershgorin bound).  The FP64 factor places them in FP32
 // first and confirms and refines that bracket in FP64.
 // ---------------------------------------------------------------------------
@@ -647,7 +634,7 @@ __device__ void eigvals(const EigTask<T> &t, int first, const double *d, const d
   const int j = min(jj, k2 - 1);
   // scaled as the arrays are
   const double thr = t.sb[0] * scf, hi0 = t.sb[1] * scf, emax = t.sb[2] * scf * scf, tnorm = *t.tnorm * scf;
-  const float pivf = sturm_pivmin<float>((float)emax);
+  const float pivf = sturm_pivmin((float)emax);
   float lo = (float)thr, hi = (float)hi0;
   const float tol = 4.f * unit_round<float>() * (float)tnorm;
   for (int round = 0; round < 12 && __any_sync(0xffffffffu, hi - lo > tol); ++round)
@@ -656,7 +643,7 @@ __device__ void eigvals(const EigTask<T> &t, int first, const double *d, const d
   if constexpr (sizeof(T) == 4) {
     if (jj < k2 && lane % LN == 0) t.lam[jj] = 0.5f * (lo + hi);
   } else {
-    const double piv = sturm_pivmin<double>(emax);
+    const double piv = sturm_pivmin(emax);
     auto above = [&](double s) { return count_above<double>(d, e2, m, s, piv) > j; };
     const double mid = 0.5 * ((double)lo + (double)hi), w = 64.0 * 1.2e-7 * tnorm;
     double l = mid - w, h = mid + w;
