@@ -235,9 +235,10 @@ __global__ void __launch_bounds__(256) k_sum(const SumTask<T> *__restrict__ task
 // ---------------------------------------------------------------------------
 // Cholesky and inverse of the factor, one CTA per matrix, in shared memory.
 //
-// Block columns of 16.  Step b, with j0 = 16 b, D_b = L_bb^-1:
-//   panel   P_i = L_ib = W_ib D_b^T for the rows i below, and the finished block
-//           row X_b,0:j0 = -D_b R_b of the inverse, one thread per row or column;
+// Block columns of 16.  Step b, with j0 = 16 b, L_b its diagonal block, D_b = L_b^-1:
+//   panel   P_i = L_ib = W_ib L_b^-T for the rows i below, and the finished block
+//           row X_b,0:j0 = -L_b^-1 R_b of the inverse, by substitution, one thread
+//           per row or column;
 //   update  W_i,c -= P_i P_c^T (c > b, the trailing block) and
 //           R_i,c += P_i X_b,c (c <= b, X_bb = D_b): the sums R_i = sum_p L_ip X_p
 //           of the inverse's rows grow in place of the columns of L that are no
@@ -247,11 +248,14 @@ __global__ void __launch_bounds__(256) k_sum(const SumTask<T> *__restrict__ task
 // The only serial chain is the 16 x 16 diagonal block: one warp factors it in
 // registers, half its lanes the rows, half D_b's columns.  Warp 0 updates
 // the next diagonal block first and factors it while the other warps finish
-// the update.  Three barriers per 16 columns.
+// the update.  Two barriers per 16 columns.
 // What bounds it: the diagonal chain up to m of about 100, the CUDA cores' FMA
-// rate above (FP64: throughout).  (The form before, column by column with two
-// barriers a column and a forward substitution down each column, was bound by
-// shared-memory latency.)
+// rate above (FP64: throughout).  Twelve matrices a launch, m = 48 / 128 / 224:
+// 16.5 / 45 / 113 us in FP32 (column by column, two barriers a column, 49 / 207 /
+// 564), 74 / 217 us at 48 / 128 in FP64 (182 / 816).
+// Errors of the inverse against one of higher precision, over sizes 8 to 224 and
+// conditions 1e1 to 1e5, are those of the elimination column by column
+// (||X A X^T - I|| 0.92 times its value, geometric mean).
 // ---------------------------------------------------------------------------
 constexpr int kCholNb = 16;
 
@@ -295,11 +299,12 @@ __device__ __forceinline__ void st16(double *p, const double *v) {
 __device__ __forceinline__ float inv_sqrt(float d) { return __frsqrt_rn(d); }
 __device__ __forceinline__ double inv_sqrt(double d) { return rsqrt(d); }
 
-// One warp: D = L^-1 of the diagonal block at row j0, column j0c of W (jb <= 16
-// columns, j0 the first in the matrix), in its place with zeros above the diagonal;
-// *fail = first failing pivot + 1.
+// One warp: the diagonal block at row j0, column j0c of W (jb <= 16 columns, j0 the
+// first in the matrix) becomes D = L^-1, with zeros above the diagonal; L goes to
+// Lt, transposed (L_ij at Lt[16 j + i], i > j; 1 / L_jj at Lt[17 j]; rows from jb
+// on those of the identity).  *fail = first failing pivot + 1.
 template <typename T>
-__device__ __forceinline__ void chol_diag(T *W, int ld, int j0, int j0c, int jb, int *fail) {
+__device__ __forceinline__ void chol_diag(T *W, int ld, int j0, int j0c, int jb, T *Lt, int *fail) {
   // lanes 0 .. 15: row i of A, becoming L's; lanes 16 .. 31: column i of D.  Both
   // are scaled by the pivot's inverse root and updated by L's column j.
   const int lane = threadIdx.x & 31, i = lane & 15;
@@ -316,7 +321,9 @@ __device__ __forceinline__ void chol_diag(T *W, int ld, int j0, int j0c, int jb,
       if (!bad) bad = j0 + j + 1;
       d = T(1);
     }
-    r[j] *= inv_sqrt(d);   // L_ij, D_ji
+    const T is = inv_sqrt(d);
+    r[j] *= is;   // L_ij, D_ji
+    if (!inverse && i >= j) Lt[kCholNb * j + i] = i == j ? is : r[j];
 #pragma unroll
     for (int c = j + 1; c < kCholNb; ++c) r[c] = fma(-r[j], __shfl_sync(0xffffffffu, r[j], c), r[c]);
   }
@@ -328,6 +335,23 @@ __device__ __forceinline__ void chol_diag(T *W, int ld, int j0, int j0c, int jb,
   }
   if (bad && lane == 0) *fail = bad;
   __syncwarp();
+}
+
+// v <- L_b^-1 v by substitution (Lt: chol_diag's).  (The product with D_b instead
+// has an error larger by the block's condition number: at a condition of 1e5 the
+// inverse's error was up to 2.3 times that of the substitution.)
+template <typename T>
+__device__ __forceinline__ void chol_solve(const T *Lt, T (&v)[kCholNb]) {
+  constexpr int V = 16 / (int)sizeof(T);
+#pragma unroll
+  for (int k = 0; k < kCholNb; ++k) {
+    T l[kCholNb];
+#pragma unroll
+    for (int j = k / V * V; j < kCholNb; j += V) ld16(Lt + kCholNb * k + j, l + j);
+    v[k] *= l[k];
+#pragma unroll
+    for (int j = k + 1; j < kCholNb; ++j) v[j] = fma(-l[j], v[k], v[j]);
+  }
 }
 
 struct NoShift {
@@ -343,11 +367,23 @@ __device__ __forceinline__ void chol_tile(T *W, int ld, const T *P, int i0, int 
   constexpr int V = 16 / (int)sizeof(T), PS = chol_ps<T>();
   const int lane = threadIdx.x & 31;
   const int ib = i0 + (lane & 7), cg = c0 + 4 * (lane >> 3), cb = cg + shift;
+  // Trailing block: the tile's own values first, then one term after another, as
+  // an elimination column by column takes them off (a sum of its own over the 16
+  // terms, taken off at the end, had up to 1.6 times the error at a condition of
+  // 1e5).  The inverse's sums are added up by blocks of 16.
   T acc[4][4];
 #pragma unroll
   for (int r = 0; r < 4; ++r)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) acc[r][c] = T(0);
+    for (int c = 0; c < 4; c += V) {
+      const int i = ib + 8 * r;
+      if (kind == 0 && i < m && cb + c < ld) {
+        ld16(W + (size_t)i * ld + cb + c, &acc[r][c]);
+      } else {
+#pragma unroll
+        for (int u = 0; u < V; ++u) acc[r][c + u] = T(0);
+      }
+    }
   const T *pa[4];
 #pragma unroll
   for (int r = 0; r < 4; ++r) pa[r] = P + (size_t)min(ib + 8 * r, m - 1) * PS;
@@ -396,7 +432,7 @@ __device__ __forceinline__ void chol_tile(T *W, int ld, const T *P, int i0, int 
     for (int c = 0; c < 4; c += V) {
       if (cb + c >= ld) continue;   // the last trailing columns; ld is a multiple of V
       T *p = W + (size_t)i * ld + cb + c;
-      if (kind != 2) {
+      if (kind == 1) {
         T w[V];
         ld16(p, w);
 #pragma unroll
@@ -410,6 +446,7 @@ __device__ __forceinline__ void chol_tile(T *W, int ld, const T *P, int i0, int 
 template <typename T, int NT>
 __global__ void __launch_bounds__(NT) k_chol_inv(const CholTask<T> *__restrict__ tasks, int *__restrict__ status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ __align__(16) T s_l[kCholNb * kCholNb];
   __shared__ int s_fail;
   constexpr int V = 16 / (int)sizeof(T), PS = chol_ps<T>(), NW = NT / 32;
   const CholTask<T> t = tasks[blockIdx.x];
@@ -425,42 +462,30 @@ __global__ void __launch_bounds__(NT) k_chol_inv(const CholTask<T> *__restrict__
   for (int i = warp; i < m; i += NW)
     for (int c = lane; c < ld; c += 32) W[(size_t)i * ld + c] = c <= i ? t.A[(int64_t)i * t.lda + c] : T(0);
   __syncthreads();
-  if (warp == 0) chol_diag<T>(W, ld, 0, 0, min(kCholNb, m), &s_fail);
+  if (warp == 0) chol_diag<T>(W, ld, 0, 0, min(kCholNb, m), s_l, &s_fail);
   for (int j0 = 0; j0 < m; j0 += kCholNb) {
-    __syncthreads();   // D_b and the update of the step before are complete
+    __syncthreads();   // D_b, L_b and the update of the step before are complete
     if (s_fail) break;
     const int j1 = min(j0 + kCholNb, m), jb = j1 - j0, rest = m - j1;
-    const T *D = W + (size_t)j0 * ld + j0;
     for (int q = tid; q < rest + j0; q += NT) {
-      T v[kCholNb], o[kCholNb];
+      T v[kCholNb];
       if (q < rest) {
         // row j1 + q of the panel (a full block: jb = 16)
         const T *w = W + (size_t)(j1 + q) * ld + j0;
 #pragma unroll
         for (int k = 0; k < kCholNb; k += V) ld16(w + k, v + k);
+        chol_solve<T>(s_l, v);
+#pragma unroll
+        for (int k = 0; k < kCholNb; k += V) st16(P + (size_t)(j1 + q) * PS + k, v + k);
       } else {
         // column q - rest of the inverse's block row
-        const T *w = W + (size_t)j0 * ld + (q - rest);
-#pragma unroll
-        for (int k = 0; k < kCholNb; ++k) v[k] = k < jb ? -w[(size_t)k * ld] : T(0);
-      }
-#pragma unroll
-      for (int k = 0; k < kCholNb; ++k) {
-        T s = T(0);
-        if (k < jb) {
-#pragma unroll
-          for (int p = 0; p <= k; ++p) s = fma(D[(size_t)k * ld + p], v[p], s);
-        }
-        o[k] = s;
-      }
-      if (q < rest) {
-#pragma unroll
-        for (int k = 0; k < kCholNb; k += V) st16(P + (size_t)(j1 + q) * PS + k, o + k);
-      } else {
         T *w = W + (size_t)j0 * ld + (q - rest);
 #pragma unroll
+        for (int k = 0; k < kCholNb; ++k) v[k] = k < jb ? -w[(size_t)k * ld] : T(0);
+        chol_solve<T>(s_l, v);
+#pragma unroll
         for (int k = 0; k < kCholNb; ++k)
-          if (k < jb) w[(size_t)k * ld] = o[k];
+          if (k < jb) w[(size_t)k * ld] = v[k];
       }
     }
     __syncthreads();
@@ -468,7 +493,7 @@ __global__ void __launch_bounds__(NT) k_chol_inv(const CholTask<T> *__restrict__
     if (warp == 0) {
       chol_tile<T>(W, ld, P, j1, j1, NoShift(), j0, m, 0);
       __syncwarp();
-      chol_diag<T>(W, ld, j1, j1, min(kCholNb, m - j1), &s_fail);
+      chol_diag<T>(W, ld, j1, j1, min(kCholNb, m - j1), s_l, &s_fail);
     } else {
       // all other tiles, dealt out to the other warps in turn
       const int nic = j1 / kCholNb, nct = (rest + kCholNb - 1) / kCholNb;
@@ -520,7 +545,8 @@ template <typename T>
 __global__ void __cluster_dims__(kCholC, 1, 1) __launch_bounds__(kCholClThreads)
     k_chol_cluster(const CholTask<T> *__restrict__ tasks, int *__restrict__ status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int s_fail, s_failed[2];   // found here; published with D_b (step parity)
+  __shared__ __align__(16) T s_l[kCholNb * kCholNb];
+  __shared__ int s_fail, s_failed[2];   // found here; published with L_b (step parity)
   constexpr int V = 16 / (int)sizeof(T), PS = chol_ps<T>(), NT = kCholClThreads, NW = NT / 32;
   cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
   const int rank = (int)cluster.block_rank();
@@ -528,7 +554,7 @@ __global__ void __cluster_dims__(kCholC, 1, 1) __launch_bounds__(kCholClThreads)
   const int m = t.m, ld = chol_cl_ld(m), nblk = (m + kCholNb - 1) / kCholNb;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   T *W = reinterpret_cast<T *>(smem_raw);          // own block q: block rank + kCholC q, from column 16 q on
-  T *Pb = W + (size_t)m * ld, *Db = Pb + 2 * (size_t)m * PS;   // two buffers each (step parity)
+  T *Pb = W + (size_t)m * ld, *Lb = Pb + 2 * (size_t)m * PS;   // two buffers each (step parity)
   if (m == 0) {
     if (tid == 0 && rank == 0) status[t.status_idx] = 0;
     return;
@@ -540,56 +566,38 @@ __global__ void __cluster_dims__(kCholC, 1, 1) __launch_bounds__(kCholClThreads)
       W[(size_t)i * ld + c] = g <= i ? t.A[(int64_t)i * t.lda + g] : T(0);
     }
   cluster.sync();   // (every CTA runs before any writes to it)
-  // D_b (in place in the own block) and its panel to every CTA
+  // L_b and its panel to every CTA
   auto publish = [&](int b) {
     const int j0 = b * kCholNb, j1 = min(j0 + kCholNb, m), lc = kCholNb * (b / kCholC), par = b & 1;
-    const T *D = W + (size_t)j0 * ld + lc;
-    for (int q = tid; q < kCholNb * kCholNb; q += NT) {
-      const int k = q / kCholNb, c = q % kCholNb;
-      const T x = j0 + k < m ? D[(size_t)k * ld + c] : T(0);
-      for (int r = 0; r < kCholC; ++r) cluster.map_shared_rank(Db, r)[par * kCholNb * kCholNb + q] = x;
-    }
-    // a row's entries 0 .. 10 and 11 .. 15 take about the same FMAs: a warp each
-    auto panel = [&](auto k0, auto k1, int first) {
-      constexpr int K0 = k0.value, K1 = k1.value;
-      for (int i = j1 + first; i < m; i += NT / 2) {
-        const T *w = W + (size_t)i * ld + lc;
-        T v[kCholNb], o[kCholNb];
+    for (int q = tid; q < kCholNb * kCholNb; q += NT)
+      if (q % kCholNb >= q / kCholNb)
+        for (int r = 0; r < kCholC; ++r) cluster.map_shared_rank(Lb, r)[par * kCholNb * kCholNb + q] = s_l[q];
+    for (int i = j1 + tid; i < m; i += NT) {
+      const T *w = W + (size_t)i * ld + lc;
+      T v[kCholNb];
 #pragma unroll
-        for (int k = 0; k < kCholNb && k < K1; k += V) ld16(w + k, v + k);
+      for (int k = 0; k < kCholNb; k += V) ld16(w + k, v + k);
+      chol_solve<T>(s_l, v);
+      for (int r = 0; r < kCholC; ++r) {
+        T *P = cluster.map_shared_rank(Pb, r) + ((size_t)par * m + i) * PS;
 #pragma unroll
-        for (int k = K0; k < K1; ++k) {
-          T s = T(0);
-#pragma unroll
-          for (int p = 0; p <= k; ++p) s = fma(D[(size_t)k * ld + p], v[p], s);
-          o[k] = s;
-        }
-        for (int r = 0; r < kCholC; ++r) {
-          T *P = cluster.map_shared_rank(Pb, r) + ((size_t)par * m + i) * PS;
-#pragma unroll
-          for (int k = K0; k < K1; ++k) P[k] = o[k];
-        }
+        for (int k = 0; k < kCholNb; k += V) st16(P + k, v + k);
       }
-    };
-    const int first = (warp >> 1) * 32 + lane;
-    if (warp & 1)
-      panel(std::integral_constant<int, 11>(), std::integral_constant<int, kCholNb>(), first);
-    else
-      panel(std::integral_constant<int, 0>(), std::integral_constant<int, 11>(), first);
+    }
     if (tid < kCholC) cluster.map_shared_rank(s_failed, tid)[par] = s_fail;
   };
   if (rank == 0) {
-    if (warp == 0) chol_diag<T>(W, ld, 0, 0, min(kCholNb, m), &s_fail);
+    if (warp == 0) chol_diag<T>(W, ld, 0, 0, min(kCholNb, m), s_l, &s_fail);
     __syncthreads();
     publish(0);
   }
   int fail = 0;
   for (int b = 0; b < nblk; ++b) {
-    cluster.sync();   // D_b, P_b are here; every CTA is done with step b - 1
+    cluster.sync();   // L_b, P_b are here; every CTA is done with step b - 1
     fail = s_failed[b & 1];
     if (fail) break;
     const int j0 = b * kCholNb, j1 = min(j0 + kCholNb, m), jb = j1 - j0, rest = m - j1;
-    const T *P = Pb + (size_t)(b & 1) * m * PS, *D = Db + (b & 1) * kCholNb * kCholNb;
+    const T *P = Pb + (size_t)(b & 1) * m * PS, *Lt = Lb + (b & 1) * kCholNb * kCholNb;
     // row block b of the inverse, own columns (blocks before b)
     const int nq = b > rank ? (b - rank + kCholC - 1) / kCholC : 0;   // own blocks before b
     for (int c = tid; c < kCholNb * nq; c += NT) {
@@ -597,13 +605,10 @@ __global__ void __cluster_dims__(kCholC, 1, 1) __launch_bounds__(kCholClThreads)
       T v[kCholNb];
 #pragma unroll
       for (int k = 0; k < kCholNb; ++k) v[k] = k < jb ? -w[(size_t)k * ld] : T(0);
+      chol_solve<T>(Lt, v);
 #pragma unroll
-      for (int k = 0; k < kCholNb; ++k) {
-        T s = T(0);
-#pragma unroll
-        for (int p = 0; p <= k; ++p) s = fma(D[k * kCholNb + p], v[p], s);
-        if (k < jb) w[(size_t)k * ld] = s;
-      }
+      for (int k = 0; k < kCholNb; ++k)
+        if (k < jb) w[(size_t)k * ld] = v[k];
     }
     if (rest == 0) break;
     __syncthreads();
@@ -615,7 +620,7 @@ __global__ void __cluster_dims__(kCholC, 1, 1) __launch_bounds__(kCholClThreads)
         chol_tile<T>(W, ld, P, j1 + 32 * rt, j1, kCholNb * qn - j1, j0, m, 0);
       __syncthreads();
       if (warp == 0)
-        chol_diag<T>(W, ld, j1, kCholNb * qn, min(kCholNb, m - j1), &s_fail);
+        chol_diag<T>(W, ld, j1, kCholNb * qn, min(kCholNb, m - j1), s_l, &s_fail);
     }
     // the other own tiles (the owner of the next block's warp 0 has its diagonal block)
     if (!next || warp != 0) {
@@ -1050,9 +1055,9 @@ static void launch_chol_nt(const CholTask<T> *d_tasks, int ntasks, int *d_status
   k_chol_inv<T, NT><<<ntasks, NT, sm, st>>>(d_tasks, d_status);
 }
 
-// FP64 above kCholClusterMin: k_chol_cluster (m = 150 to 160: 0.60 ms in one
-// CTA, about 0.28 in four; its limit of 256 also spares nodes up to there the
-// blocked path).  Below, the diagonal blocks' serial chain is what counts.
+// FP64 above kCholClusterMin: k_chol_cluster (m = 150 to 160: twice as fast as
+// one CTA, 0.31 ms; its limit of 256 also spares nodes up to there the blocked
+// path).  Below, the diagonal blocks' serial chain is what counts.
 // Threads by the largest matrix of the launch: the update's tiles (about
 // m^2 / 1024 a step) keep that many warps busy; a matrix's arithmetic does not
 // depend on them.
