@@ -1803,6 +1803,7 @@ void trunc_big(Exec &ex, const std::vector<TruncTask<T>> &all, int *d_k, int var
     }
     if (tri_cluster_enabled()) {
       const int n2 = tri_onchip_max<T>(), k0 = t.m - n2, qt = tri_class<T>(n2);
+      if (qt < 0 || k0 <= 0) fail(HS_ERR_INVALID, "internal: class of the tridiagonalisation");
       g.kend = k0;
       GridTri<T> x = g;
       x.A += (size_t)k0 * g.ld + k0;

@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "../../include/hs.h"
+#include "tri_pick.h"
 
 namespace hs {
 
@@ -354,10 +355,9 @@ void launch_tri_step(const GridTri<T> *d_tasks, int ntasks, int total_blocks, in
 // the whole tridiagonalisation of each node (or trailing block) on chip
 // (kernels_cluster.cu): class 0 in one CTA, class q in a cluster of 2^q; -1 when
 // none holds a block of size m.  All tasks of a launch are of one class.
-constexpr int kTriClasses = 5;
 template <typename T>
 int tri_class(int m);
-// the largest block any class holds
+// the largest block any class holds (tri_class is -1 above it only)
 template <typename T>
 int tri_onchip_max();
 template <typename T>

@@ -486,10 +486,10 @@ size_t cluster_room() {
   return n > 0 ? sm : 0;
 }
 
-// Largest m that one CTA (q = 0) or a cluster of 2, 4, 8 or 16 CTAs (q = 1 ..
+// Largest m that one CTA (class 0) or a cluster of 2, 4, 8 or 16 CTAs (classes 1 ..
 // 4) takes, 0 if such a cluster cannot be resident; once per device.
 template <typename T>
-int tri_max_m(int q) {
+const int (&tri_max_m())[kTriClasses] {
   static std::mutex mu;
   static int table[64][kTriClasses];
   static bool ready[64] = {false};
@@ -509,17 +509,11 @@ int tri_max_m(int q) {
     }
     ready[dev] = true;
   }
-  return table[dev][q];
+  return table[dev];
 }
 
 }  // namespace
 
-// FP32: one CTA while it fits, then 4 CTAs (a step is bound by its barriers and
-// distributed reads, which cost 2 CTAs as much), then 8, then 16.
-// FP64: the arithmetic itself (3 n^2 FMAs a step at 1/64 of the FP32 rate)
-// outgrows the barriers from about n = 112 on, so 8 CTAs share it from there (88:
-// the same) and 16 from n = 161 on (a 331 x 198 factorization 171.6 ms with 8
-// only, 166.3 with 16 from 161, 166.1 from 129, 167.0 from 113).
 // HS_TRI_CLUSTER=1 (environment) keeps to one CTA, =2 takes the smallest
 // cluster that fits.
 static int tri_mode() {
@@ -531,25 +525,12 @@ static int tri_mode() {
 }
 template <typename T>
 int tri_class(int m) {
-  const int mode = tri_mode();
-  if (mode == 1) return m <= tri_max_m<T>(0) ? 0 : -1;
-  int first = 0;
-  if (mode == 0) {
-    if (sizeof(T) == 8 && m > 112)
-      first = m > 160 ? 4 : 3;
-    else if (m > tri_max_m<T>(0))
-      first = 2;
-  }
-  for (int q = first; q < kTriClasses; ++q)
-    if (m <= tri_max_m<T>(q)) return q;
-  return -1;
+  return tri_pick(tri_max_m<T>(), m, sizeof(T) == 8, tri_mode());
 }
 
 template <typename T>
 int tri_onchip_max() {
-  int mm = 0;
-  for (int q = 0; q < (tri_mode() == 1 ? 1 : kTriClasses); ++q) mm = std::max(mm, tri_max_m<T>(q));
-  return mm;
+  return tri_pick_max(tri_max_m<T>(), tri_mode());
 }
 
 template <typename T>
