@@ -861,8 +861,9 @@ __global__ void __launch_bounds__(TRUNC_THREADS) k_trunc(const TruncTask<T> *__r
   if (variant != HS_LORASP)
     k1 = gc_basis_dev<T>(t.phi, t.a, t.np, m, variant == HS_GC_PROJ, t.eps1, t.U, (double *)A, red, s_gR, s_gW,
                          &s_gk);
-  // ---- ||A_sw||_2^2 = lambda_max(G)
-  for (int64_t e = tid; e < (int64_t)m * m; e += nt) A[e] = t.G[e];
+  // ---- ||A_sw||_2^2 = lambda_max(G), of G scaled near 1 (as J below)
+  const Pow2<T> f = gram_scale(t.G, m, red);
+  for (int64_t e = tid; e < (int64_t)m * m; e += nt) A[e] = f(t.G[e]);
   __syncthreads();
   const int max_sweeps = 40;
   double thr;
@@ -927,7 +928,7 @@ __global__ void __launch_bounds__(TRUNC_THREADS) k_trunc(const TruncTask<T> *__r
           v = fma(-ui, V[j * m + a], fma(-V[i * m + a], uj, v));
           for (int b = 0; b < k1; ++b) v = fma(ui * c[a][b], t.U[(int64_t)j * m + b], v);
         }
-        A[e] = v;
+        A[e] = f(v);
       }
     } else {
       for (int64_t e = tid; e < (int64_t)m * m; e += nt) {
@@ -938,7 +939,7 @@ __global__ void __launch_bounds__(TRUNC_THREADS) k_trunc(const TruncTask<T> *__r
           v = fma(-ui, V[j * m + a], fma(-V[i * m + a], uj, v));
           for (int b = 0; b < k1; ++b) v = fma(ui * s_c[a * kMaxK1 + b], t.U[(int64_t)j * m + b], v);
         }
-        A[e] = v;
+        A[e] = f(v);
       }
     }
     thr = eps * eps * lmax;

@@ -5,7 +5,8 @@
 //   1. k_trunc_prep (one CTA per node): GC basis U_1 = orth[phi_s, A_sw phi_w]
 //      (Sec. 6; Appendix B: its dominant left singular vectors), J = G (LoRaSp)
 //      or (I - U1 U1^T) G (I - U1 U1^T) (GC), and with C = U1^T G U1 the
-//      coupling X = (I - U1 U1^T) G U1 of the two blocks of G.
+//      coupling X = (I - U1 U1^T) G U1 of the two blocks of G; J, X and C times
+//      a power of two that brings G's largest diagonal entry near 1.
 //   2. J = Q T Q^T (kernels_cluster.cu, or the step kernels below), and
 //      Z = Q^T X (k_qmul).
 //   3. k_rank (one CTA per node): ||A_sw||_2^2 = lambda_max(G), from T (LoRaSp)
@@ -235,9 +236,10 @@ __device__ __forceinline__ int section(R &lo, R &hi, int lane, bool closed, F &&
 
 // J = G - U1 X^T - X U1^T + U1 c U1^T (the Gram matrix projected off span U_1),
 // X = G U1 in Y's columns and U1 in U's (column a at + a m), c in shared memory
-// (ld kMaxK1); one warp per row.  KB >= k1 sizes the per-row registers.
+// (ld kMaxK1), times f; one warp per row.  KB >= k1 sizes the per-row registers.
 template <typename T, int KB>
-__device__ void build_projected_gram(const T *G, const T *U, const T *Y, const T *s_c, T *A, int m, int k1) {
+__device__ void build_projected_gram(const T *G, const T *U, const T *Y, const T *s_c, T *A, int m, int k1,
+                                     const Pow2<T> &f) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
   for (int i = warp; i < m; i += nw) {
     T ui[KB], xi[KB], cu[KB];
@@ -263,7 +265,7 @@ __device__ void build_projected_gram(const T *G, const T *U, const T *Y, const T
           v = fma(-ui[a], Y[(size_t)a * m + j], fma(-xi[a], uj, v));
           v = fma(cu[a], uj, v);
         }
-      A[(int64_t)i * m + j] = v;
+      A[(int64_t)i * m + j] = f(v);
     }
   }
 }
@@ -272,8 +274,8 @@ __device__ void build_projected_gram(const T *G, const T *U, const T *Y, const T
 // allocation of the one-vector path
 template <typename T>
 __device__ __noinline__ void build_projected_gram_wide(const T *G, const T *U, const T *Y, const T *s_c, T *A,
-                                                       int m, int k1) {
-  build_projected_gram<T, kMaxK1>(G, U, Y, s_c, A, m, k1);
+                                                       int m, int k1, const Pow2<T> &f) {
+  build_projected_gram<T, kMaxK1>(G, U, Y, s_c, A, m, k1, f);
 }
 
 // U_1, J, X and C of one node, or the complete basis (eps = 0)
@@ -298,7 +300,8 @@ __global__ void __launch_bounds__(NT) k_trunc_prep(const TruncTask<T> *__restric
       if (tid == 0) kout[t.k_idx] = m;
       return;
     }
-    for (int64_t q = tid; q < (int64_t)m * m; q += nt) A[q] = t.G[q];
+    const Pow2<T> f = gram_scale(t.G, m, red);
+    for (int64_t q = tid; q < (int64_t)m * m; q += nt) A[q] = f(t.G[q]);
     if (tid == 0) L.sc_int[0] = 0;
     return;
   }
@@ -344,20 +347,21 @@ __global__ void __launch_bounds__(NT) k_trunc_prep(const TruncTask<T> *__restric
       if (tid == 0) s_c[a * kMaxK1 + bb] = cab;
     }
   __syncthreads();
+  const Pow2<T> f = gram_scale(t.G, m, red);
   if (k1 <= 2)
-    build_projected_gram<T, 2>(t.G, Uc, Y, s_c, A, m, k1);
+    build_projected_gram<T, 2>(t.G, Uc, Y, s_c, A, m, k1, f);
   else
-    build_projected_gram_wide<T>(t.G, Uc, Y, s_c, A, m, k1);
+    build_projected_gram_wide<T>(t.G, Uc, Y, s_c, A, m, k1, f);
   // X = G U1 - U1 C (the scratch in LS is no longer in use)
   T *X = L.LS;
   for (int64_t q = tid; q < (int64_t)m * k1; q += nt) {
     const int a = (int)(q / m), i = (int)(q % m);
     T x = Y[(size_t)a * m + i];
     for (int b = 0; b < k1; ++b) x = fma(-Uc[(size_t)b * m + i], s_c[b * kMaxK1 + a], x);
-    X[(size_t)a * m + i] = x;
+    X[(size_t)a * m + i] = f(x);
   }
   if (tid == 0) L.sc_int[0] = k1;
-  for (int q = tid; q < kMaxK1 * kMaxK1; q += nt) L.sc_c[q] = (double)s_c[q];
+  for (int q = tid; q < kMaxK1 * kMaxK1; q += nt) L.sc_c[q] = (double)f(s_c[q]);
 }
 
 // ---------------------------------------------------------------------------
@@ -462,42 +466,27 @@ __global__ void __launch_bounds__(kRankThreads) k_rank(const TruncTask<T> *__res
     ctr += fmax(c, 0.0);
     cmax = fmax(cmax, c);
   }
-  const double hi_u = (fmax(ghi, 0.0) + ctr) * (1.0 + 1e-4) + (sizeof(T) == 8 ? 1e-290 : 1e-30);
-  // The FP64 factor's T, Z and C times a power of two that brings the
-  // bracket's end near 1 (the values may lie outside the FP32 range, and a
-  // weakly coupled node's far below any absolute floor)
-  const double sc = sizeof(T) == 8 ? exp2(-(double)ilogb(hi_u)) : 1.0;
-  const double hi0 = hi_u * sc, lo0 = fmax(fmax(dmax, cmax), 0.0) * (1.0 - 1e-4) * sc;
-  const double emax_u = emax;
-  emax *= sc * sc;
-  if (sizeof(T) == 8)
-    for (int i = tid; i < m; i += kRankThreads) {
-      const double em = i > 0 ? eat(i - 1) * sc : 0.0;
-      d[i] *= sc;
-      e2[i] = em * em;
-      ed[i] *= sc;
-    }
+  const double hi0 = (fmax(ghi, 0.0) + ctr) * (1.0 + 1e-4) + (sizeof(T) == 8 ? 1e-290 : 1e-30);
+  const double lo0 = fmax(fmax(dmax, cmax), 0.0) * (1.0 - 1e-4);
   for (int i = tid; i < m; i += kRankThreads) {
-    const float e1 = (float)(eat(i) * sc), e0 = i > 0 ? (float)(eat(i - 1) * sc) : 0.f;
+    const float e1 = (float)eat(i), e0 = i > 0 ? (float)eat(i - 1) : 0.f;
     df[i] = (float)d[i];
     ef[i] = e1;
     e2f[i] = e0 * e0;
     if (zs)
       for (int a = 0; a < k1; ++a) {
         const T z = L.LS[(size_t)a * m + i];
-        zf[(size_t)a * mm + i] = (float)((double)z * sc);
-        if (sizeof(T) == 8) zd[(size_t)a * mm + i] = (double)z * sc;
+        zf[(size_t)a * mm + i] = (float)z;
+        if (sizeof(T) == 8) zd[(size_t)a * mm + i] = (double)z;
       }
   }
-  if (!zs && sizeof(T) == 8)   // Z is not used after this kernel
-    for (int64_t q = tid; q < (int64_t)m * k1; q += kRankThreads) L.LS[q] = (T)((double)L.LS[q] * sc);
   for (int q = tid; q < kMaxK1 * kMaxK1; q += kRankThreads) {
-    s_cf[q] = (float)(L.sc_c[q] * sc);
-    s_ct[q] = (T)(L.sc_c[q] * sc);
+    s_cf[q] = (float)L.sc_c[q];
+    s_ct[q] = (T)L.sc_c[q];
   }
   __syncthreads();
   const float pivf = sturm_pivmin((float)emax);
-  double lmax;   // of the scaled G
+  double lmax;   // (of G as k_trunc_prep scales it)
   const bool wide_global = gc && !zs;   // many preserved vectors on a huge node
   {
     float lo = (float)lo0, hi = (float)hi0 * 1.000001f + 1e-37f;
@@ -529,7 +518,7 @@ __global__ void __launch_bounds__(kRankThreads) k_rank(const TruncTask<T> *__res
         const double piv = sturm_pivmin(emax);
         auto above = [&](double sig) {
           if (k1 == 0) return count_above<double>(d, e2, m, sig, piv) >= 1;
-          const double *z = zs ? zd : (const double *)L.LS;   // (beyond shared memory: scaled in place below)
+          const double *z = zs ? zd : (const double *)L.LS;
           const int ldz = zs ? (int)mm : m;
           return (k1 == 1   ? count_above_gc<double, 1>(d, ed, e2, m, z, ldz, k1, s_ct, sig, piv)
                   : k1 == 2 ? count_above_gc<double, 2>(d, ed, e2, m, z, ldz, k1, s_ct, sig, piv)
@@ -584,12 +573,10 @@ __global__ void __launch_bounds__(kRankThreads) k_rank(const TruncTask<T> *__res
     if (fabs(q) < piv) q = -piv;
     int k2 = m - (s_cnt[0] + s_cnt[1] + (q < 0.0 ? 1 : 0));
     k2 = max(0, min(k2, min(m - k1, t.cap - k1)));   // max_rank_ratio: the largest eigenvalues are kept
-    // a block whose Gram matrix has left the FP64 range has nothing to keep
-    if (sizeof(T) == 8 && hi_u < 1e-280) k2 = 0;
     L.sc_int[1] = k2;
-    L.sc_b[0] = thr / sc;
+    L.sc_b[0] = thr;
     L.sc_b[1] = ghi + unit_round<T>() * tnorm * 2.0 * m + (sizeof(T) == 8 ? 1e-290 : 1e-30);
-    L.sc_b[2] = emax_u;
+    L.sc_b[2] = emax;
     *L.sc_tnorm = tnorm;
     kout[t.k_idx] = k1 + k2;
   }
@@ -627,13 +614,12 @@ __device__ __forceinline__ int task_of(const Task *tasks, int ntasks, int b) {
 
 template <typename T, int LN>
 __device__ void eigvals(const EigTask<T> &t, int first, const double *d, const double *e2, const float *df,
-                        const float *e2f, double scf) {
+                        const float *e2f) {
   const int m = t.m, k2 = t.sc[1];
   const int lane = threadIdx.x & 31;
   const int jj = first + (int)threadIdx.x / LN;
   const int j = min(jj, k2 - 1);
-  // scaled as the arrays are
-  const double thr = t.sb[0] * scf, hi0 = t.sb[1] * scf, emax = t.sb[2] * scf * scf, tnorm = *t.tnorm * scf;
+  const double thr = t.sb[0], hi0 = t.sb[1], emax = t.sb[2], tnorm = *t.tnorm;
   const float pivf = sturm_pivmin((float)emax);
   float lo = (float)thr, hi = (float)hi0;
   const float tol = 4.f * unit_round<float>() * (float)tnorm;
@@ -655,7 +641,7 @@ __device__ void eigvals(const EigTask<T> &t, int first, const double *d, const d
     const double told = 4.0 * unit_round<double>() * tnorm;
     for (int round = 0; round < 40 && __any_sync(0xffffffffu, h - l > told); ++round)
       section<double, LN>(l, h, lane, false, above);
-    if (jj < k2 && lane % LN == 0) t.lam[jj] = 0.5 * (l + h) / scf;
+    if (jj < k2 && lane % LN == 0) t.lam[jj] = 0.5 * (l + h);
   }
 }
 
@@ -670,23 +656,20 @@ __global__ void __launch_bounds__(kEigThreads) k_eigval(const EigTask<T> *__rest
   double *d = (double *)smem_raw, *e2 = d + m;
   float *df = sizeof(T) == 8 ? (float *)(e2 + m) : (float *)smem_raw;
   float *e2f = df + m;
-  // as in k_rank: the FP64 factor's T scaled near 1
-  const double scf = sizeof(T) == 8 ? exp2(-(double)ilogb(fmax(t.sb[1], 1e-290))) : 1.0;
   for (int i = threadIdx.x; i < m; i += kEigThreads) {
     const T di = t.dt[i], ei = i > 0 ? t.et[i - 1] : T(0);
-    df[i] = sizeof(T) == 8 ? (float)(di * scf) : (float)di;
-    const float es = sizeof(T) == 8 ? (float)(ei * scf) : (float)ei;
-    e2f[i] = es * es;
+    df[i] = (float)di;
+    e2f[i] = (float)ei * (float)ei;
     if (sizeof(T) == 8) {
-      d[i] = (double)di * scf;
-      e2[i] = ((double)ei * scf) * ((double)ei * scf);
+      d[i] = (double)di;
+      e2[i] = (double)ei * (double)ei;
     }
   }
   __syncthreads();
   if (lanes == 8)
-    eigvals<T, 8>(t, first, d, e2, df, e2f, scf);
+    eigvals<T, 8>(t, first, d, e2, df, e2f);
   else
-    eigvals<T, 32>(t, first, d, e2, df, e2f, scf);
+    eigvals<T, 32>(t, first, d, e2, df, e2f);
 }
 
 // ---------------------------------------------------------------------------

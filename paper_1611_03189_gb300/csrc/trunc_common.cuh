@@ -27,6 +27,36 @@ __device__ __forceinline__ double blk_sum(double v, double *red) {
   return s;
 }
 
+// Times 2^-e, where 2^e is the size of g (1 when g is 0, infinite or NaN): in two
+// factors, for a g near the ends of the range
+template <typename T>
+struct Pow2 {
+  T a, b;
+  __device__ explicit Pow2(T g) {
+    const int e = g > T(0) && isfinite(g) ? ilogb(g) : 0;
+    a = b = scalbn(T(1), -(e / 2));
+    if (e & 1) b *= e > 0 ? T(0.5) : T(2);
+  }
+  __device__ __forceinline__ T operator()(T x) const { return x * a * b; }
+};
+
+// The largest diagonal entry of G brought near 1.  Ranks and bases do not depend on
+// the scale of G, and a power of two changes no bit of what follows; but the
+// squares and pivots of a matrix of entries around 1e-15 (FP32; 1e-150 FP64) would
+// leave the range or fall below the recurrences' smallest pivots.  red: 33 doubles.
+template <typename T>
+__device__ Pow2<T> gram_scale(const T *G, int m, double *red) {
+  T g = T(0);
+  for (int i = threadIdx.x; i < m; i += blockDim.x) g = fmax(g, G[(int64_t)i * m + i]);
+  for (int o = 16; o > 0; o >>= 1) g = fmax(g, __shfl_xor_sync(0xffffffffu, g, o));
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = (double)g;
+  __syncthreads();
+  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) g = fmax(g, (T)red[w]);
+  __syncthreads();
+  return Pow2<T>(g);
+}
+
 // Complete the k1 <= 2 orthonormal columns U[:, 0..k1) (row-major, ld m) to an
 // orthonormal basis of R^m, writing columns k1..m-1.  Q = H1 H2 from the
 // Householder QR of U_1; its trailing m - k1 columns span the complement of
