@@ -17,7 +17,8 @@
 // column k and p from the other CTAs besides).  Measured: about 1 us a step in
 // one CTA, 3.4 us in 16 CTAs at n = 900 (8.0 us when every CTA read column k from
 // the CTA that holds it).  The reflector's scalars are kept off the FP64 pipe in
-// FP32 factors (see reflector() below), and computed by one warp in FP64 ones:
+// FP32 factors (reflector.h; the off-diagonal entries' FP64 roots are taken
+// together at the end), and computed by one warp in FP64 ones:
 // every thread computing them in FP64, at 1/64 of the FP32 rate, took more than
 // half of each step.
 // Outputs: d, e (FP64) and tau, reflector k in row k of A (v[0] = 1 implicit,
@@ -33,6 +34,7 @@
 #include <mutex>
 
 #include "hs_internal.h"
+#include "reflector.h"
 
 namespace cg = cooperative_groups;
 
@@ -41,44 +43,6 @@ namespace hs {
 namespace {
 
 constexpr int kClThreads = 512;
-
-// The reflector of x with |x|^2 = xn2 and first entry alpha: beta = -sign(alpha)
-// |x| = (beta, lo), tau = (beta - alpha) / beta, v = x * scale beyond the first
-// entry, scale = 1 / (alpha - beta); tau = 0 when x has no tail.
-// FP32: the square root and both quotients are corrected by their residuals
-// (exact through fused multiply-adds, |beta| kept as s + lo), which gives tau and
-// scale as if computed in higher precision and rounded, with no FP64 at all.
-__device__ __forceinline__ void reflector(float xn2, float alpha, float &scale, float &tau, float &beta, float &lo) {
-  if (!(fmaf(-alpha, alpha, xn2) > 0.f)) {
-    scale = tau = lo = 0.f;
-    beta = alpha;
-    return;
-  }
-  const float a = fabsf(alpha);
-  const float s = sqrtf(xn2), inv = 1.f / s;
-  const float sl = 0.5f * fmaf(-s, s, xn2) * inv;
-  const float sum = a + s, suml = (a - (sum - s)) + sl;   // a <= s
-  const float r = 1.f / sum;
-  const float sc = fmaf(r, fmaf(-sum, r, 1.f) - r * suml, r);
-  const float q = a * inv;
-  tau = 1.f + fmaf(inv, fmaf(-q, s, a) - q * sl, q);
-  scale = copysignf(sc, alpha);
-  beta = -copysignf(s, alpha);
-  lo = alpha < 0.f || (alpha == 0.f && signbit(alpha)) ? sl : -sl;
-}
-__device__ __forceinline__ void reflector(double xn2, double alpha, double &scale, double &tau, double &beta,
-                                          double &lo) {
-  lo = 0.0;
-  if (!(fma(-alpha, alpha, xn2) > 0.0)) {
-    scale = tau = 0.0;
-    beta = alpha;
-    return;
-  }
-  const double a = fabs(alpha), s = sqrt(xn2);
-  scale = copysign(1.0 / (a + s), alpha);
-  tau = 1.0 + a / s;
-  beta = -copysign(s, alpha);
-}
 
 // warp partials of a block sum into red[warp]; complete after a barrier
 template <typename T>
@@ -147,32 +111,31 @@ __global__ void __launch_bounds__(NT) k_tri_cta(const GridTri<T> *__restrict__ t
   T vpi = T(0), wpi = T(0), vk = T(0), wk = T(0);   // pending update: own column, and row k
   __syncthreads();
   for (int k = 0; k + 2 < m; ++k) {
-    // row k (columns >= k) with the pending update, and the norm of its tail
+    // row k (columns >= k) with the pending update, and the norm of its tail beyond k + 1
     T a = T(0);
     if (i >= k && i < m) a = fma(-vk, wpi, fma(-wk, vpi, W[(size_t)k * ld + i]));
     if (half == 0) {
       if (i == k + 1) s_alpha = a;
       if (i == k) s_dk = a;
     }
-    put_partial<T>(half == 0 && i > k ? a * a : T(0), red0);
+    put_partial<T>(half == 0 && i > k + 1 ? a * a : T(0), red0);
     __syncthreads();
-    T scale, tau, beta, lo;
+    T scale, tau, xn2;
     if constexpr (sizeof(T) == 4) {
-      reflector(partial_total<T, NW>(red0), s_alpha, scale, tau, beta, lo);
+      reflector(partial_total<T, NW>(red0), s_alpha, scale, tau, xn2);
     } else {
       if (warp == 0) {
-        reflector(partial_total<T, NW>(red0), s_alpha, scale, tau, beta, lo);
+        reflector(partial_total<T, NW>(red0), s_alpha, scale, tau, xn2);
         if (lane == 0) {
           s_r[0] = scale;
           s_r[1] = tau;
-          s_r[2] = beta;
+          s_r[2] = xn2;
         }
       }
       __syncthreads();
       scale = s_r[0];
       tau = s_r[1];
-      beta = s_r[2];
-      lo = T(0);
+      xn2 = s_r[2];
     }
     const T vi = i == k + 1 ? T(1) : i > k + 1 ? a * scale : T(0);
     if (half == 0 && i < m) {
@@ -181,7 +144,7 @@ __global__ void __launch_bounds__(NT) k_tri_cta(const GridTri<T> *__restrict__ t
     }
     if (tid == 0) {
       t.d[k] = (double)s_dk;
-      t.e[k] = (double)beta + (double)lo;
+      t.e[k] = beta_code(tau, xn2, s_alpha);
       t.tau[k] = tau;
     }
     __syncthreads();
@@ -237,6 +200,7 @@ __global__ void __launch_bounds__(NT) k_tri_cta(const GridTri<T> *__restrict__ t
   }
   // the last pending update on the trailing 2 x 2 block, which is written out
   __syncthreads();
+  for (int k = tid; k + 2 < m; k += NT) t.e[k] = beta_of(t.e[k], t.tau[k] != T(0));
   if (half == 0 && i < m) pk[i] = Pack<T>{vpi, wpi, T(0), T(0)};
   __syncthreads();
   if (half == 0 && i < m && i >= m - 2)
@@ -342,25 +306,24 @@ __global__ void __launch_bounds__(kClThreads) k_tri_cluster(const GridTri<T> *__
       break;
     }
     if (tid < 2) s_x[tid] = col[0];               // entries k and k + 1
-    put_rows(fma(col[1], col[1], tid > 0 ? col[0] * col[0] : T(0)), red0);
+    put_rows(fma(col[1], col[1], tid > 1 ? col[0] * col[0] : T(0)), red0);
     __syncthreads();
-    T scale, beta, lo;
+    T scale, xn2;
     if constexpr (sizeof(T) == 4) {
-      reflector(partial_total<T, NW>(red0), s_x[1], scale, tau, beta, lo);
+      reflector(partial_total<T, NW>(red0), s_x[1], scale, tau, xn2);
     } else {
       if (warp == 0) {
-        reflector(partial_total<T, NW>(red0), s_x[1], scale, tau, beta, lo);
+        reflector(partial_total<T, NW>(red0), s_x[1], scale, tau, xn2);
         if (lane == 0) {
           s_r[0] = scale;
           s_r[1] = tau;
-          s_r[2] = beta;
+          s_r[2] = xn2;
         }
       }
       __syncthreads();
       scale = s_r[0];
       tau = s_r[1];
-      beta = s_r[2];
-      lo = T(0);
+      xn2 = s_r[2];
     }
     const bool owner = (k & (C - 1)) == crank;
 #pragma unroll
@@ -374,7 +337,7 @@ __global__ void __launch_bounds__(kClThreads) k_tri_cluster(const GridTri<T> *__
     }
     if (owner && tid == 0) {
       t.d[k] = (double)col[0];
-      t.e[k] = (double)beta + (double)lo;
+      t.e[k] = beta_code(tau, xn2, s_x[1]);
       t.tau[k] = tau;
     }
     __syncthreads();
@@ -426,6 +389,9 @@ __global__ void __launch_bounds__(kClThreads) k_tri_cluster(const GridTri<T> *__
     }
     cluster.sync();   // every CTA's p is visible; every walk of step k is done
   }
+  // (the barrier also makes thread 0's words visible)
+  __syncthreads();
+  for (int k = crank + C * tid; k + 2 < m; k += C * nt) t.e[k] = beta_of(t.e[k], t.tau[k] != T(0));
   // no CTA may leave while others still read its shared memory
   cluster.sync();
 }

@@ -977,7 +977,7 @@ __global__ void __launch_bounds__(kQmWarps * 32) k_qmul(const QmulTask<T> *__res
 //   phase 0 (k_tri_update): rows i >= k get the rank-2 update of step k - 1,
 //     A_ij -= v_i w_j + w_i v_j (w = p - K v, K = tau p.v / 2 from the CTAs'
 //     partials in block order); then x_i = A_ik for i > k and d_k = A_kk, with
-//     per-CTA partials of |x|^2.
+//     per-CTA partials of |x|^2 beyond x's first entry.
 //   phase 1 (k_tri_symv): every CTA forms the reflector of x from the partials
 //     (same arithmetic in every CTA), v_i for its rows, p_i = tau sum_j A_ij v_j,
 //     and per-CTA partials of p.v; v is also kept in row k of A for the later
@@ -1055,7 +1055,7 @@ __global__ void __launch_bounds__(kTriRows * 32) k_tri_update(const GridTri<T> *
         t.d[k] = (double)x;
       } else {
         t.X[i] = x;
-        part = x * x;
+        if (i > k + 1) part = x * x;
       }
     }
   }
@@ -1080,13 +1080,12 @@ __global__ void __launch_bounds__(kTriRows * 32) k_tri_symv(const GridTri<T> *__
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (warp == 0) {
     // the reflector of x = A[k+1.., k] (as in the cluster tridiagonalisation)
-    const double xn2 = (double)warp_sum_parts<T>(t.px, t.nblk, lane);
+    const double tail2 = (double)warp_sum_parts<T>(t.px, t.nblk, lane);
     if (lane == 0) {
       const double alpha = (double)t.X[k + 1];
-      const double sig = xn2 - alpha * alpha;
       double tau = 0.0, beta = alpha, scale = 0.0;
-      if (sig > 0.0) {
-        beta = -copysign(sqrt(xn2), alpha);
+      if (tail2 > (sizeof(T) == 8 ? 1e-290 : 1e-30)) {   // (as in reflector.h)
+        beta = -copysign(sqrt(fma(alpha, alpha, tail2)), alpha);
         tau = (beta - alpha) / beta;
         scale = 1.0 / (alpha - beta);
       }
