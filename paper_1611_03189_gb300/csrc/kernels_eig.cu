@@ -683,11 +683,11 @@ __global__ void __launch_bounds__(kEigThreads) k_eigval(const EigTask<T> *__rest
 // Only the span of the selected vectors matters and the host
 // re-orthonormalises them, which tolerates the overlap u ||T|| / gap that
 // inverse iteration leaves between vectors of distinct eigenvalues.
-// One warp per CTA; a lane's LU (inverse pivots, two super-diagonals,
+// One warp per CTA; a lane's LU (pivots, two super-diagonals,
 // multipliers), vector and interchange flags sit in shared memory, element i
 // of lane s at i * st + s with st odd, so that neither the lanes' sweeps nor
 // the write-out of whole vectors conflict.  A sweep carries its two last
-// values in registers: one fused multiply-add (forward) or two and a product
+// values in registers: one fused multiply-add (forward) or two and a quotient
 // (backward) per row on the dependent chain.
 // ---------------------------------------------------------------------------
 template <typename T>
@@ -706,7 +706,7 @@ __global__ void __launch_bounds__(32) k_invit(const EigTask<T> *__restrict__ tas
   if (q0 >= k2) return;
   const int st = spc | 1;
   const size_t sm = (size_t)m * st;
-  T *iu = (T *)smem_raw + (with_t ? 2 * (size_t)m : 0), *u1 = iu + sm, *u2 = u1 + sm, *lm = u2 + sm, *y = lm + sm;
+  T *u0 = (T *)smem_raw + (with_t ? 2 * (size_t)m : 0), *u1 = u0 + sm, *u2 = u1 + sm, *lm = u2 + sm, *y = lm + sm;
   unsigned char *fl = (unsigned char *)(y + sm);
   const T *dt = t.dt, *et = t.et;   // staged when they fit beside the slots
   if (with_t) {
@@ -742,9 +742,8 @@ __global__ void __launch_bounds__(32) k_invit(const EigTask<T> *__restrict__ tas
         const size_t o = (size_t)i * st + lane;
         const bool swap = fabs(a) < fabs(b);
         T piv = swap ? b : (a == T(0) ? small : a);
-        const T inv = T(1) / piv;
-        const T mult = (swap ? a : b) * inv;
-        iu[o] = fabs(piv) < small ? T(1) / copysign(small, piv) : inv;
+        const T mult = (swap ? a : b) / piv;
+        u0[o] = fabs(piv) < small ? copysign(small, piv) : piv;
         u1[o] = swap ? an : c;
         u2[o] = swap ? cn : T(0);
         lm[o] = mult;
@@ -753,7 +752,7 @@ __global__ void __launch_bounds__(32) k_invit(const EigTask<T> *__restrict__ tas
         c = swap ? -mult * cn : cn;
         a = na;
       }
-      iu[(size_t)(m - 1) * st + lane] = T(1) / (fabs(a) < small ? copysign(small, a) : a);
+      u0[(size_t)(m - 1) * st + lane] = fabs(a) < small ? copysign(small, a) : a;
       for (int i = 0; i < m; ++i) y[(size_t)i * st + lane] = (T)hash_unit(seed, (uint32_t)i);
     }
     T scale = T(1);
@@ -770,13 +769,13 @@ __global__ void __launch_bounds__(32) k_invit(const EigTask<T> *__restrict__ tas
           y[o] = swap ? yn : cur;
           cur = swap ? fma(-l, yn, cur) : fma(-l, cur, yn);
         }
-        T y1 = cur * iu[(size_t)(m - 1) * st + lane], y2 = T(0);
+        T y1 = cur / u0[(size_t)(m - 1) * st + lane], y2 = T(0);
         y[(size_t)(m - 1) * st + lane] = y1;
         big = fabs(y1);
 #pragma unroll 4
         for (int i = m - 2; i >= 0; --i) {
           const size_t o = (size_t)i * st + lane;
-          const T s = fma(-u1[o], y1, fma(-u2[o], y2, y[o])) * iu[o];
+          const T s = fma(-u1[o], y1, fma(-u2[o], y2, y[o])) / u0[o];
           y[o] = s;
           y2 = y1;
           y1 = s;
