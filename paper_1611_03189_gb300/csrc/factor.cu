@@ -1751,7 +1751,8 @@ constexpr int kAuxL = 0, kAuxJacobi = 1, kAuxTri = 2;
 template <typename T>
 void trunc_big(Exec &ex, const std::vector<TruncTask<T>> &all, int *d_k, int variant) {
   std::vector<TruncTask<T>> prep[2], tasks;
-  int pmax[2] = {0, 0}, max_m = 0, max_np = 1;
+  int pmax[2] = {0, 0}, max_m = 0;
+  size_t rbytes = 0;
   for (const TruncTask<T> &t : all) {
     const int c = t.m <= kTruncPrepMid ? 0 : 1;
     prep[c].push_back(t);
@@ -1759,7 +1760,7 @@ void trunc_big(Exec &ex, const std::vector<TruncTask<T>> &all, int *d_k, int var
     if (t.eps > 0.0) {
       tasks.push_back(t);
       max_m = std::max(max_m, t.m);
-      max_np = std::max(max_np, t.np);
+      rbytes = std::max(rbytes, rank_bytes<T>(t.m, t.np, variant));
     }
   }
   // nested spans (phases 10-14) inside the large-truncation span (5)
@@ -1885,7 +1886,7 @@ void trunc_big(Exec &ex, const std::vector<TruncTask<T>> &all, int *d_k, int var
   ex.begin(13);
   {
     const TruncTask<T> *d = ex.list(tasks);
-    ex.op([=] { launch_rank<T>(d, n, d_k, variant, max_m, max_np, o); });
+    ex.op([=] { launch_rank<T>(d, n, d_k, variant, rbytes, o); });
   }
   {
     // eigenvalues and eigenvectors of T (at most m per node)

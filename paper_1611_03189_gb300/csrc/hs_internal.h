@@ -333,10 +333,11 @@ size_t trunc_big_work_elems(int m);
 // U_1, J and X of each node; for eps = 0 the complete basis and its rank instead
 template <typename T>
 void launch_trunc_prep(const TruncTask<T> *d_tasks, int ntasks, int *d_k, int variant, int max_m, cudaStream_t st);
-// ranks from the tridiagonals (max_np: most preserved vectors of the tasks)
+// ranks from the tridiagonals (bytes: the largest rank_bytes of the tasks)
 template <typename T>
-void launch_rank(const TruncTask<T> *d_tasks, int ntasks, int *d_k, int variant, int max_m, int max_np,
-                 cudaStream_t st);
+size_t rank_bytes(int m, int np, int variant);
+template <typename T>
+void launch_rank(const TruncTask<T> *d_tasks, int ntasks, int *d_k, int variant, size_t bytes, cudaStream_t st);
 // CTAs of launch_eigval for a node of size m
 template <typename T>
 int eigval_blocks(int m);

@@ -378,18 +378,26 @@ __global__ void __launch_bounds__(NT) k_trunc_prep(const TruncTask<T> *__restric
 constexpr int kRankThreads = 256;
 
 // dynamic shared memory: d, e2 (FP64), d, e, e2, Z in T, and for the FP64
-// factor also in FP32; Z stays in global memory when it does not fit
+// factor also in FP32; Z stays in global memory when it does not fit, and all of
+// it when the rest does not (0 bytes).  The places decide which recurrences a node
+// runs, so they depend on the node alone, not on what else is in the launch.
+struct RankPlace {
+  int zcols;      // columns of Z in shared memory (room for 2 np, or none)
+  size_t bytes;
+};
 template <typename T>
-__host__ __device__ inline size_t rank_smem_bytes(int m, int zcols) {
+__host__ __device__ inline RankPlace rank_place(int m, int np, bool gc, size_t limit) {
   const size_t mm = (size_t)m + 1;
-  size_t b = 2 * sizeof(double) * mm + (3 + (size_t)zcols) * sizeof(float) * mm;
-  if (sizeof(T) == 8) b += (1 + (size_t)zcols) * sizeof(double) * mm;
-  return b + 64;
+  const size_t base = (2 * sizeof(double) + 3 * sizeof(float) + (sizeof(T) == 8 ? sizeof(double) : 0)) * mm + 64;
+  const size_t col = (sizeof(float) + (sizeof(T) == 8 ? sizeof(double) : 0)) * mm;
+  const int z = gc ? 2 * np : 0;
+  if (base + col * z <= limit) return RankPlace{z, base + col * z};
+  return RankPlace{0, base <= limit ? base : 0};
 }
 
 template <typename T>
 __global__ void __launch_bounds__(kRankThreads) k_rank(const TruncTask<T> *__restrict__ tasks, int *__restrict__ kout,
-                                                      int variant, int zcols, int in_smem) {
+                                                      int variant, size_t limit) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double s_red[3 * kRankThreads / 32];
   __shared__ float s_cf[kMaxK1 * kMaxK1];
@@ -402,6 +410,9 @@ __global__ void __launch_bounds__(kRankThreads) k_rank(const TruncTask<T> *__res
   const BigLayout<T> L = big_layout<T>(t.work, m);
   const bool gc = variant != HS_LORASP;
   const int k1 = gc ? L.sc_int[0] : 0;
+  const RankPlace place = rank_place<T>(m, t.np, gc, limit);
+  const int zcols = place.zcols;
+  const bool in_smem = place.bytes > 0;
   const size_t mm = (size_t)m + 1;
   // (nodes beyond shared memory keep these vectors in Y, which is free until
   // the eigenvectors go there)
@@ -1224,16 +1235,15 @@ void launch_trunc_prep(const TruncTask<T> *d_tasks, int ntasks, int *d_k, int va
 }
 
 template <typename T>
-void launch_rank(const TruncTask<T> *d_tasks, int ntasks, int *d_k, int variant, int max_m, int max_np,
-                 cudaStream_t st) {
+size_t rank_bytes(int m, int np, int variant) {
+  return rank_place<T>(m, np, variant != HS_LORASP, (size_t)allow_max_dynamic_smem<&k_rank<T>>()).bytes;
+}
+
+template <typename T>
+void launch_rank(const TruncTask<T> *d_tasks, int ntasks, int *d_k, int variant, size_t bytes, cudaStream_t st) {
   if (ntasks == 0) return;
-  const int limit = allow_max_dynamic_smem<&k_rank<T>>();
-  int zcols = variant == HS_LORASP ? 0 : 2 * max_np;
-  if (rank_smem_bytes<T>(max_m, zcols) > (size_t)limit) zcols = 0;
-  size_t sm = rank_smem_bytes<T>(max_m, zcols);
-  const int in_smem = sm <= (size_t)limit;
-  if (!in_smem) sm = 0;
-  k_rank<T><<<ntasks, kRankThreads, sm, st>>>(d_tasks, d_k, variant, zcols, in_smem);
+  const size_t limit = (size_t)allow_max_dynamic_smem<&k_rank<T>>();
+  k_rank<T><<<ntasks, kRankThreads, bytes, st>>>(d_tasks, d_k, variant, limit);
   count_launch();
   HS_CUDA(cudaGetLastError());
 }
@@ -1344,7 +1354,8 @@ void launch_refl(const ReflTask<T> *d_tasks, int ntasks, int nb, int m_max, cuda
 
 #define HS_INST(T)                                                                                             \
   template void launch_trunc_prep<T>(const TruncTask<T> *, int, int *, int, int, cudaStream_t);                \
-  template void launch_rank<T>(const TruncTask<T> *, int, int *, int, int, int, cudaStream_t);                 \
+  template size_t rank_bytes<T>(int, int, int);                                                                \
+  template void launch_rank<T>(const TruncTask<T> *, int, int *, int, size_t, cudaStream_t);                   \
   template int eigval_blocks<T>(int);                                                                          \
   template void launch_eigval<T>(const EigTask<T> *, int, int, int, cudaStream_t);                             \
   template int invit_slots<T>(int);                                                                            \
