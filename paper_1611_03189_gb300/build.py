@@ -3,6 +3,8 @@
 Each translation unit is compiled in parallel, then linked into one shared
 library under paper_1611_03189_gb300/_build/.  A unit is rebuilt when its
 source or any header of csrc/ (or include/hs.h) is newer than its object.
+Objects, library and stamp are written beside their places and renamed, so that
+builds that run at the same time never read each other's half-written files.
 """
 from __future__ import annotations
 
@@ -50,10 +52,12 @@ def build(verbose: bool = False, force: bool = False) -> str:
         o = os.path.join(BUILD, src + ".o")
         if not force and os.path.exists(o) and os.path.getmtime(o) >= max(os.path.getmtime(s), hdr):
             return o, None
-        cmd = [nvcc, "-c", s, "-o", o] + common
+        tmp = o + f".tmp{os.getpid()}"
+        cmd = [nvcc, "-c", s, "-o", tmp] + common
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"nvcc failed on {src}:\n{r.stdout}\n{r.stderr}")
+        os.replace(tmp, o)
         return o, (r.stdout + r.stderr) if verbose else None
 
     with ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
