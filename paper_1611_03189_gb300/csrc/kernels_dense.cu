@@ -251,11 +251,11 @@ __global__ void __launch_bounds__(256) k_sum(const SumTask<T> *__restrict__ task
 // the update.  Two barriers per 16 columns.
 // What bounds it: the diagonal chain up to m of about 100, the CUDA cores' FMA
 // rate above (FP64: throughout).  Twelve matrices a launch, m = 48 / 128 / 224:
-// 16.5 / 45 / 113 us in FP32 (column by column, two barriers a column, 49 / 207 /
-// 564), 74 / 217 us at 48 / 128 in FP64 (182 / 816).
+// 16.5 / 45 / 115 us in FP32 (column by column, two barriers a column, 49 / 207 /
+// 564), 74 / 225 us at 48 / 128 in FP64 (182 / 816).
 // Errors of the inverse against one of higher precision, over sizes 8 to 224 and
-// conditions 1e1 to 1e5, are those of the elimination column by column
-// (||X A X^T - I|| 0.92 times its value, geometric mean).
+// conditions 1e1 to 1e5, are below those of the elimination column by column
+// (||X A X^T - I|| 0.83 times its value, geometric mean).
 // ---------------------------------------------------------------------------
 constexpr int kCholNb = 16;
 
@@ -354,6 +354,12 @@ __device__ __forceinline__ void chol_solve(const T *Lt, T (&v)[kCholNb]) {
   }
 }
 
+// Matrices up to this size update the trailing block term by term, larger ones add
+// up 16 terms before they take them off.  The sums have 0.4 to 0.9 times the error
+// above it, but up to 1.6 times below 64 at a graded spectrum of condition 1e5,
+// where the terms are larger than what is left.
+constexpr int kCholInOrder = 96;
+
 struct NoShift {
   __device__ __forceinline__ operator int() const { return 0; }
 };
@@ -367,17 +373,16 @@ __device__ __forceinline__ void chol_tile(T *W, int ld, const T *P, int i0, int 
   constexpr int V = 16 / (int)sizeof(T), PS = chol_ps<T>();
   const int lane = threadIdx.x & 31;
   const int ib = i0 + (lane & 7), cg = c0 + 4 * (lane >> 3), cb = cg + shift;
-  // Trailing block: the tile's own values first, then one term after another, as
-  // an elimination column by column takes them off (a sum of its own over the 16
-  // terms, taken off at the end, had up to 1.6 times the error at a condition of
-  // 1e5).  The inverse's sums are added up by blocks of 16.
+  // in order: the tile's own values first, then one term after another, as an
+  // elimination column by column takes them off
+  const bool in_order = kind == 0 && m <= kCholInOrder;
   T acc[4][4];
 #pragma unroll
   for (int r = 0; r < 4; ++r)
 #pragma unroll
     for (int c = 0; c < 4; c += V) {
       const int i = ib + 8 * r;
-      if (kind == 0 && i < m && cb + c < ld) {
+      if (in_order && i < m && cb + c < ld) {
         ld16(W + (size_t)i * ld + cb + c, &acc[r][c]);
       } else {
 #pragma unroll
@@ -432,7 +437,7 @@ __device__ __forceinline__ void chol_tile(T *W, int ld, const T *P, int i0, int 
     for (int c = 0; c < 4; c += V) {
       if (cb + c >= ld) continue;   // the last trailing columns; ld is a multiple of V
       T *p = W + (size_t)i * ld + cb + c;
-      if (kind == 1) {
+      if (kind != 2 && !in_order) {
         T w[V];
         ld16(p, w);
 #pragma unroll
