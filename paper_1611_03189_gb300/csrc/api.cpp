@@ -104,7 +104,6 @@ void numeric_pre(FactorHandle &h, const double *val, cudaStream_t st) {
 void numeric_failed(FactorHandle &h) {
   h.nodes.clear();
   h.waves.clear();
-  h.levels.clear();
   h.root_m = 0;
 }
 

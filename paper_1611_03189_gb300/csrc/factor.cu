@@ -19,9 +19,9 @@
 //
 // One executor (execute) drives one problem or many independent ones in lock
 // step: at every step (level from the leaves, wave) all problems that have it
-// share the launches.  Truncations of nodes with m >= 128 spread their
-// tridiagonalisation over the GPU (trunc_grid); Cholesky factors above the
-// shared-memory limit are blocked (Exec::chol_inv_blocked).
+// share the launches.  Nodes above the Jacobi limit are truncated by way of a
+// tridiagonal form (trunc_big); Cholesky factors above the shared-memory limit
+// are blocked (Exec::chol_inv_blocked).
 #include <algorithm>
 #include <cmath>
 #include <atomic>
@@ -369,7 +369,6 @@ template <typename T>
 struct CholBatch {
   std::vector<CholTask<T>> tasks;
   std::vector<Tag> what;
-  int max_m = 0;
   double flops = 0.0;
   void add(const T *A, int lda, T *Linv, int m, const Tag &w) {
     if (m <= 0) return;
@@ -382,7 +381,6 @@ struct CholBatch {
     t.status_idx = (int)tasks.size();
     tasks.push_back(t);
     what.push_back(w);
-    max_m = std::max(max_m, m);
     flops += 2.0 * (double)m * m * m / 3.0;
   }
 };
@@ -1569,7 +1567,6 @@ void Run<T>::end_level(const PlanLevel &lv, int li) {
     FlatMap<int> tix;
     std::vector<int> torder, c_t, c_node, c_col;
     int64_t t = 0;
-    wa.max_m = 0;
     for (int q = 0; q < wa.node_count; ++q, ++rp) {
       const Rec &rc = recs_[rp];
       ApplyNode &an = h_.nodes[rc.node];
@@ -1577,7 +1574,6 @@ void Run<T>::end_level(const PlanLevel &lv, int li) {
       an.xr = lv.red_made[rc.s] ? xoff(nsup + rc.s) : -1;
       an.toff = t;
       t += an.m;
-      wa.max_m = std::max(wa.max_m, an.m);
       an.nb_first = (int)h_.nbrs.size();
       an.nb_count = (int)rc.N.size();
       int col = 0;
@@ -1606,7 +1602,6 @@ void Run<T>::end_level(const PlanLevel &lv, int li) {
       std::vector<int> cur(c_start.begin(), c_start.end() - 1);
       for (size_t c = 0; c < c_t.size(); ++c) c_list[cur[c_t[c]]++] = (int)c;
     }
-    wa.tsize = t;
     h_.tmax = std::max(h_.tmax, t);
     std::vector<int> tsorted(torder.size());
     for (size_t x = 0; x < torder.size(); ++x) tsorted[x] = (int)x;
@@ -1634,11 +1629,6 @@ void Run<T>::end_level(const PlanLevel &lv, int li) {
     }
   }
   recs_.clear();
-  LevelApply la;
-  la.level = lv.level;
-  la.wave_first = wfirst;
-  la.wave_count = (int)lv.waves.size();
-  h_.levels.push_back(la);
   // parent level: red node nsup+i becomes red i
   FlatMap<BlockRef<T>> nb;
   nb.reserve(blocks_.size());
@@ -1671,7 +1661,6 @@ void Run<T>::begin() {
   h_.targets.clear();
   h_.contribs.clear();
   h_.waves.clear();
-  h_.levels.clear();
   h_.ranks.clear();
   h_.tmax = 0;
   leaf_setup();

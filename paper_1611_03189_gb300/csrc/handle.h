@@ -108,13 +108,7 @@ struct ApplyItem {
 struct WaveApply {
   int node_first, node_count;
   int tgt_first, tgt_count;
-  int max_m;
-  int64_t tsize;     // unknowns of t scratch used
   int f_first = 0, f_count = 0, b_first = 0, b_count = 0;   // items of the two launches
-};
-struct LevelApply {
-  int level;
-  int wave_first, wave_count;
 };
 
 // A recorded launch sequence (CUDA graph) of the solve.  key: the
@@ -164,7 +158,6 @@ struct FactorHandle {
   std::vector<ApplyTarget> targets;
   std::vector<ApplyContrib> contribs;
   std::vector<WaveApply> waves;        // in elimination order, levels L..2
-  std::vector<LevelApply> levels;      // levels L..2
   ApplyNode *d_nodes = nullptr;
   ApplyNbr *d_nbrs = nullptr;
   ApplyContrib *d_contribs = nullptr;

@@ -895,68 +895,55 @@ __global__ void __launch_bounds__(TRUNC_THREADS) k_trunc(const TruncTask<T> *__r
     return;
   }
   double lmax = 0.0;
-  if (eps > 0.0) {
-    jacobi_eig<T>(A, V, m, false, sh, max_sweeps);
-    for (int i = 0; i < m; ++i) lmax = fmax(lmax, (double)A[i * m + i]);
-    __syncthreads();
-  }
-  // ---- matrix whose leading eigenvectors give U_2: (I - U1 U1^T) G (I - U1 U1^T),
-  // or the projector I - U1 U1^T itself when eps == 0 (complete basis)
+  jacobi_eig<T>(A, V, m, false, sh, max_sweeps);
+  for (int i = 0; i < m; ++i) lmax = fmax(lmax, (double)A[i * m + i]);
+  __syncthreads();
+  // ---- matrix whose leading eigenvectors give U_2: (I - U1 U1^T) G (I - U1 U1^T)
   // X = G U1 (m x k1) in V's columns 0..k1-1 (scratch, ld m), all in T
-  if (eps > 0.0) {
-    for (int w = tid; w < m * k1; w += nt) {
-      const int i = w / k1, a = w % k1;
-      T s = T(0);
-      for (int j = 0; j < m; ++j) s = fma(t.G[(int64_t)i * m + j], t.U[(int64_t)j * m + a], s);
-      V[i * m + a] = s;
+  for (int w = tid; w < m * k1; w += nt) {
+    const int i = w / k1, a = w % k1;
+    T s = T(0);
+    for (int j = 0; j < m; ++j) s = fma(t.G[(int64_t)i * m + j], t.U[(int64_t)j * m + a], s);
+    V[i * m + a] = s;
+  }
+  __syncthreads();
+  // c = U1^T G U1 (k1 x k1, ld kMaxK1)
+  for (int a = 0; a < k1; ++a)
+    for (int b = 0; b < k1; ++b) {
+      double s = 0.0;
+      for (int i = tid; i < m; i += nt) s += (double)(t.U[(int64_t)i * m + a] * V[i * m + b]);
+      const T cab = (T)block_sum<T>(s, red);
+      if (tid == 0) s_c[a * kMaxK1 + b] = cab;
     }
-    __syncthreads();
-    // c = U1^T G U1 (k1 x k1, ld kMaxK1)
-    for (int a = 0; a < k1; ++a)
-      for (int b = 0; b < k1; ++b) {
-        double s = 0.0;
-        for (int i = tid; i < m; i += nt) s += (double)(t.U[(int64_t)i * m + a] * V[i * m + b]);
-        const T cab = (T)block_sum<T>(s, red);
-        if (tid == 0) s_c[a * kMaxK1 + b] = cab;
+  __syncthreads();
+  if (k1 <= 2) {
+    // one or two basis vectors (one preserved vector): c in registers
+    T c[2][2];
+    for (int a = 0; a < 2; ++a)
+      for (int b = 0; b < 2; ++b) c[a][b] = (a < k1 && b < k1) ? s_c[a * kMaxK1 + b] : T(0);
+    for (int64_t e = tid; e < (int64_t)m * m; e += nt) {
+      const int i = (int)(e / m), j = (int)(e % m);
+      T v = t.G[e];
+      for (int a = 0; a < k1; ++a) {
+        const T ui = t.U[(int64_t)i * m + a], uj = t.U[(int64_t)j * m + a];
+        v = fma(-ui, V[j * m + a], fma(-V[i * m + a], uj, v));
+        for (int b = 0; b < k1; ++b) v = fma(ui * c[a][b], t.U[(int64_t)j * m + b], v);
       }
-    __syncthreads();
-    if (k1 <= 2) {
-      // one or two basis vectors (one preserved vector): c in registers
-      T c[2][2];
-      for (int a = 0; a < 2; ++a)
-        for (int b = 0; b < 2; ++b) c[a][b] = (a < k1 && b < k1) ? s_c[a * kMaxK1 + b] : T(0);
-      for (int64_t e = tid; e < (int64_t)m * m; e += nt) {
-        const int i = (int)(e / m), j = (int)(e % m);
-        T v = t.G[e];
-        for (int a = 0; a < k1; ++a) {
-          const T ui = t.U[(int64_t)i * m + a], uj = t.U[(int64_t)j * m + a];
-          v = fma(-ui, V[j * m + a], fma(-V[i * m + a], uj, v));
-          for (int b = 0; b < k1; ++b) v = fma(ui * c[a][b], t.U[(int64_t)j * m + b], v);
-        }
-        A[e] = f(v);
-      }
-    } else {
-      for (int64_t e = tid; e < (int64_t)m * m; e += nt) {
-        const int i = (int)(e / m), j = (int)(e % m);
-        T v = t.G[e];
-        for (int a = 0; a < k1; ++a) {
-          const T ui = t.U[(int64_t)i * m + a], uj = t.U[(int64_t)j * m + a];
-          v = fma(-ui, V[j * m + a], fma(-V[i * m + a], uj, v));
-          for (int b = 0; b < k1; ++b) v = fma(ui * s_c[a * kMaxK1 + b], t.U[(int64_t)j * m + b], v);
-        }
-        A[e] = f(v);
-      }
+      A[e] = f(v);
     }
-    thr = eps * eps * lmax;
   } else {
     for (int64_t e = tid; e < (int64_t)m * m; e += nt) {
       const int i = (int)(e / m), j = (int)(e % m);
-      double v = (i == j) ? 1.0 : 0.0;
-      for (int a = 0; a < k1; ++a) v -= (double)t.U[(int64_t)i * m + a] * (double)t.U[(int64_t)j * m + a];
-      A[e] = (T)v;
+      T v = t.G[e];
+      for (int a = 0; a < k1; ++a) {
+        const T ui = t.U[(int64_t)i * m + a], uj = t.U[(int64_t)j * m + a];
+        v = fma(-ui, V[j * m + a], fma(-V[i * m + a], uj, v));
+        for (int b = 0; b < k1; ++b) v = fma(ui * s_c[a * kMaxK1 + b], t.U[(int64_t)j * m + b], v);
+      }
+      A[e] = f(v);
     }
-    thr = 0.5;
   }
+  thr = eps * eps * lmax;
   __syncthreads();
   jacobi_eig<T>(A, V, m, true, sh, max_sweeps);
   const int k2 = select_columns<T>(A, V, m, thr, t.U, k1, red);

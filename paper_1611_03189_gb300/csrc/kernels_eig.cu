@@ -1147,9 +1147,8 @@ __global__ void __launch_bounds__(kTriRows * 32) k_tri_symv(const GridTri<T> *__
   }
 }
 
-// The same products for nodes too large for a warp's registers (m > qmul_max), one CTA
-// per batch of columns held in
-// shared memory: for each reflector the block forms all the batch's dot
+// The same products for nodes too large for a warp's registers (m > kQmulMax), one CTA
+// per batch of columns held in shared memory: for each reflector the block forms all the batch's dot
 // products (fixed-order reduction), then updates the columns.
 constexpr int RT = 256;
 constexpr int RNB = 16;   // most columns per task
