@@ -218,6 +218,8 @@ void launch_trunc(const TruncTask<T> *d_tasks, int ntasks, int *d_k, int variant
 //   SC          scalars passed between the kernels: k1, k2 (ints), the norm
 //               bound of T, C = U1^T G U1 (kMaxK1 x kMaxK1 doubles), and
 //               eps^2 lambda_max, the Gershgorin bound of T, max e^2
+// (J, X, C and all that follows from them: of G times a power of two that brings its
+// largest diagonal entry near 1, k_trunc_prep)
 template <typename T>
 struct BigLayout {
   T *A, *Y, *LS;
